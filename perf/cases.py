@@ -122,15 +122,21 @@ def _empty(*shape, dtype=torch.bfloat16):
 
 # ------------------------------------------------------------------------------------------------ the kinds
 
+def _inputs_train_block(c, gen):
+    """X, W and dY of every linear, then the block outputs, in the order of the step's buffers."""
+    cfg, M = synth.CONFIGS[c["cfg"]], c["M"]
+    for l in cfg.linears:
+        yield _activation(gen, (M, l.K), cfg.x_kind)
+        yield _normal(gen, (l.N, l.K), 0.02)
+        yield _normal(gen, (M, l.N), 1e-3)
+    for _ in range(cfg.n_blocks):
+        yield _activation(gen, (M, cfg.d), cfg.x_kind)
+
+
 def _prepare_train_block(c, gen):
     b = BlockStep(c["cfg"], M=c["M"], variant=c["variant"])
-    kind = b.cfg.x_kind
-    for lb in b.linears:
-        lb.x.copy_(_activation(gen, lb.x.shape, kind))
-        lb.w.copy_(_normal(gen, lb.w.shape, 0.02))
-        lb.dy.copy_(_normal(gen, lb.dy.shape, 1e-3))
-    for a in b.a:
-        a.copy_(_activation(gen, a.shape, kind))
+    for t, v in zip([t for lb in b.linears for t in (lb.x, lb.w, lb.dy)] + b.a, _inputs_train_block(c, gen)):
+        t.copy_(v)
     if c["variant"] == "fused":        # the amax histories of a step that has run before
         b.step()
         b.step()
@@ -157,10 +163,15 @@ def _work_train_block(c):
     return {"bytes": byt, "flops": sum(6 * M * l.K * l.N for l in cfg.linears)}
 
 
+def _inputs_train_linear(c, gen):
+    M, K, N = c["M"], c["K"], c["N"]
+    return {"x": _activation(gen, (M, K), "outlier_entries"), "w": _normal(gen, (N, K), 0.02), "dy": _normal(gen, (M, N), 1e-3),
+            "a": _activation(gen, (M, K), "outlier_entries")}
+
+
 def _prepare_train_linear(c, gen):
     M, K, N = c["M"], c["K"], c["N"]
-    s = {"x": _activation(gen, (M, K), "outlier_entries"), "w": _normal(gen, (N, K), 0.02), "dy": _normal(gen, (M, N), 1e-3),
-         "a": _activation(gen, (M, K), "outlier_entries"), "y": _empty(M, N), "dx": _empty(M, K), "g": [_empty(M, K)],
+    s = {**_inputs_train_linear(c, gen), "y": _empty(M, N), "dx": _empty(M, K), "g": [_empty(M, K)],
          "f32": c["dw"] != "bf16"}
     s["dw"] = torch.zeros((N, K), dtype=torch.float32 if s["f32"] else torch.bfloat16, device="cuda")
     sc = torch.ones(9, dtype=torch.float32, device="cuda")
@@ -191,13 +202,20 @@ def _work_train_linear(c):
             "flops": 6 * M * K * N}
 
 
-def _prepare_block_fwd(c, gen):
+def _inputs_block_fwd(c, gen):
     M, d, ff = c["M"], c["d"], c["ff"]
     rows = 2 * ff if c["act"] == "swiglu" else ff
-    s = {"x": _activation(gen, (M, d)), "gamma": 1.0 + 0.1 * torch.randn(d, device="cuda", generator=gen),
-         "beta": None if c["norm"] == "rms" else 0.1 * torch.randn(d, device="cuda", generator=gen),
+    return {"x": _activation(gen, (M, d)), "gamma": 1.0 + 0.1 * torch.randn(d, device="cuda", generator=gen),
+            "beta": None if c["norm"] == "rms" else 0.1 * torch.randn(d, device="cuda", generator=gen),
+            "w1": _normal(gen, (rows, d), 0.02), "w2": _normal(gen, (d, ff), 0.02)}
+
+
+def _prepare_block_fwd(c, gen):
+    M, d, ff = c["M"], c["d"], c["ff"]
+    i = _inputs_block_fwd(c, gen)
+    s = {"x": i["x"], "gamma": i["gamma"], "beta": i["beta"],
          "norm": tw.NORM_RMS if c["norm"] == "rms" else tw.NORM_LAYER, "act": ACTS[c["act"]],
-         "w1": tw.quantize_per_tensor(_normal(gen, (rows, d), 0.02)), "w2": tw.quantize_per_tensor(_normal(gen, (d, ff), 0.02)),
+         "w1": tw.quantize_per_tensor(i["w1"]), "w2": tw.quantize_per_tensor(i["w2"]),
          "s_n": _scale(6.0), "s_h": _scale(4.0), "s_a": _scale(8.0), "amax_h": torch.zeros(1, device="cuda"),
          "nq": _empty(M, d, dtype=torch.uint8), "hq": _empty(M, ff, dtype=torch.uint8), "f": _empty(M, d), "a": _empty(M, d),
          "grad": _empty(M, d), "aq": _empty(M, d, dtype=torch.uint8), "ws": tw.new_workspace(tw.OP_LINEAR_FWD),
@@ -225,11 +243,18 @@ def _work_block_fwd(c):
     return {"bytes": 2 * M * d + (rows + ff) * d + M * d + M * ff + 7 * M * d, "flops": 2 * M * d * (rows + ff)}
 
 
+def _inputs_w8a8(c, gen):
+    M, K, N = c["M"], c["K"], c["N"]
+    w = _normal(gen, (N, K), 0.02)
+    sx = _scale(float(_normal(gen, (1024, K)).abs().max()))   # calibration
+    return _normal(gen, (M, K)), w, sx
+
+
 def _prepare_w8a8(c, gen):
     M, K, N = c["M"], c["K"], c["N"]
-    wq = tw.quantize_per_tensor(_normal(gen, (N, K), 0.02))
-    amax = float(_normal(gen, (1024, K)).abs().max())   # calibration
-    return {"x": _normal(gen, (M, K)), "sx": _scale(amax), "w": wq.q, "sw_inv": wq.scale_inv, "y": _empty(M, N),
+    x, w, sx = _inputs_w8a8(c, gen)
+    wq = tw.quantize_per_tensor(w)
+    return {"x": x, "sx": sx, "w": wq.q, "sw_inv": wq.scale_inv, "y": _empty(M, N),
             "ws": tw.new_workspace(tw.OP_W8A8, M, N, K)}
 
 
@@ -242,11 +267,18 @@ def _work_w8a8(c):
     return {"bytes": 2 * M * K + N * K + 2 * M * N, "flops": 2 * M * K * N}
 
 
+def _inputs_int8_token(c, gen):
+    M, K, N = c["M"], c["K"], c["N"]
+    w, r = _normal(gen, (N, K), 0.02), _normal(gen, (M, N))
+    return _normal(gen, (M, K)), w, r
+
+
 def _prepare_int8_token(c, gen):
     M, K, N = c["M"], c["K"], c["N"]
-    wq, sw = tw.absmax_quantize(_normal(gen, (N, K), 0.02), granularity=tw.GRAN_ROW)
-    rq, rs = tw.absmax_quantize(_normal(gen, (M, N)), granularity=tw.GRAN_ROW)
-    return {"x": _normal(gen, (M, K)), "wq": wq, "sw": sw, "rq": rq, "rs": rs, "y": _empty(M, N),
+    x, w, r = _inputs_int8_token(c, gen)
+    wq, sw = tw.absmax_quantize(w, granularity=tw.GRAN_ROW)
+    rq, rs = tw.absmax_quantize(r, granularity=tw.GRAN_ROW)
+    return {"x": x, "wq": wq, "sw": sw, "rq": rq, "rs": rs, "y": _empty(M, N),
             "out": _empty(M, N, dtype=torch.int8)}
 
 
@@ -263,11 +295,16 @@ def _work_int8_token(c):
     return {"bytes": 3 * M * K + N * K + 2 * M * N + 3 * M * N, "flops": 2 * M * K * N}
 
 
+def _inputs_w4(c, gen):
+    M, K, N = c["M"], c["K"], c["N"]
+    w, x = _normal(gen, (N, K), 0.02), _normal(gen, (M, K))
+    return x, w, _scale(float(_normal(gen, (1024, K)).abs().max()))
+
+
 def _prepare_w4(c, gen):
     M, K, N = c["M"], c["K"], c["N"]
-    w = tw.fp4_quantize(_normal(gen, (N, K), 0.02), carriers=False)
-    x = _normal(gen, (M, K))
-    sx = _scale(float(_normal(gen, (1024, K)).abs().max()))
+    x, w, sx = _inputs_w4(c, gen)
+    w = tw.fp4_quantize(w, carriers=False)
     sc = torch.empty(2, dtype=torch.float32, device="cuda")
     return {"x": x, "sx": sx, "w4": w.q4.view(N, K // 2), "sw_inv": w.scale_inv, "y": _empty(M, N),
             "q": tw.Quantized(_empty(M, K, dtype=torch.uint8), sx, sc[0:1], sc[1:2], None, tw.E4M3)}
@@ -283,12 +320,127 @@ def _work_w4(c):
     return {"bytes": 2 * M * K + N * K // 2 + 2 * M * N, "flops": 2 * M * K * N}
 
 
-_KINDS = {"train_block": (_prepare_train_block, _run_train_block, _work_train_block),
-          "train_linear": (_prepare_train_linear, _run_train_linear, _work_train_linear),
-          "block_fwd": (_prepare_block_fwd, _run_block_fwd, _work_block_fwd),
-          "w8a8": (_prepare_w8a8, _run_w8a8, _work_w8a8),
-          "int8_token": (_prepare_int8_token, _run_int8_token, _work_int8_token),
-          "w4": (_prepare_w4, _run_w4, _work_w4)}
+# ------------------------------------------------------------------------------------------------ 64-bit results
+
+# The codes, the scales and the roundings to bf16 that a later operation reads are part of what a pass is defined to do
+# (a binary32 multiplication by the scale, one rounding); everything between them is taken in binary64.  Codes have no
+# value of their own here: None.
+
+_GRID = {tw.E4M3: (448.0, torch.float8_e4m3fn), tw.E5M2: (57344.0, torch.float8_e5m2)}
+
+
+def _bf16(x):
+    return x.to(torch.bfloat16)
+
+
+def _over(top, x):
+    """top / x in binary32, rounded once (a Python number over a tensor is a reciprocal and a product)."""
+    return torch.full_like(x, top) / x
+
+
+def _fp8(x, fmt=tw.E4M3, scale=None):
+    """The dequantised FP8 values of a bf16 tensor, and its largest magnitude; `scale`: given, else the current one."""
+    top, dtype = _GRID[fmt]
+    amax = x.abs().max().float().view(1)
+    scale = _over(top, amax) if scale is None else scale
+    q = (x.float() * scale).clamp_(-top, top).to(dtype)
+    return q.double() * _over(1.0, scale).double(), amax
+
+
+def _absmax_rows(x):
+    """Codes and scales of Eq. 4 with one scale per row; x in binary32 or bf16."""
+    s = x.abs().amax(dim=1).float() + 1e-6
+    return (x.float() * _over(127.0, s)[:, None]).round_().clamp_(-127, 127).double(), s
+
+
+def _penalty(a, c, tau=3.0, eps=1e-6, p=4.0):
+    a, d = a.double(), tau + eps
+    return (a.abs() / d).pow(p).mean().view(1), c * p * a.sign() * a.abs().pow(p - 1) / (a.numel() * d ** p)
+
+
+def _exact_train_block(c, gen):
+    cfg = synth.CONFIGS[c["cfg"]]
+    inputs, L = list(_inputs_train_block(c, gen)), cfg.n_blocks
+    linears, amax_e, amax_g, n = [], [], [], len(cfg.linears)
+    for i in range(n):
+        x, w, dy = inputs[3 * i:3 * i + 3]
+        (xv, ax), (wv, aw), (dv, ad) = _fp8(x), _fp8(w), _fp8(dy, tw.E5M2)
+        y, dx, dw = xv @ wv.T, dv @ wv, dv.T @ xv
+        linears.append((y, dx, dw))
+        if c["variant"] == "fused":   # of the step before the first scales were known, and of every later one
+            one = x.new_ones(1, dtype=torch.float32)
+            x1, w1, d1 = _fp8(x, tw.E4M3, one)[0], _fp8(w, tw.E4M3, one)[0], _fp8(dy, tw.E5M2, one)[0]
+            y1, dx1 = (float(_bf16(t).abs().max()) for t in (x1 @ w1.T, d1 @ w1))
+            amax_e.append([(float(ax),) * 3, (float(aw),) * 3, (float(_bf16(y).abs().max()),) * 2 + (y1,)])
+            amax_g.append([(float(ad),) * 3, (float(_bf16(dx).abs().max()),) * 2 + (dx1,)])
+    terms = [_penalty(a, 0.01 / L) for a in inputs[3 * n:]]
+    per_block = torch.cat([t[0] for t in terms])
+    out = {"loss": per_block.mean().view(1), "loss_per_block": per_block, "grad": [t[1] for t in terms], "linears": linears}
+    if c["variant"] == "fused":
+        groups = []
+        for amax, fmt in ((amax_e, tw.E4M3), (amax_g, tw.E5M2)):
+            hist = torch.tensor([linear[k] for k in range(len(amax[0])) for linear in amax], dtype=torch.float64, device="cuda")
+            groups.append((_GRID[fmt][0] / hist.amax(dim=1), torch.cat([hist, hist.new_zeros(len(hist), 13)], dim=1)))
+        out["scales"] = (groups[0][0], groups[1][0], groups[0][1], groups[1][1])
+    return out
+
+
+def _exact_train_linear(c, gen):
+    i = _inputs_train_linear(c, gen)
+    (xv, ax), (wv, aw), (dv, ad) = _fp8(i["x"]), _fp8(i["w"]), _fp8(i["dy"], tw.E5M2)
+    loss, grad = _penalty(i["a"], 0.01)
+    return {"y": xv @ wv.T, "dx": dv @ wv, "dw": dv.T @ xv, "loss": loss, "grad": grad, "amax": [ax, aw, ad], "codes": None}
+
+
+def _exact_block_fwd(c, gen):
+    i = _inputs_block_fwd(c, gen)
+    x = i["x"].double()
+    mean = x.mean(dim=1, keepdim=True) if c["norm"] == "layer" else torch.zeros_like(x[:, :1])
+    rstd = ((x - mean).square().mean(dim=1, keepdim=True) + 1e-5).rsqrt()
+    n = (x - mean) * rstd * i["gamma"].double() + (0.0 if i["beta"] is None else i["beta"].double())
+    nv, amax_n = _fp8(_bf16(n), tw.E4M3, _scale(6.0))
+    h = nv @ _fp8(i["w1"])[0].T
+    if c["act"] == "swiglu":
+        h = torch.nn.functional.silu(h[:, :c["ff"]]) * h[:, c["ff"]:]
+    else:
+        h = torch.nn.functional.gelu(h, approximate="none" if c["act"] == "gelu" else "tanh")
+    hv, amax_h = _fp8(_bf16(h), tw.E4M3, _scale(4.0))
+    f = hv @ _fp8(i["w2"])[0].T
+    a = x + _bf16(f).double()
+    loss, grad = _penalty(_bf16(a), 0.01)
+    return {"normed": None, "mean": mean.view(-1), "rstd": rstd.view(-1), "hidden": None, "f": f, "a": a, "loss": loss,
+            "grad": grad, "aq": None, "amax": (amax_n, amax_h, _bf16(a).abs().max().view(1))}
+
+
+def _exact_w8a8(c, gen):
+    x, w, sx = _inputs_w8a8(c, gen)
+    return _fp8(x, tw.E4M3, sx)[0] @ _fp8(w)[0].T
+
+
+def _exact_int8_token(c, gen):
+    x, w, r = _inputs_int8_token(c, gen)
+    (xq, sx), (wq, sw), (rq, sr) = _absmax_rows(x), _absmax_rows(w), _absmax_rows(r)
+    f = (xq @ wq.T) * (sx.double()[:, None] / 127) * (sw.double() / 127)
+    fq, sf = _absmax_rows(_bf16(f))
+    y = fq * (sf.double()[:, None] / 127) + rq * (sr.double()[:, None] / 127)
+    return {"xq": None, "sx": x.double().abs().amax(dim=1) + 1e-6, "f": f, "fq": None,
+            "sf": _bf16(f).double().abs().amax(dim=1) + 1e-6, "yq": None, "sy": y.abs().amax(dim=1) + 1e-6}
+
+
+def _exact_w4(c, gen):
+    x, w, sx = _inputs_w4(c, gen)
+    s = _over(6.0, w.abs().max().float())
+    v = (w.float() * s).clamp_(-6.0, 6.0)
+    step = torch.where(v.abs() < 2, 0.5, torch.where(v.abs() < 4, 1.0, 2.0))   # E2M1: 0 0.5 1 1.5 2 3 4 6
+    return _fp8(x, tw.E4M3, sx)[0] @ (((v / step).round_() * step).double() * _over(1.0, s).double()).T
+
+
+_KINDS = {"train_block": (_prepare_train_block, _run_train_block, _work_train_block, _exact_train_block),
+          "train_linear": (_prepare_train_linear, _run_train_linear, _work_train_linear, _exact_train_linear),
+          "block_fwd": (_prepare_block_fwd, _run_block_fwd, _work_block_fwd, _exact_block_fwd),
+          "w8a8": (_prepare_w8a8, _run_w8a8, _work_w8a8, _exact_w8a8),
+          "int8_token": (_prepare_int8_token, _run_int8_token, _work_int8_token, _exact_int8_token),
+          "w4": (_prepare_w4, _run_w4, _work_w4, _exact_w4)}
 
 
 def prepare(case, seed):
@@ -302,6 +454,11 @@ def run(state):
 
 def work(case):
     return _KINDS[case["kind"]][2](case)
+
+
+def exact(case, seed):
+    gen = torch.Generator(device="cuda").manual_seed(int(seed))
+    return _KINDS[case["kind"]][3](case, gen)
 
 
 def tolerance(case):
