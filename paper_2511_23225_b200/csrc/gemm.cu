@@ -633,13 +633,13 @@ tweo_status_t launch_pair_act_cfg(const CUtensorMap& ma, const CUtensorMap& mb, 
 //   [8192x768].[2304x768]^T    (8,4,2) 19.3  (4,5,2) 19.1  (8,5,1) 18.3  (4,6,1) 20.7
 //   [16384x2048].[6144x2048]^T (8,4,2) 169.6 (4,5,2) 158.7 (8,5,1) 161.9 (4,6,1) 156.9
 // Short contractions are bound by the epilogue's issue rate (eight warps), long ones by the main loop, which
-// wants the deepest operand ring; one staging buffer per warp pays for the extra stage in both.
+// wants the deepest operand ring; one staging buffer per warp pays for the extra stage in both.  SwiGLU, FP8 copy and
+// amax, [16384x768].[6144x768]^T: (4,6,1) 95.9, (8,5,1) 73.4.
 template <int ACT, bool B_MN = false>
 tweo_status_t launch_pair_act(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& md,
                               const CUtensorMap& mq, GemmParams& p, cudaStream_t st) {
-  if (ACT == 3 || (p.Kc + BK - 1) / BK >= 16)          // SwiGLU (238 registers) always takes four warps
-    return launch_pair_act_cfg<ACT, B_MN, 4, 6, 1>(ma, mb, md, mq, p, st);
-  return launch_pair_act_cfg<(ACT == 3 ? 0 : ACT), B_MN, 8, 5, 1>(ma, mb, md, mq, p, st);
+  if ((p.Kc + BK - 1) / BK >= 16) return launch_pair_act_cfg<ACT, B_MN, 4, 6, 1>(ma, mb, md, mq, p, st);
+  return launch_pair_act_cfg<ACT, B_MN, 8, 5, 1>(ma, mb, md, mq, p, st);
 }
 
 // D[M,N] = A[M,K] . B with A stored [M,K]; B stored [N,K] (w_mn false: the forward product) or [K,N] (w_mn

@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "common.cuh"
+#include "tc_ptx.cuh"
 
 namespace tweo_detail {
 
@@ -125,43 +126,133 @@ __device__ __forceinline__ uint32_t quant4(float a, float b, float c, float d) {
   return cvt_fp8x2<FMT>(a, b) | (cvt_fp8x2<FMT>(c, d) << 16);
 }
 
-// Four bf16 values (two packed words) times the scale -> four FP8 codes.
+// Four bf16 values (two packed words) times the scale (both lanes of qs2) -> four FP8 codes.
 template <int FMT>
-__device__ __forceinline__ uint32_t quant_words(uint32_t w0, uint32_t w1, float qs) {
-  return quant4<FMT>(__fmul_rn(bf16lo_to_f32(w0), qs), __fmul_rn(bf16hi_to_f32(w0), qs),
-                     __fmul_rn(bf16lo_to_f32(w1), qs), __fmul_rn(bf16hi_to_f32(w1), qs));
+__device__ __forceinline__ uint32_t quant_words(uint32_t w0, uint32_t w1, uint64_t qs2) {
+  float a, b, c, d;
+  unpack_f32x2(mul_f32x2(bf16x2_to_f32x2(w0), qs2), a, b);
+  unpack_f32x2(mul_f32x2(bf16x2_to_f32x2(w1), qs2), c, d);
+  return quant4<FMT>(a, b, c, d);
+}
+
+// A row of 64 bf16 values (packed words) times the scale -> 64 codes at shared address `qrow`, in four 16-byte pieces
+// whose positions are XORed with `qswz` (the 64-byte swizzle of the store's tensor map).
+template <int FMT>
+__device__ __forceinline__ void stage_codes_fmt(uint32_t qrow, uint32_t qswz, const uint32_t (&packed)[32], uint64_t qs2) {
+#pragma unroll
+  for (int g4 = 0; g4 < 4; ++g4) {
+    uint32_t q[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) q[j] = quant_words<FMT>(packed[8 * g4 + 2 * j], packed[8 * g4 + 2 * j + 1], qs2);
+    st_shared_v4(qrow + (((uint32_t)g4 ^ qswz) << 4), q[0], q[1], q[2], q[3]);
+  }
+}
+__device__ __forceinline__ void stage_codes(int fmt, uint32_t qrow, uint32_t qswz, const uint32_t (&packed)[32], uint64_t qs2) {
+  if (fmt == TWEO_E4M3) stage_codes_fmt<TWEO_E4M3>(qrow, qswz, packed, qs2);
+  else stage_codes_fmt<TWEO_E5M2>(qrow, qswz, packed, qs2);
 }
 
 // MLP activations of the forward epilogue (Sec. 3.2: GELU in the classic MLP, a gated unit in the
-// Llama-style one), on binary32 values.
+// Llama-style one), on pairs of binary32 values: one packed instruction per pair wherever the operation has one.
 // 1: v * Phi(v).  Phi from the rational approximation of erfc by Hastings (Abramowitz & Stegun
 //    7.1.26): erfc(x) = t (a1 + t (a2 + t (a3 + t (a4 + t a5)))) exp(-x^2), t = 1 / (1 + p x), x >= 0,
-//    absolute error below 1.5e-7 -- three orders below the bf16 rounding that follows.
+//    absolute error below 1.5e-7 -- three orders below the bf16 rounding that follows.  With h = erfc(|v|/sqrt 2) / 2
+//    the result is max(v, 0) - |v| h for either sign: one rounding, no select.
 // 2: the tanh form with the hardware tanh (relative error 2^-11).
+// What bounds the kernels that use them, at short contractions: the issue slots and the latencies of the epilogue.
+// Scalar arithmetic (with the scaling for denormals of exp and of the division, which no argument here needs: results
+// of exp below 2^-126 vanish in the sum, the divisors lie in [1, 16]) took 31 warp instructions per element for the
+// erf form and 14 000 cycles per 256x256 tile, against 4 300 of the main loop at contraction 768; the packed form takes
+// 17, and eight pairs go through stage by stage, because a warp shares its scheduler with only one other and has to
+// cover its own latencies (two thirds of the stalls of the first packed version were waits for a result of the chain).
+// [12608x768].[3072x768]^T, amax and FP8 copy, microseconds: erf 74.3 scalar, 59.4 packed, 46.3 staged; tanh 45.6,
+// 39.3, 34.6; without an activation 35.
+__device__ __forceinline__ float ex2_ftz(float x) {
+  float r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float rcp_ftz(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+// the larger operand; a NaN operand gives NaN
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+
+constexpr int kActPairs = 8;
 template <int ACT>
-__device__ __forceinline__ float act_apply(float v) {
+__device__ __forceinline__ void act_pairs(uint64_t (&v)[kActPairs]) {
   if (ACT == 1) {
-    const float x = fabsf(v) * 0.70710678118654752f;
-    const float t = __fdividef(1.0f, fmaf(0.3275911f, x, 1.0f));
-    float poly = fmaf(t, 1.061405429f, -1.453152027f);
-    poly = fmaf(t, poly, 1.421413741f);
-    poly = fmaf(t, poly, -0.284496736f);
-    poly = fmaf(t, poly, 0.254829592f);
-    const float half_erfc = 0.5f * t * poly * __expf(-x * x);   // Phi(-|v|)
-    return v * (v >= 0.0f ? 1.0f - half_erfc : half_erfc);
+    uint64_t n[kActPairs], t[kActPairs], e[kActPairs], q[kActPairs];
+#pragma unroll
+    for (int i = 0; i < kActPairs; ++i) {
+      float v0, v1;
+      unpack_f32x2(v[i], v0, v1);
+      // -|v|, held above -64 (erfc vanishes long before): infinity times zero must not arise below
+      n[i] = pack_f32x2(max_nan(-fabsf(v0), -64.0f), max_nan(-fabsf(v1), -64.0f));
+      v[i] = pack_f32x2(max_nan(v0, -0.0f), max_nan(v1, -0.0f));
+    }
+#pragma unroll
+    for (int i = 0; i < kActPairs; ++i) {
+      t[i] = fma_f32x2(n[i], splat_f32x2(-0.23164187f), splat_f32x2(1.0f));   // 1 + p |v| / sqrt 2
+      e[i] = mul_f32x2(n[i], splat_f32x2(-0.72134752f));
+    }
+#pragma unroll
+    for (int i = 0; i < kActPairs; ++i) {
+      float d0, d1;
+      unpack_f32x2(t[i], d0, d1);
+      t[i] = pack_f32x2(rcp_ftz(d0), rcp_ftz(d1));
+      e[i] = mul_f32x2(e[i], n[i]);                                           // -v^2 / 2 in units of ln 2
+    }
+#pragma unroll
+    for (int i = 0; i < kActPairs; ++i) {
+      float d0, d1;
+      unpack_f32x2(e[i], d0, d1);
+      e[i] = pack_f32x2(ex2_ftz(d0), ex2_ftz(d1));
+      q[i] = fma_f32x2(t[i], splat_f32x2(0.5307027145f), splat_f32x2(-0.7265760135f));   // a5/2, a4/2, ...
+    }
+#pragma unroll
+    for (int i = 0; i < kActPairs; ++i) q[i] = fma_f32x2(t[i], q[i], splat_f32x2(0.7107068705f));
+#pragma unroll
+    for (int i = 0; i < kActPairs; ++i) q[i] = fma_f32x2(t[i], q[i], splat_f32x2(-0.142248368f));
+#pragma unroll
+    for (int i = 0; i < kActPairs; ++i) q[i] = fma_f32x2(t[i], q[i], splat_f32x2(0.127414796f));
+#pragma unroll
+    for (int i = 0; i < kActPairs; ++i) q[i] = mul_f32x2(t[i], q[i]);
+#pragma unroll
+    for (int i = 0; i < kActPairs; ++i) v[i] = fma_f32x2(mul_f32x2(q[i], e[i]), n[i], v[i]);   // - |v| Phi(-|v|)
+  } else if (ACT == 2) {
+    uint64_t c[kActPairs];
+#pragma unroll
+    for (int i = 0; i < kActPairs; ++i)
+      c[i] = fma_f32x2(mul_f32x2(v[i], splat_f32x2(0.044715f)), mul_f32x2(v[i], v[i]), v[i]);
+#pragma unroll
+    for (int i = 0; i < kActPairs; ++i) {
+      float u0, u1, t0, t1;
+      unpack_f32x2(mul_f32x2(c[i], splat_f32x2(0.79788456080286536f)), u0, u1);
+      asm("tanh.approx.f32 %0, %1;" : "=f"(t0) : "f"(u0));
+      asm("tanh.approx.f32 %0, %1;" : "=f"(t1) : "f"(u1));
+      c[i] = pack_f32x2(t0, t1);
+    }
+#pragma unroll
+    for (int i = 0; i < kActPairs; ++i) {
+      const uint64_t h = mul_f32x2(v[i], splat_f32x2(0.5f));
+      v[i] = fma_f32x2(h, c[i], h);
+    }
   }
-  if (ACT == 2) {
-    const float u = 0.79788456080286536f * fmaf(0.044715f * v * v, v, v);
-    float t;
-    asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(u));
-    const float h = 0.5f * v;
-    return fmaf(h, t, h);
-  }
-  return v;
 }
 // SiLU(gate) * up = gate * up / (1 + exp(-gate))
-__device__ __forceinline__ float swiglu(float gate, float up) {
-  return __fdividef(gate, 1.0f + __expf(-gate)) * up;
+__device__ __forceinline__ uint64_t swiglu_pair(uint64_t gate, uint64_t up) {
+  float e0, e1;
+  unpack_f32x2(mul_f32x2(gate, splat_f32x2(-1.44269504f)), e0, e1);
+  e0 = rcp_ftz(1.0f + ex2_ftz(e0));   // 0 once the sum passes 2^126
+  e1 = rcp_ftz(1.0f + ex2_ftz(e1));
+  return mul_f32x2(mul_f32x2(gate, pack_f32x2(e0, e1)), up);
 }
 
 }  // namespace tweo_detail

@@ -182,6 +182,7 @@ gemm_fp8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
     const int quarter = warp & 3;
     const float alpha = I8 ? 1.0f : dequant_alpha(p.sa_inv, p.sb_inv, p.sa_is_scale);
     const float qs = p.out_q ? (Q8 ? __fdiv_rn(p.q8_qmax, __ldg(p.q_scale)) : __ldg(p.q_scale)) : 0.0f;
+    const uint64_t alpha2 = splat_f32x2(alpha), qs2 = splat_f32x2(qs);
     constexpr int CH = OUT_F32 ? 32 : 64;
     const uint32_t epi_base = smem_u32(epi_smem) + (uint32_t)(warp - 2) * (uint32_t)EBUF * EPI_BUF;
     const uint32_t q_base = smem_u32(epi_smem) + EPI_BYTES + (uint32_t)(warp - 2) * (uint32_t)EBUF * Q_BUF;
@@ -241,9 +242,14 @@ gemm_fp8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
             tmem_ld32(taddr + 128 + 32 * h, u);
             tmem_ld_wait();
 #pragma unroll
-            for (int j = 0; j < 32; ++j)
-              r[32 * h + j] = __float_as_uint(swiglu(__fmul_rn(__uint_as_float(r[32 * h + j]), alpha),
-                                                     __fmul_rn(__uint_as_float(u[j]), alpha)));
+            for (int j = 0; j < 32; j += 2) {
+              const uint64_t gate = pack_f32x2(__uint_as_float(r[32 * h + j]), __uint_as_float(r[32 * h + j + 1]));
+              const uint64_t up = pack_f32x2(__uint_as_float(u[j]), __uint_as_float(u[j + 1]));
+              float v0, v1;
+              unpack_f32x2(swiglu_pair(mul_f32x2(gate, alpha2), mul_f32x2(up, alpha2)), v0, v1);
+              r[32 * h + j] = __float_as_uint(v0);
+              r[32 * h + j + 1] = __float_as_uint(v1);
+            }
           }
         }
         if (I8) {
@@ -271,8 +277,12 @@ gemm_fp8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
         }
         const uint32_t ebuf = EBUF == 2 ? (it & 1u) : 0u;
         const uint32_t buf = epi_base + ebuf * EPI_BUF;
-        if (lane == 0) bulk_wait_read<EBUF - 1>();
-        __syncwarp();
+        // the store that used this staging buffer last must have read it (waited for after the arithmetic)
+        auto buffer_free = [&]() {
+          if (lane == 0) bulk_wait_read<EBUF - 1>();
+          __syncwarp();
+        };
+        if (ACT == 0) buffer_free();
         if (Q8) {
           // Eq. 4 with the static output scale on the binary32 results: clamp(rne_int(y * (Q_b / s))), NaN -> 0
           const uint32_t qrow = q_base + ebuf * Q_BUF + (uint32_t)lane * 64u;
@@ -304,53 +314,48 @@ gemm_fp8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
         } else {
           uint32_t packed[CH / 2];
           const bool want_max = QST && p.out_amax != nullptr;
-          const bool whole = ACT != 3 || col0 + CH <= p.Nd;   // only a ragged SwiGLU chunk has live columns beyond Nd
-          if (ACT == 0 && want_max) {
+          if (ACT == 3 && col0 + CH > p.Nd) {   // a ragged SwiGLU chunk has live columns beyond Nd: not part of the maximum
+            if (want_max) {
+#pragma unroll
+              for (int j = 0; j < CH; ++j)
+                if (col0 + j < p.Nd) run_max = fmaxf(run_max, fabsf(__uint_as_float(r[j])));
+            }
+          } else if ((ACT == 0 || ACT == 3) && want_max) {
 #pragma unroll
             for (int j = 0; j < CH; ++j) run_max = fmaxf(run_max, fabsf(__uint_as_float(r[j])));
           }
+          constexpr int G = kActPairs;
 #pragma unroll
-          for (int j = 0; j < CH / 2; ++j) {
-            float v0, v1;
-            if (ACT == 3) {
-              v0 = __uint_as_float(r[2 * j]);
-              v1 = __uint_as_float(r[2 * j + 1]);
-            } else {
-              v0 = act_apply<ACT>(__fmul_rn(__uint_as_float(r[2 * j]), alpha));
-              v1 = act_apply<ACT>(__fmul_rn(__uint_as_float(r[2 * j + 1]), alpha));
+          for (int j0 = 0; j0 < CH / 2; j0 += G) {
+            uint64_t v[G];
+#pragma unroll
+            for (int i = 0; i < G; ++i) {
+              v[i] = pack_f32x2(__uint_as_float(r[2 * (j0 + i)]), __uint_as_float(r[2 * (j0 + i) + 1]));
+              if (ACT != 3) v[i] = mul_f32x2(v[i], alpha2);
             }
-            if (ACT != 0 && want_max) {
-              if (whole) {
-                run_max = fmaxf(run_max, fmaxf(fabsf(v0), fabsf(v1)));
-              } else {
-                if (col0 + 2 * j < p.Nd) run_max = fmaxf(run_max, fabsf(v0));
-                if (col0 + 2 * j + 1 < p.Nd) run_max = fmaxf(run_max, fabsf(v1));
-              }
+            if (ACT != 3) act_pairs<ACT>(v);
+#pragma unroll
+            for (int i = 0; i < G; ++i) {
+              float v0, v1;
+              unpack_f32x2(v[i], v0, v1);
+              if (ACT == 1 || ACT == 2) run_max = fmaxf(run_max, fmaxf(fabsf(v0), fabsf(v1)));
+              packed[j0 + i] = f32x2_to_bf16x2(v0, v1);
             }
-            packed[j] = f32x2_to_bf16x2(v0, v1);
           }
+          if (ACT != 0) buffer_free();
           if (ACT == 0 || p.d != nullptr) {
 #pragma unroll
             for (int j = 0; j < 8; ++j)
               st_shared_v4(buf + row_off + (((uint32_t)j ^ swz) << 4), packed[4 * j], packed[4 * j + 1],
                            packed[4 * j + 2], packed[4 * j + 3]);
           }
-          if (QST) {
+          if constexpr (QST && !OUT_F32) {
             if (p.out_q) {
               // 64 codes per row -> 32 rows x 64 B, 16-byte pieces XOR-swizzled with row bits 1-2
               const uint32_t qbuf = q_base + ebuf * Q_BUF;
               const uint32_t qrow = qbuf + (uint32_t)lane * 64u;
               const uint32_t qswz = ((uint32_t)lane >> 1) & 3u;
-#pragma unroll
-              for (int g4 = 0; g4 < 4; ++g4) {
-                uint32_t q[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                  const uint32_t w0 = packed[8 * g4 + 2 * j], w1 = packed[8 * g4 + 2 * j + 1];
-                  q[j] = p.q_fmt == TWEO_E4M3 ? quant_words<TWEO_E4M3>(w0, w1, qs) : quant_words<TWEO_E5M2>(w0, w1, qs);
-                }
-                st_shared_v4(qrow + (((uint32_t)g4 ^ qswz) << 4), q[0], q[1], q[2], q[3]);
-              }
+              stage_codes(p.q_fmt, qrow, qswz, packed, qs2);
             }
           }
           // (without QST the kernel has no fused outputs: the host sends those products to a QST instantiation)
