@@ -5,11 +5,13 @@
 // evaluated as X * (Q_b / s), one division per scale and one multiplication per element:
 //   s = fl32(amax + eps);  c = fl32(Q_b / s);  q = clamp(rne_int(fl32(x * c)), -Q_b, Q_b);  NaN -> 0.
 // HBM-bound streaming kernels: 16-byte loads of 8 bf16, 16-byte stores of 16 codes.
-//   per row   : one CTA per row (grid-stride over rows): maximum of the row, then the cast;
-//               the second read of the row comes from L1/L2.
+//   per row   : one CTA per row.  Rows of up to 8192 aligned elements stay in registers between the maximum and
+//               the cast (absmax_rows_reg_kernel); others are read twice, the second time from L1/L2.
 //   per tensor: kernel 1 writes per-CTA maxima to workspace slots, kernel 2 reduces them in
 //               every CTA and casts (no atomics, no reset kernel); static s skips kernel 1.
 #include <cuda_runtime.h>
+
+#include <algorithm>
 
 #include "common.cuh"
 
@@ -111,6 +113,120 @@ absmax_rows_kernel(const uint16_t* x, int64_t rows, int64_t cols, int64_t ldx, f
   }
 }
 
+// The same with the row held in registers: VPT vectors of 8 elements per thread (thread-interleaved), the block sized
+// to the row.  One read of x, and no conversion instruction: the unit that converts to integers does 16 a clock, 1.8 us
+// for 8 M elements.  With a finite row maximum no |x c| exceeds Q_b by more than one rounding, so the nearest integer
+// is read off the sum fl32(x c) + 1.5 2^23, whose low byte is the code (the addition rounds to nearest-even, as the
+// conversion does); rows with a NaN, an infinity or an infinite c take the converting path.  Launched in a chain, like
+// the residual addition below.  The per-token pass (quantise, integer linear, quantise, add) at 1999 tokens and
+// [4096x4096] went from 66.9 to 57.1 us with both, at 8192 tokens and [3072x5120] from 193.1 to 168.4.
+constexpr uint32_t kRoundMagicBits = 0x4B400000u;   // 1.5 * 2^23
+constexpr int64_t kRegRowCols = 8192;
+
+// Low bytes of four such sums -> one word of codes.
+__device__ __forceinline__ uint32_t pack_low_bytes(float a, float b, float c, float d) {
+  const uint32_t ab = __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x0040);
+  const uint32_t cd = __byte_perm(__float_as_uint(c), __float_as_uint(d), 0x0040);
+  return __byte_perm(ab, cd, 0x5410);
+}
+// four values (two pairs) times c, rounded to the nearest integers -> four codes.  Scalar instructions: a packed product
+// followed by a packed addition comes out of the assembler as one fused operation, which rounds differently at ties.
+__device__ __forceinline__ uint32_t quant4_magic(uint64_t v01, uint64_t v23, float c) {
+  const float magic = __uint_as_float(kRoundMagicBits);
+  float v[4];
+  unpack_f32x2(v01, v[0], v[1]);
+  unpack_f32x2(v23, v[2], v[3]);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) v[i] = __fadd_rn(__fmul_rn(v[i], c), magic);
+  return pack_low_bytes(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ uint32_t quant4_slow(const uint32_t w0, const uint32_t w1, float c, float Q) {
+  return (uint32_t)(quant1(bf16lo_to_f32(w0), c, Q) & 0xFF) | ((uint32_t)(quant1(bf16hi_to_f32(w0), c, Q) & 0xFF) << 8) |
+         ((uint32_t)(quant1(bf16lo_to_f32(w1), c, Q) & 0xFF) << 16) | ((uint32_t)(quant1(bf16hi_to_f32(w1), c, Q) & 0xFF) << 24);
+}
+// the maximum of m over the CTA (any number of warps up to 8)
+__device__ __forceinline__ uint32_t block_max_bits(uint32_t m, uint32_t* part) {
+  m = __reduce_max_sync(0xFFFFFFFFu, m);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = m;
+  __syncthreads();
+  const int warps = blockDim.x >> 5;
+  for (int w = 0; w < warps; ++w) m = max(m, part[w]);
+  return m;
+}
+
+template <int VPT>
+__global__ void __launch_bounds__(kThreads)
+absmax_rows_reg_kernel(const uint16_t* x, int64_t rows, int64_t cols, int64_t ldx, float eps, float Q, float* s_out, int8_t* q, int64_t ldq) {
+  __shared__ uint32_t part[kThreads / 32], part2[kThreads / 32];
+  chain_release();
+  chain_wait();
+  const int nvec = (int)(cols >> 3);
+  for (int64_t r = blockIdx.x; r < rows; r += gridDim.x) {   // one turn, unless there are more rows than a grid has CTAs
+  if (r != blockIdx.x) __syncthreads();                      // part[] may still be read from the turn before
+  const uint4* xv = reinterpret_cast<const uint4*>(x + r * ldx);
+  uint4 v[VPT];
+  uint32_t m2 = 0;   // two lanes: the largest sign-stripped patterns, NaN patterns included
+#pragma unroll
+  for (int i = 0; i < VPT; ++i) {
+    const int idx = threadIdx.x + i * blockDim.x;
+    v[i] = idx < nvec ? __ldg(xv + idx) : make_uint4(0u, 0u, 0u, 0u);
+  }
+#pragma unroll
+  for (int i = 0; i < VPT; ++i) {
+    m2 = __vmaxu2(m2, v[i].x & 0x7FFF7FFFu);
+    m2 = __vmaxu2(m2, v[i].y & 0x7FFF7FFFu);
+    m2 = __vmaxu2(m2, v[i].z & 0x7FFF7FFFu);
+    m2 = __vmaxu2(m2, v[i].w & 0x7FFF7FFFu);
+  }
+  uint32_t m = block_max_bits(absmax_fold(m2), part);
+  const bool finite = m < 0x7F80u;   // uniform over the CTA, as all that follows from m
+  if (!finite) {                     // NaN patterns do not count
+    m2 = 0;
+#pragma unroll
+    for (int i = 0; i < VPT; ++i) {
+      m2 = absmax_bits(m2, v[i].x);
+      m2 = absmax_bits(m2, v[i].y);
+      m2 = absmax_bits(m2, v[i].z);
+      m2 = absmax_bits(m2, v[i].w);
+    }
+    m = block_max_bits(absmax_fold(m2), part2);
+  }
+  const float s = __fadd_rn(__uint_as_float(m << 16), eps);
+  if (threadIdx.x == 0) s_out[r] = s;
+  const float c = __fdiv_rn(Q, s);
+  uint2* qv = reinterpret_cast<uint2*>(q + r * ldq);
+  if (finite && c < __int_as_float(0x7F800000)) {
+#pragma unroll
+    for (int i = 0; i < VPT; ++i) {
+      const int idx = threadIdx.x + i * blockDim.x;
+      if (idx < nvec)
+        qv[idx] = make_uint2(quant4_magic(bf16x2_to_f32x2(v[i].x), bf16x2_to_f32x2(v[i].y), c),
+                             quant4_magic(bf16x2_to_f32x2(v[i].z), bf16x2_to_f32x2(v[i].w), c));
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < VPT; ++i) {
+      const int idx = threadIdx.x + i * blockDim.x;
+      if (idx < nvec) qv[idx] = make_uint2(quant4_slow(v[i].x, v[i].y, c, Q), quant4_slow(v[i].z, v[i].w, c, Q));
+    }
+  }
+  }
+}
+
+// Threads per CTA for a row of `nvec` vectors, `vpt` per thread: whole warps.
+int row_threads(int64_t nvec, int vpt) { return (int)(((nvec + vpt - 1) / vpt + 31) / 32 * 32); }
+
+cudaError_t launch_rows_reg(const uint16_t* x, int64_t rows, int64_t cols, int64_t ldx, float eps, float Q, float* s, int8_t* q,
+                            int64_t ldq, cudaStream_t st) {
+  const int64_t nvec = cols >> 3;
+  const dim3 grid((unsigned)std::min<int64_t>(rows, INT32_MAX));
+  if (nvec <= kThreads)
+    return launch_chain(absmax_rows_reg_kernel<1>, grid, dim3(row_threads(nvec, 1)), 0, st, 0, x, rows, cols, ldx, eps, Q, s, q, ldq);
+  if (nvec <= 2 * kThreads)
+    return launch_chain(absmax_rows_reg_kernel<2>, grid, dim3(row_threads(nvec, 2)), 0, st, 0, x, rows, cols, ldx, eps, Q, s, q, ldq);
+  return launch_chain(absmax_rows_reg_kernel<4>, grid, dim3(row_threads(nvec, 4)), 0, st, 0, x, rows, cols, ldx, eps, Q, s, q, ldq);
+}
+
 // one scale for the whole (contiguous) tensor: per-CTA maxima ...
 __global__ void __launch_bounds__(kThreads) absmax_slots_kernel(const uint16_t* x, int64_t n, uint32_t* slots) {
   __shared__ uint32_t part[kThreads / 32];
@@ -163,6 +279,12 @@ extern "C" tweo_status_t tweo_absmax_quantize(const uint16_t* x, int64_t rows, i
   const bool given = mode == TWEO_SCALE_GIVEN;
   if (granularity == TWEO_GRAN_ROW) {
     if (rows == 0) return TWEO_OK;
+    if (!given && cols >= 8 && cols <= kRegRowCols && !(cols & 7) && !(ldx & 7) && !(ldq & 7) && aligned16(x) &&
+        !(reinterpret_cast<uintptr_t>(q) & 7u)) {
+      TWEO_CUDA_TRY(launch_rows_reg(x, rows, cols, ldx, eps, Q, s, q, ldq, st));
+      count_launch();
+      return check_launch("absmax_rows_reg_kernel");
+    }
     const int grid = grid_cap(rows, 8);
     if (given) absmax_rows_kernel<true><<<grid, kThreads, 0, st>>>(x, rows, cols, ldx, eps, Q, s, q, ldq);
     else absmax_rows_kernel<false><<<grid, kThreads, 0, st>>>(x, rows, cols, ldx, eps, Q, s, q, ldq);
@@ -263,9 +385,13 @@ extern "C" tweo_status_t tweo_residual_add_q8(const int8_t* xq, const float* sx,
 }
 
 // ------------------------------------------------------------------ per-token 8-bit residual stream (Sec. 4.4)
-// One warp per row: the row's codes of x and f(x) stay in registers (VPL 16-byte vectors of each per lane,
-// lane-interleaved), so the dequantised sum is formed once, its maximum found by shuffles, and the codes of the
-// sum written in the same pass: 2 bytes read and 1 written per element plus three scales per row.
+// One CTA per row, the block sized to the row: VPT 16-byte vectors of each input per thread, the dequantised sums formed
+// once and held in registers, their maximum found by shuffles and one barrier, the codes of the sum written in the same
+// pass: 2 bytes read and 1 written per element plus three scales per row.  Converting instructions (bytes to binary32 and
+// back) go through a unit that does 16 a clock per SM, five of them per element bounded an earlier form of one warp per
+// row (9.5 us at [1999x4096], and a row's work behind one warp: 4.4 us at 16 rows).  Instead a byte becomes binary32 by
+// placing it in the mantissa of 2^23 and subtracting, and the code is the low byte of fl32(y c) + 1.5 2^23 (see
+// absmax_rows_reg_kernel); rows whose scales are not far from overflow take the converting path.
 namespace {
 
 struct RowAddArgs {
@@ -280,74 +406,86 @@ struct RowAddArgs {
   float Q, eps;
 };
 
-template <int VPL>
-__global__ void __launch_bounds__(256) residual_add_q8_rows_kernel(const RowAddArgs a) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp_global = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int64_t warp_stride = (int64_t)gridDim.x * 8;
-  const int nvec = a.cols >> 4;
-  const int q = (int)a.Q;
-  for (int64_t row = warp_global; row < a.rows; row += warp_stride) {
-    const uint4* xv = reinterpret_cast<const uint4*>(a.xq + row * a.cols);
-    const uint4* fv = reinterpret_cast<const uint4*>(a.fq + row * a.cols);
-    uint4 vx[VPL], vf[VPL];
-#pragma unroll
-    for (int i = 0; i < VPL; ++i) {
-      const int idx = lane + 32 * i;
-      vx[i] = idx < nvec ? __ldcs(xv + idx) : make_uint4(0u, 0u, 0u, 0u);
-      vf[i] = idx < nvec ? __ldcs(fv + idx) : make_uint4(0u, 0u, 0u, 0u);
-    }
-    const float cx = __fdiv_rn(__ldg(a.sx + row), a.Q), cf = __fdiv_rn(__ldg(a.sf + row), a.Q);
-    float amax = 0.0f;  // padding lanes hold zero codes: their sum is 0
-#pragma unroll
-    for (int i = 0; i < VPL; ++i) {
-      const uint32_t wx[4] = {vx[i].x, vx[i].y, vx[i].z, vx[i].w};
-      const uint32_t wf[4] = {vf[i].x, vf[i].y, vf[i].z, vf[i].w};
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-          amax = fmaxf(amax, fabsf(__fmaf_rn(code_to_f32(wf[k], e), cf, __fmul_rn(code_to_f32(wx[k], e), cx))));
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, o));
-    const float s = __fadd_rn(amax, a.eps);
-    const float c = __fdiv_rn(a.Q, s);
-    if (lane == 0) a.sy[row] = s;
-    uint4* yv = reinterpret_cast<uint4*>(a.yq + row * a.cols);
-#pragma unroll
-    for (int i = 0; i < VPL; ++i) {
-      const int idx = lane + 32 * i;
-      if (idx < nvec) {
-        const uint32_t wx[4] = {vx[i].x, vx[i].y, vx[i].z, vx[i].w};
-        const uint32_t wf[4] = {vf[i].x, vf[i].y, vf[i].z, vf[i].w};
-        uint32_t o4[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          uint32_t w = 0u;
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const float y = __fmaf_rn(code_to_f32(wf[k], e), cf, __fmul_rn(code_to_f32(wx[k], e), cx));
-            w |= ((uint32_t)quant1(y, c, a.Q) & 0xFFu) << (8 * e);
-          }
-          o4[k] = w;
-        }
-        __stcs(yv + idx, make_uint4(o4[0], o4[1], o4[2], o4[3]));
-      }
-    }
-    (void)q;
-  }
+// codes of word w (int8) -> two binary32 pairs, exact: 2^23 + (code + 128), minus 2^23 + 128
+__device__ __forceinline__ void codes_to_f32x2(uint32_t w, uint64_t& p01, uint64_t& p23) {
+  const uint32_t u = w ^ 0x80808080u;
+  const uint64_t bias = splat_f32x2(-8388736.0f);
+  p01 = add_f32x2(pack_f32x2(__uint_as_float(__byte_perm(u, 0x4B000000u, 0x7440)),
+                             __uint_as_float(__byte_perm(u, 0x4B000000u, 0x7441))), bias);
+  p23 = add_f32x2(pack_f32x2(__uint_as_float(__byte_perm(u, 0x4B000000u, 0x7442)),
+                             __uint_as_float(__byte_perm(u, 0x4B000000u, 0x7443))), bias);
 }
 
-template <int VPL>
-cudaError_t launch_row_add(const RowAddArgs& a, cudaStream_t st) {
-  int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, residual_add_q8_rows_kernel<VPL>, 256, 0);
-  if (e != cudaSuccess) return e;
-  const int64_t want = (a.rows + 7) / 8;
-  const int64_t cap = (int64_t)tweo_detail::sm_count() * (per_sm > 0 ? per_sm : 1);
-  residual_add_q8_rows_kernel<VPL><<<tweo_detail::balanced_grid(want, cap), 256, 0, st>>>(a);
-  return cudaGetLastError();
+template <int VPT>
+__global__ void __launch_bounds__(256) residual_add_q8_rows_kernel(const RowAddArgs a) {
+  __shared__ float part[8];
+  chain_release();
+  chain_wait();
+  const int nvec = a.cols >> 4;
+  for (int64_t row = blockIdx.x; row < a.rows; row += gridDim.x) {   // one turn, as in absmax_rows_reg_kernel
+  if (row != blockIdx.x) __syncthreads();
+  const uint4* xv = reinterpret_cast<const uint4*>(a.xq + row * a.cols);
+  const uint4* fv = reinterpret_cast<const uint4*>(a.fq + row * a.cols);
+  uint4 vx[VPT], vf[VPT];
+#pragma unroll
+  for (int i = 0; i < VPT; ++i) {
+    const int idx = threadIdx.x + i * blockDim.x;
+    vx[i] = idx < nvec ? __ldcs(xv + idx) : make_uint4(0u, 0u, 0u, 0u);
+    vf[i] = idx < nvec ? __ldcs(fv + idx) : make_uint4(0u, 0u, 0u, 0u);
+  }
+  const float cx = __fdiv_rn(__ldg(a.sx + row), a.Q), cf = __fdiv_rn(__ldg(a.sf + row), a.Q);
+  const uint64_t cx2 = splat_f32x2(cx), cf2 = splat_f32x2(cf);
+  uint64_t y[VPT][8];
+  float amax = 0.0f;  // padding lanes hold zero codes: their sum is 0 (or, like any NaN, does not count)
+#pragma unroll
+  for (int i = 0; i < VPT; ++i) {
+    const uint32_t wx[4] = {vx[i].x, vx[i].y, vx[i].z, vx[i].w};
+    const uint32_t wf[4] = {vf[i].x, vf[i].y, vf[i].z, vf[i].w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      uint64_t x01, x23, f01, f23;
+      codes_to_f32x2(wx[k], x01, x23);
+      codes_to_f32x2(wf[k], f01, f23);
+      y[i][2 * k] = fma_f32x2(f01, cf2, mul_f32x2(x01, cx2));
+      y[i][2 * k + 1] = fma_f32x2(f23, cf2, mul_f32x2(x23, cx2));
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      float lo, hi;
+      unpack_f32x2(y[i][k], lo, hi);
+      amax = fmaxf(amax, fmaxf(fabsf(lo), fabsf(hi)));
+    }
+  }
+  amax = warp_max(amax);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = amax;
+  __syncthreads();
+  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) amax = fmaxf(amax, part[w]);
+  const float s = __fadd_rn(amax, a.eps);
+  const float c = __fdiv_rn(a.Q, s);
+  if (threadIdx.x == 0) a.sy[row] = s;
+  // no sum of the row can have been infinite or NaN, and Q / s is finite: |y c| stays within one rounding of Q
+  const bool plain = (fabsf(cx) + fabsf(cf)) * 256.0f < 3.0e38f && c < __int_as_float(0x7F800000);
+  uint4* yv = reinterpret_cast<uint4*>(a.yq + row * a.cols);
+#pragma unroll
+  for (int i = 0; i < VPT; ++i) {
+    const int idx = threadIdx.x + i * blockDim.x;
+    uint32_t o4[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (plain) {
+        o4[k] = quant4_magic(y[i][2 * k], y[i][2 * k + 1], c);
+      } else {
+        float v[4];
+        unpack_f32x2(y[i][2 * k], v[0], v[1]);
+        unpack_f32x2(y[i][2 * k + 1], v[2], v[3]);
+        o4[k] = 0u;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) o4[k] |= ((uint32_t)quant1(v[e], c, a.Q) & 0xFFu) << (8 * e);
+      }
+    }
+    if (idx < nvec) __stcs(yv + idx, make_uint4(o4[0], o4[1], o4[2], o4[3]));
+  }
+  }
 }
 
 }  // namespace
@@ -373,13 +511,13 @@ extern "C" tweo_status_t tweo_residual_add_q8_rows(const int8_t* xq, const float
   a.Q = (float)((1 << (bits - 1)) - 1);
   a.eps = eps;
   cudaStream_t st = (cudaStream_t)stream;
-  const int vpl = (int)((cols / 16 + 31) / 32);
+  const int64_t nvec = cols >> 4;
+  const dim3 grid((unsigned)std::min<int64_t>(rows, INT32_MAX));
   cudaError_t e;
-  if (vpl <= 1) e = launch_row_add<1>(a, st);
-  else if (vpl <= 2) e = launch_row_add<2>(a, st);
-  else if (vpl <= 4) e = launch_row_add<4>(a, st);
-  else if (vpl <= 8) e = launch_row_add<8>(a, st);
-  else e = launch_row_add<16>(a, st);
+  if (nvec <= 256)
+    e = tweo_detail::launch_chain(residual_add_q8_rows_kernel<1>, grid, dim3(row_threads(nvec, 1)), 0, st, 0, a);
+  else
+    e = tweo_detail::launch_chain(residual_add_q8_rows_kernel<2>, grid, dim3(row_threads(nvec, 2)), 0, st, 0, a);
   if (e != cudaSuccess) return tweo_detail::cuda_fail(e, "residual_add_q8_rows_kernel");
   tweo_detail::count_launch();
   return TWEO_OK;

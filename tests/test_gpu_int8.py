@@ -116,3 +116,23 @@ def test_int8_linear_rejects_bad_arguments(tw):
         tw.int8_linear(xq, one, wq, one)
     with pytest.raises(tw.TweoError):
         tw.int8_linear(xq, one, torch.zeros((48, 64), dtype=torch.int8, device="cuda"), one, bits=9)
+
+
+@pytest.mark.parametrize("cols,pitch", [(8, 8), (256, 264), (2048, 2048), (2056, 2056), (4096, 4096), (4104, 4104), (8192, 8200),
+                                        (8200, 8200), (100, 100), (96, 100)])
+def test_absmax_rows_bit_exact_at_the_edges_of_the_register_form(tw, cols, pitch):
+    """One to four vectors per thread, whole and partial warps, and the widths and pitches that are read twice; with eps = 0:
+    an all-zero row (scale 0), rows with a NaN, an infinity, only NaN, and values down to the smallest."""
+    x = synth.normal_with_extreme_outliers_bf16(220 + cols, (11, pitch))
+    x[1, :] = 0
+    x[2, cols // 2] = 0x7FC0
+    x[3, cols - 1] = 0xFF80
+    x[4, :] = 0xFFC1
+    x[5, :] = 0x8001
+    x[6, :cols // 2] = 0x3F80
+    for eps in (1e-6, 0.0):
+        q_ref, s_ref = orc.absmax_quantize_bf16(np.ascontiguousarray(x[:, :cols]), 8, eps, per_row=True)
+        q, s = tw.absmax_quantize(to_gpu_bf16(x)[:, :cols], 8, tw.GRAN_ROW, eps)
+        torch.cuda.synchronize()
+        assert np.array_equal(s.cpu().numpy().view(np.uint32), s_ref.view(np.uint32))
+        assert np.array_equal(q.cpu().numpy(), q_ref)

@@ -134,6 +134,22 @@ def test_residual_add_q8_rows_bit_exact(tw, rows, cols, bits):
         assert out is gx and np.array_equal(gx.cpu().numpy(), ref_q)
 
 
+@pytest.mark.parametrize("cols", [16, 496, 528, 4096, 4112, 8192])
+def test_residual_add_q8_rows_bit_exact_with_extreme_scales(tw, cols):
+    """Scales of ordinary size, zero, tiny, close to overflow, infinite and NaN, one row each, with eps = 0 and not."""
+    sx = np.array([1.0, 0.0, 1e-44, 3e38, np.inf, np.nan, 1.0, 1e30, 0.0], dtype=np.float32)
+    sf = np.array([0.5, 0.0, 1e-44, 3e38, 1.0, 1.0, np.nan, 1e-30, 1e-38], dtype=np.float32)
+    g = np.random.Generator(np.random.PCG64(cols))
+    xq = g.integers(-128, 128, (len(sx), cols), dtype=np.int8)
+    fq = g.integers(-128, 128, (len(sx), cols), dtype=np.int8)
+    for eps in (1e-6, 0.0):
+        ref_q, ref_s = orc.residual_add_q8_rows(xq, sx, fq, sf, 8, eps)
+        yq, sy = tw.residual_add_q8_rows(torch.from_numpy(xq).cuda(), dev(sx), torch.from_numpy(fq).cuda(), dev(sf), 8, eps)
+        torch.cuda.synchronize()
+        assert np.array_equal(sy.cpu().numpy().view(np.uint32), ref_s.view(np.uint32))
+        assert np.array_equal(yq.cpu().numpy(), ref_q)
+
+
 def test_per_token_chain_linear_quantise_add(tw):
     """A8(K): x codes per token -> integer linear (per-token x per-channel scales) -> per-token codes of f(x) ->
     per-token codes of x + f(x); every stage against the oracle's stage on the oracle's own inputs."""
