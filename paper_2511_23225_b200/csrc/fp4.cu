@@ -16,7 +16,7 @@ namespace tweo_detail {
 tweo_status_t gemm_fwd_codes(const uint8_t* xq, int64_t ldx, int fmt_x, const uint8_t* wq, int64_t ldw, int fmt_w,
                              const float* sx_inv, const float* sw_inv, uint16_t* y, int64_t ldy, int64_t M,
                              int64_t N, int64_t K, const tweo_epilogue_t* epi, void* ws, size_t ws_bytes,
-                             cudaStream_t st, bool sx_is_scale);
+                             cudaStream_t st, bool sx_is_scale, bool inference, bool w_early);
 // amax reset (+ reciprocal of a given scale) and, for current scaling, the amax pass: shared with the FP8 casts
 tweo_status_t launch_amax_prologue(const uint16_t* x, int64_t n, float* amax, uint32_t* sat_count, const float* scale_in,
                                    float* scale_inv, cudaStream_t st);
@@ -82,8 +82,7 @@ __device__ __forceinline__ float e2m1_scale_from_amax(float amax) {
 template <bool GIVEN, int U>
 __global__ void __launch_bounds__(kThreads)
 fp4_cast_kernel(const uint16_t* x, int64_t n, float* scale, float* scale_inv, float* amax, uint8_t* q4, uint8_t* q8) {
-  chain_release();
-  chain_wait();
+  chain_wait();   // and no chain_release(): the packed-weight linear loads its weight, maybe these codes, before its own wait
   float s;
   if (GIVEN) {
     s = *scale;
@@ -260,5 +259,5 @@ extern "C" tweo_status_t tweo_w4a4_static_gemm(const uint16_t* x, int64_t ldx, c
   if (s != TWEO_OK) return s;
   const size_t used = 256 + (((size_t)M * (size_t)K + 255) & ~(size_t)255);
   return gemm_fwd_codes(carriers, K, TWEO_E4M3, wq8, ldw, TWEO_E4M3, scalars, sw_inv, y, ldy, M, N, K, nullptr,
-                        reinterpret_cast<char*>(ws) + used, ws_bytes - used, (cudaStream_t)stream, false);
+                        reinterpret_cast<char*>(ws) + used, ws_bytes - used, (cudaStream_t)stream, false, true, false);
 }

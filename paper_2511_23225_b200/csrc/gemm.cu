@@ -681,66 +681,162 @@ tweo_status_t run_fwd_act(const uint8_t* xq, int64_t ldx, int fmt_x, const uint8
   }
 }
 
-// Forward product for M <= 128 (see gemm_skinny.cuh): W is streamed once, K is sliced over CTAs.  The caller has
-// filled the scale fields of `p`; this fills the shape, the ring and the slicing, and launches.
+// How the few-token kernel (gemm_skinny.cuh) would split a product of M tokens, N output columns and `k_blocks`
+// contraction blocks.
+struct SkinnyPlan {
+  int m_tiles, tokens;   // token tiles, and tokens per tile (a multiple of 16, at most 256)
+  int slices;            // slices of the contraction
+  int stages;
+  uint32_t stage_bytes;
+  double clocks;         // estimate, see below
+};
+
+// Clusters of `slices` CTAs that are resident at once, with rings of 100 KB or (wide) 200 KB.  A cluster lives within one
+// group of SMs, whose size is no multiple of most counts (148 SMs hold 15 clusters of eight 200 KB CTAs, not 18).
+// Asked for once per device.
+int resident_clusters(int slices, bool wide) {
+  struct Table {
+    std::atomic<bool> known{false};
+    int n[2][9];
+  };
+  static Table tables[64];
+  static std::mutex mu;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return sm_count() * (wide ? 1 : 2) / slices;
+  Table& t = tables[dev];
+  if (!t.known.load(std::memory_order_acquire)) {
+    std::lock_guard<std::mutex> lock(mu);
+    auto kern = gemm_fp8_skinny_kernel<false, false>;
+    const int bytes[2] = {100 * 1024 + 1024 + 256, 200 * 1024 + 1024 + 256};
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes[1]);
+    for (int w = 0; w < 2; ++w)
+      for (int c = 1; c <= 8; ++c) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)c);
+        cfg.blockDim = dim3(kThreads);
+        cfg.dynamicSmemBytes = (size_t)bytes[w];
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)c;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) n = sm_count() * (w ? 1 : 2) / c;
+        t.n[w][c] = n;
+      }
+    (void)cudaGetLastError();
+    t.known.store(true, std::memory_order_release);
+  }
+  return t.n[wide ? 1 : 0][slices];
+}
+
+SkinnyPlan plan_skinny(int64_t M, int64_t N, int k_blocks) {
+  const int sms = sm_count();
+  const int slabs = (int)((N + 127) / 128);
+  SkinnyPlan pl{};
+  pl.m_tiles = (int)((M + 255) / 256);
+  // above 128 tokens a CTA has an SM to itself (a deep ring of wide stages); up to 128 two share one
+  pl.tokens = (int)(((M + pl.m_tiles - 1) / pl.m_tiles + 15) / 16 * 16);
+  const bool wide = pl.tokens > 128;
+  pl.stage_bytes = (uint32_t)((BM * BK + pl.tokens * 128 + 1023) / 1024 * 1024);
+  pl.stages = (int)((wide ? 200 : 100) * 1024 / pl.stage_bytes);
+  if (pl.stages > kSkinnyMaxStages) pl.stages = kSkinnyMaxStages;
+  if (pl.stages < 2) pl.stages = 2;
+  // slices = CTAs per cluster: the largest count up to the portable cluster size whose clusters are all resident at
+  // once and that leaves every slice at least four k-blocks
+  const int64_t tiles = (int64_t)slabs * pl.m_tiles;
+  pl.slices = 1;
+  for (int sl = 2; sl <= 8; ++sl)
+    if (tiles <= resident_clusters(sl, wide) && k_blocks / sl >= 4) pl.slices = sl;
+  // Operand bytes per SM at 46 B a clock (what the CTA-pair kernel's main loop draws from L2), the reduction at 32 B
+  // a clock, set-up and the two cluster barriers at 6000 clocks.
+  const int64_t ctas = tiles * pl.slices;
+  const int64_t rounds = (ctas + sms - 1) / sms;
+  const double kb = (double)((k_blocks + pl.slices - 1) / pl.slices);
+  pl.clocks = (double)rounds * (kb * pl.stage_bytes / 46.0 + pl.tokens * 512.0 / 32.0) + 6000.0;
+  return pl;
+}
+
+// Estimate for the CTA-pair kernel on whole tiles: 630 clocks per k-block of a 256 x 256 tile, 5000 for
+// set-up, the first tile's loads and the last tile's epilogue (fitted to the measurements below skinny_pays).
+double pair_clocks(int64_t M, int64_t N, int k_blocks) {
+  const int64_t tiles = ((M + 255) / 256) * ((N + 255) / 256), pairs = sm_count() / 2;
+  return (double)((tiles + pairs - 1) / pairs) * k_blocks * 630.0 + 5000.0;
+}
+
+// Whether an inference product of M tokens takes the few-token kernel: always up to 128 tokens; above, where the
+// 256 x 256 tiles of the pair kernel leave most of the chip idle (few tiles, long contractions).  The products of the
+// training step stay on the pair kernel above 128 tokens: they have to equal those of a grouped launch bit for bit.
+// Static W8A8 pass, us, few-token kernel against pair kernel: M = 160 [4096x4096] 11.2 / 16.7, [4096x11008] 18.6 / 34.9,
+// [1024x1024] 8.7 / 8.9; M = 300 14.0 / 17.7, 26.8 / 36.5, 9.2 / 9.2; M = 512 16.6 / 18.7, 33.8 / 38.4, 11.2 / 9.2.
+bool skinny_pays(int64_t M, int64_t N, int64_t Kc) {
+  if (M <= 128) return true;
+  if (M > 2048 || N > INT32_MAX || Kc > INT32_MAX) return false;
+  const int k_blocks = (int)((Kc + BK - 1) / BK);
+  return plan_skinny(M, N, k_blocks).clocks < pair_clocks(M, N, k_blocks);
+}
+
+// Fills the shape, the ring and the split of `p` (the caller has filled the scale fields and the operand formats of the
+// instruction descriptor), and launches.  wq: [N, Kc] (K contiguous), or [Kc, N] for W_MN.
 // w_packed4: W holds packed E2M1 codes (two per byte, ldw in BYTES); the ring and the kernel are the same, only the
 // tensor map of W differs (and the operand format in p.idesc, set by the caller).
-template <bool I8>
+// w_early: W may be loaded before the kernels before this one have completed (see gemm_skinny.cuh).
+template <bool I8, bool W_MN = false>
 tweo_status_t launch_skinny(SkinnyParams& p, const void* xq, int64_t ldx, const void* wq, int64_t ldw, int64_t M, int64_t N,
-                            int64_t K, cudaStream_t st, bool w_packed4 = false) {
-  if (N > INT32_MAX || K > INT32_MAX) return TWEO_ERR_UNSUPPORTED_SHAPE;
+                            int64_t K, cudaStream_t st, bool w_early, bool w_packed4 = false) {
+  if (M > INT32_MAX || N > INT32_MAX || K > INT32_MAX) return TWEO_ERR_UNSUPPORTED_SHAPE;
   if (!aligned16(xq) || !aligned16(wq) || (ldx & 15) || (ldw & 15)) return TWEO_ERR_ALIGNMENT;
   if (w_packed4 && ((reinterpret_cast<uintptr_t>(wq) & 31u) || (ldw & 31) || (K & 127))) return TWEO_ERR_ALIGNMENT;
   p.M = (int32_t)M;
   p.N = (int32_t)N;
-  p.Mpad = (int32_t)((M + 15) / 16 * 16);
   p.k_blocks = (int32_t)((K + BK - 1) / BK);
-  p.stage_bytes = (uint32_t)((BM * BK + p.Mpad * 128 + 1023) / 1024 * 1024);
+  const SkinnyPlan pl = plan_skinny(M, N, p.k_blocks);
+  p.Mpad = pl.tokens;
+  p.slabs = (int32_t)((N + 127) / 128);
+  p.slices = pl.slices;
+  p.stages = pl.stages;
+  p.stage_bytes = pl.stage_bytes;
   p.w_tx_bytes = (uint32_t)(w_packed4 ? BM * BK / 2 : BM * BK);
-  // A ring of at most 100 KB, so that two CTAs fit an SM: the CTAs of the next kernel of a launch chain become
-  // resident (and fetch their first ring of W) while this kernel's are still reducing and writing.
-  p.stages = (int32_t)((100 * 1024) / p.stage_bytes);
-  if (p.stages > kSkinnyMaxStages) p.stages = kSkinnyMaxStages;
-  if (p.stages < 2) p.stages = 2;
-  p.tmem_cols = p.Mpad <= 32 ? 32u : (p.Mpad <= 64 ? 64u : 128u);
-  const int sms = sm_count();
-  const int slabs = (int)((N + 127) / 128);
-  // slices of K per slab = CTAs per cluster: the largest count up to the portable cluster size that keeps the grid
-  // within two CTAs per SM and leaves every slice at least four k-blocks
-  p.slices = 1;
-  for (int sl = 2; sl <= 8; ++sl)
-    if (slabs * sl <= 2 * sms && p.k_blocks / sl >= 4) p.slices = sl;
+  p.tmem_cols = p.Mpad <= 32 ? 32u : (p.Mpad <= 64 ? 64u : (p.Mpad <= 128 ? 128u : 256u));
+  p.vec_out = (reinterpret_cast<uintptr_t>(p.y) & 7u) == 0 && (p.ldy & 3) == 0;
+  p.idesc |= (uint32_t)(p.Mpad >> 3) << 17;
+  p.w_early = w_early ? 1 : 0;
   CUtensorMap mw, mx;
-  const bool w_ok = w_packed4 ? make_map_packed4(&mw, wq, K, N, ldw, BM) : make_map(&mw, wq, K, N, ldw, BM);
+  const bool w_ok = w_packed4 ? make_map_packed4(&mw, wq, K, N, ldw, BM)
+                              : (W_MN ? make_map(&mw, wq, N, K, ldw, BK) : make_map(&mw, wq, K, N, ldw, BM));
   if (!w_ok || !make_map(&mx, xq, K, M, ldx, p.Mpad)) {
     cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
     return TWEO_ERR_CUDA;
   }
   const size_t smem = (size_t)p.stages * p.stage_bytes + 1024 + 256;
-  auto kern = gemm_fp8_skinny_kernel<I8>;
+  auto kern = gemm_fp8_skinny_kernel<I8, W_MN>;
   static std::atomic<uint64_t> attr_done{0};  // per device
   int attr_dev = 0;
   if (device_once_pending(attr_done, &attr_dev)) {
-    TWEO_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(100 * 1024 + 1024 + 256)));
+    TWEO_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(200 * 1024 + 1024 + 256)));
     device_once_done(attr_done, attr_dev);
   }
-  TWEO_CUDA_TRY(launch_chain(kern, dim3((unsigned)(slabs * p.slices)), dim3(kThreads), smem, st, (unsigned)p.slices, mw,
-                             mx, p));
+  TWEO_CUDA_TRY(launch_chain(kern, dim3((unsigned)(p.slabs * pl.m_tiles * p.slices)), dim3(kThreads), smem, st,
+                             (unsigned)p.slices, mw, mx, p));
   count_launch();
   return check_launch("gemm_fp8_skinny_kernel");
 }
 
-tweo_status_t run_skinny(const uint8_t* xq, int64_t ldx, int fmt_x, const uint8_t* wq, int64_t ldw, int fmt_w,
+// FP8 operands: the forward product, or with w_mn the data gradient (N: output columns, K: contraction).
+tweo_status_t run_skinny(const uint8_t* xq, int64_t ldx, int fmt_x, const uint8_t* wq, int64_t ldw, int fmt_w, bool w_mn,
                          const float* sx_inv, const float* sw_inv, bool sx_is_scale, uint16_t* y, int64_t ldy, int64_t M,
-                         int64_t N, int64_t K, cudaStream_t st) {
+                         int64_t N, int64_t K, bool w_early, cudaStream_t st) {
   SkinnyParams p{};
   p.y = y;
   p.ldy = ldy;
-  p.idesc = make_idesc(fmt_w, fmt_x, false, false, (int)((M + 15) / 16 * 16), BM);
+  p.idesc = make_idesc(fmt_w, fmt_x, w_mn, false, 0, BM);
   p.sx_inv = sx_inv;
   p.sw_inv = sw_inv;
   p.sx_is_scale = sx_is_scale ? 1 : 0;
-  return launch_skinny<false>(p, xq, ldx, wq, ldw, M, N, K, st);
+  return w_mn ? launch_skinny<false, true>(p, xq, ldx, wq, ldw, M, N, K, st, w_early)
+              : launch_skinny<false>(p, xq, ldx, wq, ldw, M, N, K, st, w_early);
 }
 
 // The same with W as packed E2M1 codes: half the bytes of the stream that bounds the call.
@@ -750,11 +846,12 @@ tweo_status_t run_skinny_w4(const uint8_t* xq, int64_t ldx, int fmt_x, const uin
   SkinnyParams p{};
   p.y = y;
   p.ldy = ldy;
-  p.idesc = make_idesc(kFmtE2M1, fmt_x, false, false, (int)((M + 15) / 16 * 16), BM);
+  p.idesc = make_idesc(kFmtE2M1, fmt_x, false, false, 0, BM);
   p.sx_inv = sx_inv;
   p.sw_inv = sw_inv;
   p.sx_is_scale = 0;
-  return launch_skinny<false>(p, xq, ldx, w4, ldw_bytes, M, N, K, st, true);
+  // packed weights come from the FP4 cast alone, which lets no later kernel start before it has completed
+  return launch_skinny<false>(p, xq, ldx, w4, ldw_bytes, M, N, K, st, true, true);
 }
 
 // Up to kGroupMaxProblems independent products in ONE launch of the CTA-pair kernel (see gemm_pair_group.cuh).
@@ -972,10 +1069,11 @@ unsigned int* device_status_word() {
 tweo_status_t gemm_fwd_codes(const uint8_t* xq, int64_t ldx, int fmt_x, const uint8_t* wq, int64_t ldw, int fmt_w,
                              const float* sx_inv, const float* sw_inv, uint16_t* y, int64_t ldy, int64_t M,
                              int64_t N, int64_t K, const tweo_epilogue_t* epi, void* ws, size_t ws_bytes,
-                             cudaStream_t st, bool sx_is_scale) {
+                             cudaStream_t st, bool sx_is_scale, bool inference, bool w_early) {
   const bool fused = epi && (epi->out_amax || epi->out_q);
-  if (M <= 128 && !fused)  // few tokens: stream W once, tokens on the MMA's N side
-    return run_skinny(xq, ldx, fmt_x, wq, ldw, fmt_w, sx_inv, sw_inv, sx_is_scale, y, ldy, M, N, K, st);
+  if (M > 128 && (!aligned16(y) || (ldy & 7))) return TWEO_ERR_ALIGNMENT;
+  if (!fused && (inference ? skinny_pays(M, N, K) : M <= 128))  // few tokens: stream W once, tokens on the MMA's N side
+    return run_skinny(xq, ldx, fmt_x, wq, ldw, fmt_w, false, sx_inv, sw_inv, sx_is_scale, y, ldy, M, N, K, w_early, st);
   GemmParams p{};
   p.d = y;
   p.ldd = ldy;
@@ -1003,21 +1101,21 @@ tweo_status_t run_int8_linear(const int8_t* xq, int64_t ldx, const float* sx, in
   if (y && (!aligned16(y) || (ldy & 7))) return TWEO_ERR_ALIGNMENT;
   if (yq && (!aligned16(yq) || (ldq & 15))) return TWEO_ERR_ALIGNMENT;
   const bool q8 = yq != nullptr;
-  if (!q8 && M <= 128) {
+  if (!q8 && skinny_pays(M, N, K)) {
     // few tokens (small-batch inference, Sec. 4.4): the weight-streaming kernel with integer operands
     const int Q_ = (1 << (bits - 1)) - 1;
-    const int Mpad = (int)((M + 15) / 16 * 16);
     SkinnyParams sp{};
     sp.y = y;
     sp.ldy = ldy;
-    // kind::i8 descriptor: int32 accumulators, signed 8-bit A and B, K-major, M = 128 (rows of W), N = padded tokens
-    sp.idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(Mpad >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+    // kind::i8 descriptor: int32 accumulators, signed 8-bit A and B, K-major, M = 128 (rows of W); N is filled in at launch
+    sp.idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BM >> 4) << 24);
     sp.row_scale = sx;
     sp.col_scale = sw;
     sp.row_scale_per_row = sx_per_row ? 1 : 0;
     sp.col_scale_per_col = sw_per_row ? 1 : 0;
     sp.post_scale = 1.0f / ((float)Q_ * (float)Q_);
-    return launch_skinny<true>(sp, xq, ldx, wq, ldw, M, N, K, stream);
+    // integer codes come from the AbsMax casts alone, which let no later kernel start before they have completed
+    return launch_skinny<true>(sp, xq, ldx, wq, ldw, M, N, K, stream, true);
   }
   constexpr size_t smem6 = (size_t)6 * (BM * BK + 128 * BK) + 4 * 2 * 32 * 128 + 1024 + 256;
   constexpr size_t smem5q = (size_t)5 * (BM * BK + 128 * BK) + 4 * 2 * 32 * 128 + 4 * 2 * 32 * 64 + 1024 + 256;
@@ -1064,20 +1162,8 @@ tweo_status_t run_int8_linear(const int8_t* xq, int64_t ldx, const float* sx, in
     cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
     return TWEO_ERR_CUDA;
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(2 * pairs));
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = q8 ? smem5q : smem6;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (q8) TWEO_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern_q8, ma, mb, md, md, p));   // md doubles as the 8-bit output map
-  else TWEO_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern_bf16, ma, mb, md, md, p));
+  TWEO_CUDA_TRY(launch_chain(q8 ? kern_q8 : kern_bf16, dim3((unsigned)(2 * pairs)), dim3(kThreads), q8 ? smem5q : smem6, stream, 2,
+                             ma, mb, md, md, p));   // md doubles as the 8-bit output map
   count_launch();
   return check_launch("gemm_fp8_pair_kernel (int8)");
 }
@@ -1095,7 +1181,7 @@ tweo_status_t tweo_fp8_linear_fwd(const uint8_t* xq, int64_t ldx, const uint8_t*
   if (M < 1 || N < 1 || K < 1) return TWEO_ERR_INVALID_ARG;
   if ((N & 15) || (K & 15)) return TWEO_ERR_UNSUPPORTED_SHAPE;
   return tweo_detail::gemm_fwd_codes(xq, ldx, fmt_x, wq, ldw, fmt_w, sx_inv, sw_inv, y, ldy, M, N, K, epi, ws,
-                                     ws_bytes, (cudaStream_t)stream, false);
+                                     ws_bytes, (cudaStream_t)stream, false, false, false);
 }
 
 tweo_status_t tweo_fp8_linear_fwd_act(const uint8_t* xq, int64_t ldx, const uint8_t* wq, int64_t ldw,
@@ -1138,6 +1224,9 @@ tweo_status_t tweo_fp8_linear_bwd_dgrad(const uint8_t* dyq, int64_t lddy, int32_
   // dX[M,K] = dYq[M,N] . Wq[N,K]: contraction over N; Wq is stored [N(contraction), K(out)] = MN-major
   if (epi && (epi->out_amax || epi->out_q) && M > 128 && K > 128)  // extra outputs leave through shared memory and TMA
     return run_fwd_act(dyq, lddy, fmt_dy, wq, ldw, fmt_w, true, TWEO_ACT_NONE, M, K, N, p, (cudaStream_t)stream);
+  if (!aligned16(dx) || (lddx & 7)) return TWEO_ERR_ALIGNMENT;
+  if (!(epi && (epi->out_amax || epi->out_q)) && M <= 128)
+    return run_skinny(dyq, lddy, fmt_dy, wq, ldw, fmt_w, true, sdy_inv, sw_inv, false, dx, lddx, M, K, N, false, (cudaStream_t)stream);
   return run_gemm(Operand{dyq, lddy, fmt_dy, false}, Operand{wq, ldw, fmt_w, true}, M, K, N, p, ws, ws_bytes,
                   (cudaStream_t)stream);
 }

@@ -1,20 +1,19 @@
-// Forward product for few tokens (M <= 128): Y[M,N] = Xq[M,K] . Wq[N,K]^T, the shape of a
-// static W8A8 inference linear at small batch.  The work is streaming W once from HBM, so
-// the kernel is organised around that: the operands are swapped -- 128 rows of W are the
-// MMA's M dimension, the (padded) tokens its N dimension -- so the accumulator is only
-// 128 x Mpad and nothing but W moves in bulk.  Each CTA takes one 128-row slab of W and one
-// slice of K; slabs x slices is chosen to give every SM one or two CTAs, each with a ring of TMA stages of
-// up to 100 KB (two CTAs fit an SM, so in a launch chain the next kernel's CTAs fetch their first ring of W
-// while this kernel's still reduce and write).
+// Products with few tokens: Y[M,N] = Xq[M,K] . Wq[N,K]^T (forward) and dX[M,K] = dYq[M,N] . Wq[N,K] (data gradient,
+// W_MN: the weight in its forward layout as an MN-major operand).  The work is streaming W once from HBM, so
+// the kernel is organised around that: the operands are swapped -- 128 output columns (rows of W, or columns of it
+// for the data gradient) are the MMA's M dimension, a tile of up to 256 (padded) tokens its N dimension -- so the
+// accumulator is 128 x tokens and for few tokens nothing but W moves in bulk.  Each CTA takes one 128-wide slab of W,
+// one token tile and one slice of the contraction; the split is chosen by the launcher (plan_skinny).  Rings of up to
+// 100 KB leave room for two CTAs per SM, so that in a launch chain the next kernel's CTAs settle (and bring their
+// share of W into L2) while this kernel's still reduce and write; token tiles above 128 take up to 200 KB.
 //
-// CTA = 192 threads: warp 0 issues TMA loads (W slab 128 x 128 B and X 'Mpad' x 128 B per
+// CTA = 192 threads: warp 0 issues TMA loads (W slab 128 x 128 B and tokens x 128 B of X per
 // k-block, 128-byte swizzle, rows beyond M zero-filled), warp 1 owns tensor memory and issues
-// tcgen05.mma kind::f8f6f4 128 x Mpad x 32, warps 2-5 read the accumulator (lane = row of W =
-// output column) and write Y.  With K sliced, the slices of one slab form a thread-block cluster:
-// every CTA parks its fp32 partial sums in its own shared memory ([token][128 columns], in the
-// ring the loads no longer need), the cluster synchronises, and CTA r sums tokens r, r + S, ...
-// over all S slices in slice order through distributed shared memory and writes those rows of Y
-// (64 contiguous bytes per warp).  No workspace, no atomics, and the sum does not depend on
+// tcgen05.mma kind::f8f6f4 128 x tokens x 32, warps 2-5 read the accumulator (lane = output column), park it in the
+// CTA's own shared memory ([token][128 columns] fp32, in the ring the loads no longer need) and write Y.  The slices
+// of one tile form a thread-block cluster: the cluster synchronises, and CTA r sums tokens r, r + S, ...
+// over all S slices in slice order through distributed shared memory, 16 bytes per lane, and writes those rows of Y
+// (256 contiguous bytes per warp).  No workspace, no atomics, and the sum does not depend on
 // timing.  All mbarrier waits are bounded; the cluster barrier is reached by every thread.
 #pragma once
 
@@ -30,14 +29,17 @@ constexpr int kSkinnyMaxStages = 11;
 struct SkinnyParams {
   uint16_t* y;
   int64_t ldy;
-  int32_t M, N, Mpad;      // Mpad: M rounded up to a multiple of 16 (<= 128)
-  int32_t k_blocks;        // ceil(K / 128)
-  int32_t slices;          // slices of K = CTAs per cluster (1, 2, 4 or 8)
+  int32_t M, N, Mpad;      // N: output columns; Mpad: tokens per tile, a multiple of 16 (<= 256)
+  int32_t slabs;           // ceil(N / 128)
+  int32_t k_blocks;        // contraction blocks of 128
+  int32_t slices;          // slices of the contraction = CTAs per cluster (1 .. 8)
+  int32_t vec_out;         // y and ldy allow 8-byte stores
+  int32_t w_early;         // no kernel that may still run when this one starts can be writing W
   int32_t stages;          // TMA ring depth (<= kSkinnyMaxStages)
   uint32_t stage_bytes;    // 16 KB of W + Mpad * 128 B of X, rounded up to 1 KB
   uint32_t w_tx_bytes;     // bytes one W load reports to its barrier: the 16 KB it writes, or 8 KB for packed 4-bit
                            // codes (the load counts the bytes it fetched, not the padded groups it writes)
-  uint32_t tmem_cols;      // power of two >= max(32, Mpad)
+  uint32_t tmem_cols;      // power of two >= max(32, Mpad), at most 256
   uint32_t idesc;
   const float* sx_inv;
   const float* sw_inv;
@@ -49,9 +51,10 @@ struct SkinnyParams {
   float post_scale;
 };
 
-__device__ __forceinline__ uint32_t ld_shared_cluster_b32(uint32_t cluster_addr) {
-  uint32_t v;
-  asm volatile("ld.shared::cluster.b32 %0, [%1];" : "=r"(v) : "r"(cluster_addr) : "memory");
+__device__ __forceinline__ uint4 ld_shared_cluster_v4(uint32_t cluster_addr) {
+  uint4 v;
+  asm volatile("ld.shared::cluster.v4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(cluster_addr) : "memory");
   return v;
 }
 
@@ -76,49 +79,66 @@ __device__ __forceinline__ float skinny_out(const SkinnyParams& p, uint32_t acc,
   return __fmul_rn(__fmul_rn(__int2float_rn((int)acc), ar), alpha);
 }
 
-// The cluster's reduction for one output column (this thread's): CTA `slice` of the cluster sums tokens slice,
-// slice + S, ... over all S slices in slice order, reading the partial sums the CTAs parked in their shared memory
-// ([token][128 columns] fp32) through distributed shared memory, TOK tokens at a time (TOK * SL loads in flight).
-// SL: the slice count rounded up to 2, 4 or 8.
+// The cluster's reduction for four adjacent output columns (this lane's): CTA `slice` of the cluster sums tokens slice,
+// slice + S, ... of the tile over all S slices in slice order, reading the partial sums the CTAs parked in their shared
+// memory through distributed shared memory; the epilogue warps (wrp 0..3) take them in turn, TOK at a time
+// (TOK * SL 16-byte loads in flight per lane).  SL: the slice count rounded up to 1, 2, 4 or 8.
 template <bool I8, int TOK, int SL>
-__device__ __forceinline__ void skinny_reduce(const SkinnyParams& p, uint32_t mine, int slice, int n, float alpha) {
+__device__ __forceinline__ void skinny_reduce(const SkinnyParams& p, uint32_t mine, int slice, int wrp, int n, int m0,
+                                              int tokens, const float (&alpha)[4]) {
   uint32_t peer[SL];
 #pragma unroll
   for (int sl = 0; sl < SL; ++sl) peer[sl] = map_to_cta(mine, (uint32_t)(sl < p.slices ? sl : 0));
-  for (int t0 = slice; t0 < p.M; t0 += TOK * p.slices) {
-    uint32_t v[TOK][SL];
+  const int step = 4 * p.slices;
+  for (int t0 = slice + wrp * p.slices; t0 < tokens; t0 += TOK * step) {
+    uint4 v[TOK][SL];
 #pragma unroll
     for (int u = 0; u < TOK; ++u) {
-      const int t = t0 + u * p.slices;
+      const int t = t0 + u * step;
 #pragma unroll
       for (int sl = 0; sl < SL; ++sl)
-        v[u][sl] = (sl < p.slices && t < p.M) ? ld_shared_cluster_b32(peer[sl] + (uint32_t)t * 512u) : 0u;
+        v[u][sl] = (sl < p.slices && t < tokens) ? ld_shared_cluster_v4(peer[sl] + (uint32_t)t * 512u) : make_uint4(0u, 0u, 0u, 0u);
     }
 #pragma unroll
     for (int u = 0; u < TOK; ++u) {
-      const int t = t0 + u * p.slices;
-      uint32_t acc;
-      if (I8) {
-        int a = (int)v[u][0];
+      const int t = t0 + u * step;
+      uint4 acc = v[u][0];
 #pragma unroll
-        for (int sl = 1; sl < SL; ++sl)
-          if (sl < p.slices) a += (int)v[u][sl];   // exact
-        acc = (uint32_t)a;
-      } else {
-        float a = __uint_as_float(v[u][0]);
-#pragma unroll
-        for (int sl = 1; sl < SL; ++sl)
-          if (sl < p.slices) a += __uint_as_float(v[u][sl]);  // slice order
-        acc = __float_as_uint(a);
+      for (int sl = 1; sl < SL; ++sl)
+        if (sl < p.slices) {
+          if (I8) {   // exact
+            acc.x += v[u][sl].x;
+            acc.y += v[u][sl].y;
+            acc.z += v[u][sl].z;
+            acc.w += v[u][sl].w;
+          } else {    // slice order
+            acc.x = __float_as_uint(__uint_as_float(acc.x) + __uint_as_float(v[u][sl].x));
+            acc.y = __float_as_uint(__uint_as_float(acc.y) + __uint_as_float(v[u][sl].y));
+            acc.z = __float_as_uint(__uint_as_float(acc.z) + __uint_as_float(v[u][sl].z));
+            acc.w = __float_as_uint(__uint_as_float(acc.w) + __uint_as_float(v[u][sl].w));
+          }
+        }
+      if (t < tokens && n < p.N) {   // N is a multiple of 16: the four columns are in or out together
+        const int row = m0 + t;
+        const uint32_t lo = f32x2_to_bf16x2(skinny_out<I8>(p, acc.x, row, alpha[0]), skinny_out<I8>(p, acc.y, row, alpha[1]));
+        const uint32_t hi = f32x2_to_bf16x2(skinny_out<I8>(p, acc.z, row, alpha[2]), skinny_out<I8>(p, acc.w, row, alpha[3]));
+        uint16_t* dst = p.y + (int64_t)row * p.ldy + n;
+        if (p.vec_out) {
+          *reinterpret_cast<uint2*>(dst) = make_uint2(lo, hi);
+        } else {
+          dst[0] = (uint16_t)lo;
+          dst[1] = (uint16_t)(lo >> 16);
+          dst[2] = (uint16_t)hi;
+          dst[3] = (uint16_t)(hi >> 16);
+        }
       }
-      if (t < p.M && n < p.N) p.y[(int64_t)t * p.ldy + n] = (uint16_t)f32_to_bf16_bits(skinny_out<I8>(p, acc, t, alpha));
     }
   }
 }
 
 // I8: signed 8-bit operands (tcgen05 kind::i8, int32 accumulators: partial sums of K slices add exactly) with the
 // Eq. 4 dequantisation in the epilogue, per tensor or per token (activation rows) / per channel (weight rows).
-template <bool I8>
+template <bool I8, bool W_MN>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_fp8_skinny_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x,
                        const __grid_constant__ SkinnyParams p) {
@@ -152,38 +172,47 @@ gemm_fp8_skinny_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  const int slab = blockIdx.x / p.slices;
-  const int slice = blockIdx.x - slab * p.slices;
-  const int n0 = slab * 128;
+  const int tile = blockIdx.x / p.slices;
+  const int slice = blockIdx.x - tile * p.slices;
+  const int mt = tile / p.slabs;
+  const int n0 = (tile - mt * p.slabs) * 128;
+  const int m0 = mt * p.Mpad;
+  const int tokens = min(p.Mpad, p.M - m0);
   const int kb0 = (int)((int64_t)p.k_blocks * slice / p.slices);
   const int kb1 = (int)((int64_t)p.k_blocks * (slice + 1) / p.slices);
   const uint32_t x_bytes = (uint32_t)p.Mpad * 128u;
 
-  // The kernel may have been launched while the kernel before it on the stream is still running (programmatic
-  // dependent launch).  W is a static weight, not something that kernel produced, so the first ring of W loads is
-  // issued at once; everything that can depend on the previous kernel -- the activations, the two scales, the
-  // output buffer -- is touched only after chain_wait().
+  // The kernel may have been launched while the kernels before it on the stream are still running (programmatic
+  // dependent launch): the activations, the scales and the output are touched only after chain_wait().  So is W where
+  // one of those kernels may be the cast that writes it; until then it is brought into L2, which is safe whoever
+  // writes it.  Where none can be (w_early, see the callers), the first ring of W is loaded at once: L2 to shared memory
+  // takes 3 of 13 us at [11008x4096] after the wait.
   chain_release();
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
     if (lane == 0) {
-      const int pre = min(p.stages, kb1 - kb0);   // the ring is empty: these stages need no wait
+      auto load_w = [&](int stage, int kb) {
+        tma_load_2d(smem_base + stage * p.stage_bytes, &tmap_w, W_MN ? n0 : kb * BK, W_MN ? kb * BK : n0, full_bar(stage));
+      };
+      auto load_x = [&](int stage, int kb) {
+        tma_load_2d(smem_base + stage * p.stage_bytes + BM * BK, &tmap_x, kb * BK, m0, full_bar(stage));
+      };
+      const int pre = p.w_early ? min(p.stages, kb1 - kb0) : 0;   // the ring is empty: these stages need no wait
       for (int i = 0; i < pre; ++i) {
         mbar_expect_tx(full_bar(i), p.w_tx_bytes + x_bytes);
-        tma_load_2d(smem_base + i * p.stage_bytes, &tmap_w, (kb0 + i) * BK, n0, full_bar(i));
+        load_w(i, kb0 + i);
       }
+      if (!p.w_early && mt == 0)   // the token tiles of a slab read the same W
+        for (int kb = kb0; kb < kb1; ++kb) tma_prefetch_2d(&tmap_w, W_MN ? n0 : kb * BK, W_MN ? kb * BK : n0);
       chain_wait();
-      for (int i = 0; i < pre; ++i)
-        tma_load_2d(smem_base + i * p.stage_bytes + BM * BK, &tmap_x, (kb0 + i) * BK, 0, full_bar(i));
+      for (int i = 0; i < pre; ++i) load_x(i, kb0 + i);
       int stage = pre == p.stages ? 0 : pre;
       uint32_t phase = pre == p.stages ? 1u : 0u;
       for (int kb = kb0 + pre; kb < kb1; ++kb) {
         if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag)) break;
-        const uint32_t fb = full_bar(stage);
-        mbar_expect_tx(fb, p.w_tx_bytes + x_bytes);
-        const uint32_t sw = smem_base + stage * p.stage_bytes;
-        tma_load_2d(sw, &tmap_w, kb * BK, n0, fb);
-        tma_load_2d(sw + BM * BK, &tmap_x, kb * BK, 0, fb);
+        mbar_expect_tx(full_bar(stage), p.w_tx_bytes + x_bytes);
+        load_w(stage, kb);
+        load_x(stage, kb);
         if (++stage == p.stages) { stage = 0; phase ^= 1u; }
       }
     }
@@ -201,7 +230,7 @@ gemm_fp8_skinny_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
         const uint32_t sx = sw + BM * BK;
 #pragma unroll
         for (int k = 0; k < BK / UMMA_K; ++k) {
-          const uint64_t adesc = make_smem_desc(sw + k * UMMA_K, BK * 128), bdesc = make_smem_desc(sx + k * UMMA_K, BK * 128);
+          const uint64_t adesc = make_smem_desc(sw + (W_MN ? k * UMMA_K * 128 : k * UMMA_K), BK * 128), bdesc = make_smem_desc(sx + k * UMMA_K, BK * 128);
           if (I8) umma_i8(tmem_base, adesc, bdesc, p.idesc, (uint32_t)(kb != kb0 || k != 0));
           else umma_f8(tmem_base, adesc, bdesc, p.idesc, (uint32_t)(kb != kb0 || k != 0));
         }
@@ -214,57 +243,43 @@ gemm_fp8_skinny_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
     // ------------------------------------------------------------ epilogue (warps 2..5)
     chain_wait();
     const int quarter = warp & 3;  // tensor-memory lanes [32*quarter, 32*quarter+32) belong to this warp
-    const int col = n0 + quarter * 32 + lane;  // output column of this lane (= row of W)
-    const float alpha = I8 ? __ldg(p.col_scale + (p.col_scale_per_col ? min(col, p.N - 1) : 0))
-                           : dequant_alpha(p.sx_inv, p.sw_inv, p.sx_is_scale);
     if (mbar_wait(done_bar, 0, abort_flag)) {
       tc_fence_after();
       const uint32_t tacc = tmem_base + ((uint32_t)(quarter * 32) << 16);
-      if (p.slices == 1) {
-        for (int c = 0; c < p.Mpad; c += 16) {
-          uint32_t r[16];
-          tmem_ld16(tacc + (uint32_t)c, r);
-          tmem_ld_wait();
-          if (col < p.N) {
+      // park the sums in this CTA's shared memory: [token][128 columns] fp32 (the operand ring is
+      // free: the accumulator-complete signal comes after the last MMA has read it)
+      const uint32_t park = smem_base + (uint32_t)(quarter * 32 + lane) * 4u;
+      for (int c = 0; c < tokens; c += 16) {
+        uint32_t r[16];
+        tmem_ld16(tacc + (uint32_t)c, r);
+        tmem_ld_wait();
 #pragma unroll
-            for (int j = 0; j < 16; ++j)
-              if (c + j < p.M)
-                p.y[(int64_t)(c + j) * p.ldy + col] = (uint16_t)f32_to_bf16_bits(skinny_out<I8>(p, r[j], c + j, alpha));
-          }
-        }
-      } else {
-        // park the partial sums in this CTA's shared memory: [token][128 columns] fp32 (the operand ring is
-        // free: the accumulator-complete signal comes after the last MMA has read it)
-        const uint32_t park = smem_base + (uint32_t)(quarter * 32 + lane) * 4u;
-        for (int c = 0; c < p.Mpad; c += 16) {
-          uint32_t r[16];
-          tmem_ld16(tacc + (uint32_t)c, r);
-          tmem_ld_wait();
-#pragma unroll
-          for (int j = 0; j < 16; ++j)
-            asm volatile("st.shared.b32 [%0], %1;" ::"r"(park + (uint32_t)(c + j) * 512u), "r"(r[j]) : "memory");
-        }
+        for (int j = 0; j < 16; ++j)
+          asm volatile("st.shared.b32 [%0], %1;" ::"r"(park + (uint32_t)(c + j) * 512u), "r"(r[j]) : "memory");
       }
     }
   }
 
-  if (p.slices > 1) {
-    // every thread of every CTA of the cluster gets here, whatever happened above
-    cluster_sync_all();  // all partial sums are parked and visible
-    if (warp >= 2) {
-      const int quarter = warp & 3;
-      const int col = quarter * 32 + lane;
-      const int n = n0 + col;
-      const float alpha = I8 ? __ldg(p.col_scale + (p.col_scale_per_col ? min(n, p.N - 1) : 0))
-                             : dequant_alpha(p.sx_inv, p.sw_inv, p.sx_is_scale);
-      const uint32_t mine = smem_base + (uint32_t)col * 4u;
-      // 64 remote loads in flight per thread whatever the slice count: 8, 16 or 32 tokens at a time
-      if (p.slices > 4) skinny_reduce<I8, 8, 8>(p, mine, slice, n, alpha);
-      else if (p.slices > 2) skinny_reduce<I8, 16, 4>(p, mine, slice, n, alpha);
-      else skinny_reduce<I8, 32, 2>(p, mine, slice, n, alpha);
+  // every thread of every CTA of the cluster gets here, whatever happened above
+  if (p.slices > 1) cluster_sync_all();  // all partial sums are parked and visible
+  else __syncthreads();
+  if (warp >= 2) {
+    const int n = n0 + 4 * lane;
+    float alpha[4];
+    if (I8) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) alpha[j] = __ldg(p.col_scale + (p.col_scale_per_col ? min(n + j, p.N - 1) : 0));
+    } else {
+      alpha[0] = alpha[1] = alpha[2] = alpha[3] = dequant_alpha(p.sx_inv, p.sw_inv, p.sx_is_scale);
     }
-    cluster_sync_all();  // nobody leaves while a peer may still read its shared memory
+    const uint32_t mine = smem_base + (uint32_t)lane * 16u;
+    // 16 loads of 16 bytes in flight per lane whatever the slice count
+    if (p.slices > 4) skinny_reduce<I8, 2, 8>(p, mine, slice, warp - 2, n, m0, tokens, alpha);
+    else if (p.slices > 2) skinny_reduce<I8, 4, 4>(p, mine, slice, warp - 2, n, m0, tokens, alpha);
+    else if (p.slices > 1) skinny_reduce<I8, 8, 2>(p, mine, slice, warp - 2, n, m0, tokens, alpha);
+    else skinny_reduce<I8, 8, 1>(p, mine, slice, warp - 2, n, m0, tokens, alpha);
   }
+  if (p.slices > 1) cluster_sync_all();  // nobody leaves while a peer may still read its shared memory
 
   tc_fence_before();
   __syncthreads();

@@ -14,6 +14,7 @@
 // next call (so no reset kernel).  A linear layer's three casts (X, W, dY) then cost two
 // launches instead of nine, which matters because the tensors of a transformer block are
 // small enough for launch cost to rival streaming time.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -163,6 +164,41 @@ cast_kernel(const uint16_t* x, int64_t n, float* scale, float* scale_inv, float*
   if (GIVEN) cta_amax_to_global(absmax_f32_bits(m0, m1), amax);
 }
 
+// The codes alone, with a given scale: the activations of a static linear, whose amax nobody reads.  One launch instead
+// of a reset and a cast.
+template <int FMT, int U>
+__global__ void __launch_bounds__(kThreads) cast_codes_kernel(const uint16_t* x, int64_t n, const float* scale, uint8_t* q) {
+  chain_wait();
+  chain_release();   // in this order: when the next kernel starts, those before this one have completed
+  const float s = __ldg(scale);
+  const int64_t n16 = n >> 4;
+  const uint4* xv = reinterpret_cast<const uint4*>(x);
+  uint4* qv = reinterpret_cast<uint4*>(q);
+  const int64_t stride = (int64_t)gridDim.x * kThreads * U;
+  uint32_t sat = 0;
+  float m0 = 0.0f, m1 = 0.0f;
+  for (int64_t base = (int64_t)blockIdx.x * kThreads * U + threadIdx.x; base < n16; base += stride) {
+    uint4 v[U][2];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t i = base + (int64_t)u * kThreads;
+      if (i < n16) {
+        v[u][0] = __ldcs(xv + 2 * i);
+        v[u][1] = __ldcs(xv + 2 * i + 1);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t i = base + (int64_t)u * kThreads;
+      if (i < n16) qv[i] = cast16<FMT, false, false>(v[u][0], v[u][1], s, sat, m0, m1);
+    }
+  }
+  if (blockIdx.x == 0 && threadIdx.x < 16) {  // ragged tail: n % 16 elements
+    const int64_t i = (n16 << 4) + threadIdx.x;
+    if (i < n) q[i] = (uint8_t)(cvt_fp8x2<FMT>(__fmul_rn(bf16lo_to_f32((uint32_t)x[i]), s), 0.0f) & 0xFFu);
+  }
+}
+
 // ---------------------------------------------------------------------------------------
 // Batched form with a workspace (CURRENT scaling): no reset kernel and no atomics.
 //   kernel 1: every CTA writes the maximum of its share of each tensor to its own workspace
@@ -178,7 +214,7 @@ struct QTensor {
   float* scale_inv;
   float* amax;
   int32_t fmt;
-  int32_t pad;
+  int32_t mode;
 };
 struct QBatch {
   QTensor t[TWEO_MAX_QUANT_BATCH];
@@ -350,7 +386,129 @@ __global__ void __launch_bounds__(kThreads) cast_given_batch_kernel(const __grid
   }
 }
 
+// ---------------------------------------------------------------------------------------
+// Small tensors, either kind of scale, up to TWEO_MAX_QUANT_BATCH in ONE launch and without a workspace: a cluster of
+// eight CTAs per tensor, whose maxima meet through distributed shared memory.  At these sizes the launches are the cost
+// (2 to 4 us each in a chain, two to four of them in the other forms), not the bytes: eight SMs read a tensor twice, the
+// second time from L1 or L2.
+constexpr int kSmallCluster = 8;
+constexpr int kSmallThreads = 512;
+
+template <int FMT, bool AMAX>
+__device__ __forceinline__ void small_cast_share(const QTensor& t, float s, int rank, float& m0, float& m1) {
+  const int64_t n16 = t.n >> 4;
+  const uint4* xv = reinterpret_cast<const uint4*>(t.x);
+  uint4* qv = reinterpret_cast<uint4*>(t.q);
+  uint32_t sat = 0;
+  constexpr int stride = kSmallCluster * kSmallThreads;
+  for (int64_t i = rank * kSmallThreads + threadIdx.x; i < n16; i += 2 * stride) {
+    const int64_t j = i + stride;
+    const uint4 a0 = __ldg(xv + 2 * i), b0 = __ldg(xv + 2 * i + 1);
+    uint4 a1 = a0, b1 = b0;
+    if (j < n16) {
+      a1 = __ldg(xv + 2 * j);
+      b1 = __ldg(xv + 2 * j + 1);
+    }
+    qv[i] = cast16<FMT, false, AMAX>(a0, b0, s, sat, m0, m1);
+    if (j < n16) qv[j] = cast16<FMT, false, AMAX>(a1, b1, s, sat, m0, m1);
+  }
+  if (rank == 0 && threadIdx.x < 16) {  // ragged tail: n % 16 elements
+    const int64_t i = (n16 << 4) + threadIdx.x;
+    if (i < t.n) {
+      const uint32_t w = t.x[i];
+      t.q[i] = (uint8_t)(cvt_fp8x2<FMT>(__fmul_rn(bf16lo_to_f32(w), s), 0.0f) & 0xFFu);
+      if (AMAX) absmax_f32(m0, m1, w);
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kSmallThreads) small_cast_kernel(const __grid_constant__ QBatch b) {
+  namespace cg = cooperative_groups;
+  __shared__ uint32_t part[kSmallThreads / 32];
+  __shared__ uint32_t mine;
+  cg::cluster_group cluster = cg::this_cluster();
+  chain_release();
+  chain_wait();
+  const int ti = blockIdx.x / kSmallCluster;
+  const int rank = blockIdx.x - ti * kSmallCluster;
+  const QTensor& t = b.t[ti];
+  const bool given = t.mode == TWEO_SCALE_GIVEN;   // uniform over the cluster
+  float m0 = 0.0f, m1 = 0.0f;
+  float s = 1.0f;
+  if (given) {
+    s = *t.scale;
+    if (t.fmt == TWEO_E4M3) small_cast_share<TWEO_E4M3, true>(t, s, rank, m0, m1);
+    else small_cast_share<TWEO_E5M2, true>(t, s, rank, m0, m1);
+  } else {
+    const int64_t n16 = t.n >> 4;
+    const uint4* xv = reinterpret_cast<const uint4*>(t.x);
+    constexpr int stride = kSmallCluster * kSmallThreads;
+    for (int64_t i = rank * kSmallThreads + threadIdx.x; i < n16; i += 2 * stride) {
+      const int64_t j = i + stride < n16 ? i + stride : i;
+      const uint4 v[4] = {__ldg(xv + 2 * i), __ldg(xv + 2 * i + 1), __ldg(xv + 2 * j), __ldg(xv + 2 * j + 1)};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        absmax_f32(m0, m1, v[u].x);
+        absmax_f32(m0, m1, v[u].y);
+        absmax_f32(m0, m1, v[u].z);
+        absmax_f32(m0, m1, v[u].w);
+      }
+    }
+    if (rank == 0 && threadIdx.x < 16) {
+      const int64_t i = (n16 << 4) + threadIdx.x;
+      if (i < t.n) absmax_f32(m0, m1, (uint32_t)t.x[i]);
+    }
+  }
+  uint32_t m = __reduce_max_sync(0xFFFFFFFFu, absmax_f32_bits(m0, m1));
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    m = __reduce_max_sync(0xFFFFFFFFu, threadIdx.x < kSmallThreads / 32 ? part[threadIdx.x] : 0u);
+    if (threadIdx.x == 0) mine = m;
+  }
+  cluster.sync();
+  if (threadIdx.x < 32) {
+    m = __reduce_max_sync(0xFFFFFFFFu, threadIdx.x < kSmallCluster ? *cluster.map_shared_rank(&mine, threadIdx.x) : 0u);
+    if (threadIdx.x == 0) part[0] = m;
+  }
+  __syncthreads();
+  const float amax = __uint_as_float(part[0] << 16);   // non-negative bf16 pattern -> binary32
+  if (!given) s = scale_from_amax(amax, t.fmt);
+  if (rank == 0 && threadIdx.x == 0) {
+    *t.amax = amax;
+    if (!given) *t.scale = s;
+    *t.scale_inv = __fdiv_rn(1.0f, s);
+  }
+  if (!given) {
+    if (t.fmt == TWEO_E4M3) small_cast_share<TWEO_E4M3, false>(t, s, rank, m0, m1);
+    else small_cast_share<TWEO_E5M2, false>(t, s, rank, m0, m1);
+  }
+  cluster.sync();   // nobody leaves while a peer may still read its maximum
+}
+
 int grid_for(int64_t work_items, int per_cta, int ctas_per_sm);
+
+// Where one cluster per tensor is the faster form (see launch_small's measurements).
+constexpr int64_t kSmallElems = 1 << 19;
+
+bool all_small(const tweo_quant_desc_t* descs, int count) {
+  for (int i = 0; i < count; ++i)
+    if (descs[i].n > kSmallElems || descs[i].sat_count) return false;
+  return true;
+}
+
+tweo_status_t launch_small(const tweo_quant_desc_t* descs, int count, cudaStream_t st) {
+  QBatch b;
+  b.count = count;
+  b.amax_grid = 0;
+  for (int i = 0; i < count; ++i) {
+    const tweo_quant_desc_t& d = descs[i];
+    b.t[i] = QTensor{d.x, d.q, d.n, d.scale, d.scale_inv, d.amax, d.fmt, d.mode};
+  }
+  TWEO_CUDA_TRY(launch_chain(small_cast_kernel, dim3((unsigned)(kSmallCluster * count)), dim3(kSmallThreads), 0, st, kSmallCluster, b));
+  count_launch();
+  return check_launch("small_cast_kernel");
+}
 
 // Launches the batched form for descs[idx[0..count)] (all CURRENT scaling, no saturation count).
 tweo_status_t launch_batch(const tweo_quant_desc_t* descs, const int* idx, int count, void* ws, cudaStream_t st) {
@@ -359,7 +517,7 @@ tweo_status_t launch_batch(const tweo_quant_desc_t* descs, const int* idx, int c
   int64_t vec8 = 0, vec16[2] = {0, 0};
   for (int i = 0; i < count; ++i) {
     const tweo_quant_desc_t& d = descs[idx[i]];
-    b.t[i] = QTensor{d.x, d.q, d.n, d.scale, d.scale_inv, d.amax, d.fmt, 0};
+    b.t[i] = QTensor{d.x, d.q, d.n, d.scale, d.scale_inv, d.amax, d.fmt, d.mode};
     vec8 += d.n >> 3;
     vec16[d.fmt] += d.n >> 4;
   }
@@ -403,7 +561,7 @@ tweo_status_t launch_given_batch(const tweo_quant_desc_t* descs, const int* idx,
   int64_t vec16[2] = {0, 0};
   for (int i = 0; i < count; ++i) {
     const tweo_quant_desc_t& d = descs[idx[i]];
-    b.t[i] = QTensor{d.x, d.q, d.n, d.scale, d.scale_inv, d.amax, d.fmt, 0};
+    b.t[i] = QTensor{d.x, d.q, d.n, d.scale, d.scale_inv, d.amax, d.fmt, d.mode};
     vec16[d.fmt] += d.n >> 4;
   }
   TWEO_CUDA_TRY(launch_chain(init_batch_kernel, dim3(1), dim3(32), 0, st, 0, b));
@@ -486,6 +644,7 @@ tweo_status_t quantize_many(const tweo_quant_desc_t* descs, int count, void* ws,
     tweo_status_t s = check_desc(descs[i]);
     if (s != TWEO_OK) return s;
   }
+  if (all_small(descs, count)) return launch_small(descs, count, st);
   const bool have_ws = ws && ws_bytes >= kBatchWsBytes && aligned16(ws);
   int idx[TWEO_MAX_QUANT_BATCH], idxg[TWEO_MAX_QUANT_BATCH];
   int nb = 0, ng = 0;
@@ -522,6 +681,19 @@ tweo_status_t launch_amax_prologue(const uint16_t* x, int64_t n, float* amax, ui
     count_launch();
   }
   return TWEO_OK;
+}
+
+// E4M3 codes of x with a given scale, nothing else (see cast_codes_kernel).
+tweo_status_t launch_cast_codes(const uint16_t* x, int64_t n, const float* scale, uint8_t* q, cudaStream_t st) {
+  const int64_t n16 = n >> 4;
+  if (n16 >= 2 * (int64_t)sm_count() * 8 * kThreads * 4)
+    TWEO_CUDA_TRY(launch_chain(cast_codes_kernel<TWEO_E4M3, 4>, dim3(grid_for(n16, kThreads * 4, 8)), dim3(kThreads), 0, st, 0, x, n, scale, q));
+  else if (n16 >= (int64_t)sm_count() * 8 * kThreads)
+    TWEO_CUDA_TRY(launch_chain(cast_codes_kernel<TWEO_E4M3, 2>, dim3(grid_for(n16, kThreads * 2, 8)), dim3(kThreads), 0, st, 0, x, n, scale, q));
+  else   // less than a sweep of the chip: one group of 16 per thread, on as many SMs as there are
+    TWEO_CUDA_TRY(launch_chain(cast_codes_kernel<TWEO_E4M3, 1>, dim3(grid_for(n16, kThreads, 8)), dim3(kThreads), 0, st, 0, x, n, scale, q));
+  count_launch();
+  return check_launch("cast_codes_kernel");
 }
 
 size_t quantize_workspace_bytes() { return kBatchWsBytes; }

@@ -4,10 +4,11 @@
 #include "common.cuh"
 
 namespace tweo_detail {
+tweo_status_t launch_cast_codes(const uint16_t* x, int64_t n, const float* scale, uint8_t* q, cudaStream_t st);
 tweo_status_t gemm_fwd_codes(const uint8_t* xq, int64_t ldx, int fmt_x, const uint8_t* wq, int64_t ldw, int fmt_w,
                              const float* sx_inv, const float* sw_inv, uint16_t* y, int64_t ldy, int64_t M,
                              int64_t N, int64_t K, const tweo_epilogue_t* epi, void* ws, size_t ws_bytes,
-                             cudaStream_t st, bool sx_is_scale);
+                             cudaStream_t st, bool sx_is_scale, bool inference, bool w_early);
 }
 
 extern "C" tweo_status_t tweo_w8a8_static_gemm(const void* x, int32_t x_dtype, int64_t ldx, const float* sx,
@@ -23,7 +24,6 @@ extern "C" tweo_status_t tweo_w8a8_static_gemm(const void* x, int32_t x_dtype, i
   if (!ws || ws_bytes < tweo_workspace_bytes(TWEO_OP_W8A8, M, N, K)) return TWEO_ERR_WORKSPACE_TOO_SMALL;
   if (!aligned16(ws) || !aligned16(x)) return TWEO_ERR_ALIGNMENT;
   cudaStream_t st = (cudaStream_t)stream;
-  float* scalars = reinterpret_cast<float*>(ws);  // [0] = 1/sx, [1] = amax of x (by-product), [2] = scale_inv scratch
   const uint8_t* xq;
   int64_t ldxq;
   if (x_dtype == TWEO_BF16) {
@@ -32,20 +32,19 @@ extern "C" tweo_status_t tweo_w8a8_static_gemm(const void* x, int32_t x_dtype, i
       return TWEO_ERR_UNSUPPORTED_SHAPE;
     }
     uint8_t* codes = reinterpret_cast<uint8_t*>(ws) + 256;
-    tweo_status_t s = tweo_quantize_per_tensor(reinterpret_cast<const uint16_t*>(x), M * K, TWEO_E4M3,
-                                               TWEO_SCALE_GIVEN, const_cast<float*>(sx), scalars, scalars + 1,
-                                               codes, nullptr, nullptr, 0, stream);
+    tweo_status_t s = launch_cast_codes(reinterpret_cast<const uint16_t*>(x), M * K, sx, codes, st);
     if (s != TWEO_OK) return s;
     xq = codes;
     ldxq = K;
   } else {
-    xq = reinterpret_cast<const uint8_t*>(x);   // the GEMM's epilogue forms 1 / *sx itself: no extra launch
+    xq = reinterpret_cast<const uint8_t*>(x);
     ldxq = ldx;
   }
-  // what follows the scalars and the codes serves the GEMM's stream-K fix-up
+  // what follows the codes serves the GEMM's stream-K fix-up; its epilogue forms 1 / *sx itself: no extra launch
   size_t used = 256;
   if (x_dtype == TWEO_BF16) used += ((size_t)M * (size_t)K + 255) & ~(size_t)255;
-  const bool pre_cast = x_dtype != TWEO_BF16;
-  return gemm_fwd_codes(xq, ldxq, TWEO_E4M3, wq, ldw, TWEO_E4M3, pre_cast ? sx : scalars, sw_inv, y, ldy, M, N, K, nullptr,
-                        reinterpret_cast<char*>(ws) + used, ws_bytes - used, st, pre_cast);
+  // With the cast of this call in between, every kernel enqueued before the call has completed when the product starts
+  // (cast_codes_kernel lets it start only then): W can be loaded without waiting for the cast.
+  return gemm_fwd_codes(xq, ldxq, TWEO_E4M3, wq, ldw, TWEO_E4M3, sx, sw_inv, y, ldy, M, N, K, nullptr,
+                        reinterpret_cast<char*>(ws) + used, ws_bytes - used, st, true, true, x_dtype == TWEO_BF16);
 }
