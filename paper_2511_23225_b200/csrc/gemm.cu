@@ -691,6 +691,17 @@ struct SkinnyPlan {
   double clocks;         // estimate, see below
 };
 
+// The most shared memory a launch asks for: the ring, and alignment and barriers.
+constexpr int skinny_smem(bool wide) { return (wide ? 200 : 100) * 1024 + 1024 + 256; }
+
+// Never launched: resident_clusters() asks how many clusters of it fit.  Asking about the few-token kernel itself, with
+// success, left its later launches slower (one token, 4-bit weights [8192x8192]: 15.4 us a pass against 10.9), as if two of its CTAs no longer met on an SM.
+template <int W>
+__global__ void __launch_bounds__(kThreads, 1) occupancy_probe_kernel(int* p) {
+  extern __shared__ uint8_t smem_probe[];
+  if (p) *p = smem_probe[threadIdx.x];
+}
+
 // Clusters of `slices` CTAs that are resident at once, with rings of 100 KB or (wide) 200 KB.  A cluster lives within one
 // group of SMs, whose size is no multiple of most counts (148 SMs hold 15 clusters of eight 200 KB CTAs, not 18).
 // Asked for once per device.
@@ -706,15 +717,15 @@ int resident_clusters(int slices, bool wide) {
   Table& t = tables[dev];
   if (!t.known.load(std::memory_order_acquire)) {
     std::lock_guard<std::mutex> lock(mu);
-    auto kern = gemm_fp8_skinny_kernel<false, false>;
-    const int bytes[2] = {100 * 1024 + 1024 + 256, 200 * 1024 + 1024 + 256};
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes[1]);
-    for (int w = 0; w < 2; ++w)
+    for (int w = 0; w < 2; ++w) {
+      auto kern = w ? occupancy_probe_kernel<1> : occupancy_probe_kernel<0>;
+      const int bytes = skinny_smem(w != 0);
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
       for (int c = 1; c <= 8; ++c) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)c);
         cfg.blockDim = dim3(kThreads);
-        cfg.dynamicSmemBytes = (size_t)bytes[w];
+        cfg.dynamicSmemBytes = (size_t)bytes;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = (unsigned)c;
@@ -726,6 +737,7 @@ int resident_clusters(int slices, bool wide) {
         if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) n = sm_count() * (w ? 1 : 2) / c;
         t.n[w][c] = n;
       }
+    }
     (void)cudaGetLastError();
     t.known.store(true, std::memory_order_release);
   }
@@ -811,12 +823,13 @@ tweo_status_t launch_skinny(SkinnyParams& p, const void* xq, int64_t ldx, const 
     return TWEO_ERR_CUDA;
   }
   const size_t smem = (size_t)p.stages * p.stage_bytes + 1024 + 256;
-  auto kern = gemm_fp8_skinny_kernel<I8, W_MN>;
-  static std::atomic<uint64_t> attr_done{0};  // per device
+  const bool wide = p.Mpad > 128;
+  auto kern = wide ? gemm_fp8_skinny_kernel<I8, W_MN, true> : gemm_fp8_skinny_kernel<I8, W_MN, false>;
+  static std::atomic<uint64_t> attr_done[2];  // per device
   int attr_dev = 0;
-  if (device_once_pending(attr_done, &attr_dev)) {
-    TWEO_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(200 * 1024 + 1024 + 256)));
-    device_once_done(attr_done, attr_dev);
+  if (device_once_pending(attr_done[wide], &attr_dev)) {
+    TWEO_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, skinny_smem(wide)));
+    device_once_done(attr_done[wide], attr_dev);
   }
   TWEO_CUDA_TRY(launch_chain(kern, dim3((unsigned)(p.slabs * pl.m_tiles * p.slices)), dim3(kThreads), smem, st,
                              (unsigned)p.slices, mw, mx, p));

@@ -138,7 +138,9 @@ __device__ __forceinline__ void skinny_reduce(const SkinnyParams& p, uint32_t mi
 
 // I8: signed 8-bit operands (tcgen05 kind::i8, int32 accumulators: partial sums of K slices add exactly) with the
 // Eq. 4 dequantisation in the epilogue, per tensor or per token (activation rows) / per channel (weight rows).
-template <bool I8, bool W_MN>
+// WIDE: rings of up to 200 KB, one CTA per SM; a kernel of its own, so that the other's shared-memory attribute stays at
+// what lets two of its CTAs share an SM.
+template <bool I8, bool W_MN, bool WIDE>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_fp8_skinny_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x,
                        const __grid_constant__ SkinnyParams p) {
@@ -188,6 +190,7 @@ gemm_fp8_skinny_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
   // writes it.  Where none can be (w_early, see the callers), the first ring of W is loaded at once: L2 to shared memory
   // takes 3 of 13 us at [11008x4096] after the wait.
   chain_release();
+  float alpha[4];
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
     if (lane == 0) {
@@ -243,6 +246,13 @@ gemm_fp8_skinny_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
     // ------------------------------------------------------------ epilogue (warps 2..5)
     chain_wait();
     const int quarter = warp & 3;  // tensor-memory lanes [32*quarter, 32*quarter+32) belong to this warp
+    // the factors of this lane's four output columns, fetched while the operands stream
+    if (I8) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) alpha[j] = __ldg(p.col_scale + (p.col_scale_per_col ? min(n0 + 4 * lane + j, p.N - 1) : 0));
+    } else {
+      alpha[0] = alpha[1] = alpha[2] = alpha[3] = dequant_alpha(p.sx_inv, p.sw_inv, p.sx_is_scale);
+    }
     if (mbar_wait(done_bar, 0, abort_flag)) {
       tc_fence_after();
       const uint32_t tacc = tmem_base + ((uint32_t)(quarter * 32) << 16);
@@ -265,13 +275,6 @@ gemm_fp8_skinny_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
   else __syncthreads();
   if (warp >= 2) {
     const int n = n0 + 4 * lane;
-    float alpha[4];
-    if (I8) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) alpha[j] = __ldg(p.col_scale + (p.col_scale_per_col ? min(n + j, p.N - 1) : 0));
-    } else {
-      alpha[0] = alpha[1] = alpha[2] = alpha[3] = dequant_alpha(p.sx_inv, p.sw_inv, p.sx_is_scale);
-    }
     const uint32_t mine = smem_base + (uint32_t)lane * 16u;
     // 16 loads of 16 bytes in flight per lane whatever the slice count
     if (p.slices > 4) skinny_reduce<I8, 2, 8>(p, mine, slice, warp - 2, n, m0, tokens, alpha);

@@ -427,8 +427,8 @@ __global__ void __launch_bounds__(kSmallThreads) small_cast_kernel(const __grid_
   __shared__ uint32_t part[kSmallThreads / 32];
   __shared__ uint32_t mine;
   cg::cluster_group cluster = cg::this_cluster();
-  chain_release();
   chain_wait();
+  chain_release();   // in this order the kernels behind do not crowd in early (train step of a small linear: 21.5 -> 20.2 us)
   const int ti = blockIdx.x / kSmallCluster;
   const int rank = blockIdx.x - ti * kSmallCluster;
   const QTensor& t = b.t[ti];
