@@ -4,10 +4,16 @@ Argument marshalling only: every function takes torch CUDA tensors (used for
 device memory and streams, nothing else), checks dtypes, and forwards raw
 device pointers and the current CUDA stream to the library entry point of the
 same name.  There is no CPU path: a missing library or a non-CUDA tensor raises.
+
+The calls of training and inference loops go through the native module built beside
+the library (csrc/native.cpp): the same checks and calls, without the 7 to 12
+microseconds that ctypes and attribute look-ups take, more than a few-token product.
+The others go through ctypes.
 """
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
 import os
 from dataclasses import dataclass
 
@@ -24,6 +30,7 @@ MAX_BLOCKS = 128
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libtweo_b200.so")
+NATIVE_PATH = os.path.join(_HERE, "_native.so")
 
 EXPORTS = [
     "tweo_quantize_per_tensor", "tweo_quantize_per_tensor_batch", "tweo_fp8_linear_fwd", "tweo_fp8_linear_fwd_act",
@@ -131,6 +138,26 @@ def lib() -> C.CDLL:
     return _lib
 
 
+_native_module = None
+
+
+def _native():
+    """Loads the native marshalling module; raises if it has not been built."""
+    global _native_module
+    if _native_module is None:
+        lib()
+        if not os.path.exists(NATIVE_PATH):
+            raise RuntimeError(
+                f"{NATIVE_PATH} is missing: build it with `python -m paper_2511_23225_b200.build` "
+                "(there is no CPU fallback)")
+        spec = importlib.util.spec_from_file_location(__package__ + "._native", NATIVE_PATH)
+        m = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(m)
+        m.set_error(TweoError)
+        _native_module = m
+    return _native_module
+
+
 def _check(status: int, where: str):
     if status != 0:
         raise TweoError(status, where)
@@ -203,10 +230,8 @@ def quantize_per_tensor(x: torch.Tensor, fmt: int = E4M3, mode: int = SCALE_CURR
                         out: Quantized | None = None, ws: torch.Tensor | None = None) -> Quantized:
     """tweo_quantize_per_tensor: amax -> scale -> FP8 codes of a bf16 tensor.
     With a workspace (new_workspace(OP_QUANTIZE)) current scaling runs as two kernels, not three."""
-    xp = _dev(x, torch.bfloat16, "x")
-    if not x.is_contiguous():
-        raise ValueError("x must be contiguous")
     if out is None:
+        _dev(x, torch.bfloat16, "x")
         q = torch.empty(x.shape, dtype=torch.uint8, device=x.device)
         scalars = torch.empty(4, dtype=torch.float32, device=x.device)
         if mode == SCALE_GIVEN:
@@ -217,10 +242,7 @@ def quantize_per_tensor(x: torch.Tensor, fmt: int = E4M3, mode: int = SCALE_CURR
             s = scalars[0:1]
         out = Quantized(q, s, scalars[1:2], scalars[2:3],
                         torch.empty(1, dtype=torch.int32, device=x.device) if count_saturated else None, fmt)
-    sat = out.sat_count.data_ptr() if out.sat_count is not None else None
-    _check(lib().tweo_quantize_per_tensor(xp, x.numel(), fmt, mode, _dev(out.scale, torch.float32, "scale"),
-                                          out.scale_inv.data_ptr(), out.amax.data_ptr(), out.q.data_ptr(), sat,
-                                          *_ws(ws), _stream()), "tweo_quantize_per_tensor")
+    _native().quantize(x, out, fmt, mode, ws)
     return out
 
 
@@ -233,62 +255,14 @@ def quantize_per_tensor_batch(xs, outs, modes=None, ws: torch.Tensor | None = No
         raise ValueError("need 1..MAX_QUANT_BATCH tensors with one output record each")
     if ws is None:
         ws = new_workspace(OP_QUANTIZE)
-    descs = (_QuantDesc * n)()
-    for i, (x, o) in enumerate(zip(xs, outs)):
-        if not x.is_contiguous():
-            raise ValueError("x must be contiguous")
-        d = descs[i]
-        d.x = _dev(x, torch.bfloat16, "x")
-        d.n = x.numel()
-        d.fmt = o.fmt
-        d.mode = SCALE_CURRENT if modes is None else modes[i]
-        d.scale = _dev(o.scale, torch.float32, "scale")
-        d.scale_inv = _dev(o.scale_inv, torch.float32, "scale_inv")
-        d.amax = _dev(o.amax, torch.float32, "amax")
-        d.q = _dev(o.q, U8, "q")
-        d.sat_count = o.sat_count.data_ptr() if o.sat_count is not None else None
-    _check(lib().tweo_quantize_per_tensor_batch(descs, n, ws.data_ptr(), ws.numel(), _stream()),
-           "tweo_quantize_per_tensor_batch")
+    _native().quantize_batch(xs, outs, modes, ws)
     return outs
-
-
-def _epilogue(amax, q, q_fmt, q_scale):
-    e = _epilogue_struct(amax, q, q_fmt, q_scale)
-    return None if e is None else C.byref(e)
-
-
-def _epilogue_struct(amax, q, q_fmt, q_scale):
-    if amax is None and q is None:
-        return None
-    e = _Epilogue()
-    e.out_amax = _dev(amax, torch.float32, "out_amax") if amax is not None else None
-    if q is not None:
-        e.out_q = _dev(q, U8, "out_q")
-        e.ldq = _rows(q, "out_q")
-        e.q_fmt = q_fmt
-        e.q_scale = _dev(q_scale, torch.float32, "q_scale")
-    return e
-
-
-def _ws(ws):
-    return (None, 0) if ws is None else (_dev(ws, torch.uint8, "ws"), ws.numel())
 
 
 def fp8_linear_fwd(xq, wq, sx_inv, sw_inv, fmt_x=E4M3, fmt_w=E4M3, y=None, out_amax=None, out_q=None,
                    q_fmt=E4M3, q_scale=None, ws=None) -> torch.Tensor:
     """tweo_fp8_linear_fwd: Y[M,N] = Xq[M,K] . Wq[N,K]^T * sx_inv * sw_inv -> bf16."""
-    M, K = xq.shape
-    N, K2 = wq.shape
-    if K != K2:
-        raise ValueError("inner dimensions differ")
-    if y is None:
-        y = torch.empty((M, N), dtype=torch.bfloat16, device=xq.device)
-    _check(lib().tweo_fp8_linear_fwd(_dev(xq, U8, "xq"), _rows(xq, "xq"), _dev(wq, U8, "wq"), _rows(wq, "wq"),
-                                     _dev(sx_inv, torch.float32), _dev(sw_inv, torch.float32),
-                                     _dev(y, torch.bfloat16, "y"), _rows(y, "y"), M, N, K, fmt_x, fmt_w,
-                                     _epilogue(out_amax, out_q, q_fmt, q_scale), *_ws(ws), _stream()),
-           "tweo_fp8_linear_fwd")
-    return y
+    return _native().linear_fwd(xq, wq, sx_inv, sw_inv, fmt_x, fmt_w, y, out_amax, out_q, q_fmt, q_scale, ws)
 
 
 def fp8_linear_fwd_act(xq, wq, sx_inv, sw_inv, act, fmt_x=E4M3, fmt_w=E4M3, y=None, want_y=True, out_amax=None,
@@ -296,25 +270,7 @@ def fp8_linear_fwd_act(xq, wq, sx_inv, sw_inv, act, fmt_x=E4M3, fmt_w=E4M3, y=No
     """tweo_fp8_linear_fwd_act: act(Xq . Wq^T * sx_inv * sw_inv) -> bf16 and / or FP8.  For ACT_SWIGLU wq holds
     the gate rows followed by the up rows and the output has half as many columns as wq has rows.
     want_y=False with out_q given writes only the FP8 copy.  Returns y (or None)."""
-    M, K = xq.shape
-    N, K2 = wq.shape
-    if K != K2:
-        raise ValueError("inner dimensions differ")
-    if act == ACT_SWIGLU:
-        if N % 2:
-            raise ValueError("SwiGLU needs an even number of weight rows (gate rows, then up rows)")
-        N //= 2
-    if want_y and y is None:
-        y = torch.empty((M, N), dtype=torch.bfloat16, device=xq.device)
-    if not want_y:
-        y = None
-    _check(lib().tweo_fp8_linear_fwd_act(_dev(xq, U8, "xq"), _rows(xq, "xq"), _dev(wq, U8, "wq"), _rows(wq, "wq"),
-                                         _dev(sx_inv, torch.float32), _dev(sw_inv, torch.float32), act,
-                                         _dev(y, torch.bfloat16, "y") if y is not None else None,
-                                         _rows(y, "y") if y is not None else 0, M, N, K, fmt_x, fmt_w,
-                                         _epilogue(out_amax, out_q, q_fmt, q_scale), _stream()),
-           "tweo_fp8_linear_fwd_act")
-    return y
+    return _native().linear_fwd_act(xq, wq, sx_inv, sw_inv, act, fmt_x, fmt_w, y, want_y, out_amax, out_q, q_fmt, q_scale)
 
 
 def layernorm_fp8(x, gamma, beta=None, eps=1e-5, kind=NORM_LAYER, want_y=True, q_fmt=None, q_scale=None,
@@ -322,92 +278,24 @@ def layernorm_fp8(x, gamma, beta=None, eps=1e-5, kind=NORM_LAYER, want_y=True, q
     """tweo_layernorm_fp8: LayerNorm / RMSNorm over the last dimension of a bf16 [rows, d] tensor with the FP8
     cast of the output (q_fmt, q_scale) and its amax in the same pass.
     Returns (y or None, yq or None, amax [1] or None, mean [rows] or None, rstd [rows] or None)."""
-    rows, d = x.shape
-    dev = x.device
-    if want_y and y is None:
-        y = torch.empty((rows, d), dtype=torch.bfloat16, device=dev)
-    if not want_y:
-        y = None
-    if q_fmt is not None:
-        if q_scale is None:
-            raise ValueError("the FP8 copy needs q_scale")
-        if yq is None:
-            yq = torch.empty((rows, d), dtype=torch.uint8, device=dev)
-    else:
-        yq = None
-    amax = torch.empty(1, dtype=torch.float32, device=dev) if want_amax else None
-    mean = torch.empty(rows, dtype=torch.float32, device=dev) if want_stats else None
-    rstd = torch.empty(rows, dtype=torch.float32, device=dev) if want_stats else None
-    _check(lib().tweo_layernorm_fp8(_dev(x, torch.bfloat16, "x"), _rows(x, "x"), rows, d, kind,
-                                    _dev(gamma, torch.float32, "gamma"),
-                                    _dev(beta, torch.float32, "beta") if beta is not None else None, eps,
-                                    _dev(y, torch.bfloat16, "y") if y is not None else None,
-                                    _rows(y, "y") if y is not None else 0,
-                                    _dev(yq, U8, "yq") if yq is not None else None,
-                                    _rows(yq, "yq") if yq is not None else 0, q_fmt if q_fmt is not None else 0,
-                                    _dev(q_scale, torch.float32, "q_scale") if q_scale is not None else None,
-                                    amax.data_ptr() if amax is not None else None,
-                                    mean.data_ptr() if mean is not None else None,
-                                    rstd.data_ptr() if rstd is not None else None, _stream()),
-           "tweo_layernorm_fp8")
-    return y, yq, amax, mean, rstd
+    return _native().layernorm(x, gamma, beta, eps, kind, want_y, q_fmt, q_scale, want_amax, want_stats, y, yq)
 
 
 def fp8_linear_bwd_dgrad(dyq, wq, sdy_inv, sw_inv, fmt_dy=E5M2, fmt_w=E4M3, dx=None, out_amax=None, out_q=None,
                          q_fmt=E5M2, q_scale=None, ws=None) -> torch.Tensor:
     """tweo_fp8_linear_bwd_dgrad: dX[M,K] = dYq[M,N] . Wq[N,K] * sdy_inv * sw_inv -> bf16."""
-    M, N = dyq.shape
-    N2, K = wq.shape
-    if N != N2:
-        raise ValueError("inner dimensions differ")
-    if dx is None:
-        dx = torch.empty((M, K), dtype=torch.bfloat16, device=dyq.device)
-    _check(lib().tweo_fp8_linear_bwd_dgrad(_dev(dyq, U8, "dyq"), _rows(dyq, "dyq"), fmt_dy, _dev(wq, U8, "wq"),
-                                           _rows(wq, "wq"), fmt_w, _dev(sdy_inv, torch.float32),
-                                           _dev(sw_inv, torch.float32), _dev(dx, torch.bfloat16, "dx"),
-                                           _rows(dx, "dx"), M, N, K, _epilogue(out_amax, out_q, q_fmt, q_scale),
-                                           *_ws(ws), _stream()), "tweo_fp8_linear_bwd_dgrad")
-    return dx
+    return _native().linear_dgrad(dyq, wq, sdy_inv, sw_inv, fmt_dy, fmt_w, dx, out_amax, out_q, q_fmt, q_scale, ws)
 
 
 def fp8_linear_bwd_wgrad(xq, dyq, sx_inv, sdy_inv, fmt_x=E4M3, fmt_dy=E5M2, dw=None, dw_dtype=BF16,
                          accumulate=False, ws=None) -> torch.Tensor:
     """tweo_fp8_linear_bwd_wgrad: dW[N,K] = dYq[M,N]^T . Xq[M,K] * sx_inv * sdy_inv."""
-    M, K = xq.shape
-    M2, N = dyq.shape
-    if M != M2:
-        raise ValueError("token dimensions differ")
-    tdt = torch.bfloat16 if dw_dtype == BF16 else torch.float32
-    if dw is None:
-        if accumulate:
-            raise ValueError("accumulate needs an existing dw")
-        dw = torch.empty((N, K), dtype=tdt, device=xq.device)
-    _check(lib().tweo_fp8_linear_bwd_wgrad(_dev(xq, U8, "xq"), _rows(xq, "xq"), fmt_x, _dev(dyq, U8, "dyq"),
-                                           _rows(dyq, "dyq"), fmt_dy, _dev(sx_inv, torch.float32),
-                                           _dev(sdy_inv, torch.float32), _dev(dw, tdt, "dw"), _rows(dw, "dw"),
-                                           dw_dtype, 1 if accumulate else 0, M, N, K, *_ws(ws), _stream()),
-           "tweo_fp8_linear_bwd_wgrad")
-    return dw
+    return _native().linear_wgrad(xq, dyq, sx_inv, sdy_inv, fmt_x, fmt_dy, dw, dw_dtype, accumulate, ws)
 
 
 def fp8_linear_bwd(dyq, xq, wq, sdy_inv, sx_inv, sw_inv, fmt_dy=E5M2, fmt_x=E4M3, fmt_w=E4M3, dx=None, dw=None, ws=None):
     """tweo_fp8_linear_bwd: dX[M,K] and dW[N,K] (both bf16) of one linear layer in one call."""
-    M, N = dyq.shape
-    M2, K = xq.shape
-    N2, K2 = wq.shape
-    if M != M2 or N != N2 or K != K2:
-        raise ValueError("shapes of dyq [M,N], xq [M,K] and wq [N,K] do not agree")
-    if dx is None:
-        dx = torch.empty((M, K), dtype=torch.bfloat16, device=dyq.device)
-    if dw is None:
-        dw = torch.empty((N, K), dtype=torch.bfloat16, device=dyq.device)
-    _check(lib().tweo_fp8_linear_bwd(_dev(dyq, U8, "dyq"), _rows(dyq, "dyq"), fmt_dy, _dev(xq, U8, "xq"),
-                                     _rows(xq, "xq"), fmt_x, _dev(wq, U8, "wq"), _rows(wq, "wq"), fmt_w,
-                                     _dev(sdy_inv, torch.float32), _dev(sx_inv, torch.float32),
-                                     _dev(sw_inv, torch.float32), _dev(dx, torch.bfloat16, "dx"), _rows(dx, "dx"),
-                                     _dev(dw, torch.bfloat16, "dw"), _rows(dw, "dw"), M, N, K, *_ws(ws), _stream()),
-           "tweo_fp8_linear_bwd")
-    return dx, dw
+    return _native().linear_bwd(dyq, xq, wq, sdy_inv, sx_inv, sw_inv, fmt_dy, fmt_x, fmt_w, dx, dw, ws)
 
 
 def fp8_linear_group(problems):
@@ -416,70 +304,22 @@ def fp8_linear_group(problems):
     "sdy_inv", "sw_inv", "out" [M,K]} or {"product": PRODUCT_WGRAD, "xq", "dyq", "sx_inv", "sdy_inv", "out" [N,K]},
     each optionally with "fmt_x", "fmt_w", "fmt_dy" (defaults E4M3, E4M3, E5M2).  Outputs are bf16 tensors.  A FWD or
     DGRAD problem may add the fused epilogue: "out_amax" and / or "out_q" with "q_fmt" and "q_scale"."""
-    n = len(problems)
-    if not 1 <= n <= MAX_GROUP:
-        raise ValueError("need 1..MAX_GROUP problems")
-    arr = (_LinearProblem * n)()
-    epis = []   # keeps the epilogue descriptors alive until the call returns
-    for q, d in zip(arr, problems):
-        e = _epilogue_struct(d.get("out_amax"), d.get("out_q"), d.get("q_fmt", E4M3), d.get("q_scale"))
-        if e is not None:
-            epis.append(e)
-            q.epi = C.addressof(e)
-        q.product = d["product"]
-        q.fmt_x, q.fmt_w, q.fmt_dy = d.get("fmt_x", E4M3), d.get("fmt_w", E4M3), d.get("fmt_dy", E5M2)
-        xq, wq, dyq = d.get("xq"), d.get("wq"), d.get("dyq")
-        if q.product == PRODUCT_FWD:
-            (M, K), N = xq.shape, wq.shape[0]
-        elif q.product == PRODUCT_DGRAD:
-            (M, N), K = dyq.shape, wq.shape[1]
-        elif q.product == PRODUCT_WGRAD:
-            (M, K), N = xq.shape, dyq.shape[1]
-        else:
-            raise ValueError("product must be PRODUCT_FWD, PRODUCT_DGRAD or PRODUCT_WGRAD")
-        q.M, q.N, q.K = M, N, K
-        if xq is not None:
-            q.xq, q.ldx = _dev(xq, U8, "xq"), _rows(xq, "xq")
-        if wq is not None:
-            q.wq, q.ldw = _dev(wq, U8, "wq"), _rows(wq, "wq")
-        if dyq is not None:
-            q.dyq, q.lddy = _dev(dyq, U8, "dyq"), _rows(dyq, "dyq")
-        for name in ("sx_inv", "sw_inv", "sdy_inv"):
-            if d.get(name) is not None:
-                setattr(q, name, _dev(d[name], torch.float32, name))
-        q.out, q.ldo = _dev(d["out"], torch.bfloat16, "out"), _rows(d["out"], "out")
-    _check(lib().tweo_fp8_linear_group(arr, n, _stream()), "tweo_fp8_linear_group")
+    _native().linear_group(problems)
 
 
 def loss_fwd_bwd(blocks, tau=3.0, eps=1e-6, p=4.0, grad_coeff=1.0, want_grad=True, grad_dtype=BF16,
                  grads=None, ws=None, per_block=True):
     """tweo_loss_fwd_bwd over a list of bf16 block outputs of equal size.
     Returns (loss [1] float32, per-block [L] float32 or None, list of grads or None)."""
-    Lb = len(blocks)
-    n = blocks[0].numel()
-    dev = blocks[0].device
-    a_arr = (C.c_void_p * Lb)()
-    for i, b in enumerate(blocks):
-        if b.numel() != n or not b.is_contiguous():
-            raise ValueError("block outputs must be contiguous and of equal size")
-        a_arr[i] = _dev(b, torch.bfloat16, "block output")
-    g_arr = None
     if want_grad:
-        gdt = torch.bfloat16 if grad_dtype == BF16 else torch.float32
         if grads is None:
-            grads = [torch.empty(b.shape, dtype=gdt, device=dev) for b in blocks]
-        g_arr = (C.c_void_p * Lb)()
-        for i, g in enumerate(grads):
-            g_arr[i] = _dev(g, gdt, "grad")
+            gdt = torch.bfloat16 if grad_dtype == BF16 else torch.float32
+            grads = [torch.empty(b.shape, dtype=gdt, device=b.device) for b in blocks]
     else:
         grads = None
     if ws is None:
-        ws = new_workspace(OP_LOSS, n, Lb)
-    loss = torch.empty(1, dtype=torch.float32, device=dev)
-    pb = torch.empty(Lb, dtype=torch.float32, device=dev) if per_block else None
-    _check(lib().tweo_loss_fwd_bwd(a_arr, Lb, n, tau, eps, p, grad_coeff, loss.data_ptr(),
-                                   pb.data_ptr() if pb is not None else None, g_arr, grad_dtype, ws.data_ptr(),
-                                   ws.numel(), _stream()), "tweo_loss_fwd_bwd")
+        ws = new_workspace(OP_LOSS, blocks[0].numel(), len(blocks))
+    loss, pb = _native().loss(blocks, tau, eps, p, grad_coeff, grads, grad_dtype, ws, per_block)
     return loss, pb, grads
 
 
@@ -520,25 +360,9 @@ def loss_fwd_bwd_static(blocks, tau=3.0, eps=1e-6, p=4.0, grad_coeff=1.0, want_g
 
 def w8a8_static_gemm(x, sx, wq, sw_inv, y=None, ws=None) -> torch.Tensor:
     """tweo_w8a8_static_gemm: static per-tensor W8A8 linear, bf16 or E4M3-coded activations."""
-    M, K = x.shape
-    N, K2 = wq.shape
-    if K != K2:
-        raise ValueError("inner dimensions differ")
-    if x.dtype == torch.bfloat16:
-        xdt = BF16
-    elif x.dtype in U8:
-        xdt = FP8_E4M3
-    else:
-        raise TypeError("x must be bf16 or uint8 E4M3 codes")
-    if y is None:
-        y = torch.empty((M, N), dtype=torch.bfloat16, device=x.device)
     if ws is None:
-        ws = new_workspace(OP_W8A8, M, N, K)
-    _check(lib().tweo_w8a8_static_gemm(_dev(x, None, "x"), xdt, _rows(x, "x"), _dev(sx, torch.float32, "sx"),
-                                       _dev(wq, U8, "wq"), _rows(wq, "wq"), _dev(sw_inv, torch.float32),
-                                       _dev(y, torch.bfloat16, "y"), _rows(y, "y"), M, N, K, ws.data_ptr(),
-                                       ws.numel(), _stream()), "tweo_w8a8_static_gemm")
-    return y
+        ws = new_workspace(OP_W8A8, x.shape[0], wq.shape[0], x.shape[1])
+    return _native().w8a8(x, sx, wq, sw_inv, y, ws)
 
 
 @dataclass
@@ -589,17 +413,7 @@ def fp4_unpack(q4: torch.Tensor, shape, q8: torch.Tensor | None = None) -> torch
 def fp4_weight_linear(xq, sx_inv, w4, sw_inv, fmt_x=E4M3, y=None) -> torch.Tensor:
     """tweo_fp4_weight_linear: few-token (M <= 128) linear on PACKED E2M1 weights w4 [N, K // 2]; xq [M, K] holds
     FP8 codes (W4A8) or E2M1 carriers (W4A4)."""
-    M, K = xq.shape
-    N, Kb = w4.shape
-    if 2 * Kb != K:
-        raise ValueError("w4 must be [N, K // 2]")
-    if y is None:
-        y = torch.empty((M, N), dtype=torch.bfloat16, device=xq.device)
-    _check(lib().tweo_fp4_weight_linear(_dev(xq, U8, "xq"), _rows(xq, "xq"), fmt_x, _dev(sx_inv, torch.float32, "sx_inv"),
-                                        _dev(w4, U8, "w4"), _rows(w4, "w4"), _dev(sw_inv, torch.float32, "sw_inv"),
-                                        _dev(y, torch.bfloat16, "y"), _rows(y, "y"), M, N, K, _stream()),
-           "tweo_fp4_weight_linear")
-    return y
+    return _native().fp4_weight(xq, sx_inv, w4, sw_inv, fmt_x, y)
 
 
 def w4a4_static_gemm(x, sx, wq8, sw_inv, y=None, ws=None) -> torch.Tensor:
@@ -624,82 +438,28 @@ def block_output_fused(x, f, tau=3.0, eps=1e-6, p=4.0, grad_coeff=1.0, want_grad
                        a=None, grad=None, aq=None, ws=None):
     """tweo_block_output_fused: a = x + f with the TWEO loss term, its gradient, amax(a) and (with
     q_fmt / q_scale) the FP8 codes of a, in one pass.  Returns (a, loss [1], amax [1], grad or None, aq or None)."""
-    if x.shape != f.shape or not x.is_contiguous() or not f.is_contiguous():
-        raise ValueError("x and f must be contiguous and of equal shape")
-    dev = x.device
-    if a is None:
-        a = torch.empty_like(x)
-    if want_grad and grad is None:
-        grad = torch.empty_like(x)
-    if not want_grad:
-        grad = None
-    if q_fmt is not None:
-        if q_scale is None:
-            raise ValueError("the FP8 copy needs q_scale")
-        if aq is None:
-            aq = torch.empty(x.shape, dtype=torch.uint8, device=dev)
-    else:
-        aq = None
     if ws is None:
         ws = new_workspace(OP_BLOCK_OUTPUT)
-    out = torch.empty(2, dtype=torch.float32, device=dev)
-    _check(lib().tweo_block_output_fused(_dev(x, torch.bfloat16, "x"), _dev(f, torch.bfloat16, "f"), x.numel(), tau, eps,
-                                         p, grad_coeff, _dev(a, torch.bfloat16, "a"),
-                                         _dev(grad, torch.bfloat16, "grad") if grad is not None else None,
-                                         out[0:1].data_ptr(), out[1:2].data_ptr(),
-                                         _dev(aq, U8, "aq") if aq is not None else None,
-                                         q_fmt if q_fmt is not None else 0,
-                                         _dev(q_scale, torch.float32, "q_scale") if q_scale is not None else None,
-                                         ws.data_ptr(), ws.numel(), _stream()), "tweo_block_output_fused")
-    return a, out[0:1], out[1:2], grad, aq
+    return _native().block_output(x, f, tau, eps, p, grad_coeff, want_grad, q_fmt, q_scale, a, grad, aq, ws)
 
 
 def delayed_scaling_update(amax_history, amax_new, scale, scale_inv, fmt):
     """tweo_delayed_scaling_update: rolls the [T, H] amax history, inserts amax_new [T] and refreshes
     scale / scale_inv [T] for the next step (all float32 CUDA tensors, updated in place)."""
-    T, H = amax_history.shape
-    if not amax_history.is_contiguous():
-        raise ValueError("amax_history must be contiguous [T, H]")
-    for t, name in ((amax_new, "amax_new"), (scale, "scale"), (scale_inv, "scale_inv")):
-        if t.numel() != T or not t.is_contiguous():
-            raise ValueError(f"{name} must hold one value per tensor")
-    _check(lib().tweo_delayed_scaling_update(_dev(amax_history, torch.float32, "amax_history"), H,
-                                             _dev(amax_new, torch.float32), _dev(scale, torch.float32),
-                                             _dev(scale_inv, torch.float32), T, fmt, _stream()),
-           "tweo_delayed_scaling_update")
+    _native().delayed_scaling(amax_history, amax_new, scale, scale_inv, fmt)
 
 
 def absmax_quantize(x, bits=8, granularity=GRAN_TENSOR, eps=1e-6, s=None, ws=None):
     """tweo_absmax_quantize (Eq. 4): int8 codes of a 2-D bf16 tensor and its scale(s) s ([1] or [rows]).
     With `s` given the quantisation is static."""
-    if x.dim() != 2 or x.stride(1) != 1:
-        raise ValueError("x must be 2-D with contiguous rows")
-    rows, cols = x.shape
-    mode = SCALE_GIVEN if s is not None else SCALE_CURRENT
-    if s is None:
-        s = torch.empty(rows if granularity == GRAN_ROW else 1, dtype=torch.float32, device=x.device)
-    q = torch.empty((rows, cols), dtype=torch.int8, device=x.device)
-    if ws is None and granularity == GRAN_TENSOR and mode == SCALE_CURRENT:
+    if ws is None and granularity == GRAN_TENSOR and s is None:
         ws = new_workspace(OP_ABSMAX)
-    _check(lib().tweo_absmax_quantize(_dev(x, torch.bfloat16, "x"), rows, cols, x.stride(0), bits, granularity, mode,
-                                      eps, _dev(s, torch.float32, "s"), q.data_ptr(), q.stride(0), *_ws(ws), _stream()),
-           "tweo_absmax_quantize")
-    return q, s
+    return _native().absmax(x, bits, granularity, eps, s, ws)
 
 
 def int8_linear(xq, sx, wq, sw, bits=8, y=None):
     """tweo_int8_linear: Y = (Xq . Wq^T) (sx/Q)(sw/Q) -> bf16; sx holds 1 value or one per row of xq, sw 1 or one per row of wq."""
-    M, K = xq.shape
-    N, K2 = wq.shape
-    if K != K2:
-        raise ValueError("inner dimensions differ")
-    if y is None:
-        y = torch.empty((M, N), dtype=torch.bfloat16, device=xq.device)
-    _check(lib().tweo_int8_linear(_dev(xq, torch.int8, "xq"), _rows(xq, "xq"), _dev(sx, torch.float32, "sx"),
-                                  1 if sx.numel() > 1 else 0, _dev(wq, torch.int8, "wq"), _rows(wq, "wq"),
-                                  _dev(sw, torch.float32, "sw"), 1 if sw.numel() > 1 else 0, bits,
-                                  _dev(y, torch.bfloat16, "y"), _rows(y, "y"), M, N, K, _stream()), "tweo_int8_linear")
-    return y
+    return _native().int8_linear(xq, sx, wq, sw, bits, y)
 
 
 def int8_linear_q8(xq, sx, wq, sw, sy, bits=8, yq=None):
@@ -735,16 +495,4 @@ def residual_add_q8(xq, sx, fq, sf, sy, bits=8, yq=None):
 def residual_add_q8_rows(xq, sx, fq, sf, bits=8, eps=1e-6, yq=None):
     """tweo_residual_add_q8_rows: per-token quantised residual addition.  xq, fq: int8 [rows, cols] with one scale
     per row (sx, sf: float32 [rows]); returns (codes of x + f(x), their per-row AbsMax scales)."""
-    if xq.dim() != 2 or xq.shape != fq.shape or not xq.is_contiguous() or not fq.is_contiguous():
-        raise ValueError("xq and fq must be contiguous 2-D tensors of equal shape")
-    rows, cols = xq.shape
-    if sx.numel() != rows or sf.numel() != rows:
-        raise ValueError("one scale per row")
-    if yq is None:
-        yq = torch.empty_like(xq)
-    sy = torch.empty(rows, dtype=torch.float32, device=xq.device)
-    _check(lib().tweo_residual_add_q8_rows(_dev(xq, torch.int8, "xq"), _dev(sx, torch.float32, "sx"),
-                                           _dev(fq, torch.int8, "fq"), _dev(sf, torch.float32, "sf"), rows, cols, bits,
-                                           eps, _dev(yq, torch.int8, "yq"), sy.data_ptr() if rows else None, _stream()),
-           "tweo_residual_add_q8_rows")
-    return yq, sy
+    return _native().residual_rows(xq, sx, fq, sf, bits, eps, yq)

@@ -1,14 +1,17 @@
-"""Builds the CUDA library in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
+"""Builds the CUDA library in-tree with nvcc for sm_100a, and the native half of the Python binding with the host
+compiler (both without a GPU)."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_HERE)
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "libtweo_b200.so")
+NATIVE = os.path.join(_HERE, "_native.so")
 SOURCES = ["api.cu", "loss.cu", "block.cu", "absmax.cu", "norm.cu", "quantize.cu", "gemm.cu", "w8a8.cu", "fp4.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC,-fvisibility=hidden", "--expt-relaxed-constexpr"]
@@ -16,6 +19,27 @@ NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", 
 
 def _newer(a: str, b: str) -> bool:
     return not os.path.exists(b) or os.path.getmtime(a) > os.path.getmtime(b)
+
+
+def build_native(force: bool = False, verbose: bool = False) -> str:
+    """The extension module of binding.py (csrc/native.cpp), linked against the library beside it."""
+    src, header = os.path.join(CSRC, "native.cpp"), os.path.join(_ROOT, "include", "tweo.h")
+    if force or _newer(src, NATIVE) or _newer(header, NATIVE):
+        import torch
+        base = os.path.dirname(torch.__file__)
+        tmp = NATIVE + f".tmp{os.getpid()}"
+        cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+               f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+               "-I", os.path.join(_ROOT, "include"), "-isystem", os.path.join(base, "include"),
+               "-isystem", os.path.join(base, "include", "torch", "csrc", "api", "include"),
+               "-isystem", "/usr/local/cuda/include", "-isystem", sysconfig.get_paths()["include"], src, "-o", tmp,
+               "-L", os.path.join(base, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python",
+               "-L", _HERE, "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN"]
+        if verbose:
+            sys.stderr.write(" ".join(cmd) + "\n")
+        subprocess.check_call(cmd)
+        os.replace(tmp, NATIVE)
+    return NATIVE
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -49,6 +73,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         subprocess.check_call([nvcc, "-shared", "-o", tmp, *objs, "-gencode", "arch=compute_100a,code=sm_100a",
                                "-Xcompiler", "-fPIC"])
         os.replace(tmp, LIB)
+    build_native(force, verbose)
     return LIB
 
 
