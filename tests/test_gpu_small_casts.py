@@ -1,0 +1,47 @@
+"""The one-launch cast of small tensors at its edges: less than a vector, ragged tails, one and several turns of the cluster,
+the largest size it takes and the first one beyond, both formats and kinds of scale in one call; bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import tweo_oracle as orc
+from paper_2511_23225_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def tw():
+    from paper_2511_23225_b200 import binding
+    binding.lib()
+    return binding
+
+
+def word(t):
+    return int(np.float32(t.item()).view(np.uint32))
+
+
+@pytest.mark.parametrize("n", [1, 15, 16, 17, 65535, 65536, 65553, 131072 + 7, 1 << 19, (1 << 19) + 16])
+def test_small_casts_bit_exact(tw, n):
+    bits = [synth.normal_with_extreme_outliers_bf16(900 + i, (n,), frac=1e-2) for i in range(4)]
+    bits[1][n // 2] = 0x7FC0            # a NaN, and an infinity in the last place
+    bits[3][n - 1] = 0xFF80
+    fmts = [tw.E4M3, tw.E5M2, tw.E4M3, tw.E5M2]
+    modes = [tw.SCALE_CURRENT, tw.SCALE_CURRENT, tw.SCALE_GIVEN, tw.SCALE_GIVEN]
+    given = np.float32(0.37)
+    xs = [torch.from_numpy(b.view(np.int16)).cuda().view(torch.bfloat16) for b in bits]
+    outs = []
+    for x, f in zip(xs, fmts):
+        sc = torch.tensor([float(given), 5.0, 123.0], dtype=torch.float32, device="cuda")   # a stale amax
+        outs.append(tw.Quantized(torch.full((n,), 0x55, dtype=torch.uint8, device="cuda"), sc[0:1], sc[1:2], sc[2:3], None, f))
+    for _ in range(2):
+        tw.quantize_per_tensor_batch(xs, outs, modes)
+        torch.cuda.synchronize()
+        for b, f, m, o in zip(bits, fmts, modes, outs):
+            if m == tw.SCALE_GIVEN:
+                ref = {"q": orc.quantize_bf16(b, f, given)[0], "amax": orc.amax_bf16(b), "scale": given, "scale_inv": np.float32(1) / given}
+            else:
+                ref = orc.quantize_per_tensor_current(b, f)
+            assert np.array_equal(o.q.cpu().numpy(), ref["q"])
+            for name in ("amax", "scale", "scale_inv"):
+                assert word(getattr(o, name)) == int(np.float32(ref[name]).view(np.uint32))
