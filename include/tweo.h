@@ -120,7 +120,8 @@ typedef struct tweo_epilogue_t {
  *     cast).  With a workspace of tweo_workspace_bytes(TWEO_OP_QUANTIZE) bytes (any
  *     contents) a CURRENT-scaling call without sat_count runs as two kernels: per-CTA
  *     maxima go to workspace slots and every CTA of the cast reduces them itself, so
- *     there is no reset kernel and no atomic.  Results are identical bit for bit.
+ *     there is no reset kernel and no atomic.  A tensor of up to 2^17 elements without
+ *     sat_count runs as one kernel, with or without a workspace.  Results are identical bit for bit.
  */
 TWEO_API tweo_status_t tweo_quantize_per_tensor(const uint16_t* x, int64_t n, int32_t fmt, int32_t mode,
                                        float* scale, float* scale_inv, float* amax, uint8_t* q,
@@ -137,7 +138,8 @@ TWEO_API tweo_status_t tweo_quantize_per_tensor(const uint16_t* x, int64_t n, in
  *   ws: tweo_workspace_bytes(TWEO_OP_QUANTIZE) bytes, any contents.  The tensors with
  *     CURRENT scaling and no sat_count share one amax kernel and one cast kernel per FP8
  *     format; GIVEN-scale tensors and those with a sat_count (and all of them when ws is
- *     NULL or too small) are launched one by one as tweo_quantize_per_tensor does.
+ *     NULL or too small) are launched one by one as tweo_quantize_per_tensor does.  A
+ *     batch of tensors of up to 2^20 elements, none with a sat_count, is one launch.
  *   Errors: TWEO_ERR_INVALID_ARG (count out of range, NULL pointers, bad enums),
  *     TWEO_ERR_ALIGNMENT.
  */

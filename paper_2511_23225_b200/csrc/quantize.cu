@@ -488,12 +488,16 @@ __global__ void __launch_bounds__(kSmallThreads) small_cast_kernel(const __grid_
 
 int grid_for(int64_t work_items, int per_cta, int ctas_per_sm);
 
-// Where one cluster per tensor is the faster form (see launch_small's measurements).
-constexpr int64_t kSmallElems = 1 << 19;
+// Where one cluster per tensor is the faster form.  Microseconds per call in a chain, this form / the others:
+//   one tensor, given scale       2^16 2.6 / 2.4   2^17 2.9 / 2.5   2^19 4.6 / 2.6      current  2^17 3.4 / 3.4   2^19 6.3 / 3.5
+//   three, both formats, current  2^16 3.2 / 7.7   2^19 6.5 / 9.4   2^20 10.1 / 12.7    2^21 17.2 / 15.8
+//   three, given                  2^16 2.9 / 5.6   2^19 4.9 / 5.8   2^20 6.9 / 7.4      2^21 10.9 / 8.5
+// One tensor gains launches (each costs its host 2 us), not device time; several gain both.
+constexpr int64_t kSmallElemsOne = 1 << 17, kSmallElemsBatch = 1 << 20;
 
 bool all_small(const tweo_quant_desc_t* descs, int count) {
   for (int i = 0; i < count; ++i)
-    if (descs[i].n > kSmallElems || descs[i].sat_count) return false;
+    if (descs[i].n > (count == 1 ? kSmallElemsOne : kSmallElemsBatch) || descs[i].sat_count) return false;
   return true;
 }
 

@@ -21,7 +21,7 @@ def word(t):
     return int(np.float32(t.item()).view(np.uint32))
 
 
-@pytest.mark.parametrize("n", [1, 15, 16, 17, 65535, 65536, 65553, 131072 + 7, 1 << 19, (1 << 19) + 16])
+@pytest.mark.parametrize("n", [1, 15, 16, 17, 65535, 65536, 65553, 131072 + 7, 1 << 20, (1 << 20) + 16])
 def test_small_casts_bit_exact(tw, n):
     bits = [synth.normal_with_extreme_outliers_bf16(900 + i, (n,), frac=1e-2) for i in range(4)]
     bits[1][n // 2] = 0x7FC0            # a NaN, and an infinity in the last place
