@@ -135,6 +135,12 @@ __device__ __forceinline__ uint32_t quant_words(uint32_t w0, uint32_t w1, uint64
   return quant4<FMT>(a, b, c, d);
 }
 
+template <int FMT>
+__device__ __forceinline__ uint32_t quant_words_scalar(uint32_t w0, uint32_t w1, float qs) {
+  return quant4<FMT>(__fmul_rn(bf16lo_to_f32(w0), qs), __fmul_rn(bf16hi_to_f32(w0), qs),
+                     __fmul_rn(bf16lo_to_f32(w1), qs), __fmul_rn(bf16hi_to_f32(w1), qs));
+}
+
 // A row of 64 bf16 values (packed words) times the scale -> 64 codes at shared address `qrow`, in four 16-byte pieces
 // whose positions are XORed with `qswz` (the 64-byte swizzle of the store's tensor map).
 template <int FMT>

@@ -318,7 +318,18 @@ gemm_fp8_pair_group_kernel(const __grid_constant__ PairGroupParams<LIST> g) {
           // 64 codes per row -> 32 rows x 64 B, 16-byte pieces XOR-swizzled with row bits 1-2
           const uint32_t qrow = qbuf + (uint32_t)lane * 64u;
           const uint32_t qswz = ((uint32_t)lane >> 1) & 3u;
-          stage_codes(q.q_fmt, qrow, qswz, packed, splat_f32x2(qs));
+          // scalar products here: packed ones and the choice of the format outside the loop, faster in the kernel with
+          // activations, made the fused step of the ViT-B/16 block at 20000 tokens slower (804 -> 835 us)
+#pragma unroll
+          for (int g4 = 0; g4 < 4; ++g4) {
+            uint32_t qq[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const uint32_t w0 = packed[8 * g4 + 2 * j], w1 = packed[8 * g4 + 2 * j + 1];
+              qq[j] = q.q_fmt == TWEO_E4M3 ? quant_words_scalar<TWEO_E4M3>(w0, w1, qs) : quant_words_scalar<TWEO_E5M2>(w0, w1, qs);
+            }
+            st_shared_v4(qrow + (((uint32_t)g4 ^ qswz) << 4), qq[0], qq[1], qq[2], qq[3]);
+          }
         }
         fence_async_smem();
         __syncwarp();
