@@ -268,20 +268,38 @@ class BlockStep:
             self.side = torch.cuda.Stream()
         side = self.side
         side.wait_stream(main)
-        ready, cast_pos = [], {}
-        with torch.cuda.stream(side):
-            for pos, batch in enumerate(self.cast_batches()):
+        ready, cast_pos, gemms = [], {}, self.gemm_batches()
+
+        def launch_gemms():
+            """The GEMM batches whose casts have been issued; returns an event in front of the first, None if none."""
+            begun = None
+            while gemms and all(i in cast_pos for i in gemms[0]):
+                # the last cast batch that holds one of this GEMM batch's linears: the earlier ones are done too
+                main.wait_event(ready[max(cast_pos[i] for i in gemms[0])])
+                if begun is None:
+                    begun = torch.cuda.Event()
+                    begun.record(main)
+                self.run_gemm_batch(gemms.pop(0))
+            return begun
+
+        for pos, batch in enumerate(self.cast_batches()):
+            with torch.cuda.stream(side):
                 self.quantize_all([self.linears[i] for i in batch])
                 ev = torch.cuda.Event()
                 ev.record(side)
-                ready.append(ev)
-                for i in batch:
-                    cast_pos[i] = pos
+            ready.append(ev)
+            for i in batch:
+                cast_pos[i] = pos
+            if self.variant != "plain":
+                # With given scales the next casts start one hop behind the event that frees the GEMM: they fill every SM
+                # and would keep it waiting.  Step of the ViT-B/16 block, 20000 tokens, fused: 806 -> 765 us.  The two
+                # passes of current scaling gain nothing from coming second (GPT-2-small block 291 -> 295).
+                begun = launch_gemms()
+                if begun is not None:
+                    side.wait_event(begun)
+        with torch.cuda.stream(side):
             self.tweo()
-        for batch in self.gemm_batches():
-            # the last cast batch that holds one of this GEMM batch's linears: the earlier ones are done too
-            main.wait_event(ready[max(cast_pos[i] for i in batch)])
-            self.run_gemm_batch(batch)
+        launch_gemms()
         self.update_output_scales()
         main.wait_stream(side)
 
