@@ -163,19 +163,25 @@ __device__ __forceinline__ void stage_codes(int fmt, uint32_t qrow, uint32_t qsw
 // 1: v * Phi(v).  Phi from the rational approximation of erfc by Hastings (Abramowitz & Stegun
 //    7.1.26): erfc(x) = t (a1 + t (a2 + t (a3 + t (a4 + t a5)))) exp(-x^2), t = 1 / (1 + p x), x >= 0,
 //    absolute error below 1.5e-7 -- three orders below the bf16 rounding that follows.  With h = erfc(|v|/sqrt 2) / 2
-//    the result is max(v, 0) - |v| h for either sign: one rounding, no select.
+//    the result is v (1 - h) for v >= 0 and v h below, every operation rounded by itself: the same bits as the scalar
+//    form (-infinity gives NaN, as the definition does).
 // 2: the tanh form with the hardware tanh (relative error 2^-11).
 // What bounds the kernels that use them, at short contractions: the issue slots and the latencies of the epilogue.
-// Scalar arithmetic (with the scaling for denormals of exp and of the division, which no argument here needs: results
-// of exp below 2^-126 vanish in the sum, the divisors lie in [1, 16]) took 31 warp instructions per element for the
-// erf form and 14 000 cycles per 256x256 tile, against 4 300 of the main loop at contraction 768; the packed form takes
-// 17, and eight pairs go through stage by stage, because a warp shares its scheduler with only one other and has to
-// cover its own latencies (two thirds of the stalls of the first packed version were waits for a result of the chain).
-// [12608x768].[3072x768]^T, amax and FP8 copy, microseconds: erf 74.3 scalar, 59.4 packed, 46.3 staged; tanh 45.6,
-// 39.3, 34.6; without an activation 35.
+// Scalar arithmetic took 31 warp instructions per element for the erf form (part of it the scaling for denormals of the
+// division, which divisors of 1 and above never need, and of exp) and 14 000 cycles per 256x256 tile, against 4 300 of
+// the main loop at contraction 768.  G packed pairs go through stage by stage, because a warp shares its scheduler with
+// only one other and has to cover its own latencies.  exp with denormal results runs only where a chunk has a value
+// below -13: everywhere it costs 62 us where the choice costs 46.
+// [12608x768].[3072x768]^T, amax and FP8 copy, microseconds: erf 74.3 scalar, 59.4 packed, 46.1 staged by four pairs (48.0
+// by eight); tanh 45.6, 39.3, 34.6 by eight; without an activation 35.  The erf form as max(v, 0) - |v| h takes 41.1, but moves roundings.
 __device__ __forceinline__ float ex2_ftz(float x) {
   float r;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float ex2_denormal(float x) {
+  float r;
+  asm("ex2.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
 __device__ __forceinline__ float rcp_ftz(float x) {
@@ -183,62 +189,62 @@ __device__ __forceinline__ float rcp_ftz(float x) {
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
-// the larger operand; a NaN operand gives NaN
-__device__ __forceinline__ float max_nan(float a, float b) {
-  float r;
-  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-  return r;
-}
 
-constexpr int kActPairs = 8;
-template <int ACT>
-__device__ __forceinline__ void act_pairs(uint64_t (&v)[kActPairs]) {
+// LOW: values below -13 count, where h is denormal.
+template <int ACT, bool LOW, int G>
+__device__ __forceinline__ void act_pairs(uint64_t (&v)[G]) {
   if (ACT == 1) {
-    uint64_t n[kActPairs], t[kActPairs], e[kActPairs], q[kActPairs];
+    uint64_t t[G], e[G], q[G];
 #pragma unroll
-    for (int i = 0; i < kActPairs; ++i) {
+    for (int i = 0; i < G; ++i) {
       float v0, v1;
       unpack_f32x2(v[i], v0, v1);
-      // -|v|, held above -64 (erfc vanishes long before): infinity times zero must not arise below
-      n[i] = pack_f32x2(max_nan(-fabsf(v0), -64.0f), max_nan(-fabsf(v1), -64.0f));
-      v[i] = pack_f32x2(max_nan(v0, -0.0f), max_nan(v1, -0.0f));
+      e[i] = pack_f32x2(__fmul_rn(fabsf(v0), 0.70710678118654752f), __fmul_rn(fabsf(v1), 0.70710678118654752f));   // x
     }
 #pragma unroll
-    for (int i = 0; i < kActPairs; ++i) {
-      t[i] = fma_f32x2(n[i], splat_f32x2(-0.23164187f), splat_f32x2(1.0f));   // 1 + p |v| / sqrt 2
-      e[i] = mul_f32x2(n[i], splat_f32x2(-0.72134752f));
+    for (int i = 0; i < G; ++i) {
+      t[i] = fma_f32x2(e[i], splat_f32x2(0.3275911f), splat_f32x2(1.0f));
+      e[i] = mul_f32x2(e[i], e[i]);
     }
 #pragma unroll
-    for (int i = 0; i < kActPairs; ++i) {
+    for (int i = 0; i < G; ++i) {
       float d0, d1;
       unpack_f32x2(t[i], d0, d1);
       t[i] = pack_f32x2(rcp_ftz(d0), rcp_ftz(d1));
-      e[i] = mul_f32x2(e[i], n[i]);                                           // -v^2 / 2 in units of ln 2
+      e[i] = mul_f32x2(e[i], splat_f32x2(-1.44269504f));                        // -x^2 in units of ln 2
     }
 #pragma unroll
-    for (int i = 0; i < kActPairs; ++i) {
+    for (int i = 0; i < G; ++i) {
       float d0, d1;
       unpack_f32x2(e[i], d0, d1);
-      e[i] = pack_f32x2(ex2_ftz(d0), ex2_ftz(d1));
+      e[i] = LOW ? pack_f32x2(ex2_denormal(d0), ex2_denormal(d1)) : pack_f32x2(ex2_ftz(d0), ex2_ftz(d1));
       q[i] = fma_f32x2(t[i], splat_f32x2(0.5307027145f), splat_f32x2(-0.7265760135f));   // a5/2, a4/2, ...
     }
 #pragma unroll
-    for (int i = 0; i < kActPairs; ++i) q[i] = fma_f32x2(t[i], q[i], splat_f32x2(0.7107068705f));
+    for (int i = 0; i < G; ++i) q[i] = fma_f32x2(t[i], q[i], splat_f32x2(0.7107068705f));
 #pragma unroll
-    for (int i = 0; i < kActPairs; ++i) q[i] = fma_f32x2(t[i], q[i], splat_f32x2(-0.142248368f));
+    for (int i = 0; i < G; ++i) q[i] = fma_f32x2(t[i], q[i], splat_f32x2(-0.142248368f));
 #pragma unroll
-    for (int i = 0; i < kActPairs; ++i) q[i] = fma_f32x2(t[i], q[i], splat_f32x2(0.127414796f));
+    for (int i = 0; i < G; ++i) q[i] = fma_f32x2(t[i], q[i], splat_f32x2(0.127414796f));
 #pragma unroll
-    for (int i = 0; i < kActPairs; ++i) q[i] = mul_f32x2(t[i], q[i]);
+    for (int i = 0; i < G; ++i) q[i] = mul_f32x2(t[i], q[i]);
 #pragma unroll
-    for (int i = 0; i < kActPairs; ++i) v[i] = fma_f32x2(mul_f32x2(q[i], e[i]), n[i], v[i]);   // - |v| Phi(-|v|)
+    for (int i = 0; i < G; ++i) q[i] = mul_f32x2(q[i], e[i]);           // h
+#pragma unroll
+    for (int i = 0; i < G; ++i) {
+      float v0, v1, h0, h1, p0, p1;
+      unpack_f32x2(v[i], v0, v1);
+      unpack_f32x2(q[i], h0, h1);
+      unpack_f32x2(fma_f32x2(q[i], splat_f32x2(-1.0f), splat_f32x2(1.0f)), p0, p1);
+      v[i] = mul_f32x2(v[i], pack_f32x2(v0 >= 0.0f ? p0 : h0, v1 >= 0.0f ? p1 : h1));
+    }
   } else if (ACT == 2) {
-    uint64_t c[kActPairs];
+    uint64_t c[G];
 #pragma unroll
-    for (int i = 0; i < kActPairs; ++i)
-      c[i] = fma_f32x2(mul_f32x2(v[i], splat_f32x2(0.044715f)), mul_f32x2(v[i], v[i]), v[i]);
+    for (int i = 0; i < G; ++i)
+      c[i] = fma_f32x2(mul_f32x2(mul_f32x2(v[i], splat_f32x2(0.044715f)), v[i]), v[i], v[i]);
 #pragma unroll
-    for (int i = 0; i < kActPairs; ++i) {
+    for (int i = 0; i < G; ++i) {
       float u0, u1, t0, t1;
       unpack_f32x2(mul_f32x2(c[i], splat_f32x2(0.79788456080286536f)), u0, u1);
       asm("tanh.approx.f32 %0, %1;" : "=f"(t0) : "f"(u0));
@@ -246,7 +252,7 @@ __device__ __forceinline__ void act_pairs(uint64_t (&v)[kActPairs]) {
       c[i] = pack_f32x2(t0, t1);
     }
 #pragma unroll
-    for (int i = 0; i < kActPairs; ++i) {
+    for (int i = 0; i < G; ++i) {
       const uint64_t h = mul_f32x2(v[i], splat_f32x2(0.5f));
       v[i] = fma_f32x2(h, c[i], h);
     }

@@ -13,6 +13,8 @@
 //                            arrival: a releasing one would wait for the warp's TMA stores to drain)
 #pragma once
 
+#include <type_traits>
+
 #include <cuda.h>
 
 #include "gemm_common.cuh"
@@ -324,22 +326,39 @@ gemm_fp8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
 #pragma unroll
             for (int j = 0; j < CH; ++j) run_max = fmaxf(run_max, fabsf(__uint_as_float(r[j])));
           }
-          constexpr int G = kActPairs;
+          constexpr int G = ACT == 1 ? 4 : 8;   // pairs per pass of act_pairs()
+          float least = 0.0f;
+          auto arithmetic = [&](auto low) {
 #pragma unroll
-          for (int j0 = 0; j0 < CH / 2; j0 += G) {
-            uint64_t v[G];
+            for (int j0 = 0; j0 < CH / 2; j0 += G) {
+              uint64_t v[G];
 #pragma unroll
-            for (int i = 0; i < G; ++i) {
-              v[i] = pack_f32x2(__uint_as_float(r[2 * (j0 + i)]), __uint_as_float(r[2 * (j0 + i) + 1]));
-              if (ACT != 3) v[i] = mul_f32x2(v[i], alpha2);
+              for (int i = 0; i < G; ++i) {
+                v[i] = pack_f32x2(__uint_as_float(r[2 * (j0 + i)]), __uint_as_float(r[2 * (j0 + i) + 1]));
+                if (ACT != 3) v[i] = mul_f32x2(v[i], alpha2);
+                if (ACT == 1) {
+                  float v0, v1;
+                  unpack_f32x2(v[i], v0, v1);
+                  least = fminf(least, fminf(v0, v1));
+                }
+              }
+              if (ACT != 3) act_pairs<ACT, decltype(low)::value>(v);
+#pragma unroll
+              for (int i = 0; i < G; ++i) {
+                float v0, v1;
+                unpack_f32x2(v[i], v0, v1);
+                if (ACT == 1 || ACT == 2) run_max = fmaxf(run_max, fmaxf(fabsf(v0), fabsf(v1)));
+                packed[j0 + i] = f32x2_to_bf16x2(v0, v1);
+              }
             }
-            if (ACT != 3) act_pairs<ACT>(v);
-#pragma unroll
-            for (int i = 0; i < G; ++i) {
-              float v0, v1;
-              unpack_f32x2(v[i], v0, v1);
-              if (ACT == 1 || ACT == 2) run_max = fmaxf(run_max, fmaxf(fabsf(v0), fabsf(v1)));
-              packed[j0 + i] = f32x2_to_bf16x2(v0, v1);
+          };
+          arithmetic(std::false_type{});
+          if constexpr (ACT == 1) {
+            if (__any_sync(0xFFFFFFFFu, least < -13.0f)) {   // rare: once more, from tensor memory, with denormal results of exp
+              tmem_ld32(taddr, *reinterpret_cast<uint32_t(*)[32]>(&r[0]));
+              tmem_ld32(taddr + 32, *reinterpret_cast<uint32_t(*)[32]>(&r[CH - 32]));
+              tmem_ld_wait();
+              arithmetic(std::true_type{});
             }
           }
           if (ACT != 0) buffer_free();
