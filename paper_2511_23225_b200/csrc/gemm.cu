@@ -794,7 +794,7 @@ bool skinny_pays(int64_t M, int64_t N, int64_t Kc) {
 // instruction descriptor), and launches.  wq: [N, Kc] (K contiguous), or [Kc, N] for W_MN.
 // w_packed4: W holds packed E2M1 codes (two per byte, ldw in BYTES); the ring and the kernel are the same, only the
 // tensor map of W differs (and the operand format in p.idesc, set by the caller).
-// w_early: W may be loaded before the kernels before this one have completed (see gemm_skinny.cuh).
+// w_early: see gemm_skinny.cuh; only for a call whose own kernel in front waits before it releases.
 template <bool I8, bool W_MN = false>
 tweo_status_t launch_skinny(SkinnyParams& p, const void* xq, int64_t ldx, const void* wq, int64_t ldw, int64_t M, int64_t N,
                             int64_t K, cudaStream_t st, bool w_early, bool w_packed4 = false) {
@@ -1127,8 +1127,8 @@ tweo_status_t run_int8_linear(const int8_t* xq, int64_t ldx, const float* sx, in
     sp.row_scale_per_row = sx_per_row ? 1 : 0;
     sp.col_scale_per_col = sw_per_row ? 1 : 0;
     sp.post_scale = 1.0f / ((float)Q_ * (float)Q_);
-    // integer codes come from the AbsMax casts alone, which let no later kernel start before they have completed
-    return launch_skinny<true>(sp, xq, ldx, wq, ldw, M, N, K, stream, true);
+    // wq may be the output of the kernel just before (an 8-bit linear, an addition, a cast): not before the wait
+    return launch_skinny<true>(sp, xq, ldx, wq, ldw, M, N, K, stream, false);
   }
   constexpr size_t smem6 = (size_t)6 * (BM * BK + 128 * BK) + 4 * 2 * 32 * 128 + 1024 + 256;
   constexpr size_t smem5q = (size_t)5 * (BM * BK + 128 * BK) + 4 * 2 * 32 * 128 + 4 * 2 * 32 * 64 + 1024 + 256;

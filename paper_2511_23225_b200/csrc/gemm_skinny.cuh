@@ -34,7 +34,7 @@ struct SkinnyParams {
   int32_t k_blocks;        // contraction blocks of 128
   int32_t slices;          // slices of the contraction = CTAs per cluster (1 .. 8)
   int32_t vec_out;         // y and ldy allow 8-byte stores
-  int32_t w_early;         // no kernel that may still run when this one starts can be writing W
+  int32_t w_early;         // every kernel enqueued before this call has completed, its writes visible, when this kernel starts
   int32_t stages;          // TMA ring depth (<= kSkinnyMaxStages)
   uint32_t stage_bytes;    // 16 KB of W + Mpad * 128 B of X, rounded up to 1 KB
   uint32_t w_tx_bytes;     // bytes one W load reports to its barrier: the 16 KB it writes, or 8 KB for packed 4-bit
@@ -185,10 +185,12 @@ gemm_fp8_skinny_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
   const uint32_t x_bytes = (uint32_t)p.Mpad * 128u;
 
   // The kernel may have been launched while the kernels before it on the stream are still running (programmatic
-  // dependent launch): the activations, the scales and the output are touched only after chain_wait().  So is W where
-  // one of those kernels may be the cast that writes it; until then it is brought into L2, which is safe whoever
-  // writes it.  Where none can be (w_early, see the callers), the first ring of W is loaded at once: L2 to shared memory
-  // takes 3 of 13 us at [11008x4096] after the wait.
+  // dependent launch), and any of them may write an operand: activations, scales, W and the output are touched only after
+  // chain_wait().  Until then W is brought into L2, which is safe whoever writes it.  An exception is a call with a
+  // kernel of its own in front that does chain_wait() first and chain_release() then (w_early): when this kernel starts,
+  // what was enqueued before the call has completed, and the first ring of W is loaded at once (L2 to shared memory takes 3 of 13 us
+  // at [11008x4096] after the wait).  That no kernel before releases early is not enough: without a wait the
+  // writes of a kernel that has just ended need not be visible.
   chain_release();
   float alpha[4];
   if (warp == 0) {

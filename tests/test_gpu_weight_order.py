@@ -1,0 +1,68 @@
+"""A product whose weight operand the call just before it writes, without a host synchronisation in between: the few-token
+kernel starts while that call is still running and must not take the weight's former contents.  Every step writes other codes
+into the same buffer.  Reference: the same product on a copy of the codes, after everything has completed (the products do
+not depend on timing)."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+STEPS = 12
+
+
+@pytest.fixture(scope="module")
+def tw():
+    from paper_2511_23225_b200 import binding
+    binding.lib()
+    return binding
+
+
+def i8(shape, seed):
+    return torch.randint(-127, 128, shape, generator=torch.Generator().manual_seed(seed), dtype=torch.int8).cuda()
+
+
+def run(tw, weight_of, product):
+    """weight_of(step) enqueues the call that writes the weight and returns it; product(w) is checked for every step."""
+    torch.cuda.synchronize()
+    got = []
+    for s in range(STEPS):
+        w = weight_of(s)
+        got.append((product(w), w.clone()))
+    torch.cuda.synchronize()
+    assert tw.read_device_status() == 0
+    for s, (y, w) in enumerate(got):
+        torch.cuda.synchronize()
+        assert torch.equal(y, product(w)), f"step {s} used other codes"
+        assert s == 0 or not torch.equal(w, got[s - 1][1])
+
+
+# tokens: the narrow ring, and (above 128) the wide one with a ragged last tile
+@pytest.mark.parametrize("M", [1, 16, 128, 300])
+@pytest.mark.parametrize("writer", ["int8_linear_q8", "residual_add_q8", "residual_add_q8_rows", "absmax_rows", "absmax_tensor",
+                                    "linear_behind_an_addition"])
+def test_integer_linear_behind_the_call_that_writes_its_weight(tw, writer, M):
+    N, K, C = 1024, 1024, 2048           # weight [N, K]; C: the contraction of the linear that writes it
+    one = torch.ones(1, device="cuda")
+    rows = torch.rand(N, generator=torch.Generator().manual_seed(9)).cuda() + 0.5
+    src, mat = [i8((N, C), 20 + s) for s in range(STEPS)], i8((K, C), 3)
+    a, b = [i8((N, K), 50 + s) for s in range(STEPS)], i8((N, K), 4)
+    act = [torch.randn((N, K), generator=torch.Generator().manual_seed(80 + s)).to(torch.bfloat16).cuda() for s in range(STEPS)]
+    x, w = i8((M, K), 7), torch.zeros((N, K), dtype=torch.int8, device="cuda")
+    other = torch.zeros_like(w)
+    big = one * 60.0
+
+    def weight_of(s):
+        if writer in ("int8_linear_q8", "linear_behind_an_addition"):
+            tw.int8_linear_q8(src[s], one, mat, one, big, yq=w)
+            if writer == "linear_behind_an_addition":   # does not touch w, but starts early itself
+                tw.residual_add_q8_rows(a[s], rows, b, rows, yq=other)
+            return w
+        if writer == "residual_add_q8":
+            tw.residual_add_q8(a[s], one, b, one, one * 2.0, yq=w)
+            return w
+        if writer == "residual_add_q8_rows":
+            tw.residual_add_q8_rows(a[s], rows, b, rows, yq=w)
+            return w
+        return tw.absmax_quantize(act[s], granularity=tw.GRAN_ROW if writer == "absmax_rows" else tw.GRAN_TENSOR)[0]
+
+    run(tw, weight_of, lambda v: tw.int8_linear(x, one, v, rows))
