@@ -82,7 +82,8 @@ __device__ __forceinline__ float e2m1_scale_from_amax(float amax) {
 template <bool GIVEN, int U>
 __global__ void __launch_bounds__(kThreads)
 fp4_cast_kernel(const uint16_t* x, int64_t n, float* scale, float* scale_inv, float* amax, uint8_t* q4, uint8_t* q8) {
-  chain_wait();   // and no chain_release(): the packed-weight linear loads its weight, maybe these codes, before its own wait
+  chain_wait();
+  chain_release();
   float s;
   if (GIVEN) {
     s = *scale;

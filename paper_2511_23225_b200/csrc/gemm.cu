@@ -863,8 +863,8 @@ tweo_status_t run_skinny_w4(const uint8_t* xq, int64_t ldx, int fmt_x, const uin
   p.sx_inv = sx_inv;
   p.sw_inv = sw_inv;
   p.sx_is_scale = 0;
-  // packed weights come from the FP4 cast alone, which lets no later kernel start before it has completed
-  return launch_skinny<false>(p, xq, ldx, w4, ldw_bytes, M, N, K, st, true, true);
+  // w4 may have been cast or copied by the kernel just before: not before the wait
+  return launch_skinny<false>(p, xq, ldx, w4, ldw_bytes, M, N, K, st, false, true);
 }
 
 // Up to kGroupMaxProblems independent products in ONE launch of the CTA-pair kernel (see gemm_pair_group.cuh).

@@ -66,3 +66,23 @@ def test_integer_linear_behind_the_call_that_writes_its_weight(tw, writer, M):
         return tw.absmax_quantize(act[s], granularity=tw.GRAN_ROW if writer == "absmax_rows" else tw.GRAN_TENSOR)[0]
 
     run(tw, weight_of, lambda v: tw.int8_linear(x, one, v, rows))
+
+
+@pytest.mark.parametrize("M", [1, 16, 128])
+@pytest.mark.parametrize("writer", ["fp4_quantize", "copy"])
+def test_packed_weight_linear_behind_the_call_that_writes_its_weight(tw, writer, M):
+    N, K = 2048, 2048
+    one = torch.ones(1, device="cuda")
+    ws = [torch.randn((N, K), generator=torch.Generator().manual_seed(30 + s)).to(torch.bfloat16).cuda() for s in range(STEPS)]
+    packed = [tw.fp4_quantize(w, carriers=False).q4.view(N, K // 2) for w in ws]
+    x = torch.randint(0, 0x70, (M, K), generator=torch.Generator().manual_seed(5), dtype=torch.uint8).cuda()
+    out = tw.QuantizedFP4(torch.zeros(N * K // 2, dtype=torch.uint8, device="cuda"), None, *(torch.ones(1, device="cuda") for _ in range(3)))
+
+    def weight_of(s):
+        if writer == "fp4_quantize":
+            tw.fp4_quantize(ws[s], carriers=False, out=out)
+        else:
+            out.q4.copy_(packed[s].view(-1))
+        return out.q4.view(N, K // 2)
+
+    run(tw, weight_of, lambda w: tw.fp4_weight_linear(x, one, w, one))
