@@ -77,15 +77,17 @@ __device__ __forceinline__ float e2m1_scale_from_amax(float amax) {
 }
 
 // 16 elements per thread and pass: two 16-byte loads -> 8 bytes of packed codes and / or 16 carrier bytes.
-// CURRENT mode reads *amax (finished by the kernel before) and derives the scale; GIVEN mode reads *scale
-// and folds |x| into *amax while casting.
-template <bool GIVEN, int U>
+// CURRENT reads *amax (finished by the kernel before) and derives the scale; GIVEN reads *scale
+// and folds |x| into *amax while casting; CODES reads *scale and writes the codes alone (the activations of a static
+// linear, whose amax nobody reads: one launch instead of a reset and a cast).
+enum CastMode { CURRENT, GIVEN, CODES };
+template <CastMode MODE, int U>
 __global__ void __launch_bounds__(kThreads)
 fp4_cast_kernel(const uint16_t* x, int64_t n, float* scale, float* scale_inv, float* amax, uint8_t* q4, uint8_t* q8) {
   chain_wait();
-  chain_release();
+  chain_release();   // in this order: when the next kernel starts, those before this one have completed
   float s;
-  if (GIVEN) {
+  if (MODE != CURRENT) {
     s = *scale;
   } else {
     s = e2m1_scale_from_amax(*amax);
@@ -122,7 +124,7 @@ fp4_cast_kernel(const uint16_t* x, int64_t n, float* scale, float* scale_inv, fl
           float lo, hi;
           unpack_f32x2(mul_f32x2(bf16x2_to_f32x2(w[j]), ss), lo, hi);  // each lane rounded once
           cvt_e2m1x2(lo, hi, code[j], car[j]);
-          if (GIVEN) absmax_f32(m0, m1, w[j]);
+          if (MODE == GIVEN) absmax_f32(m0, m1, w[j]);
         }
         if (q4)
           __stcs(q4v + i, make_uint2(code[0] | (code[1] << 8) | (code[2] << 16) | (code[3] << 24),
@@ -144,10 +146,10 @@ fp4_cast_kernel(const uint16_t* x, int64_t n, float* scale, float* scale_inv, fl
         q8[i] = (uint8_t)(car & 0xFFu);
         if (i + 1 < n) q8[i + 1] = (uint8_t)(car >> 8);
       }
-      if (GIVEN) absmax_f32(m0, m1, w0 | (w1 << 16));
+      if (MODE == GIVEN) absmax_f32(m0, m1, w0 | (w1 << 16));
     }
   }
-  if (GIVEN) {
+  if (MODE == GIVEN) {
     uint32_t m = absmax_f32_bits(m0, m1);
     __shared__ uint32_t part[kThreads / 32];
 #pragma unroll
@@ -223,11 +225,11 @@ extern "C" tweo_status_t tweo_fp4_quantize(const uint16_t* x, int64_t n, int32_t
   const bool deep = n16 >= (int64_t)sm_count() * 8 * kThreads * 8;
   const dim3 grid(cast_grid(n16, deep ? 4 : 2));
   if (given) {
-    if (deep) TWEO_CUDA_TRY(launch_chain(fp4_cast_kernel<true, 4>, grid, dim3(kThreads), 0, st, 0, x, n, scale, scale_inv, amax, q4, q8));
-    else TWEO_CUDA_TRY(launch_chain(fp4_cast_kernel<true, 2>, grid, dim3(kThreads), 0, st, 0, x, n, scale, scale_inv, amax, q4, q8));
+    if (deep) TWEO_CUDA_TRY(launch_chain(fp4_cast_kernel<GIVEN, 4>, grid, dim3(kThreads), 0, st, 0, x, n, scale, scale_inv, amax, q4, q8));
+    else TWEO_CUDA_TRY(launch_chain(fp4_cast_kernel<GIVEN, 2>, grid, dim3(kThreads), 0, st, 0, x, n, scale, scale_inv, amax, q4, q8));
   } else {
-    if (deep) TWEO_CUDA_TRY(launch_chain(fp4_cast_kernel<false, 4>, grid, dim3(kThreads), 0, st, 0, x, n, scale, scale_inv, amax, q4, q8));
-    else TWEO_CUDA_TRY(launch_chain(fp4_cast_kernel<false, 2>, grid, dim3(kThreads), 0, st, 0, x, n, scale, scale_inv, amax, q4, q8));
+    if (deep) TWEO_CUDA_TRY(launch_chain(fp4_cast_kernel<CURRENT, 4>, grid, dim3(kThreads), 0, st, 0, x, n, scale, scale_inv, amax, q4, q8));
+    else TWEO_CUDA_TRY(launch_chain(fp4_cast_kernel<CURRENT, 2>, grid, dim3(kThreads), 0, st, 0, x, n, scale, scale_inv, amax, q4, q8));
   }
   count_launch();
   return check_launch("tweo_fp4_quantize");
@@ -253,12 +255,18 @@ extern "C" tweo_status_t tweo_w4a4_static_gemm(const uint16_t* x, int64_t ldx, c
   if ((N & 15) || (K & 15) || ldx != K) return TWEO_ERR_UNSUPPORTED_SHAPE;
   if (!ws || ws_bytes < tweo_workspace_bytes(TWEO_OP_W8A8, M, N, K)) return TWEO_ERR_WORKSPACE_TOO_SMALL;
   if (!aligned16(ws) || !aligned16(x)) return TWEO_ERR_ALIGNMENT;
-  float* scalars = reinterpret_cast<float*>(ws);  // [0] = 1 / sx, [1] = amax of x (by-product)
   uint8_t* carriers = reinterpret_cast<uint8_t*>(ws) + 256;
-  tweo_status_t s = tweo_fp4_quantize(x, M * K, TWEO_SCALE_GIVEN, const_cast<float*>(sx), scalars, scalars + 1, nullptr,
-                                      carriers, stream);
+  cudaStream_t st = (cudaStream_t)stream;
+  const int64_t n16 = M * K >> 4, sweep = (int64_t)sm_count() * 8 * kThreads;
+  auto cast = n16 >= 8 * sweep ? fp4_cast_kernel<CODES, 4> : n16 >= sweep ? fp4_cast_kernel<CODES, 2> : fp4_cast_kernel<CODES, 1>;
+  const dim3 grid(cast_grid(n16, n16 >= 8 * sweep ? 4 : n16 >= sweep ? 2 : 1));
+  TWEO_CUDA_TRY(launch_chain(cast, grid, dim3(kThreads), 0, st, 0, x, M * K, const_cast<float*>(sx), (float*)nullptr, (float*)nullptr,
+                             (uint8_t*)nullptr, carriers));
+  count_launch();
+  tweo_status_t s = check_launch("tweo_w4a4_static_gemm");
   if (s != TWEO_OK) return s;
   const size_t used = 256 + (((size_t)M * (size_t)K + 255) & ~(size_t)255);
-  return gemm_fwd_codes(carriers, K, TWEO_E4M3, wq8, ldw, TWEO_E4M3, scalars, sw_inv, y, ldy, M, N, K, nullptr,
-                        reinterpret_cast<char*>(ws) + used, ws_bytes - used, (cudaStream_t)stream, false, true, false);
+  // fp4_cast_kernel waits before it releases: what was enqueued before this call has completed when the product starts
+  return gemm_fwd_codes(carriers, K, TWEO_E4M3, wq8, ldw, TWEO_E4M3, sx, sw_inv, y, ldy, M, N, K, nullptr,
+                        reinterpret_cast<char*>(ws) + used, ws_bytes - used, st, true, true, true);
 }

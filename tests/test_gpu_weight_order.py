@@ -86,3 +86,15 @@ def test_packed_weight_linear_behind_the_call_that_writes_its_weight(tw, writer,
         return out.q4.view(N, K // 2)
 
     run(tw, weight_of, lambda w: tw.fp4_weight_linear(x, one, w, one))
+
+
+# the product behind the call's own cast loads its weight at once: the call before has to have completed by then
+@pytest.mark.parametrize("M", [1, 16, 128, 300])
+def test_static_4_bit_linear_behind_the_cast_of_its_weight(tw, M):
+    N, K = 2048, 4096
+    one = torch.ones(1, device="cuda")
+    ws = [torch.randn((N, K), generator=torch.Generator().manual_seed(40 + s)).to(torch.bfloat16).cuda() for s in range(STEPS)]
+    x = torch.randn((M, K), generator=torch.Generator().manual_seed(6)).to(torch.bfloat16).cuda()
+    out = tw.QuantizedFP4(None, torch.zeros((N, K), dtype=torch.uint8, device="cuda"), *(torch.ones(1, device="cuda") for _ in range(3)))
+    buf = tw.new_workspace(tw.OP_W8A8, M, N, K)
+    run(tw, lambda s: tw.fp4_quantize(ws[s], packed=False, out=out).q8, lambda w: tw.w4a4_static_gemm(x, one, w, one, ws=buf))
