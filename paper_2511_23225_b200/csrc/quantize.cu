@@ -18,6 +18,8 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace tweo_detail {
@@ -388,7 +390,7 @@ __global__ void __launch_bounds__(kThreads) cast_given_batch_kernel(const __grid
 
 // ---------------------------------------------------------------------------------------
 // Small tensors, either kind of scale, up to TWEO_MAX_QUANT_BATCH in ONE launch and without a workspace: a cluster of
-// eight CTAs per tensor, whose maxima meet through distributed shared memory.  At these sizes the launches are the cost
+// eight CTAs per tensor, which write their maxima into each other's shared memory.  At these sizes the launches are the cost
 // (2 to 4 us each in a chain, two to four of them in the other forms), not the bytes: eight SMs read a tensor twice, the
 // second time from L1 or L2.
 constexpr int kSmallCluster = 8;
@@ -425,8 +427,9 @@ __device__ __forceinline__ void small_cast_share(const QTensor& t, float s, int 
 __global__ void __launch_bounds__(kSmallThreads) small_cast_kernel(const __grid_constant__ QBatch b) {
   namespace cg = cooperative_groups;
   __shared__ uint32_t part[kSmallThreads / 32];
-  __shared__ uint32_t mine;
+  __shared__ uint32_t maxima[kSmallCluster];   // one per CTA of the cluster, written by it
   cg::cluster_group cluster = cg::this_cluster();
+  cluster.barrier_arrive();   // this CTA has started: its peers may write into its maxima[]
   chain_wait();
   chain_release();   // in this order the kernels behind do not crowd in early (train step of a small linear: 21.5 -> 20.2 us)
   const int ti = blockIdx.x / kSmallCluster;
@@ -461,18 +464,15 @@ __global__ void __launch_bounds__(kSmallThreads) small_cast_kernel(const __grid_
   }
   uint32_t m = __reduce_max_sync(0xFFFFFFFFu, absmax_f32_bits(m0, m1));
   if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = m;
+  cluster.barrier_wait();
   __syncthreads();
   if (threadIdx.x < 32) {
     m = __reduce_max_sync(0xFFFFFFFFu, threadIdx.x < kSmallThreads / 32 ? part[threadIdx.x] : 0u);
-    if (threadIdx.x == 0) mine = m;
+    if (threadIdx.x < kSmallCluster) *cluster.map_shared_rank(&maxima[rank], threadIdx.x) = m;
   }
-  cluster.sync();
-  if (threadIdx.x < 32) {
-    m = __reduce_max_sync(0xFFFFFFFFu, threadIdx.x < kSmallCluster ? *cluster.map_shared_rank(&mine, threadIdx.x) : 0u);
-    if (threadIdx.x == 0) part[0] = m;
-  }
-  __syncthreads();
-  const float amax = __uint_as_float(part[0] << 16);   // non-negative bf16 pattern -> binary32
+  cluster.sync();   // all maxima are there; nobody reaches into another CTA after this
+  m = __reduce_max_sync(0xFFFFFFFFu, (threadIdx.x & 31) < kSmallCluster ? maxima[threadIdx.x & 31] : 0u);
+  const float amax = __uint_as_float(m << 16);   // non-negative bf16 pattern -> binary32
   if (!given) s = scale_from_amax(amax, t.fmt);
   if (rank == 0 && threadIdx.x == 0) {
     *t.amax = amax;
@@ -483,21 +483,34 @@ __global__ void __launch_bounds__(kSmallThreads) small_cast_kernel(const __grid_
     if (t.fmt == TWEO_E4M3) small_cast_share<TWEO_E4M3, false>(t, s, rank, m0, m1);
     else small_cast_share<TWEO_E5M2, false>(t, s, rank, m0, m1);
   }
-  cluster.sync();   // nobody leaves while a peer may still read its maximum
 }
 
 int grid_for(int64_t work_items, int per_cta, int ctas_per_sm);
 
-// Where one cluster per tensor is the faster form.  Microseconds per call in a chain, this form / the others:
-//   one tensor, given scale       2^16 2.6 / 2.4   2^17 2.9 / 2.5   2^19 4.6 / 2.6      current  2^17 3.4 / 3.4   2^19 6.3 / 3.5
-//   three, both formats, current  2^16 3.2 / 7.7   2^19 6.5 / 9.4   2^20 10.1 / 12.7    2^21 17.2 / 15.8
-//   three, given                  2^16 2.9 / 5.6   2^19 4.9 / 5.8   2^20 6.9 / 7.4      2^21 10.9 / 8.5
-// One tensor gains launches (each costs its host 2 us), not device time; several gain both.
-constexpr int64_t kSmallElemsOne = 1 << 17, kSmallElemsBatch = 1 << 20;
+// Where one cluster per tensor is no slower than the other forms.  Microseconds per call replayed from a graph, this form /
+// the others (all tensors in one format; in parentheses: in both):
+//   one, given       2^10 1.8 / 2.2   2^14 2.1 / 2.3   2^17 2.35 / 2.40  2^19 4.2 / 2.4
+//   one, current     2^10 2.2 / 2.9   2^14 2.6 / 3.3   2^17 2.9 / 3.5    2^19 6.0 / 3.6
+//   two, given       2^16 2.1 / 3.5   2^18 3.1 / 3.7   2^19 4.3 / 3.9 (4.3 / 5.1)   2^20 6.2 / 4.9 (6.2 / 6.1)
+//   three, given     2^16 2.2 / 4.6   2^19 4.3 / 5.5   2^20 6.3 / 6.2 (6.4 / 7.6)
+//   four, given      2^16 2.3 / 5.4   2^19 4.2 / 7.2   2^20 6.4 / 9.1
+//   two, current     2^16 2.7 / 5.1   2^19 6.0 / 6.2   2^20 9.7 / 8.4
+//   three, current   2^16 2.7 / 6.8   2^19 6.0 / 10.2  2^20 9.7 / 14.0   2^21 17 / 16
+// Issued call by call the one launch also saves its host the others, 2 us each.
+int64_t small_limit(const tweo_quant_desc_t* descs, int count) {
+  if (count == 1) return 1 << 17;
+  bool given = true, both = false;
+  for (int i = 0; i < count; ++i) {
+    given &= descs[i].mode == TWEO_SCALE_GIVEN;
+    both |= descs[i].fmt != descs[0].fmt;
+  }
+  return (int64_t)1 << std::min(given ? 16 + count + (both ? 1 : 0) : 17 + count, 20);
+}
 
 bool all_small(const tweo_quant_desc_t* descs, int count) {
+  const int64_t limit = small_limit(descs, count);
   for (int i = 0; i < count; ++i)
-    if (descs[i].n > (count == 1 ? kSmallElemsOne : kSmallElemsBatch) || descs[i].sat_count) return false;
+    if (descs[i].n > limit || descs[i].sat_count) return false;
   return true;
 }
 

@@ -45,3 +45,24 @@ def test_small_casts_bit_exact(tw, n):
             assert np.array_equal(o.q.cpu().numpy(), ref["q"])
             for name in ("amax", "scale", "scale_inv"):
                 assert word(getattr(o, name)) == int(np.float32(ref[name]).view(np.uint32))
+
+
+# up to these sizes one launch is no slower than the separate kernels, beyond them they are the faster form
+@pytest.mark.parametrize("count,given,both,top", [(1, True, False, 17), (1, False, False, 17), (2, True, False, 18), (2, True, True, 19),
+                                                  (3, True, False, 19), (3, True, True, 20), (4, True, False, 20), (2, False, False, 19),
+                                                  (3, False, True, 20), (8, False, False, 20)])
+def test_the_one_launch_form_is_taken_where_it_pays(tw, count, given, both, top):
+    mode = tw.SCALE_GIVEN if given else tw.SCALE_CURRENT
+    ws = tw.new_workspace(tw.OP_QUANTIZE)
+    for n, one in ((1 << top, True), ((1 << top) + 16, False)):
+        xs = [torch.full((n,), 1.0 + i, dtype=torch.bfloat16, device="cuda") for i in range(count)]
+        outs = [tw.Quantized(torch.empty(n, dtype=torch.uint8, device="cuda"), *(torch.ones(1, device="cuda") for _ in range(3)), None,
+                             tw.E5M2 if both and i == 0 else tw.E4M3) for i in range(count)]
+        before = tw.launch_count()
+        if count == 1:
+            tw.quantize_per_tensor(xs[0], tw.E4M3, mode, out=outs[0], ws=ws)
+        else:
+            tw.quantize_per_tensor_batch(xs, outs, [mode] * count, ws=ws)
+        assert (tw.launch_count() - before == 1) == one
+        torch.cuda.synchronize()
+        assert all(o.amax.item() == 1.0 + i for i, o in enumerate(outs))
