@@ -290,10 +290,14 @@ class BlockStep:
             ready.append(ev)
             for i in batch:
                 cast_pos[i] = pos
-            if self.variant != "plain":
-                # With given scales the next casts start one hop behind the event that frees the GEMM: they fill every SM
-                # and would keep it waiting.  Step of the ViT-B/16 block, 20000 tokens, fused: 806 -> 765 us.  The two
-                # passes of current scaling gain nothing from coming second (GPT-2-small block 291 -> 295).
+            if self.variant == "unfused":
+                # Here a GEMM batch goes ahead of the next casts, which wait for the event in front of it: for what frees
+                # the GEMM and, from the second batch on, for the GEMM batch before.  Replayed from a graph / call by call,
+                # all casts first -> this, us: ViT-B/16 block, 20000 tokens, 809 -> 680 / 798 -> 761; LLaMA-1B block, 16384
+                # tokens, 2767 -> 2595 / 2887 -> 2685; GPT-2-small block, 8192 tokens, 263 -> 261 / 298 -> 308.  The other
+                # variants issue all casts first.  Fused, the same three: 689 -> 681 / 756 -> 763, 2414 -> 2437 /
+                # 2531 -> 2549, 245 -> 249 / 272 -> 272 (at 32768 tokens 965 -> 962 / 954 -> 1013); plain: 756 -> 721 /
+                # 720 -> 756, 2684 -> 2414 / 2636 -> 2621, 268 -> 268 / 272 -> 283.
                 begun = launch_gemms()
                 if begun is not None:
                     side.wait_event(begun)
