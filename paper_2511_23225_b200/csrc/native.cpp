@@ -12,6 +12,7 @@
 
 #include <exception>
 #include <string>
+#include <vector>
 
 #include "tweo.h"
 
@@ -173,7 +174,7 @@ PyObject* guarded(Py_ssize_t n, Py_ssize_t want, F&& f) {
 // Names of attributes and dictionary keys, interned once at import.
 struct Names {
   PyObject *q, *scale, *scale_inv, *amax, *sat_count, *fmt;
-  PyObject *product, *fmt_x, *fmt_w, *fmt_dy, *xq, *wq, *dyq, *sx_inv, *sw_inv, *sdy_inv, *out, *out_amax, *out_q, *q_fmt, *q_scale;
+  PyObject *product, *fmt_x, *fmt_w, *fmt_dy, *xq, *wq, *dyq, *sx_inv, *sw_inv, *sdy_inv, *out, *out_amax, *out_q, *q_fmt, *q_scale, *get;
 } N;
 
 struct Epi {
@@ -381,14 +382,29 @@ FN(linear_bwd, 12, {
   return PyTuple_Pack(2, dx.o, dw.o);
 })
 
-// A problem's value for a key; None where there is none (borrowed).
-PyObject* item(PyObject* dict, PyObject* key) {
-  PyObject* v = PyDict_GetItemWithError(dict, key);
+// What the mappings of a group handed out; kept until the call returns.
+struct Held {
+  std::vector<PyObject*> v;
+  ~Held() {
+    for (PyObject* o : v) Py_DECREF(o);
+  }
+  PyObject* keep(PyObject* o) {
+    if (!o) throw PyFailure{};
+    v.push_back(o);
+    return o;
+  }
+};
+
+// A problem's value for a key; None where there is none (borrowed).  A dict is read directly, another mapping through get().
+PyObject* item(PyObject* map, PyObject* key, Held& held) {
+  if (!PyDict_CheckExact(map)) return held.keep(PyObject_CallMethodOneArg(map, N.get, key));
+  PyObject* v = PyDict_GetItemWithError(map, key);
   if (!v && PyErr_Occurred()) throw PyFailure{};
   return v ? v : Py_None;
 }
-int32_t item_i32(PyObject* dict, PyObject* key, int32_t otherwise) {
-  PyObject* v = item(dict, key);
+PyObject* required(PyObject* map, PyObject* key, Held& held) { return held.keep(PyObject_GetItem(map, key)); }
+int32_t item_i32(PyObject* map, PyObject* key, int32_t otherwise, Held& held) {
+  PyObject* v = item(map, key, held);
   return v == Py_None ? otherwise : i32(v);
 }
 
@@ -400,24 +416,19 @@ FN(linear_group, 1, {
   if (count < 1 || count > most) fail(PyExc_ValueError, "need 1..MAX_GROUP problems");
   tweo_linear_problem_t pr[most] = {};
   Epi epi[most];
+  Held held;
   for (Py_ssize_t i = 0; i < count; ++i) {
     PyObject* d = PySequence_Fast_GET_ITEM(list.o, i);
-    if (!PyDict_Check(d)) fail(PyExc_TypeError, "a problem is a dict");
     tweo_linear_problem_t& p = pr[i];
-    PyObject* fmt = item(d, N.q_fmt);
+    PyObject* fmt = item(d, N.q_fmt, held);
     Ref q_fmt(fmt == Py_None ? PyLong_FromLong(TWEO_E4M3) : Py_NewRef(fmt));
-    epi[i].fill(item(d, N.out_amax), item(d, N.out_q), q_fmt.o, item(d, N.q_scale));
+    epi[i].fill(item(d, N.out_amax, held), item(d, N.out_q, held), q_fmt.o, item(d, N.q_scale, held));
     p.epi = epi[i].p;
-    PyObject* product = item(d, N.product);
-    if (product == Py_None) {
-      PyErr_SetObject(PyExc_KeyError, N.product);
-      throw PyFailure{};
-    }
-    p.product = i32(product);
-    p.fmt_x = item_i32(d, N.fmt_x, TWEO_E4M3);
-    p.fmt_w = item_i32(d, N.fmt_w, TWEO_E4M3);
-    p.fmt_dy = item_i32(d, N.fmt_dy, TWEO_E5M2);
-    PyObject *xq = item(d, N.xq), *wq = item(d, N.wq), *dyq = item(d, N.dyq);
+    p.product = i32(required(d, N.product, held));
+    p.fmt_x = item_i32(d, N.fmt_x, TWEO_E4M3, held);
+    p.fmt_w = item_i32(d, N.fmt_w, TWEO_E4M3, held);
+    p.fmt_dy = item_i32(d, N.fmt_dy, TWEO_E5M2, held);
+    PyObject *xq = item(d, N.xq, held), *wq = item(d, N.wq, held), *dyq = item(d, N.dyq, held);
     Mat x{}, w{}, dy{};
     if (xq != Py_None || p.product == TWEO_PRODUCT_FWD || p.product == TWEO_PRODUCT_WGRAD) x = mat(xq, kCodes, "xq");
     if (wq != Py_None || p.product == TWEO_PRODUCT_FWD || p.product == TWEO_PRODUCT_DGRAD) w = mat(wq, kCodes, "wq");
@@ -434,10 +445,10 @@ FN(linear_group, 1, {
     p.xq = (const uint8_t*)x.p, p.ldx = x.ld;
     p.wq = (const uint8_t*)w.p, p.ldw = w.ld;
     p.dyq = (const uint8_t*)dy.p, p.lddy = dy.ld;
-    p.sx_inv = f32_or_null(item(d, N.sx_inv), "sx_inv");
-    p.sw_inv = f32_or_null(item(d, N.sw_inv), "sw_inv");
-    p.sdy_inv = f32_or_null(item(d, N.sdy_inv), "sdy_inv");
-    const Mat o = mat(item(d, N.out), kBf16, "out");
+    p.sx_inv = f32_or_null(item(d, N.sx_inv, held), "sx_inv");
+    p.sw_inv = f32_or_null(item(d, N.sw_inv, held), "sw_inv");
+    p.sdy_inv = f32_or_null(item(d, N.sdy_inv, held), "sdy_inv");
+    const Mat o = mat(required(d, N.out, held), kBf16, "out");
     p.out = (uint16_t*)o.p;
     p.ldo = o.ld;
   }
@@ -682,7 +693,7 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", "Argument marshalling of
 
 PyMODINIT_FUNC PyInit__native(void) {
   const char* const text[] = {"q", "scale", "scale_inv", "amax", "sat_count", "fmt", "product", "fmt_x", "fmt_w", "fmt_dy", "xq", "wq",
-                              "dyq", "sx_inv", "sw_inv", "sdy_inv", "out", "out_amax", "out_q", "q_fmt", "q_scale"};
+                              "dyq", "sx_inv", "sw_inv", "sdy_inv", "out", "out_amax", "out_q", "q_fmt", "q_scale", "get"};
   PyObject** const slot = reinterpret_cast<PyObject**>(&N);
   static_assert(sizeof(text) / sizeof(text[0]) == sizeof(Names) / sizeof(PyObject*), "one name per slot");
   for (size_t i = 0; i < sizeof(text) / sizeof(text[0]); ++i)

@@ -1,0 +1,36 @@
+"""What the calls of the native marshalling module accept and refuse."""
+import collections
+import types
+
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def tw():
+    from paper_2511_23225_b200 import binding
+    binding.lib()
+    return binding
+
+
+def codes(shape, seed):
+    return torch.randint(0, 0x70, shape, generator=torch.Generator().manual_seed(seed), dtype=torch.uint8).cuda()
+
+
+@pytest.mark.parametrize("kind", [dict, collections.OrderedDict, collections.UserDict, types.MappingProxyType, lambda d: collections.ChainMap({}, d),
+                                  lambda d: collections.defaultdict(lambda: None, d)])
+def test_a_grouped_problem_is_any_mapping(tw, kind):
+    x, w, one = codes((256, 256), 1), codes((384, 256), 2), torch.ones(1, device="cuda")
+    y, amax, copy = torch.zeros((256, 384), dtype=torch.bfloat16, device="cuda"), torch.zeros(1, device="cuda"), torch.zeros((256, 384), dtype=torch.uint8, device="cuda")
+    problem = dict(product=tw.PRODUCT_FWD, xq=x, wq=w, sx_inv=one, sw_inv=one, out=y, out_amax=amax, out_q=copy, q_scale=one)
+    tw.fp8_linear_group([kind(problem)])
+    torch.cuda.synchronize()
+    assert torch.equal(y, tw.fp8_linear_fwd(x, w, one, one)) and amax.item() == y.float().abs().max().item() and copy.any()
+    for missing in ("product", "out"):
+        if kind is dict or kind is collections.UserDict:
+            with pytest.raises(KeyError):
+                tw.fp8_linear_group([kind({k: v for k, v in problem.items() if k != missing})])
+    with pytest.raises(TypeError):
+        tw.fp8_linear_group([kind({**problem, "wq": w.cpu()})])
