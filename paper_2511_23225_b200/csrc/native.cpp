@@ -27,7 +27,7 @@ struct PyFailure {};   // a Python exception is set
   throw PyFailure{};
 }
 
-enum Kind : unsigned { kBf16 = 1, kF32 = 2, kU8 = 4, kI8 = 8, kCodes = 16 };   // kCodes: uint8 or an FP8 type
+enum Kind : unsigned { kBf16 = 1, kF32 = 2, kU8 = 4, kI8 = 8, kCodes = 16, kAny = 32 };   // kCodes: uint8 or an FP8 type
 
 const char* kind_text(unsigned k) {
   switch (k) {
@@ -58,7 +58,7 @@ const at::Tensor& tensor(PyObject* o, const char* name) {
 }
 
 void check_kind(const at::Tensor& t, unsigned want, const char* name) {
-  if (!(kind_of(t.scalar_type()) & want))
+  if (want != kAny && !(kind_of(t.scalar_type()) & want))
     fail(PyExc_TypeError, std::string(name) + " has dtype " + c10::toString(t.scalar_type()) + ", expected " + kind_text(want));
 }
 
@@ -201,8 +201,9 @@ const at::Tensor& contiguous_bf16(PyObject* o, const char* name) {
   return t;
 }
 
-// What a Quantized record holds, for the cast of x.
-void fill_desc(tweo_quant_desc_t& d, PyObject* x, PyObject* out, int32_t fmt, int32_t mode) {
+// What a Quantized record holds, for the cast of x.  typed: the outputs must have the types the cast writes (a batch); a single
+// cast writes into the memory of any CUDA tensors, bytes of int8 storage for instance.
+void fill_desc(tweo_quant_desc_t& d, PyObject* x, PyObject* out, int32_t fmt, int32_t mode, bool typed) {
   const at::Tensor& t = contiguous_bf16(x, "x");
   Ref scale(PyObject_GetAttr(out, N.scale)), inv(PyObject_GetAttr(out, N.scale_inv)), amax(PyObject_GetAttr(out, N.amax)),
       q(PyObject_GetAttr(out, N.q)), sat(PyObject_GetAttr(out, N.sat_count));
@@ -211,16 +212,16 @@ void fill_desc(tweo_quant_desc_t& d, PyObject* x, PyObject* out, int32_t fmt, in
   d.fmt = fmt;
   d.mode = mode;
   d.scale = f32(scale.o, "scale");
-  d.scale_inv = f32(inv.o, "scale_inv");
-  d.amax = f32(amax.o, "amax");
-  d.q = dev<uint8_t>(q.o, kCodes, "q");
+  d.scale_inv = dev<float>(inv.o, typed ? kF32 : kAny, "scale_inv");
+  d.amax = dev<float>(amax.o, typed ? kF32 : kAny, "amax");
+  d.q = dev<uint8_t>(q.o, typed ? kCodes : kAny, "q");
   d.sat_count = sat.o == Py_None ? nullptr : (uint32_t*)tensor(sat.o, "sat_count").data_ptr();
 }
 
 // quantize(x, out, fmt, mode, ws)
 FN(quantize, 5, {
   tweo_quant_desc_t d;
-  fill_desc(d, a[0], a[1], i32(a[2]), i32(a[3]));
+  fill_desc(d, a[0], a[1], i32(a[2]), i32(a[3]), false);
   const Ws w = workspace(a[4]);
   void* st = stream();
   call("tweo_quantize_per_tensor", [&] {
@@ -242,7 +243,7 @@ FN(quantize_batch, 4, {
     PyObject* o = PySequence_Fast_GET_ITEM(outs.o, i);
     Ref fmt(PyObject_GetAttr(o, N.fmt));
     fill_desc(d[i], PySequence_Fast_GET_ITEM(xs.o, i), o, i32(fmt.o),
-              modes.o == Py_None ? TWEO_SCALE_CURRENT : i32(PySequence_Fast_GET_ITEM(modes.o, i)));
+              modes.o == Py_None ? TWEO_SCALE_CURRENT : i32(PySequence_Fast_GET_ITEM(modes.o, i)), true);
   }
   const Ws w = workspace(a[3]);
   void* st = stream();

@@ -34,3 +34,22 @@ def test_a_grouped_problem_is_any_mapping(tw, kind):
                 tw.fp8_linear_group([kind({k: v for k, v in problem.items() if k != missing})])
     with pytest.raises(TypeError):
         tw.fp8_linear_group([kind({**problem, "wq": w.cpu()})])
+
+
+def test_a_single_cast_writes_into_storage_of_any_type(tw):
+    x = torch.randn(4096, generator=torch.Generator().manual_seed(3)).to(torch.bfloat16).cuda()
+    ref = tw.quantize_per_tensor(x)
+    for qt in (torch.uint8, torch.int8, torch.float8_e4m3fn):
+        cell = lambda: torch.zeros(1, dtype=torch.int32, device="cuda")
+        out = tw.Quantized(torch.zeros(4096, dtype=qt, device="cuda"), torch.zeros(1, device="cuda"), cell(), cell(), cell(), tw.E4M3)
+        assert tw.quantize_per_tensor(x, out=out) is out
+        torch.cuda.synchronize()
+        assert torch.equal(out.q.view(torch.uint8), ref.q) and torch.equal(out.scale, ref.scale)
+        assert torch.equal(out.amax.view(torch.float32), ref.amax) and torch.equal(out.scale_inv.view(torch.float32), ref.scale_inv)
+        assert out.sat_count.item() == 0
+        if qt == torch.int8:
+            with pytest.raises(TypeError):        # a batch states what it takes
+                tw.quantize_per_tensor_batch([x], [out])
+        out.q = out.q.cpu()
+        with pytest.raises(TypeError):
+            tw.quantize_per_tensor(x, out=out)
