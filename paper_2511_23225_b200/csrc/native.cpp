@@ -88,10 +88,11 @@ struct Ws {
   void* p;
   size_t n;
 };
-Ws workspace(PyObject* o) {
+// any: storage of any type, of which a byte per element is used (the calls whose workspace is no option).
+Ws workspace(PyObject* o, bool any = false) {
   if (o == Py_None) return Ws{nullptr, 0};
   const at::Tensor& t = tensor(o, "ws");
-  check_kind(t, kU8, "ws");
+  if (!any) check_kind(t, kU8, "ws");
   return Ws{t.data_ptr(), (size_t)t.numel()};
 }
 
@@ -245,7 +246,7 @@ FN(quantize_batch, 4, {
     fill_desc(d[i], PySequence_Fast_GET_ITEM(xs.o, i), o, i32(fmt.o),
               modes.o == Py_None ? TWEO_SCALE_CURRENT : i32(PySequence_Fast_GET_ITEM(modes.o, i)), true);
   }
-  const Ws w = workspace(a[3]);
+  const Ws w = workspace(a[3], true);
   void* st = stream();
   call("tweo_quantize_per_tensor_batch", [&] { return tweo_quantize_per_tensor_batch(d, (int32_t)count, w.p, w.n, st); });
   Py_RETURN_NONE;
@@ -481,7 +482,7 @@ FN(loss, 9, {
     if (i < ng) pg[i] = dev(PySequence_Fast_GET_ITEM(grads.o, i), gdt == TWEO_BF16 ? kBf16 : kF32, "grad");
   }
   const float tau = flt(a[1]), eps = flt(a[2]), p = flt(a[3]), c = flt(a[4]);
-  const Ws w = workspace(a[7]);
+  const Ws w = workspace(a[7], true);
   const at::Device device = tensor(PySequence_Fast_GET_ITEM(blocks.o, 0), "block output").device();
   const at::Tensor out = empty({1}, at::kFloat, device);
   at::Tensor pb;
@@ -504,7 +505,7 @@ FN(w8a8, 6, {
   same(x.cols, w.cols, "inner dimensions differ");
   Out y(a[4], x.rows, w.rows, t.device(), "y");
   const float *sx = f32(a[1], "sx"), *sw = f32(a[3]);
-  const Ws ws = workspace(a[5]);
+  const Ws ws = workspace(a[5], true);
   void* st = stream();
   call("tweo_w8a8_static_gemm", [&] {
     return tweo_w8a8_static_gemm(x.p, k & kBf16 ? TWEO_BF16 : TWEO_FP8_E4M3, x.ld, sx, (const uint8_t*)w.p, w.ld, sw, (uint16_t*)y.m.p,
@@ -548,7 +549,7 @@ FN(block_output, 13, {
   uint8_t* pq = cast ? dev<uint8_t>(aq.o, kCodes, "aq") : nullptr;
   const int32_t fmt = cast ? i32(a[7]) : 0;
   const float* qs = f32_or_null(a[8], "q_scale");
-  const Ws w = workspace(a[12]);
+  const Ws w = workspace(a[12], true);
   const float tau = flt(a[2]), eps = flt(a[3]), p = flt(a[4]), c = flt(a[5]);
   const at::Tensor two = empty({2}, at::kFloat, device);
   float* scalars = (float*)two.data_ptr();

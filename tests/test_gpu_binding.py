@@ -53,3 +53,22 @@ def test_a_single_cast_writes_into_storage_of_any_type(tw):
         out.q = out.q.cpu()
         with pytest.raises(TypeError):
             tw.quantize_per_tensor(x, out=out)
+
+
+def test_a_required_workspace_is_storage_of_any_type(tw):
+    def both(op, call, *shape):
+        ws = tw.new_workspace(op, *shape)
+        ref = call(ws)
+        got = call(torch.zeros(ws.numel(), dtype=torch.int32, device="cuda"))
+        torch.cuda.synchronize()
+        assert all(torch.equal(a.view(torch.uint8), b.view(torch.uint8)) for a, b in zip(ref, got))
+        with pytest.raises(TypeError):
+            call(ws.cpu())
+
+    x, f = (torch.randn((16, 256), generator=torch.Generator().manual_seed(s)).to(torch.bfloat16).cuda() for s in (1, 2))
+    w, one = codes((272, 256), 3), torch.ones(1, device="cuda")
+    record = lambda: tw.Quantized(torch.zeros(x.shape, dtype=torch.uint8, device="cuda"), *(torch.zeros(1, device="cuda") for _ in range(3)), None, tw.E4M3)
+    both(tw.OP_QUANTIZE, lambda ws: [tw.quantize_per_tensor_batch([x], [record()], ws=ws)[0].q])
+    both(tw.OP_LOSS, lambda ws: [tw.loss_fwd_bwd([x, f], ws=ws)[0]], x.numel(), 2)
+    both(tw.OP_W8A8, lambda ws: [tw.w8a8_static_gemm(x, one, w, one, ws=ws)], 16, 272, 256)
+    both(tw.OP_BLOCK_OUTPUT, lambda ws: tw.block_output_fused(x, f, ws=ws)[:4])
