@@ -19,6 +19,8 @@ from dataclasses import dataclass
 
 import torch
 
+from .build import native_target
+
 E4M3, E5M2 = 0, 1
 SCALE_CURRENT, SCALE_GIVEN = 0, 1
 BF16, F32, FP8_E4M3 = 0, 1, 2
@@ -153,6 +155,11 @@ def _native():
         spec = importlib.util.spec_from_file_location(__package__ + "._native", NATIVE_PATH)
         m = importlib.util.module_from_spec(spec)
         spec.loader.exec_module(m)
+        built_for = getattr(m, "BUILT_FOR", "another version")
+        if built_for != native_target():
+            raise RuntimeError(
+                f"{NATIVE_PATH} was built for {built_for}, this is {native_target()}: build it again with "
+                "`python -m paper_2511_23225_b200.build`")
         m.set_error(TweoError)
         _native_module = m
     return _native_module

@@ -21,15 +21,23 @@ def _newer(a: str, b: str) -> bool:
     return not os.path.exists(b) or os.path.getmtime(a) > os.path.getmtime(b)
 
 
+def native_target() -> str:
+    """What the extension module is compiled against beside its sources: torch's C++ interface and Python's C interface."""
+    import torch
+    return f"torch {torch.__version__} cxx11_abi {int(torch._C._GLIBCXX_USE_CXX11_ABI)} python {sysconfig.get_config_var('EXT_SUFFIX')}"
+
+
 def build_native(force: bool = False, verbose: bool = False) -> str:
     """The extension module of binding.py (csrc/native.cpp), linked against the library beside it."""
     src, header = os.path.join(CSRC, "native.cpp"), os.path.join(_ROOT, "include", "tweo.h")
-    if force or _newer(src, NATIVE) or _newer(header, NATIVE):
+    target, stamp = native_target(), os.path.join(_HERE, "_build", "native.target")
+    built_for = open(stamp).read() if os.path.exists(stamp) else None
+    if force or built_for != target or _newer(src, NATIVE) or _newer(header, NATIVE):
         import torch
         base = os.path.dirname(torch.__file__)
         tmp = NATIVE + f".tmp{os.getpid()}"
         cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
-               f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+               f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", f'-DTWEO_BUILT_FOR="{target}"',
                "-I", os.path.join(_ROOT, "include"), "-isystem", os.path.join(base, "include"),
                "-isystem", os.path.join(base, "include", "torch", "csrc", "api", "include"),
                "-isystem", "/usr/local/cuda/include", "-isystem", sysconfig.get_paths()["include"], src, "-o", tmp,
@@ -39,6 +47,9 @@ def build_native(force: bool = False, verbose: bool = False) -> str:
             sys.stderr.write(" ".join(cmd) + "\n")
         subprocess.check_call(cmd)
         os.replace(tmp, NATIVE)
+        os.makedirs(os.path.dirname(stamp), exist_ok=True)
+        with open(stamp, "w") as f:
+            f.write(target)
     return NATIVE
 
 

@@ -700,5 +700,7 @@ PyMODINIT_FUNC PyInit__native(void) {
   static_assert(sizeof(text) / sizeof(text[0]) == sizeof(Names) / sizeof(PyObject*), "one name per slot");
   for (size_t i = 0; i < sizeof(text) / sizeof(text[0]); ++i)
     if (!(slot[i] = PyUnicode_InternFromString(text[i]))) return nullptr;
-  return PyModule_Create(&module);
+  PyObject* m = PyModule_Create(&module);
+  if (m && PyModule_AddStringConstant(m, "BUILT_FOR", TWEO_BUILT_FOR) < 0) Py_CLEAR(m);
+  return m;
 }
