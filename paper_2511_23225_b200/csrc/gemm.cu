@@ -695,7 +695,7 @@ struct SkinnyPlan {
 constexpr int skinny_smem(bool wide) { return (wide ? 200 : 100) * 1024 + 1024 + 256; }
 
 // Never launched: resident_clusters() asks how many clusters of it fit.  Asking about the few-token kernel itself, with
-// success, left its later launches slower (one token, 4-bit weights [8192x8192]: 15.4 us a pass against 10.9), as if two of its CTAs no longer met on an SM.
+// success, left its later launches slower (one token, 4-bit weights [8192x8192]: 15.4 us a pass against 10.9); the cause is not known.
 template <int W>
 __global__ void __launch_bounds__(kThreads, 1) occupancy_probe_kernel(int* p) {
   extern __shared__ uint8_t smem_probe[];
@@ -707,16 +707,14 @@ __global__ void __launch_bounds__(kThreads, 1) occupancy_probe_kernel(int* p) {
 // Asked for once per device.
 int resident_clusters(int slices, bool wide) {
   struct Table {
-    std::atomic<bool> known{false};
+    std::once_flag once;
     int n[2][9];
   };
   static Table tables[64];
-  static std::mutex mu;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return sm_count() * (wide ? 1 : 2) / slices;
   Table& t = tables[dev];
-  if (!t.known.load(std::memory_order_acquire)) {
-    std::lock_guard<std::mutex> lock(mu);
+  std::call_once(t.once, [&t] {
     for (int w = 0; w < 2; ++w) {
       auto kern = w ? occupancy_probe_kernel<1> : occupancy_probe_kernel<0>;
       const int bytes = skinny_smem(w != 0);
@@ -739,8 +737,7 @@ int resident_clusters(int slices, bool wide) {
       }
     }
     (void)cudaGetLastError();
-    t.known.store(true, std::memory_order_release);
-  }
+  });
   return t.n[wide ? 1 : 0][slices];
 }
 

@@ -57,3 +57,32 @@ def test_few_token_data_gradient(tw, M, N, K):
     torch.cuda.synchronize()
     assert tw.read_device_status() == 0
     close(dx, dy.double() @ w.double())
+
+
+def test_first_calls_from_several_threads():
+    """The split of a process's first few-token products, asked for by eight threads at once, each on a stream of its own."""
+    import subprocess
+    import sys
+    code = """
+import threading
+import torch
+from paper_2511_23225_b200 import binding as tw
+x = torch.randint(0, 0x70, (8, 4096), dtype=torch.uint8, device="cuda")
+w = torch.randint(0, 0x70, (4096, 4096), dtype=torch.uint8, device="cuda")
+one, out, gate = torch.ones(1, device="cuda"), [None] * 8, threading.Barrier(8)
+torch.cuda.synchronize()
+def work(i):
+    with torch.cuda.stream(torch.cuda.Stream()):
+        gate.wait()
+        out[i] = tw.fp8_linear_fwd(x[i:i + 1], w, one, one)
+        torch.cuda.current_stream().synchronize()
+ts = [threading.Thread(target=work, args=(i,)) for i in range(8)]
+[t.start() for t in ts]
+[t.join() for t in ts]
+assert tw.read_device_status() == 0
+for i in range(8):
+    assert torch.equal(out[i], tw.fp8_linear_fwd(x[i:i + 1], w, one, one))
+print("same")
+"""
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and r.stdout.split() == ["same"], r.stderr[-2000:]
