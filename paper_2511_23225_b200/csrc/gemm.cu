@@ -715,10 +715,12 @@ int resident_clusters(int slices, bool wide) {
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return sm_count() * (wide ? 1 : 2) / slices;
   Table& t = tables[dev];
   std::call_once(t.once, [&t] {
+    const bool clean = cudaPeekAtLastError() == cudaSuccess;
+    bool failed = false;
     for (int w = 0; w < 2; ++w) {
       auto kern = w ? occupancy_probe_kernel<1> : occupancy_probe_kernel<0>;
       const int bytes = skinny_smem(w != 0);
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+      failed |= cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess;
       for (int c = 1; c <= 8; ++c) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)c);
@@ -732,11 +734,14 @@ int resident_clusters(int slices, bool wide) {
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) n = sm_count() * (w ? 1 : 2) / c;
+        if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) {
+          failed = true;
+          n = sm_count() * (w ? 1 : 2) / c;
+        }
         t.n[w][c] = n;
       }
     }
-    (void)cudaGetLastError();
+    if (failed && clean) (void)cudaGetLastError();   // an error of these queries; one that was there before stays
   });
   return t.n[wide ? 1 : 0][slices];
 }
