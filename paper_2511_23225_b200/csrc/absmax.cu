@@ -384,7 +384,8 @@ extern "C" tweo_status_t tweo_residual_add_q8(const int8_t* xq, const float* sx,
 }
 
 // ------------------------------------------------------------------ per-token 8-bit residual stream (Sec. 4.4)
-// One CTA per row, the block sized to the row: VPT 16-byte vectors of each input per thread, the dequantised sums formed
+// One CTA per row, the block sized to the row, or one warp (the launcher says where): VPT 16-byte vectors of each input per
+// thread, the dequantised sums formed
 // once and held in registers, their maximum found by shuffles and one barrier, the codes of the sum written in the same
 // pass: 2 bytes read and 1 written per element plus three scales per row.  Converting instructions (bytes to binary32 and
 // back) go through a unit that does 16 a clock per SM, five of them per element bounded an earlier form of one warp per
@@ -415,20 +416,24 @@ __device__ __forceinline__ void codes_to_f32x2(uint32_t w, uint64_t& p01, uint64
                              __uint_as_float(__byte_perm(u, 0x4B000000u, 0x7443))), bias);
 }
 
-template <int VPT>
+// WARP: a warp per row, eight rows per CTA (short rows); otherwise the CTA per row.
+template <int VPT, bool WARP>
 __global__ void __launch_bounds__(256) residual_add_q8_rows_kernel(const RowAddArgs a) {
   __shared__ float part[8];
-  chain_release();
+  if (gridDim.x <= 148) chain_release();   // it costs each CTA about 1 ns ([16384x256] 9.9 -> 17.4 us): not with more CTAs than SMs
   chain_wait();
   const int nvec = a.cols >> 4;
-  for (int64_t row = blockIdx.x; row < a.rows; row += gridDim.x) {   // one turn, as in absmax_rows_reg_kernel
-  if (row != blockIdx.x) __syncthreads();
+  const int tid = WARP ? threadIdx.x & 31 : threadIdx.x, threads = WARP ? 32 : blockDim.x;
+  const int64_t first = WARP ? (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5) : blockIdx.x;
+  const int64_t step = WARP ? (int64_t)gridDim.x * 8 : gridDim.x;
+  for (int64_t row = first; row < a.rows; row += step) {   // one turn, as in absmax_rows_reg_kernel
+  if (!WARP && row != first) __syncthreads();
   const uint4* xv = reinterpret_cast<const uint4*>(a.xq + row * a.cols);
   const uint4* fv = reinterpret_cast<const uint4*>(a.fq + row * a.cols);
   uint4 vx[VPT], vf[VPT];
 #pragma unroll
   for (int i = 0; i < VPT; ++i) {
-    const int idx = threadIdx.x + i * blockDim.x;
+    const int idx = tid + i * threads;
     vx[i] = idx < nvec ? __ldcs(xv + idx) : make_uint4(0u, 0u, 0u, 0u);
     vf[i] = idx < nvec ? __ldcs(fv + idx) : make_uint4(0u, 0u, 0u, 0u);
   }
@@ -456,18 +461,20 @@ __global__ void __launch_bounds__(256) residual_add_q8_rows_kernel(const RowAddA
     }
   }
   amax = warp_max(amax);
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = amax;
-  __syncthreads();
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) amax = fmaxf(amax, part[w]);
+  if (!WARP) {
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = amax;
+    __syncthreads();
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) amax = fmaxf(amax, part[w]);
+  }
   const float s = __fadd_rn(amax, a.eps);
   const float c = __fdiv_rn(a.Q, s);
-  if (threadIdx.x == 0) a.sy[row] = s;
+  if (tid == 0) a.sy[row] = s;
   // no sum of the row can have been infinite or NaN, and Q / s is finite: |y c| stays within one rounding of Q
   const bool plain = (fabsf(cx) + fabsf(cf)) * 256.0f < 3.0e38f && c < __int_as_float(0x7F800000);
   uint4* yv = reinterpret_cast<uint4*>(a.yq + row * a.cols);
 #pragma unroll
   for (int i = 0; i < VPT; ++i) {
-    const int idx = threadIdx.x + i * blockDim.x;
+    const int idx = tid + i * threads;
     uint32_t o4[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -511,12 +518,20 @@ extern "C" tweo_status_t tweo_residual_add_q8_rows(const int8_t* xq, const float
   a.eps = eps;
   cudaStream_t st = (cudaStream_t)stream;
   const int64_t nvec = cols >> 4;
-  const dim3 grid((unsigned)std::min<int64_t>(rows, INT32_MAX));
+  const dim3 grid((unsigned)std::min<int64_t>(rows, INT32_MAX)), grid8((unsigned)std::min<int64_t>((rows + 7) / 8, INT32_MAX));
   cudaError_t e;
-  if (nvec <= 256)
-    e = tweo_detail::launch_chain(residual_add_q8_rows_kernel<1>, grid, dim3(row_threads(nvec, 1)), 0, st, 0, a);
+  // A warp per row where a row gives it one vector per lane, or two and there are rows for every SM's warps: with a CTA per
+  // row the start of the CTAs bounds many short rows.  Microseconds, CTA per row / warp per row: [16x512] 1.6 / 1.5,
+  // [16384x256] 9.9 / 6.0, [131072x64] 68.8 / 38.5, [131072x512] 69.2 / 45.3; two vectors [16x1024] 1.6 / 1.8,
+  // [512x768] 1.8 / 2.0, [2048x768] 2.7 / 2.4, [16384x1024] 11.3 / 9.6; four [16384x2048] 21.4 / 21.5.
+  if (nvec <= 32)
+    e = tweo_detail::launch_chain(residual_add_q8_rows_kernel<1, true>, grid8, dim3(256), 0, st, 0, a);
+  else if (nvec <= 64 && rows >= 2048)
+    e = tweo_detail::launch_chain(residual_add_q8_rows_kernel<2, true>, grid8, dim3(256), 0, st, 0, a);
+  else if (nvec <= 256)
+    e = tweo_detail::launch_chain(residual_add_q8_rows_kernel<1, false>, grid, dim3(row_threads(nvec, 1)), 0, st, 0, a);
   else
-    e = tweo_detail::launch_chain(residual_add_q8_rows_kernel<2>, grid, dim3(row_threads(nvec, 2)), 0, st, 0, a);
+    e = tweo_detail::launch_chain(residual_add_q8_rows_kernel<2, false>, grid, dim3(row_threads(nvec, 2)), 0, st, 0, a);
   if (e != cudaSuccess) return tweo_detail::cuda_fail(e, "residual_add_q8_rows_kernel");
   tweo_detail::count_launch();
   return TWEO_OK;

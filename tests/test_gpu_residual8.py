@@ -150,6 +150,25 @@ def test_residual_add_q8_rows_bit_exact_with_extreme_scales(tw, cols):
         assert np.array_equal(yq.cpu().numpy(), ref_q)
 
 
+# a warp per row up to 512 columns, and up to 1024 from 2048 rows on; a block of warps per row elsewhere
+@pytest.mark.parametrize("rows,cols", [(1, 512), (7, 512), (8, 496), (9, 16), (2047, 528), (2048, 528), (2049, 1024), (2055, 512), (2048, 1040)])
+def test_residual_add_q8_rows_at_the_edges_of_its_forms(tw, rows, cols):
+    g = np.random.Generator(np.random.PCG64(rows * 7 + cols))
+    xq = g.integers(-128, 128, (rows, cols), dtype=np.int8)
+    fq = g.integers(-128, 128, (rows, cols), dtype=np.int8)
+    sx = (0.5 + 3.0 * g.random(rows)).astype(np.float32)
+    sf = (0.05 + 0.5 * g.random(rows)).astype(np.float32)
+    for r, (a, b) in zip(range(0, rows, 5), ((0.0, 0.0), (3e38, 3e38), (np.inf, 1.0), (np.nan, 1.0), (1e-44, 1e-44))):
+        sx[r], sf[r] = a, b
+    ref_q, ref_s = orc.residual_add_q8_rows(xq, sx, fq, sf, 8, 1e-6)
+    gx, gf = torch.from_numpy(xq).cuda(), torch.from_numpy(fq).cuda()
+    for out in (None, gx):       # a new tensor, then over x
+        yq, sy = tw.residual_add_q8_rows(gx, dev(sx), gf, dev(sf), 8, 1e-6, yq=out)
+        torch.cuda.synchronize()
+        assert np.array_equal(sy.cpu().numpy().view(np.uint32), ref_s.view(np.uint32))
+        assert np.array_equal(yq.cpu().numpy(), ref_q)
+
+
 def test_per_token_chain_linear_quantise_add(tw):
     """A8(K): x codes per token -> integer linear (per-token x per-channel scales) -> per-token codes of f(x) ->
     per-token codes of x + f(x); every stage against the oracle's stage on the oracle's own inputs."""
