@@ -38,6 +38,33 @@ def test_static_linear_matches_the_product_of_the_codes(tw, M, K, N):
     close(y, x.double() @ w.double().T * (0.125 / 16.0))
 
 
+# the form inference takes: bf16 activations, whose cast the product overlaps (its weight is loaded while the cast runs)
+@pytest.mark.parametrize("M,K,N", [(1, 4096, 1040), (128, 1040, 272), (129, 2064, 528), (257, 4096, 128), (300, 4096, 4096), (777, 3344, 880)])
+def test_static_linear_on_bf16_activations(tw, M, K, N):
+    x = torch.randn((M, K), generator=torch.Generator().manual_seed(M * 3 + K)).to(torch.bfloat16)
+    w, s = codes((N, K), N, std=30.0), 100.0
+    sx, sw = torch.full((1,), s), torch.full((1,), 0.125)
+    y = tw.w8a8_static_gemm(x.cuda(), sx.cuda(), w.view(torch.uint8).cuda(), sw.cuda())
+    again = tw.w8a8_static_gemm(x.cuda(), sx.cuda(), w.view(torch.uint8).cuda(), sw.cuda())
+    torch.cuda.synchronize()
+    assert tw.read_device_status() == 0 and torch.equal(y, again)
+    xq = (x.float() * s).clamp(-448, 448).to(torch.float8_e4m3fn)
+    close(y, xq.double() @ w.double().T * (0.125 / s))
+
+
+# integer sums are exact: the two scales and the bf16 rounding are all that may differ (three roundings of 2^-24, one of 2^-8)
+@pytest.mark.parametrize("M,K,N", [(1, 16, 16), (128, 4096, 272), (129, 2064, 528), (257, 4096, 128), (300, 4096, 4096), (777, 3344, 880)])
+def test_integer_linear_matches_the_product_of_the_codes(tw, M, K, N):
+    g = torch.Generator().manual_seed(M + K + N)
+    x, w = (torch.randint(-127, 128, shape, generator=g, dtype=torch.int8) for shape in ((M, K), (N, K)))
+    sx, sw = torch.rand(M, generator=g) + 0.5, torch.rand(N, generator=g) + 0.5
+    y = tw.int8_linear(x.cuda(), sx.cuda(), w.cuda(), sw.cuda())
+    torch.cuda.synchronize()
+    assert tw.read_device_status() == 0
+    ref = (x.double() @ w.double().T) * (sx.double()[:, None] / 127.0) * (sw.double() / 127.0)
+    assert torch.all((y.double().cpu() - ref).abs() <= ref.abs() * (2.0 ** -8 + 2.0 ** -21))
+
+
 def test_static_linear_into_rows_that_allow_no_wide_stores(tw):
     M, K, N = 5, 512, 144
     x, w = codes((M, K), 3), codes((N, K), 4)

@@ -98,3 +98,18 @@ def test_static_4_bit_linear_behind_the_cast_of_its_weight(tw, M):
     out = tw.QuantizedFP4(None, torch.zeros((N, K), dtype=torch.uint8, device="cuda"), *(torch.ones(1, device="cuda") for _ in range(3)))
     buf = tw.new_workspace(tw.OP_W8A8, M, N, K)
     run(tw, lambda s: tw.fp4_quantize(ws[s], packed=False, out=out).q8, lambda w: tw.w4a4_static_gemm(x, one, w, one, ws=buf))
+
+
+@pytest.mark.parametrize("M", [1, 16, 128, 300])
+@pytest.mark.parametrize("call", ["fwd", "dgrad", "w8a8_codes", "w8a8_bf16"])
+def test_fp8_product_behind_the_cast_of_its_weight(tw, call, M):
+    N, K = 2048, 4096
+    one = torch.ones(1, device="cuda")
+    ws = [torch.randn((N, K), generator=torch.Generator().manual_seed(60 + s)).to(torch.bfloat16).cuda() for s in range(STEPS)]
+    out = tw.Quantized(torch.zeros((N, K), dtype=torch.uint8, device="cuda"), *(torch.ones(1, device="cuda") for _ in range(3)), None, tw.E4M3)
+    g = torch.Generator().manual_seed(8)
+    xb, buf = torch.randn((M, K), generator=g).to(torch.bfloat16).cuda(), tw.new_workspace(tw.OP_W8A8, M, N, K)
+    xq, dy = (torch.randint(0, 0x70, (M, c), generator=g, dtype=torch.uint8).cuda() for c in (K, N))
+    product = {"fwd": lambda w: tw.fp8_linear_fwd(xq, w, one, one), "dgrad": lambda w: tw.fp8_linear_bwd_dgrad(dy, w, one, one),
+               "w8a8_codes": lambda w: tw.w8a8_static_gemm(xq, one, w, one, ws=buf), "w8a8_bf16": lambda w: tw.w8a8_static_gemm(xb, one, w, one, ws=buf)}[call]
+    run(tw, lambda s: tw.quantize_per_tensor(ws[s], out=out).q, product)
