@@ -8,6 +8,7 @@
 #include <ATen/core/Tensor.h>
 #include <ATen/ops/empty.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <exception>
@@ -159,11 +160,8 @@ PyObject* guarded(Py_ssize_t n, Py_ssize_t want, F&& f) {
     return f();
   } catch (const PyFailure&) {
     return nullptr;
-  } catch (const std::exception& e) {
-    PyErr_SetString(PyExc_RuntimeError, e.what());
-    return nullptr;
-  } catch (...) {
-    PyErr_SetString(PyExc_RuntimeError, "unknown C++ exception");
+  } catch (...) {   // as torch's own functions report it: torch.OutOfMemoryError where an output does not fit, and so on
+    torch::translate_exception_to_python(std::current_exception());
     return nullptr;
   }
 }

@@ -72,3 +72,19 @@ def test_a_required_workspace_is_storage_of_any_type(tw):
     both(tw.OP_LOSS, lambda ws: [tw.loss_fwd_bwd([x, f], ws=ws)[0]], x.numel(), 2)
     both(tw.OP_W8A8, lambda ws: [tw.w8a8_static_gemm(x, one, w, one, ws=ws)], 16, 272, 256)
     both(tw.OP_BLOCK_OUTPUT, lambda ws: tw.block_output_fused(x, f, ws=ws)[:4])
+
+
+def test_an_output_that_does_not_fit_is_an_out_of_memory_error(tw):
+    """Under a limit of the allocator's own, so that the device is not driven out of memory."""
+    x = torch.zeros((4096, 8192), dtype=torch.bfloat16, device="cuda")
+    torch.cuda.empty_cache()
+    total = torch.cuda.get_device_properties(0).total_memory
+    torch.cuda.set_per_process_memory_fraction((torch.cuda.memory_reserved() + (1 << 20)) / total)
+    try:
+        with pytest.raises(torch.OutOfMemoryError):
+            tw.absmax_quantize(x, granularity=tw.GRAN_ROW)
+    finally:
+        torch.cuda.set_per_process_memory_fraction(1.0)
+    q, s = tw.absmax_quantize(x, granularity=tw.GRAN_ROW)
+    torch.cuda.synchronize()
+    assert not q.any() and s.shape == (4096,)
