@@ -148,39 +148,38 @@ gemm_fp8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
       }
     }
   } else if (warp == 1) {
-    // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      int acc = 0;
-      uint32_t acc_phase = 0;
-      bool ok = true;
-      Sched sched(p, blockIdx.x, gridDim.x);
-      int tile, kb0, kb1;
-      while (ok && sched.next(tile, kb0, kb1)) {
-        if (!mbar_wait(tempty_bar(acc), acc_phase ^ 1u, abort_flag)) { ok = false; break; }
+    // ------------------------------------------------------------ MMA issuer (the whole warp, see gemm_pair.cuh)
+    const bool elected = elect_one();
+    int stage = 0;
+    uint32_t phase = 0;
+    int acc = 0;
+    uint32_t acc_phase = 0;
+    bool ok = true;
+    Sched sched(p, blockIdx.x, gridDim.x);
+    const uint64_t adesc0 = make_smem_desc(smem_base, BK * 128), bdesc0 = make_smem_desc(smem_base + A_BYTES, BK * 128);
+    // K-major: step 32 bytes inside the swizzle span; MN-major: step 32 rows of 128 B
+    constexpr uint32_t A_STEP = (A_MN ? UMMA_K * 128 : UMMA_K) >> 4, B_STEP = (B_MN ? UMMA_K * 128 : UMMA_K) >> 4;
+    int tile, kb0, kb1;
+    while (ok && sched.next(tile, kb0, kb1)) {
+      if (!mbar_wait_warp(tempty_bar(acc), acc_phase ^ 1u, abort_flag)) { ok = false; break; }
+      tc_fence_after();
+      const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
+      for (int kb = kb0; kb < kb1; ++kb) {
+        if (!mbar_wait_warp(full_bar(stage), phase, abort_flag)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
-        for (int kb = kb0; kb < kb1; ++kb) {
-          if (!mbar_wait(full_bar(stage), phase, abort_flag)) { ok = false; break; }
-          tc_fence_after();
-          const uint32_t sa = smem_base + stage * STAGE_BYTES;
-          const uint32_t sb = sa + A_BYTES;
+        const uint64_t adesc = adesc0 + (uint32_t)stage * (STAGE_BYTES >> 4), bdesc = bdesc0 + (uint32_t)stage * (STAGE_BYTES >> 4);
+        if (elected) {
 #pragma unroll
-          for (int k = 0; k < BK / UMMA_K; ++k) {
-            // K-major: step 32 bytes inside the swizzle span; MN-major: step 32 rows of 128 B
-            const uint64_t adesc = make_smem_desc(sa + (A_MN ? k * UMMA_K * 128 : k * UMMA_K), BK * 128);
-            const uint64_t bdesc = make_smem_desc(sb + (B_MN ? k * UMMA_K * 128 : k * UMMA_K), BK * 128);
-            umma_f8(d_tmem, adesc, bdesc, p.idesc, (uint32_t)(kb != kb0 || k != 0));
-          }
+          for (int k = 0; k < BK / UMMA_K; ++k)
+            umma_f8(d_tmem, adesc + k * A_STEP, bdesc + k * B_STEP, p.idesc, (uint32_t)(kb != kb0 || k != 0));
           umma_commit(empty_bar(stage));  // frees the stage once these MMAs have read it
-          if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
-        if (!ok) break;
-        umma_commit(tfull_bar(acc));      // accumulator complete -> epilogue
-        acc ^= 1;
-        if (acc == 0) acc_phase ^= 1u;
+        if (++stage == STAGES) { stage = 0; phase ^= 1u; }
       }
+      if (!ok) break;
+      if (elected) umma_commit(tfull_bar(acc));      // accumulator complete -> epilogue
+      acc ^= 1;
+      if (acc == 0) acc_phase ^= 1u;
     }
   } else {
     // ------------------------------------------------------------ epilogue (warps 2..5)

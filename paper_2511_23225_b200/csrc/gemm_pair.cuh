@@ -112,68 +112,79 @@ gemm_fp8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (both CTAs)
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      TileWalk walk(p, pair, num_pairs);
+    const bool elected = elect_one();
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    TileWalk walk(p, pair, num_pairs);
+    if (elected) {
       tma_prefetch_desc(&tmap_a);
       tma_prefetch_desc(&tmap_b);
-      chain_wait();
-      int tile, tm, tn, kb0, kb1;
-      while (ok && walk.next(p, tile, tm, tn, kb0, kb1)) {
-        const int m0 = tm * (2 * BM) + (int)rank * BM;  // this CTA's rows
-        const int n0 = ACT == 3 ? tn * 128 + (int)rank * p.Nd  // gate rows (leader) / up rows (peer)
-                                : tn * BN + (int)rank * 128;   // this CTA's half of B
-        for (int kb = kb0; kb < kb1; ++kb) {
-          const int k0 = kb * BK;
-          if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; break; }
+    }
+    const uint32_t fb0 = map_to_cta(full_bar(0), 0);
+    // an MN-major slab is 128 columns wide whatever the tile takes of it
+    const uint32_t stage_tx = 2 * (A_BYTES + (B_MN ? B_BYTES : (uint32_t)(bn >> 1) * BK));
+    chain_wait();
+    int tile, tm, tn, kb0, kb1;
+    while (ok && walk.next(p, tile, tm, tn, kb0, kb1)) {
+      const int m0 = tm * (2 * BM) + (int)rank * BM;  // this CTA's rows
+      const int n0 = ACT == 3 ? tn * 128 + (int)rank * p.Nd  // gate rows (leader) / up rows (peer)
+                              : tn * bn + (int)rank * (bn >> 1);   // this CTA's half of B
+      for (int kb = kb0; kb < kb1; ++kb) {
+        const int k0 = kb * BK;
+        if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; break; }
+        if (elected) {
           if (leader) mbar_expect_tx(full_bar(stage), 2 * STAGE_BYTES);
-          const uint32_t fb = map_to_cta(full_bar(stage), 0);
+          const uint32_t fb = fb0 + 8u * stage;
           const uint32_t sa = smem_base + stage * STAGE_BYTES;
           const uint32_t sb = sa + A_BYTES;
           if (A_MN) tma_load_2d_pair(sa, &tmap_a, m0, k0, fb);
           else tma_load_2d_pair(sa, &tmap_a, k0, m0, fb);
           if (B_MN) tma_load_2d_pair(sb, &tmap_b, n0, k0, fb);
           else tma_load_2d_pair(sb, &tmap_b, k0, n0, fb);
-          if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
+        if (++stage == STAGES) { stage = 0; phase ^= 1u; }
       }
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (leader CTA only)
-    if (lane == 0 && leader) {
+    // What paces the loop.  One lane in a divergent branch, four descriptors built per k-block and two commits took 600 cycles a
+    // k-block whatever the tile's width (715 with 512 of tensor work).  With the whole warp in the loop, so that the operands of
+    // the instructions are warp-uniform, an offset per instruction and one commit for both CTAs the tensor pipe sets the pace: 495 to 525
+    // cycles where the contraction is long (the clock is 1.45 to 1.6 GHz meanwhile).  [2048x4096].[4096x4096]^T 27.5 -> 25.9 us,
+    // int8 [8192x3072].[5120x3072]^T 88.9 -> 82.5, gradients of [2000x2048].[2048x2048]^T 17.5 -> 15.6.
+    if (leader) {
+      const bool elected = elect_one();
       int stage = 0;
       uint32_t phase = 0;
       int acc = 0;
       uint32_t acc_phase = 0;
       bool ok = true;
       TileWalk walk(p, pair, num_pairs);
+      const uint64_t adesc0 = make_smem_desc(smem_base, BK * 128), bdesc0 = make_smem_desc(smem_base + A_BYTES, BK * 128);
+      constexpr uint32_t A_STEP = (A_MN ? UMMA_K * 128 : UMMA_K) >> 4, B_STEP = (B_MN ? UMMA_K * 128 : UMMA_K) >> 4;
       chain_wait();
       int tile, tm, tn, kb0, kb1;
       while (ok && walk.next(p, tile, tm, tn, kb0, kb1)) {
-        if (!mbar_wait(tempty_bar(acc), acc_phase ^ 1u, abort_flag)) { ok = false; break; }
+        if (!mbar_wait_warp(tempty_bar(acc), acc_phase ^ 1u, abort_flag)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
         for (int kb = kb0; kb < kb1; ++kb) {
-          if (!mbar_wait(full_bar(stage), phase, abort_flag)) { ok = false; break; }
+          if (!mbar_wait_warp(full_bar(stage), phase, abort_flag)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t sa = smem_base + stage * STAGE_BYTES;
-          const uint32_t sb = sa + A_BYTES;
+          const uint64_t adesc = adesc0 + (uint32_t)stage * (STAGE_BYTES >> 4), bdesc = bdesc0 + (uint32_t)stage * (STAGE_BYTES >> 4);
+          if (elected) {
 #pragma unroll
-          for (int k = 0; k < BK / UMMA_K; ++k) {
-            const uint64_t adesc = make_smem_desc(sa + (A_MN ? k * UMMA_K * 128 : k * UMMA_K), BK * 128);
-            const uint64_t bdesc = make_smem_desc(sb + (B_MN ? k * UMMA_K * 128 : k * UMMA_K), BK * 128);
-            if (I8) umma_i8_pair(d_tmem, adesc, bdesc, p.idesc, (uint32_t)(kb != kb0 || k != 0));
-            else umma_f8_pair(d_tmem, adesc, bdesc, p.idesc, (uint32_t)(kb != kb0 || k != 0));
+            for (int k = 0; k < BK / UMMA_K; ++k) {
+              if (I8) umma_i8_pair(d_tmem, adesc + k * A_STEP, bdesc + k * B_STEP, p.idesc, (uint32_t)(kb != kb0 || k != 0));
+              else umma_f8_pair(d_tmem, adesc + k * A_STEP, bdesc + k * B_STEP, p.idesc, (uint32_t)(kb != kb0 || k != 0));
+            }
+            umma_commit_both(empty_bar(stage));  // frees the stage in both CTAs
           }
-          umma_commit_pair(map_to_cta(empty_bar(stage), 0));  // frees the stage in both CTAs
-          umma_commit_pair(map_to_cta(empty_bar(stage), 1));
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;
-        umma_commit_pair(map_to_cta(tfull_bar(acc), 0));      // accumulator complete, both CTAs
-        umma_commit_pair(map_to_cta(tfull_bar(acc), 1));
+        if (elected) umma_commit_both(tfull_bar(acc));      // accumulator complete, both CTAs
         acc ^= 1;
         if (acc == 0) acc_phase ^= 1u;
       }

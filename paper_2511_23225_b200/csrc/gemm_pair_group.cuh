@@ -158,30 +158,37 @@ gemm_fp8_pair_group_kernel(const __grid_constant__ PairGroupParams<LIST> g) {
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (both CTAs)
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      GroupSched sched(g, pair, num_pairs);
+    const bool elected = elect_one();
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    GroupSched sched(g, pair, num_pairs);
+    if (elected) {
       for (int i = 0; i < g.n_problems; ++i) {
         tma_prefetch_desc(&g.ma[i]);
         tma_prefetch_desc(&g.mb[i]);
       }
-      chain_wait();
-      int prob, tile;
-      while (ok && sched.next(g, prob, tile)) {
-        const GroupProblem& q = g.pr[prob];
-        int tm, tn;
-        group_tile_coords(q, tile, tm, tn);
-        const int m0 = tm * (2 * BM) + (int)rank * BM;  // this CTA's rows
-        const int n0 = tn * BN + (int)rank * 128;       // this CTA's half of B
-        const bool a_mn = q.a_mn != 0, b_mn = q.b_mn != 0;
-        const CUtensorMap* ma = &g.ma[prob];
-        const CUtensorMap* mb = &g.mb[prob];
-        for (int kb = 0; kb < q.k_blocks; ++kb) {
-          if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; break; }
+    }
+    const uint32_t fb0 = map_to_cta(full_bar(0), 0);
+    chain_wait();
+    int prob, tile;
+    while (ok && sched.next(g, prob, tile)) {
+      const GroupProblem& q = g.pr[prob];
+      int tm, tn;
+      group_tile_coords(q, tile, tm, tn);
+      const int m0 = tm * (2 * BM) + (int)rank * BM;       // this CTA's rows
+      const int n0 = tn * q.bn + (int)rank * (q.bn >> 1);  // this CTA's half of B
+      const bool a_mn = q.a_mn != 0, b_mn = q.b_mn != 0;
+      // an MN-major slab is 128 columns wide whatever the tile takes of it
+      const uint32_t stage_tx = 2 * (A_BYTES + (b_mn ? B_BYTES : (uint32_t)(q.bn >> 1) * BK));
+      const CUtensorMap* ma = &g.ma[prob];
+      const CUtensorMap* mb = &g.mb[prob];
+      const int k_blocks = q.k_blocks;
+      for (int kb = 0; kb < k_blocks; ++kb) {
+        if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; break; }
+        if (elected) {
           if (leader) mbar_expect_tx(full_bar(stage), 2 * STAGE_BYTES);
-          const uint32_t fb = map_to_cta(full_bar(stage), 0);
+          const uint32_t fb = fb0 + 8u * stage;
           const uint32_t sa = smem_base + stage * STAGE_BYTES;
           const uint32_t sb = sa + A_BYTES;
           const int k0 = kb * BK;
@@ -189,47 +196,47 @@ gemm_fp8_pair_group_kernel(const __grid_constant__ PairGroupParams<LIST> g) {
           else tma_load_2d_pair(sa, ma, k0, m0, fb);
           if (b_mn) tma_load_2d_pair(sb, mb, n0, k0, fb);
           else tma_load_2d_pair(sb, mb, k0, n0, fb);
-          if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
+        if (++stage == STAGES) { stage = 0; phase ^= 1u; }
       }
     }
   } else if (warp == 1) {
-    // ------------------------------------------------------------ MMA issuer (leader CTA only)
-    if (lane == 0 && leader) {
+    // ------------------------------------------------------------ MMA issuer (leader CTA only; see gemm_pair.cuh for what paces it)
+    if (leader) {
+      const bool elected = elect_one();
       int stage = 0;
       uint32_t phase = 0;
       int acc = 0;
       uint32_t acc_phase = 0;
       bool ok = true;
       GroupSched sched(g, pair, num_pairs);
+      const uint64_t adesc0 = make_smem_desc(smem_base, BK * 128), bdesc0 = make_smem_desc(smem_base + A_BYTES, BK * 128);
       chain_wait();
       int prob, tile;
       while (ok && sched.next(g, prob, tile)) {
         const GroupProblem& q = g.pr[prob];
         // K-major: step 32 bytes inside the swizzle span; MN-major: step 32 rows of 128 B
-        const uint32_t a_step = q.a_mn ? UMMA_K * 128 : UMMA_K;
-        const uint32_t b_step = q.b_mn ? UMMA_K * 128 : UMMA_K;
+        const uint32_t a_step = (q.a_mn ? UMMA_K * 128 : UMMA_K) >> 4;
+        const uint32_t b_step = (q.b_mn ? UMMA_K * 128 : UMMA_K) >> 4;
         const uint32_t idesc = q.idesc;
         const int k_blocks = q.k_blocks;
-        if (!mbar_wait(tempty_bar(acc), acc_phase ^ 1u, abort_flag)) { ok = false; break; }
+        if (!mbar_wait_warp(tempty_bar(acc), acc_phase ^ 1u, abort_flag)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
         for (int kb = 0; kb < k_blocks; ++kb) {
-          if (!mbar_wait(full_bar(stage), phase, abort_flag)) { ok = false; break; }
+          if (!mbar_wait_warp(full_bar(stage), phase, abort_flag)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t sa = smem_base + stage * STAGE_BYTES;
-          const uint32_t sb = sa + A_BYTES;
+          const uint64_t adesc = adesc0 + (uint32_t)stage * (STAGE_BYTES >> 4), bdesc = bdesc0 + (uint32_t)stage * (STAGE_BYTES >> 4);
+          if (elected) {
 #pragma unroll
-          for (int k = 0; k < BK / UMMA_K; ++k)
-            umma_f8_pair(d_tmem, make_smem_desc(sa + k * a_step, BK * 128), make_smem_desc(sb + k * b_step, BK * 128),
-                         idesc, (uint32_t)((kb | k) != 0));
-          umma_commit_pair(map_to_cta(empty_bar(stage), 0));  // frees the stage in both CTAs
-          umma_commit_pair(map_to_cta(empty_bar(stage), 1));
+            for (int k = 0; k < BK / UMMA_K; ++k)
+              umma_f8_pair(d_tmem, adesc + k * a_step, bdesc + k * b_step, idesc, (uint32_t)((kb | k) != 0));
+            umma_commit_both(empty_bar(stage));  // frees the stage in both CTAs
+          }
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;
-        umma_commit_pair(map_to_cta(tfull_bar(acc), 0));      // accumulator complete, both CTAs
-        umma_commit_pair(map_to_cta(tfull_bar(acc), 1));
+        if (elected) umma_commit_both(tfull_bar(acc));      // accumulator complete, both CTAs
         acc ^= 1;
         if (acc == 0) acc_phase ^= 1u;
       }

@@ -222,28 +222,29 @@ gemm_fp8_skinny_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
       }
     }
   } else if (warp == 1) {
-    // ------------------------------------------------------------ MMA issuer
+    // ------------------------------------------------------------ MMA issuer (the whole warp, see gemm_pair.cuh)
+    const bool elected = elect_one();
+    const uint64_t wdesc0 = make_smem_desc(smem_base, BK * 128), xdesc0 = make_smem_desc(smem_base + BM * BK, BK * 128);
+    constexpr uint32_t W_STEP = (W_MN ? UMMA_K * 128 : UMMA_K) >> 4, X_STEP = UMMA_K >> 4;
     chain_wait();
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      for (int kb = kb0; kb < kb1; ++kb) {
-        if (!mbar_wait(full_bar(stage), phase, abort_flag)) { ok = false; break; }
-        tc_fence_after();
-        const uint32_t sw = smem_base + stage * p.stage_bytes;
-        const uint32_t sx = sw + BM * BK;
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int kb = kb0; kb < kb1; ++kb) {
+      if (!mbar_wait_warp(full_bar(stage), phase, abort_flag)) { ok = false; break; }
+      tc_fence_after();
+      const uint32_t at = (uint32_t)stage * (p.stage_bytes >> 4);
+      if (elected) {
 #pragma unroll
         for (int k = 0; k < BK / UMMA_K; ++k) {
-          const uint64_t adesc = make_smem_desc(sw + (W_MN ? k * UMMA_K * 128 : k * UMMA_K), BK * 128), bdesc = make_smem_desc(sx + k * UMMA_K, BK * 128);
-          if (I8) umma_i8(tmem_base, adesc, bdesc, p.idesc, (uint32_t)(kb != kb0 || k != 0));
-          else umma_f8(tmem_base, adesc, bdesc, p.idesc, (uint32_t)(kb != kb0 || k != 0));
+          if (I8) umma_i8(tmem_base, wdesc0 + at + k * W_STEP, xdesc0 + at + k * X_STEP, p.idesc, (uint32_t)(kb != kb0 || k != 0));
+          else umma_f8(tmem_base, wdesc0 + at + k * W_STEP, xdesc0 + at + k * X_STEP, p.idesc, (uint32_t)(kb != kb0 || k != 0));
         }
         umma_commit(empty_bar(stage));
-        if (++stage == p.stages) { stage = 0; phase ^= 1u; }
       }
-      if (ok) umma_commit(done_bar);
+      if (++stage == p.stages) { stage = 0; phase ^= 1u; }
     }
+    if (ok && elected) umma_commit(done_bar);
   } else {
     // ------------------------------------------------------------ epilogue (warps 2..5)
     chain_wait();
