@@ -122,14 +122,12 @@ gemm_fp8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
       tma_prefetch_desc(&tmap_b);
     }
     const uint32_t fb0 = map_to_cta(full_bar(0), 0);
-    // an MN-major slab is 128 columns wide whatever the tile takes of it
-    const uint32_t stage_tx = 2 * (A_BYTES + (B_MN ? B_BYTES : (uint32_t)(bn >> 1) * BK));
     chain_wait();
     int tile, tm, tn, kb0, kb1;
     while (ok && walk.next(p, tile, tm, tn, kb0, kb1)) {
       const int m0 = tm * (2 * BM) + (int)rank * BM;  // this CTA's rows
       const int n0 = ACT == 3 ? tn * 128 + (int)rank * p.Nd  // gate rows (leader) / up rows (peer)
-                              : tn * bn + (int)rank * (bn >> 1);   // this CTA's half of B
+                              : tn * BN + (int)rank * 128;   // this CTA's half of B
       for (int kb = kb0; kb < kb1; ++kb) {
         const int k0 = kb * BK;
         if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; break; }

@@ -177,10 +177,8 @@ gemm_fp8_pair_group_kernel(const __grid_constant__ PairGroupParams<LIST> g) {
       int tm, tn;
       group_tile_coords(q, tile, tm, tn);
       const int m0 = tm * (2 * BM) + (int)rank * BM;       // this CTA's rows
-      const int n0 = tn * q.bn + (int)rank * (q.bn >> 1);  // this CTA's half of B
+      const int n0 = tn * BN + (int)rank * 128;       // this CTA's half of B
       const bool a_mn = q.a_mn != 0, b_mn = q.b_mn != 0;
-      // an MN-major slab is 128 columns wide whatever the tile takes of it
-      const uint32_t stage_tx = 2 * (A_BYTES + (b_mn ? B_BYTES : (uint32_t)(q.bn >> 1) * BK));
       const CUtensorMap* ma = &g.ma[prob];
       const CUtensorMap* mb = &g.mb[prob];
       const int k_blocks = q.k_blocks;
