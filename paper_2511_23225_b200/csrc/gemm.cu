@@ -496,6 +496,46 @@ int pair_split_tiles(int tiles, int workers, int k_blocks) {
   return rem;
 }
 
+// Estimate, in nanoseconds, of one tile of the CTA-pair kernels: 256 rows and bn columns (a multiple of 64), k_blocks of the
+// contraction; b_mn: the B operand is MN-major, whose slabs are 128 columns wide whatever the tile takes of them; chunk_ns: what the
+// epilogue needs per 64 columns where it outlasts the main loop.  At 256 columns the tensor pipe bounds a k-block (and, through the
+// power it draws, the clock: 1.45 to 1.6 GHz), below 192 the operand loads.  Fitted to launches of 1 to 20 tiles per pair, K = 256 to 11008;
+// us at 256 / 192 / 128 / 64 columns: [512x256].[1024x256]^T 4.9 / 4.4 / 3.9 / 3.5, [1024x1024].[1024x1024]^T 6.7 / 5.7 / 5.0 / 5.5,
+// [8192x768].[768x768]^T 8.4 / 8.1 / 8.6 / 11.1, [12608x3072].[768x3072]^T 27.2 / 23.2 / 27.5 / 42.1,
+// [700x2048].[8192x2048]^T 14.6 / 12.9 / 14.3 / 21.1, [2048x4096].[4096x4096]^T 26.0 / 27.5 / 28.2 / 43.3.
+double tile_ns(int bn, int k_blocks, bool b_mn, double chunk_ns) {
+  static const double per_block[2][4] = {{172.0, 179.0, 220.0, 312.0}, {232.0, 244.0, 243.0, 312.0}};
+  static const double once[4] = {300.0, 600.0, 800.0, 800.0};
+  const int n = bn / 64;
+  return std::max(k_blocks * per_block[b_mn ? 1 : 0][n - 1] + once[n - 1], chunk_ns * n);
+}
+
+// Columns of the tiles of one product: a narrower tile costs more per column, but where the 256-wide ones leave the last wave (or the
+// only one) mostly empty it ends sooner, and a launch's last epilogue is shorter (430 ns per 64 columns).  The results are the same bits.
+int pair_width(int64_t Md, int64_t Nd, int k_blocks, bool b_mn, double chunk_ns) {
+  const int64_t pairs = sm_count() / 2, tiles_m = (Md + 2 * BM - 1) / (2 * BM);
+  int best = 256;
+  double best_ns = 0.0;
+  for (int bn = 256; bn >= 64; bn -= 64) {
+    const int64_t tiles = tiles_m * ((Nd + bn - 1) / bn);
+    double ns = 2700.0 + 430.0 * (bn / 64) + (double)((tiles + pairs - 1) / pairs) * tile_ns(bn, k_blocks, b_mn, chunk_ns);
+    if (bn == 64 && 2 * tiles > pairs) ns += 110.0 * k_blocks;   // the narrowest tiles read A once per 64 columns: only with pairs to spare
+    if (bn == 256 || ns < 0.95 * best_ns) {
+      best = bn;
+      best_ns = ns;
+    }
+  }
+  return best;
+}
+
+// What an epilogue needs per 64 columns of a tile, by its work per element (clock counters; four or eight warps by launch_pair_act()'s rule).
+double epilogue_chunk_ns(int act, bool fp8_copy, int k_blocks) {
+  const bool eight = k_blocks < 16;
+  if (act == TWEO_ACT_GELU) return eight ? 1190.0 : 1500.0;
+  if (act == TWEO_ACT_GELU_TANH) return eight ? 760.0 : 940.0;
+  return fp8_copy ? (eight ? 550.0 : 1050.0) : 0.0;
+}
+
 template <bool A_MN, bool B_MN, bool OUT_F32>
 tweo_status_t launch_pair(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& md, GemmParams& p,
                           void* ws, size_t ws_bytes, cudaStream_t st) {
@@ -511,7 +551,7 @@ tweo_status_t launch_pair(const CUtensorMap& ma, const CUtensorMap& mb, const CU
     device_once_done(attr_done, attr_dev);
   }
   p.tiles_m = (p.Md + 2 * BM - 1) / (2 * BM);
-  p.tiles_n = (p.Nd + 255) / 256;
+  p.tiles_n = (p.Nd + p.bn - 1) / p.bn;
   p.k_blocks = (p.Kc + BK - 1) / BK;
   p.sk_tiles = 0;
   p.sk_partials = nullptr;
@@ -520,7 +560,7 @@ tweo_status_t launch_pair(const CUtensorMap& ma, const CUtensorMap& mb, const CU
   const int sms = sm_count();
   int pairs = sms / 2;
   p.raster_g = raster_band(p.tiles_m, pairs);
-  if (ws && ws_bytes >= kWsPartialsOffset + (size_t)sms * kWsPartialBytesPerSm && aligned16(ws)) {
+  if (p.bn == 256 && ws && ws_bytes >= kWsPartialsOffset + (size_t)sms * kWsPartialBytesPerSm && aligned16(ws)) {
     p.sk_tiles = pair_split_tiles(tiles, pairs, p.k_blocks);
     if (p.sk_tiles > 0) {
       p.sk_counters = reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(ws) + kWsCountersOffset);
@@ -554,7 +594,12 @@ tweo_status_t run_gemm(const Operand& A, const Operand& B, int64_t Md, int64_t N
   const int BN = Nd > 128 ? 256 : 128;
   // CTA pairs (256 x 256 tiles) whenever the output has more than one 128-row block and is wide enough
   const bool use_pair = Md > 128 && Nd > 128;
-  p.idesc = use_pair ? make_idesc(A.fmt, B.fmt, A.mn_major, B.mn_major, 256, 256)
+  const int k_blocks = (int)((Kc + BK - 1) / BK);
+  // where 256-wide tiles can be split along the contraction they are (launch_pair decides)
+  const bool split = ws && ws_bytes >= kWsPartialsOffset + (size_t)sm_count() * kWsPartialBytesPerSm && aligned16(ws) &&
+                     pair_split_tiles((int)(((Md + 255) / 256) * ((Nd + 255) / 256)), sm_count() / 2, k_blocks) > 0;
+  p.bn = split ? 256 : pair_width(Md, Nd, k_blocks, B.mn_major, 0.0);
+  p.idesc = use_pair ? make_idesc(A.fmt, B.fmt, A.mn_major, B.mn_major, p.bn, 256)
                      : make_idesc(A.fmt, B.fmt, A.mn_major, B.mn_major, BN);
 
   CUtensorMap ma, mb, md;
@@ -566,7 +611,7 @@ tweo_status_t run_gemm(const Operand& A, const Operand& B, int64_t Md, int64_t N
   if (A.mn_major) ok = make_map(&ma, A.ptr, Md, Kc, A.ld, BK);   // [Kc, Md]: box 128 (Md) x BK rows
   else ok = make_map(&ma, A.ptr, Kc, Md, A.ld, BM);              // [Md, Kc]: box 128 (Kc) x BM rows
   if (B.mn_major) ok = ok && make_map(&mb, B.ptr, Nd, Kc, B.ld, BK);
-  else ok = ok && make_map(&mb, B.ptr, Kc, Nd, B.ld, use_pair ? 128 : BN);  // a pair CTA loads half of B
+  else ok = ok && make_map(&mb, B.ptr, Kc, Nd, B.ld, use_pair ? p.bn / 2 : BN);  // a pair CTA loads half of B
   if (!ok) {
     cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
     return TWEO_ERR_CUDA;
@@ -613,7 +658,7 @@ tweo_status_t launch_pair_act_cfg(const CUtensorMap& ma, const CUtensorMap& mb, 
     device_once_done(attr_done, attr_dev);
   }
   p.tiles_m = (p.Md + 2 * BM - 1) / (2 * BM);
-  p.tiles_n = ACT == 3 ? (p.Nd + 127) / 128 : (p.Nd + 255) / 256;
+  p.tiles_n = ACT == 3 ? (p.Nd + 127) / 128 : (p.Nd + p.bn - 1) / p.bn;
   p.k_blocks = (p.Kc + BK - 1) / BK;
   p.sk_tiles = 0;
   p.sk_partials = nullptr;
@@ -653,7 +698,8 @@ tweo_status_t run_fwd_act(const uint8_t* xq, int64_t ldx, int fmt_x, const uint8
   p.Md = (int32_t)M;
   p.Nd = (int32_t)N;
   p.Kc = (int32_t)K;
-  p.idesc = make_idesc(fmt_x, fmt_w, false, w_mn, 256, 256);
+  p.bn = act == TWEO_ACT_SWIGLU ? 256 : pair_width(M, N, (int)((K + BK - 1) / BK), w_mn, epilogue_chunk_ns(act, p.out_q != nullptr, (int)((K + BK - 1) / BK)));
+  p.idesc = make_idesc(fmt_x, fmt_w, false, w_mn, p.bn, 256);
   CUtensorMap ma, mb, md, mq;
   // without a bf16 output the store is skipped; the map then describes the FP8 output's memory and is never used
   bool ok = p.d ? make_out_map(&md, p.d, N, M, p.ldd, false) : make_out_map(&md, p.out_q, N / 2, M, p.ldq / 2, false);
@@ -661,7 +707,7 @@ tweo_status_t run_fwd_act(const uint8_t* xq, int64_t ldx, int fmt_x, const uint8
   else mq = md;
   ok = ok && make_map(&ma, xq, K, M, ldx, BM);
   if (w_mn) ok = ok && make_map(&mb, wq, N, K, ldw, BK);
-  else ok = ok && make_map(&mb, wq, K, act == TWEO_ACT_SWIGLU ? 2 * N : N, ldw, 128);
+  else ok = ok && make_map(&mb, wq, K, act == TWEO_ACT_SWIGLU ? 2 * N : N, ldw, p.bn / 2);
   if (!ok) {
     cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
     return TWEO_ERR_CUDA;
@@ -884,6 +930,8 @@ struct GroupDesc {
   int64_t ldq = 0;
   int q_fmt = TWEO_E4M3;
   const float* q_scale = nullptr;
+  int bn = 256;          // columns of a tile (group_widths)
+  double tile_ns = 0.0;  // and what one takes
 };
 
 struct FloatPtrs {
@@ -895,6 +943,50 @@ __global__ void zero_floats_kernel(const FloatPtrs f) {
   chain_release();
   chain_wait();
   if ((int)threadIdx.x < f.n) *f.p[threadIdx.x] = 0.0f;
+}
+
+int64_t group_tiles(const GroupDesc& d) { return ((d.Md + 2 * BM - 1) / (2 * BM)) * ((d.Nd + d.bn - 1) / d.bn); }
+
+// Widths of the tiles of a group's products, and what one tile of each takes (ns).  The launch ends no sooner than its longest tile: a
+// weight gradient of a small linear has few tiles and a contraction of all tokens ([8192x768] and [768x768]: nine of 64 k-blocks, while the
+// data gradient's 96 take 6).  So the product with the longest tile is narrowed as long as that brings the estimate down: gradients of
+// [8192x768].[768x768]^T 23.3 -> 18.6 us, [4096x768].[768x768]^T 13.9 -> 11.2, [512x256].[1024x256]^T 6.6 -> 5.1.
+void group_widths(GroupDesc* d, int n) {
+  const double pairs = sm_count() / 2;
+  auto measure = [&](int i) {
+    const int kb = (int)((d[i].Kc + BK - 1) / BK);
+    d[i].tile_ns = tile_ns(d[i].bn, kb, d[i].b_mn, epilogue_chunk_ns(TWEO_ACT_NONE, d[i].out_q != nullptr, kb));
+  };
+  auto estimate = [&](int& longest) {
+    double total = 0.0, shortest = 1e30;
+    longest = 0;
+    for (int i = 0; i < n; ++i) {
+      total += d[i].tile_ns * (double)group_tiles(d[i]);
+      shortest = std::min(shortest, d[i].tile_ns);
+      if (d[i].tile_ns > d[longest].tile_ns) longest = i;
+    }
+    return std::max(d[longest].tile_ns, total / pairs + 0.5 * shortest) + 430.0 * (d[longest].bn / 64);
+  };
+  int best_width[kGroupMaxProblems];
+  for (int i = 0; i < n; ++i) {
+    best_width[i] = d[i].bn = 256;
+    measure(i);
+  }
+  int longest;
+  double best = estimate(longest);
+  while (d[longest].bn > 64) {
+    d[longest].bn -= 64;
+    measure(longest);
+    const double t = estimate(longest);
+    if (t < 0.97 * best) {
+      best = t;
+      for (int i = 0; i < n; ++i) best_width[i] = d[i].bn;
+    }
+  }
+  for (int i = 0; i < n; ++i) {
+    d[i].bn = best_width[i];
+    measure(i);
+  }
 }
 
 // QST: fused epilogue outputs (amax, FP8 copy) on some products.  EPIW / EBUF as in the kernel; the operand ring
@@ -916,34 +1008,32 @@ tweo_status_t run_group_list(GroupDesc* d, int n, cudaStream_t st) {
   const int pairs_all = sm_count() / 2;
   static thread_local PairGroupParams<LIST> g;   // 8 - 20 KB: kept off the stack
   g.n_problems = n;
-  int cost[kGroupMaxProblems];
   g.tile_start[0] = 0;
   for (int i = 0; i < n; ++i) {
     GroupProblem& q = g.pr[i];
     q.Md = (int32_t)d[i].Md;
     q.Nd = (int32_t)d[i].Nd;
     q.tiles_m = (int32_t)((d[i].Md + 2 * BM - 1) / (2 * BM));
-    q.tiles_n = (int32_t)((d[i].Nd + 255) / 256);
+    q.bn = d[i].bn;
+    q.tiles_n = (int32_t)((d[i].Nd + q.bn - 1) / q.bn);
     q.k_blocks = (int32_t)((d[i].Kc + BK - 1) / BK);
     q.raster_g = raster_band(q.tiles_m, pairs_all);
     q.a_mn = d[i].a_mn ? 1 : 0;
     q.b_mn = d[i].b_mn ? 1 : 0;
-    q.idesc = make_idesc(d[i].fa, d[i].fb, d[i].a_mn, d[i].b_mn, 256, 256);
+    q.idesc = make_idesc(d[i].fa, d[i].fb, d[i].a_mn, d[i].b_mn, q.bn, 256);
     q.sa_inv = d[i].sa;
     q.sb_inv = d[i].sb;
     q.out_amax = d[i].out_amax;
     q.q_scale = d[i].out_q ? d[i].q_scale : nullptr;
     q.q_fmt = d[i].q_fmt;
-    q.pad = 0;
     g.tile_start[i + 1] = g.tile_start[i] + q.tiles_m * q.tiles_n;
-    cost[i] = (q.k_blocks < 8 ? 8 : q.k_blocks) + 2;  // k-blocks, with a floor for the epilogue of short tiles
     bool ok = make_out_map(&g.md[i], d[i].d, d[i].Nd, d[i].Md, d[i].ldd, false);
     if (QST && d[i].out_q) ok = ok && make_q_map(&g.mq[i], d[i].out_q, d[i].Nd, d[i].Md, d[i].ldq);
     else g.mq[i] = g.md[i];
     if (d[i].a_mn) ok = ok && make_map(&g.ma[i], d[i].a, d[i].Md, d[i].Kc, d[i].lda, BK);
     else ok = ok && make_map(&g.ma[i], d[i].a, d[i].Kc, d[i].Md, d[i].lda, BM);
     if (d[i].b_mn) ok = ok && make_map(&g.mb[i], d[i].b, d[i].Nd, d[i].Kc, d[i].ldb, BK);
-    else ok = ok && make_map(&g.mb[i], d[i].b, d[i].Kc, d[i].Nd, d[i].ldb, 128);   // a pair CTA loads half of B
+    else ok = ok && make_map(&g.mb[i], d[i].b, d[i].Kc, d[i].Nd, d[i].ldb, q.bn / 2);   // a pair CTA loads half of B
     if (!ok) {
       cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
       return TWEO_ERR_CUDA;
@@ -968,7 +1058,7 @@ tweo_status_t run_group_list(GroupDesc* d, int n, cudaStream_t st) {
       heap.pop();
       owner[t] = (uint8_t)l.second;
       ++count[l.second];
-      l.first += cost[prob];
+      l.first += (int64_t)d[prob].tile_ns;
       heap.push(l);
     }
     int fill[kGroupMaxPairs + 1];
@@ -996,12 +1086,11 @@ tweo_status_t run_group_list(GroupDesc* d, int n, cudaStream_t st) {
 
 tweo_status_t run_group(GroupDesc* d, int n, cudaStream_t st) {
   if (n < 1 || n > kGroupMaxProblems) return TWEO_ERR_INVALID_ARG;
+  group_widths(d, n);
   // the products with the longer tiles go first in the tile list (stable: equal lengths keep the caller's order)
-  std::stable_sort(d, d + n, [](const GroupDesc& x, const GroupDesc& y) {
-    return (x.Kc + BK - 1) / BK > (y.Kc + BK - 1) / BK;
-  });
+  std::stable_sort(d, d + n, [](const GroupDesc& x, const GroupDesc& y) { return x.tile_ns > y.tile_ns; });
   int64_t tiles = 0;
-  for (int i = 0; i < n; ++i) tiles += ((d[i].Md + 2 * BM - 1) / (2 * BM)) * ((d[i].Nd + 255) / 256);
+  for (int i = 0; i < n; ++i) tiles += group_tiles(d[i]);
   bool fused = false;
   int64_t fused_kb_min = INT64_MAX;
   for (int i = 0; i < n; ++i)
@@ -1149,7 +1238,8 @@ tweo_status_t run_int8_linear(const int8_t* xq, int64_t ldx, const float* sx, in
   p.Nd = (int32_t)N;
   p.Kc = (int32_t)K;
   p.tiles_m = (int32_t)((M + 2 * BM - 1) / (2 * BM));
-  p.tiles_n = (int32_t)((N + 255) / 256);
+  p.bn = pair_width(M, N, (int)((K + BK - 1) / BK), false, 0.0);
+  p.tiles_n = (int32_t)((N + p.bn - 1) / p.bn);
   p.k_blocks = (int32_t)((K + BK - 1) / BK);
   const int tiles = p.tiles_m * p.tiles_n;
   int pairs = sm_count() / 2;
@@ -1167,11 +1257,11 @@ tweo_status_t run_int8_linear(const int8_t* xq, int64_t ldx, const float* sx, in
     p.ldq = ldq;
     p.q_scale = sy;
   }
-  // instruction descriptor of kind::i8: int32 accumulators, signed 8-bit A and B, K-major, N = 256, M = 256
-  p.idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(256 >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
+  // instruction descriptor of kind::i8: int32 accumulators, signed 8-bit A and B, K-major, N = bn, M = 256
+  p.idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.bn >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
   CUtensorMap ma, mb, md;
   bool ok = q8 ? make_q_map(&md, yq, N, M, ldq) : make_out_map(&md, y, N, M, ldy, false);
-  ok = ok && make_map(&ma, xq, K, M, ldx, BM) && make_map(&mb, wq, K, N, ldw, 128);
+  ok = ok && make_map(&ma, xq, K, M, ldx, BM) && make_map(&mb, wq, K, N, ldw, p.bn / 2);
   if (!ok) {
     cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
     return TWEO_ERR_CUDA;

@@ -20,6 +20,7 @@ struct GemmParams {
   int64_t ldd;
   int32_t Md, Nd, Kc;
   int32_t tiles_m, tiles_n, k_blocks;
+  int32_t bn;          // CTA-pair kernel: columns of a tile, a multiple of 64 up to 256
   int32_t raster_g;    // tiles are numbered in bands of raster_g tile rows (see tile_coords)
   const float* sa_inv;
   const float* sb_inv;

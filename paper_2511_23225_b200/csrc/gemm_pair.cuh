@@ -53,11 +53,12 @@ __global__ void __launch_bounds__(64 + 32 * EPIW, 1)
 gemm_fp8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
                      const __grid_constant__ CUtensorMap tmap_d, const __grid_constant__ CUtensorMap tmap_q,
                      const __grid_constant__ GemmParams p) {
-  constexpr int BN = 256;                 // tile columns of the pair
+  constexpr int BN = 256;                 // tile columns of the pair, at most
   constexpr uint32_t A_BYTES = BM * BK;   // this CTA's 128 rows of A
-  constexpr uint32_t B_BYTES = 128 * BK;  // this CTA's 128 of the 256 columns of B
+  constexpr uint32_t B_BYTES = 128 * BK;  // this CTA's half of the columns of B, at most 128
   constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
   constexpr uint32_t TMEM_COLS = 512;
+  const int bn = ACT == 3 ? BN : p.bn;    // tile columns of this launch (see pair_width() for the choice)
 
   extern __shared__ uint8_t smem_dyn[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~(uintptr_t)1023);
@@ -122,17 +123,19 @@ gemm_fp8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
       tma_prefetch_desc(&tmap_b);
     }
     const uint32_t fb0 = map_to_cta(full_bar(0), 0);
+    // an MN-major slab is 128 columns wide whatever the tile takes of it
+    const uint32_t stage_tx = 2 * (A_BYTES + (B_MN ? B_BYTES : (uint32_t)(bn >> 1) * BK));
     chain_wait();
     int tile, tm, tn, kb0, kb1;
     while (ok && walk.next(p, tile, tm, tn, kb0, kb1)) {
       const int m0 = tm * (2 * BM) + (int)rank * BM;  // this CTA's rows
       const int n0 = ACT == 3 ? tn * 128 + (int)rank * p.Nd  // gate rows (leader) / up rows (peer)
-                              : tn * BN + (int)rank * 128;   // this CTA's half of B
+                              : tn * bn + (int)rank * (bn >> 1);   // this CTA's half of B
       for (int kb = kb0; kb < kb1; ++kb) {
         const int k0 = kb * BK;
         if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; break; }
         if (elected) {
-          if (leader) mbar_expect_tx(full_bar(stage), 2 * STAGE_BYTES);
+          if (leader) mbar_expect_tx(full_bar(stage), stage_tx);
           const uint32_t fb = fb0 + 8u * stage;
           const uint32_t sa = smem_base + stage * STAGE_BYTES;
           const uint32_t sb = sa + A_BYTES;
@@ -211,11 +214,12 @@ gemm_fp8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
     int acc = 0;
     uint32_t acc_phase = 0;
     bool ok = true;
+    int turn = (warp - 2) >> 2;   // eight epilogue warps: which of two adjacent chunks this warp takes
     TileWalk walk(p, pair, num_pairs);
     int tile, tm, tn, kb0, kb1;
     while (ok && walk.next(p, tile, tm, tn, kb0, kb1)) {
       const int m0 = tm * (2 * BM) + (int)rank * BM;
-      const int n0 = ACT == 3 ? tn * 128 : tn * BN;
+      const int n0 = ACT == 3 ? tn * 128 : tn * bn;
       if (!mbar_wait(tfull_bar(acc), acc_phase, abort_flag)) { ok = false; break; }
       tc_fence_after();
       const int row0 = m0 + quarter * 32;
@@ -232,11 +236,12 @@ gemm_fp8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
         if (acc == 0) acc_phase ^= 1u;
         continue;
       }
-      // with 8 epilogue warps, warps 2-5 take the first half of the tile's chunks and warps 6-9 the second
-      constexpr int NC = (ACT == 3 ? 128 : BN) / CH, NC_W = NC / (EPIW / 4);
-      const int c_first = ((warp - 2) >> 2) * NC_W;
+      // with 8 epilogue warps, warps 2-5 and 6-9 take the chunks in turn, across tiles where their number is odd
+      const int nc = (ACT == 3 ? 128 : bn) / CH;
+      const int c_first = EPIW == 8 ? turn : 0;
+      turn ^= nc & 1;
 #pragma unroll 1
-      for (int c = c_first; c < c_first + NC_W; ++c) {
+      for (int c = c_first; c < nc; c += EPIW / 4) {
         const int col0 = n0 + c * CH;
         if (col0 >= p.Nd) break;
         uint32_t r[CH];

@@ -41,7 +41,7 @@ struct GroupProblem {
   float* out_amax;        // nullptr: none
   const float* q_scale;   // nullptr: no FP8 copy
   int32_t q_fmt;
-  int32_t pad;
+  int32_t bn;             // columns of a tile, a multiple of 64 up to 256
 };
 
 template <int LIST>
@@ -98,9 +98,9 @@ __device__ __forceinline__ void group_tile_coords(const GroupProblem& q, int til
 template <int STAGES, int LIST, bool QST = false, int EPIW = 4, int EBUF = 2>
 __global__ void __launch_bounds__(64 + 32 * EPIW, 1)
 gemm_fp8_pair_group_kernel(const __grid_constant__ PairGroupParams<LIST> g) {
-  constexpr int BN = 256;                 // tile columns of the pair
+  constexpr int BN = 256;                 // tile columns of the pair, at most
   constexpr uint32_t A_BYTES = BM * BK;   // this CTA's 128 rows of A
-  constexpr uint32_t B_BYTES = 128 * BK;  // this CTA's 128 of the 256 columns of B
+  constexpr uint32_t B_BYTES = 128 * BK;  // this CTA's half of the columns of B, at most 128
   constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
   constexpr uint32_t TMEM_COLS = 512;
   constexpr int CH = 64;                  // bf16 columns per 128-byte staging row
@@ -177,15 +177,17 @@ gemm_fp8_pair_group_kernel(const __grid_constant__ PairGroupParams<LIST> g) {
       int tm, tn;
       group_tile_coords(q, tile, tm, tn);
       const int m0 = tm * (2 * BM) + (int)rank * BM;       // this CTA's rows
-      const int n0 = tn * BN + (int)rank * 128;       // this CTA's half of B
+      const int n0 = tn * q.bn + (int)rank * (q.bn >> 1);  // this CTA's half of B
       const bool a_mn = q.a_mn != 0, b_mn = q.b_mn != 0;
+      // an MN-major slab is 128 columns wide whatever the tile takes of it
+      const uint32_t stage_tx = 2 * (A_BYTES + (b_mn ? B_BYTES : (uint32_t)(q.bn >> 1) * BK));
       const CUtensorMap* ma = &g.ma[prob];
       const CUtensorMap* mb = &g.mb[prob];
       const int k_blocks = q.k_blocks;
       for (int kb = 0; kb < k_blocks; ++kb) {
         if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; break; }
         if (elected) {
-          if (leader) mbar_expect_tx(full_bar(stage), 2 * STAGE_BYTES);
+          if (leader) mbar_expect_tx(full_bar(stage), stage_tx);
           const uint32_t fb = fb0 + 8u * stage;
           const uint32_t sa = smem_base + stage * STAGE_BYTES;
           const uint32_t sb = sa + A_BYTES;
@@ -248,9 +250,7 @@ gemm_fp8_pair_group_kernel(const __grid_constant__ PairGroupParams<LIST> g) {
     const uint32_t swz = (uint32_t)(lane & 7);
     const uint32_t tlane = (uint32_t)(quarter * 32) << 16;
     const uint32_t q_base = smem_u32(epi_smem) + EPI_BYTES + (uint32_t)(warp - 2) * (uint32_t)EBUF * Q_BUF;
-    // with 8 epilogue warps, warps 2-5 take the first half of a tile's chunks and warps 6-9 the second
-    constexpr int NC_W = (BN / CH) / (EPIW / 4);
-    const int c_first = ((warp - 2) >> 2) * NC_W;
+    int turn = (warp - 2) >> 2;   // eight epilogue warps: which of two adjacent chunks this warp takes
     uint32_t it = 0;
     int acc = 0;
     uint32_t acc_phase = 0;
@@ -286,12 +286,16 @@ gemm_fp8_pair_group_kernel(const __grid_constant__ PairGroupParams<LIST> g) {
       int tm, tn;
       group_tile_coords(q, tile, tm, tn);
       const int m0 = tm * (2 * BM) + (int)rank * BM;
-      const int n0 = tn * BN;
+      const int n0 = tn * q.bn;
       if (!mbar_wait(tfull_bar(acc), acc_phase, abort_flag)) { ok = false; break; }
       tc_fence_after();
       const int row0 = m0 + quarter * 32;
+      // with 8 epilogue warps, warps 2-5 and 6-9 take the chunks in turn, across tiles where their number is odd
+      const int nc = q.bn / CH;
+      const int c_first = EPIW == 8 ? turn : 0;
+      turn ^= nc & 1;
 #pragma unroll 1
-      for (int c = c_first; c < c_first + NC_W; ++c) {
+      for (int c = c_first; c < nc; c += EPIW / 4) {
         const int col0 = n0 + c * CH;
         if (col0 >= Nd) break;
         uint32_t r[CH];
