@@ -913,7 +913,7 @@ def run_cuda(args):
                     "linears": [f"{l.name}:{l.K}x{l.N}" for l in bs.cfg.linears], "tweo_blocks": bs.n_blocks,
                     "parallelism": f"replicas x{world} (token shards, no data-path collective)",
                     "l2": f"working set {bs.working_set_bytes() / 1e6:.0f} MB per step > 126 MB L2, no flush",
-                    "launch": "cuda graph replay of one captured step; two streams inside it: the casts of linear "
+                    "launch": "cuda graph replay of one captured step; the casts of linear "
                               "i+1 and the TWEO pass overlap the GEMMs of linear i" if overlap
                     else "cuda graph replay of one captured step, one stream"}
     if args.variant != "fused":

@@ -74,7 +74,8 @@ typedef enum {
   TWEO_OP_LOSS = 4,
   TWEO_OP_W8A8 = 5,
   TWEO_OP_BLOCK_OUTPUT = 6,
-  TWEO_OP_ABSMAX = 7
+  TWEO_OP_ABSMAX = 7,
+  TWEO_OP_BESIDE = 8
 } tweo_op_t;
 typedef enum { TWEO_GRAN_TENSOR = 0, TWEO_GRAN_ROW = 1 } tweo_granularity_t;
 typedef enum { TWEO_ACT_NONE = 0, TWEO_ACT_GELU = 1, TWEO_ACT_GELU_TANH = 2, TWEO_ACT_SWIGLU = 3 } tweo_act_t;
@@ -309,6 +310,28 @@ typedef struct tweo_linear_problem_t {
   const tweo_epilogue_t* epi;           /* optional fused outputs of Y (FWD) or dX (DGRAD); NULL: none */
 } tweo_linear_problem_t;
 TWEO_API tweo_status_t tweo_fp8_linear_group(const tweo_linear_problem_t* problems, int32_t count, void* stream);
+
+/*
+ * tweo_fp8_linear_group_beside -- the same launch, which also carries out independent streaming work while the
+ * products run: per-tensor casts (as tweo_quantize_per_tensor_batch, without sat_count: the same codes, scales and amax)
+ * and / or the penalty of block outputs with its gradient (as tweo_loss_fwd_bwd with p = 4 and bf16 gradients).  The casts are
+ * bound by HBM and the products by the tensor cores: a training step gives the casts of its next linears here.
+ * Nothing the work reads may be written by the products and the other way round.
+ *   ws: tweo_workspace_bytes(TWEO_OP_BESIDE, n_per_tensor, L, 0) bytes, any contents.
+ */
+typedef struct tweo_beside_t {
+  const tweo_quant_desc_t* casts;       /* n_casts of them (0 to TWEO_MAX_QUANT_BATCH) */
+  int32_t n_casts;
+  int32_t L;                            /* block outputs (0 to TWEO_MAX_BLOCKS) */
+  const uint16_t* const* a;             /* bf16 [n_per_tensor] each */
+  void* const* grad;                    /* bf16, one per block output */
+  int64_t n_per_tensor;
+  float tau, eps, grad_coeff;
+  float* loss;
+  float* loss_per_block;                /* float[L], or NULL */
+} tweo_beside_t;
+TWEO_API tweo_status_t tweo_fp8_linear_group_beside(const tweo_linear_problem_t* problems, int32_t count,
+                                           const tweo_beside_t* work, void* ws, size_t ws_bytes, void* stream);
 
 /*
  * tweo_loss_fwd_bwd -- TWEO penalty and its gradient in one pass (Eq. 3, and

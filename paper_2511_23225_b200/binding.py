@@ -24,7 +24,7 @@ from .build import native_target
 E4M3, E5M2 = 0, 1
 SCALE_CURRENT, SCALE_GIVEN = 0, 1
 BF16, F32, FP8_E4M3 = 0, 1, 2
-OP_QUANTIZE, OP_LINEAR_FWD, OP_LINEAR_DGRAD, OP_LINEAR_WGRAD, OP_LOSS, OP_W8A8, OP_BLOCK_OUTPUT, OP_ABSMAX = range(8)
+OP_QUANTIZE, OP_LINEAR_FWD, OP_LINEAR_DGRAD, OP_LINEAR_WGRAD, OP_LOSS, OP_W8A8, OP_BLOCK_OUTPUT, OP_ABSMAX, OP_BESIDE = range(9)
 GRAN_TENSOR, GRAN_ROW = 0, 1
 ACT_NONE, ACT_GELU, ACT_GELU_TANH, ACT_SWIGLU = 0, 1, 2, 3
 NORM_LAYER, NORM_RMS = 0, 1
@@ -37,7 +37,7 @@ NATIVE_PATH = os.path.join(_HERE, "_native.so")
 EXPORTS = [
     "tweo_quantize_per_tensor", "tweo_quantize_per_tensor_batch", "tweo_fp8_linear_fwd", "tweo_fp8_linear_fwd_act",
     "tweo_layernorm_fp8", "tweo_fp8_linear_bwd_dgrad",
-    "tweo_fp8_linear_bwd_wgrad", "tweo_fp8_linear_bwd", "tweo_fp8_linear_group", "tweo_loss_fwd_bwd", "tweo_loss_fwd_bwd_static", "tweo_w8a8_static_gemm",
+    "tweo_fp8_linear_bwd_wgrad", "tweo_fp8_linear_bwd", "tweo_fp8_linear_group", "tweo_fp8_linear_group_beside", "tweo_loss_fwd_bwd", "tweo_loss_fwd_bwd_static", "tweo_w8a8_static_gemm",
     "tweo_fp4_quantize", "tweo_fp4_unpack", "tweo_w4a4_static_gemm", "tweo_fp4_weight_linear",
     "tweo_block_output_fused", "tweo_delayed_scaling_update", "tweo_absmax_quantize", "tweo_int8_linear", "tweo_int8_linear_q8", "tweo_residual_add_q8", "tweo_residual_add_q8_rows",
     "tweo_workspace_bytes", "tweo_workspace_init", "tweo_read_device_status", "tweo_selftest_bounded_wait",
@@ -312,6 +312,15 @@ def fp8_linear_group(problems):
     each optionally with "fmt_x", "fmt_w", "fmt_dy" (defaults E4M3, E4M3, E5M2).  Outputs are bf16 tensors.  A FWD or
     DGRAD problem may add the fused epilogue: "out_amax" and / or "out_q" with "q_fmt" and "q_scale"."""
     _native().linear_group(problems)
+
+
+def fp8_linear_group_beside(problems, xs=(), outs=(), modes=None, blocks=None, grads=None, tau=3.0, eps=1e-6, grad_coeff=1.0, ws=None):
+    """tweo_fp8_linear_group_beside: the grouped launch, and beside its products the casts of `xs` into the records `outs` (as
+    quantize_per_tensor_batch) and / or the penalty (p = 4) of `blocks` with its bf16 gradients `grads` (as loss_fwd_bwd).
+    Returns (loss [1], per-block [L]) with blocks, else None."""
+    if ws is None:
+        ws = new_workspace(OP_BESIDE, blocks[0].numel() if blocks else 0, len(blocks) if blocks else 0)
+    return _native().linear_group_beside(problems, xs, outs, modes, blocks, grads, tau, eps, grad_coeff, ws)
 
 
 def loss_fwd_bwd(blocks, tau=3.0, eps=1e-6, p=4.0, grad_coeff=1.0, want_grad=True, grad_dtype=BF16,

@@ -104,6 +104,8 @@ size_t tweo_workspace_bytes(int32_t op, int64_t M, int64_t N, int64_t K) {
       return tweo_detail::absmax_workspace_bytes();
     case TWEO_OP_BLOCK_OUTPUT:
       return tweo_detail::block_output_workspace_bytes();
+    case TWEO_OP_BESIDE:   // counters, means, one binary64 sum per 8192 elements of each block output
+      return 2048 + sizeof(double) * (size_t)(N < 0 ? 0 : N) * (size_t)((M < 0 ? 0 : M) / 8192 + 1);
     case TWEO_OP_W8A8: {
       // scalars + codes of the activations (a bf16 input is cast inside) + the GEMM's stream-K area
       size_t codes = (size_t)(M < 0 ? 0 : M) * (size_t)(K < 0 ? 0 : K);

@@ -1,0 +1,316 @@
+// Streaming work beside a grouped GEMM: per-tensor casts and the penalty with its gradient, done by warps of the GEMM's own
+// CTAs.  The casts of a training step are bound by HBM and its products by the tensor pipe, so the two should share the time;
+// as kernels of two streams they hardly did (ViT-B/16 step at 12017 tokens: products 220 us, streaming 227 us, together
+// 447 us): a cast kernel holds the SMs while a GEMM that is ready waits for 200 KB of shared memory, and once the GEMM is there
+// one streaming CTA fits beside it.  Here every CTA of the GEMM brings eight warps for the streaming work.
+//
+// Work is cut into chunks of 8192 elements.  A warp draws the next chunk from a counter (the next ticket is drawn while it works), so the SMs share it evenly whatever the GEMM leaves them.  Chunks are ordered: the maximum of a tensor before its cast, with the
+// maximum of the next tensor in between, so that the second read of a tensor finds much of it in L2.  A cast with current
+// scaling waits (bounded) until all chunks of its tensor's maximum are counted; those have smaller tickets, so some warp is at the smallest
+// unfinished one and never waits: no co-residency is needed.  The sums of the penalty are kept per chunk and added in
+// a fixed order by the warp that finishes a tensor last.
+#pragma once
+
+#include "stream_ops.cuh"
+#include "tc_ptx.cuh"
+
+namespace tweo_detail {
+
+constexpr int kBesideWarps = 8;
+constexpr int kBesideChunk = 8192;                 // elements
+constexpr int kBesideMaxSegments = 2 * TWEO_MAX_QUANT_BATCH + 1;
+constexpr int kBesideWords = 192;                  // counters, cleared by a kernel in front:
+constexpr int kBesideTicket = 0, kBesideTensorsDone = 1, kBesideAmax = 8, kBesideDone = 16, kBesideLossDone = 32;
+static_assert(kBesideLossDone + TWEO_MAX_BLOCKS <= kBesideWords, "counters");
+// workspace: counters, the mean of each block output (binary64), then the sums of the chunks
+constexpr size_t kBesideBlockLossOffset = 1024, kBesidePartialsOffset = 1024 + 8 * TWEO_MAX_BLOCKS;
+
+enum BesideKind { kBesideKindAmax = 0, kBesideKindCast = 1, kBesideKindLoss = 2 };
+
+struct Beside {
+  QTensor t[TWEO_MAX_QUANT_BATCH];
+  uint32_t chunks[TWEO_MAX_QUANT_BATCH];
+  uint32_t start[kBesideMaxSegments + 1];          // first ticket of a segment
+  uint8_t kind[kBesideMaxSegments + 3], tensor[kBesideMaxSegments + 3];
+  uint32_t total;
+  uint32_t* words;
+  // penalty, p = 4, bf16 gradient
+  const uint16_t* a[TWEO_MAX_BLOCKS];
+  uint16_t* g[TWEO_MAX_BLOCKS];
+  int64_t n;
+  int32_t L;
+  uint32_t loss_chunks;                            // per block output
+  float k_grad;
+  double inv_norm;
+  float* loss;
+  float* loss_per_block;
+  double* block_loss;
+  double* partials;
+};
+
+__device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
+// Lane 0: every chunk of tensor `ti`'s maximum is counted (bounded).  The answer is the warp's.
+__device__ __forceinline__ bool beside_wait(const Beside& b, int ti, int lane, volatile int* abort_flag) {
+  bool ok = true;
+  if (lane == 0) {
+    const uint32_t* done = b.words + kBesideDone + ti;
+    uint64_t t0 = 0;
+    for (uint32_t it = 0; ld_acquire(done) < b.chunks[ti]; ++it) {
+      if (t0 == 0) t0 = globaltimer_ns();
+      __nanosleep(100);
+      if ((it & 63u) == 63u && (*abort_flag || globaltimer_ns() - t0 > kWaitLimitNs)) {
+        *abort_flag = 1;
+        atomicExch(&g_device_status, (unsigned int)TWEO_ERR_TIMEOUT);
+        ok = false;
+        break;
+      }
+    }
+  }
+  return __all_sync(0xFFFFFFFFu, ok);
+}
+
+// The three kinds of chunk, from element `first` on.  A batch of loads is under way while the one before it is worked on, and no more: with
+// the loads of 16 vectors in flight all the time, or the next chunk brought into L2 ahead, the streaming alone is faster (5.1 for 4.2 TB/s)
+// and the products beside it are slower by more than that.
+__device__ __forceinline__ uint32_t beside_amax(const uint16_t* x, int64_t n, int64_t first, int lane) {
+  const int64_t nvec = n >> 3;
+  const uint4* xv = reinterpret_cast<const uint4*>(x) + (first >> 3) + lane;
+  const int left = (int)min(nvec - (first >> 3) - lane, (int64_t)kBesideChunk);   // vectors from this lane's first one on
+  float m0 = 0.0f, m1 = 0.0f;
+  uint4 v[8];
+  auto load = [&](int j) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = j + 32 * u < left ? __ldg(xv + j + 32 * u) : make_uint4(0u, 0u, 0u, 0u);
+  };
+  load(0);
+#pragma unroll 1
+  for (int j = 0; j < kBesideChunk / 8; j += 256) {
+    uint4 w[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) w[u] = v[u];
+    if (j + 256 < kBesideChunk / 8) load(j + 256);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      absmax_f32(m0, m1, w[u].x);
+      absmax_f32(m0, m1, w[u].y);
+      absmax_f32(m0, m1, w[u].z);
+      absmax_f32(m0, m1, w[u].w);
+    }
+  }
+  if (first == 0 && lane < 8 && (nvec << 3) + lane < n) absmax_f32(m0, m1, (uint32_t)x[(nvec << 3) + lane]);
+  return __reduce_max_sync(0xFFFFFFFFu, absmax_f32_bits(m0, m1));
+}
+
+// One body for both formats, chosen around the converting instructions, and with the maximum whether it is wanted or not: with a body
+// for each case the compiler interleaves them and needs twice the registers there are.
+__device__ __forceinline__ uint32_t beside_cast(const uint16_t* x, uint8_t* q, int64_t n, int64_t first, float s, bool e4m3, int lane) {
+  const int64_t n16 = n >> 4;
+  const uint4* xv = reinterpret_cast<const uint4*>(x) + (first >> 3) + 2 * lane;
+  uint4* qv = reinterpret_cast<uint4*>(q) + (first >> 4) + lane;
+  const int left = (int)min(n16 - (first >> 4) - lane, (int64_t)kBesideChunk);
+  const uint64_t ss = splat_f32x2(s);
+  float m0 = 0.0f, m1 = 0.0f;
+  uint4 v[4][2];
+  auto load = [&](int j) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const bool in = j + 32 * u < left;
+      v[u][0] = in ? __ldcs(xv + 2 * (j + 32 * u)) : make_uint4(0u, 0u, 0u, 0u);
+      v[u][1] = in ? __ldcs(xv + 2 * (j + 32 * u) + 1) : make_uint4(0u, 0u, 0u, 0u);
+    }
+  };
+  load(0);
+#pragma unroll 1
+  for (int j = 0; j < kBesideChunk / 16; j += 128) {
+    uint4 c[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const uint32_t w[8] = {v[u][0].x, v[u][0].y, v[u][0].z, v[u][0].w, v[u][1].x, v[u][1].y, v[u][1].z, v[u][1].w};
+      float p[16];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        unpack_f32x2(mul_f32x2(bf16x2_to_f32x2(w[k]), ss), p[2 * k], p[2 * k + 1]);
+        absmax_f32(m0, m1, w[k]);
+      }
+      uint32_t h[4];
+      if (e4m3) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) h[k] = cvt_fp8x2<TWEO_E4M3>(p[4 * k], p[4 * k + 1]) | (cvt_fp8x2<TWEO_E4M3>(p[4 * k + 2], p[4 * k + 3]) << 16);
+      } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) h[k] = cvt_fp8x2<TWEO_E5M2>(p[4 * k], p[4 * k + 1]) | (cvt_fp8x2<TWEO_E5M2>(p[4 * k + 2], p[4 * k + 3]) << 16);
+      }
+      c[u] = make_uint4(h[0], h[1], h[2], h[3]);
+    }
+    if (j + 128 < kBesideChunk / 16) load(j + 128);
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (j + 32 * u < left) __stcs(qv + j + 32 * u, c[u]);
+  }
+  if (first == 0 && lane < 16 && (n16 << 4) + lane < n) {   // ragged tail: n % 16 elements
+    const int64_t i = (n16 << 4) + lane;
+    const uint32_t w = x[i];
+    const float p = __fmul_rn(bf16lo_to_f32(w), s);
+    q[i] = (uint8_t)((e4m3 ? cvt_fp8x2<TWEO_E4M3>(p, 0.0f) : cvt_fp8x2<TWEO_E5M2>(p, 0.0f)) & 0xFFu);
+    absmax_f32(m0, m1, w);
+  }
+  return __reduce_max_sync(0xFFFFFFFFu, absmax_f32_bits(m0, m1));
+}
+
+// The sum of a^4 over the chunk, and the gradient.  The grouping of the binary32 sums is that of the streaming kernel (four vectors,
+// 256 apart).
+__device__ __forceinline__ double beside_penalty(const uint16_t* a, uint16_t* g, int64_t n, int64_t first, float k_grad, int lane) {
+  const int64_t nvec = n >> 3;
+  const uint4* av = reinterpret_cast<const uint4*>(a) + (first >> 3) + lane;
+  uint4* gv = reinterpret_cast<uint4*>(g) + (first >> 3) + lane;
+  const int left = (int)min(nvec - (first >> 3) - lane, (int64_t)kBesideChunk);
+  double acc = 0.0;
+  uint4 v[4];
+  auto load = [&](int j) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = j + 256 * u < left ? __ldcs(av + j + 256 * u) : make_uint4(0u, 0u, 0u, 0u);
+  };
+  load(0);
+#pragma unroll 1
+  for (int j = 0; j < 256; j += 32) {
+    uint64_t acc2 = 0ull;
+    uint4 out[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      uint64_t g2[4];
+      penalty4_vec<true>(v[u], k_grad, acc2, g2);
+      out[u] = make_uint4(f32x2_pair_to_bf16x2(g2[0]), f32x2_pair_to_bf16x2(g2[1]), f32x2_pair_to_bf16x2(g2[2]), f32x2_pair_to_bf16x2(g2[3]));
+    }
+    if (j + 32 < 256) load(j + 32);
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (j + 256 * u < left) __stcs(gv + j + 256 * u, out[u]);
+    float lo, hi;
+    unpack_f32x2(acc2, lo, hi);
+    acc += (double)lo + (double)hi;
+  }
+  if (first == 0 && lane < 8 && (nvec << 3) + lane < n) {   // ragged tail: n % 8 elements
+    const int64_t i = (nvec << 3) + lane;
+    const float af = bf16lo_to_f32((uint32_t)a[i]);
+    const float s = af * af;
+    acc += (double)(s * s);
+    g[i] = (uint16_t)f32_to_bf16_bits(__fmul_rn(k_grad, s * af));
+  }
+  return warp_sum(acc);
+}
+
+// One chunk of block output l, and where it is the last one, the sums.
+__device__ __forceinline__ void beside_loss(const Beside& b, int l, uint32_t chunk, int lane) {
+  const double acc = beside_penalty(b.a[l], b.g[l], b.n, (int64_t)chunk * kBesideChunk, b.k_grad, lane);
+  double* part = b.partials + (size_t)l * b.loss_chunks;
+  uint32_t last = 0;
+  if (lane == 0) {
+    part[chunk] = acc;
+    __threadfence();
+    last = atomicAdd(b.words + kBesideLossDone + l, 1u) + 1u == b.loss_chunks;
+  }
+  if (!__shfl_sync(0xFFFFFFFFu, last, 0)) return;
+  // the last chunk of this tensor: add all of them in a fixed order
+  __threadfence();
+  double s = 0.0;
+  for (uint32_t b0 = lane; b0 < b.loss_chunks; b0 += 32 * 8) {
+    double w[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) w[j] = b0 + 32u * j < b.loss_chunks ? __ldcg(part + b0 + 32u * j) : 0.0;
+    s += ((w[0] + w[1]) + (w[2] + w[3])) + ((w[4] + w[5]) + (w[6] + w[7]));
+  }
+  s = warp_sum(s);
+  if (lane == 0) {
+    b.block_loss[l] = s * b.inv_norm;
+    __threadfence();
+    if (atomicAdd(b.words + kBesideTensorsDone, 1u) + 1u == (uint32_t)b.L) {   // and the last tensor
+      __threadfence();
+      double sum = 0.0;
+      for (int i = 0; i < b.L; ++i) {
+        const double m = __ldcg(b.block_loss + i);
+        sum += m;
+        if (b.loss_per_block) b.loss_per_block[i] = (float)m;
+      }
+      *b.loss = (float)(sum / (double)b.L);
+    }
+  }
+}
+
+// A ticket's chunk.
+struct BesideTask {
+  int kind, tensor;     // of a penalty: the block output
+  uint32_t chunk;
+};
+__device__ __forceinline__ BesideTask beside_task(const Beside& b, uint32_t ticket) {
+  int seg = 0;
+  while (ticket >= b.start[seg + 1]) ++seg;
+  BesideTask t{b.kind[seg], b.tensor[seg], ticket - b.start[seg]};
+  if (t.kind == kBesideKindLoss) {
+    t.tensor = (int)(t.chunk / b.loss_chunks);
+    t.chunk -= (uint32_t)t.tensor * b.loss_chunks;
+  }
+  return t;
+}
+// What a streaming warp does: chunk after chunk until none is left.
+__device__ __forceinline__ void beside_work(const Beside& b, int lane, volatile int* abort_flag) {
+  uint32_t ticket = 0, complete = 0;   // complete: a bit per tensor whose maximum is known to be complete
+  if (lane == 0) ticket = atomicAdd(b.words + kBesideTicket, 1u);
+  for (;;) {
+    const uint32_t now = __shfl_sync(0xFFFFFFFFu, ticket, 0);
+    if (now >= b.total) return;
+    if (lane == 0) ticket = atomicAdd(b.words + kBesideTicket, 1u);
+    const BesideTask task = beside_task(b, now);
+    const uint32_t chunk = task.chunk;
+    const int ti = task.tensor;
+    if (task.kind == kBesideKindLoss) {
+      beside_loss(b, ti, chunk, lane);
+      continue;
+    }
+    const QTensor& t = b.t[ti];
+    const int64_t first = (int64_t)chunk * kBesideChunk;
+    uint32_t* slot = b.words + kBesideAmax + ti;
+    uint32_t* done = b.words + kBesideDone + ti;
+    if (task.kind == kBesideKindAmax) {
+      const uint32_t m = beside_amax(t.x, t.n, first, lane);
+      if (lane == 0) {
+        if (m) atomicMax(slot, m << 16);
+        __threadfence();
+        atomicAdd(done, 1u);
+      }
+      continue;
+    }
+    const bool given = t.mode == TWEO_SCALE_GIVEN;
+    float s;
+    if (given) {
+      s = *t.scale;
+    } else {
+      if (!((complete >> ti) & 1u)) {
+        if (!beside_wait(b, ti, lane, abort_flag)) return;
+        complete |= 1u << ti;
+      }
+      const float amax = __uint_as_float(__ldcg(slot));
+      s = scale_from_amax(amax, t.fmt);
+      if (chunk == 0 && lane == 0) {
+        *t.amax = amax;
+        *t.scale = s;
+      }
+    }
+    if (chunk == 0 && lane == 0) *t.scale_inv = __fdiv_rn(1.0f, s);
+    const uint32_t m = beside_cast(t.x, t.q, t.n, first, s, t.fmt == TWEO_E4M3, lane);
+    if (given && lane == 0) {
+      if (m) atomicMax(slot, m << 16);
+      __threadfence();
+      if (atomicAdd(done, 1u) + 1u == b.chunks[ti]) {   // the last chunk: the maximum is complete
+        __threadfence();
+        *t.amax = __uint_as_float(__ldcg(slot));
+      }
+    }
+  }
+}
+
+}  // namespace tweo_detail

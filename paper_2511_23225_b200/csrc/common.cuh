@@ -28,6 +28,12 @@ void log_call(const char* fmt, ...) __attribute__((format(printf, 1, 2)));
 tweo_status_t read_and_clear_device_status(cudaStream_t stream);
 unsigned int* device_status_word();  // its device address on the current device (nullptr on failure)
 
+// Shared checks and numbers of the casts and the penalty (quantize.cu, loss.cu).
+tweo_status_t check_quant_desc(const tweo_quant_desc_t& d);
+tweo_status_t check_loss_args(const uint16_t* const* a, int32_t L, int64_t n_per_tensor, float tau, float eps, float p, const float* loss,
+                              void* const* grad, int32_t grad_dtype);
+void loss_factors(int64_t n, float tau, float eps, float p, float grad_coeff, float* k_grad, double* inv_norm);
+
 // Grid of a streaming kernel whose CTAs walk `iters` equal pieces of work with a grid-stride loop, at most `cap`
 // CTAs: every CTA gets the same number of pieces (or one less), so no SM waits for a straggler that drew one more
 // sweep than the average -- with iters = 3.5 x cap a capped grid would finish at 4 sweeps, 13 % late.

@@ -38,11 +38,13 @@
 #include <cstdlib>
 #include <mutex>
 #include <queue>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
 #include "common.cuh"
 
+#include "beside.cuh"
 #include "gemm_common.cuh"
 #include "gemm_pair.cuh"
 #include "gemm_pair_group.cuh"
@@ -938,11 +940,12 @@ struct FloatPtrs {
   float* p[kGroupMaxProblems];
   int n;
 };
-// Clears the amax cells of a group's fused epilogues (in the chain, like zero_float_kernel).
-__global__ void zero_floats_kernel(const FloatPtrs f) {
+// Clears the amax cells of a group's fused epilogues and the counters of the work beside it (in the chain, like zero_float_kernel).
+__global__ void group_clear_kernel(const FloatPtrs f, uint32_t* words) {
   chain_release();
   chain_wait();
   if ((int)threadIdx.x < f.n) *f.p[threadIdx.x] = 0.0f;
+  if (words) words[threadIdx.x] = 0u;
 }
 
 int64_t group_tiles(const GroupDesc& d) { return ((d.Md + 2 * BM - 1) / (2 * BM)) * ((d.Nd + d.bn - 1) / d.bn); }
@@ -991,14 +994,16 @@ void group_widths(GroupDesc* d, int n) {
 
 // QST: fused epilogue outputs (amax, FP8 copy) on some products.  EPIW / EBUF as in the kernel; the operand ring
 // takes what the staging buffers leave of the shared memory.
-template <int LIST, bool QST, int EPIW, int EBUF>
-tweo_status_t run_group_list(GroupDesc* d, int n, cudaStream_t st) {
+template <int LIST, bool QST, int EPIW, int EBUF, typename B>
+tweo_status_t run_group_list(GroupDesc* d, int n, const B& beside, cudaStream_t st) {
   constexpr size_t staging = (size_t)EPIW * EBUF * (32 * 128 + (QST ? 32 * 64 : 0));
   constexpr int STAGES = (int)((227 * 1024 - 1024 - 256 - staging) / (BM * BK + 128 * BK)) > 6
                              ? 6 : (int)((227 * 1024 - 1024 - 256 - staging) / (BM * BK + 128 * BK));
   static_assert(STAGES >= 4, "operand ring too short");
   constexpr size_t smem = (size_t)STAGES * (BM * BK + 128 * BK) + staging + 1024 + 256;
-  auto kern = gemm_fp8_pair_group_kernel<STAGES, LIST, QST, EPIW, EBUF>;
+  constexpr bool BESIDE = std::is_same<B, Beside>::value;
+  constexpr int THREADS = 64 + 32 * EPIW + (BESIDE ? 32 * kBesideWarps : 0);
+  auto kern = gemm_fp8_pair_group_kernel<STAGES, LIST, QST, EPIW, EBUF, B>;
   static std::atomic<uint64_t> attr_done{0};  // per device
   int attr_dev = 0;
   if (device_once_pending(attr_done, &attr_dev)) {
@@ -1041,14 +1046,16 @@ tweo_status_t run_group_list(GroupDesc* d, int n, cudaStream_t st) {
   }
   for (int i = n; i <= kGroupMaxProblems; ++i) g.tile_start[i] = g.tile_start[n];
   g.total_tiles = g.tile_start[n];
-  g.pad = 0;
-  int pairs = pairs_all < g.total_tiles ? pairs_all : g.total_tiles;
+  // the streaming warps are wanted on every SM, whether it has a tile or not
+  const int gemm_pairs = pairs_all < g.total_tiles ? pairs_all : g.total_tiles;
+  const int pairs = BESIDE ? pairs_all : gemm_pairs;
   g.use_lists = (g.total_tiles <= LIST && pairs <= kGroupMaxPairs) ? 1 : 0;
+  g.gemm_pairs = gemm_pairs;
   if (g.use_lists) {
     // longest processing time first: every tile goes to the pair with the least work so far
     typedef std::pair<int64_t, int> Load;  // (work, pair); smallest on top, ties to the lower pair index
     std::priority_queue<Load, std::vector<Load>, std::greater<Load>> heap;
-    for (int p = 0; p < pairs; ++p) heap.push(Load(0, p));
+    for (int p = 0; p < gemm_pairs; ++p) heap.push(Load(0, p));
     static thread_local uint8_t owner[LIST];
     int count[kGroupMaxPairs + 1] = {0};
     int prob = 0;
@@ -1069,22 +1076,23 @@ tweo_status_t run_group_list(GroupDesc* d, int n, cudaStream_t st) {
     }
     for (int t = 0; t < g.total_tiles; ++t) g.list[fill[owner[t]]++] = (uint16_t)t;  // ascending t within a pair
   }
-  if (QST) {
-    FloatPtrs z;
-    z.n = 0;
-    for (int i = 0; i < n; ++i)
-      if (d[i].out_amax) z.p[z.n++] = d[i].out_amax;
-    if (z.n) {
-      TWEO_CUDA_TRY(launch_chain(zero_floats_kernel, dim3(1), dim3(32), 0, st, 0, z));
-      count_launch();
-    }
+  FloatPtrs z;
+  z.n = 0;
+  for (int i = 0; i < n; ++i)
+    if (d[i].out_amax) z.p[z.n++] = d[i].out_amax;
+  uint32_t* words = nullptr;
+  if constexpr (BESIDE) words = beside.words;
+  if (z.n || words) {
+    TWEO_CUDA_TRY(launch_chain(group_clear_kernel, dim3(1), dim3(kBesideWords), 0, st, 0, z, words));
+    count_launch();
   }
-  TWEO_CUDA_TRY(launch_chain(kern, dim3((unsigned)(2 * pairs)), dim3(64 + 32 * EPIW), smem, st, 2, g));
+  TWEO_CUDA_TRY(launch_chain(kern, dim3((unsigned)(2 * pairs)), dim3(THREADS), smem, st, 2, g, beside));
   count_launch();
   return check_launch("gemm_fp8_pair_group_kernel");
 }
 
-tweo_status_t run_group(GroupDesc* d, int n, cudaStream_t st) {
+template <typename B>
+tweo_status_t run_group_beside(GroupDesc* d, int n, const B& b, cudaStream_t st) {
   if (n < 1 || n > kGroupMaxProblems) return TWEO_ERR_INVALID_ARG;
   group_widths(d, n);
   // the products with the longer tiles go first in the tile list (stable: equal lengths keep the caller's order)
@@ -1100,12 +1108,58 @@ tweo_status_t run_group(GroupDesc* d, int n, cudaStream_t st) {
     }
   const bool small = tiles <= kGroupListSmall;
   if (!fused)
-    return small ? run_group_list<kGroupListSmall, false, 4, 2>(d, n, st) : run_group_list<kGroupListLarge, false, 4, 2>(d, n, st);
+    return small ? run_group_list<kGroupListSmall, false, 4, 2>(d, n, b, st) : run_group_list<kGroupListLarge, false, 4, 2>(d, n, b, st);
   // the fused epilogue computes per element: at short contractions it outlasts the tile's main loop unless eight
   // warps share it (the rule of the single fused products)
   if (fused_kb_min < 16)
-    return small ? run_group_list<kGroupListSmall, true, 8, 1>(d, n, st) : run_group_list<kGroupListLarge, true, 8, 1>(d, n, st);
-  return small ? run_group_list<kGroupListSmall, true, 4, 1>(d, n, st) : run_group_list<kGroupListLarge, true, 4, 1>(d, n, st);
+    return small ? run_group_list<kGroupListSmall, true, 8, 1>(d, n, b, st) : run_group_list<kGroupListLarge, true, 8, 1>(d, n, b, st);
+  return small ? run_group_list<kGroupListSmall, true, 4, 1>(d, n, b, st) : run_group_list<kGroupListLarge, true, 4, 1>(d, n, b, st);
+}
+
+tweo_status_t run_group(GroupDesc* d, int n, cudaStream_t st) { return run_group_beside(d, n, NothingBeside{}, st); }
+
+// The checked work of a tweo_beside_t as the kernel takes it.
+Beside make_beside(const tweo_beside_t& w, void* ws) {
+  Beside b{};
+  b.words = reinterpret_cast<uint32_t*>(ws);
+  b.block_loss = reinterpret_cast<double*>(reinterpret_cast<char*>(ws) + kBesideBlockLossOffset);
+  b.partials = reinterpret_cast<double*>(reinterpret_cast<char*>(ws) + kBesidePartialsOffset);
+  int segs = 0;
+  uint32_t at = 0;
+  auto segment = [&](BesideKind kind, int tensor, uint32_t chunks) {
+    b.start[segs] = at;
+    b.kind[segs] = (uint8_t)kind;
+    b.tensor[segs] = (uint8_t)tensor;
+    ++segs;
+    at += chunks;
+  };
+  auto chunks_of = [](int64_t n) { return (uint32_t)std::max<int64_t>(1, (n + kBesideChunk - 1) / kBesideChunk); };
+  int waiting = -1;   // a tensor whose maximum is listed and whose cast is not yet
+  for (int i = 0; i < w.n_casts; ++i) {
+    const tweo_quant_desc_t& d = w.casts[i];
+    b.t[i] = QTensor{d.x, d.q, d.n, d.scale, d.scale_inv, d.amax, d.fmt, d.mode};
+    b.chunks[i] = chunks_of(d.n);
+    if (d.mode == TWEO_SCALE_CURRENT) segment(kBesideKindAmax, i, b.chunks[i]);
+    if (waiting >= 0) segment(kBesideKindCast, waiting, b.chunks[waiting]);
+    waiting = i;
+  }
+  if (waiting >= 0) segment(kBesideKindCast, waiting, b.chunks[waiting]);
+  if (w.L > 0) {
+    for (int l = 0; l < w.L; ++l) {
+      b.a[l] = w.a[l];
+      b.g[l] = reinterpret_cast<uint16_t*>(w.grad[l]);
+    }
+    b.n = w.n_per_tensor;
+    b.L = w.L;
+    b.loss_chunks = chunks_of(w.n_per_tensor);
+    loss_factors(w.n_per_tensor, w.tau, w.eps, 4.0f, w.grad_coeff, &b.k_grad, &b.inv_norm);
+    b.loss = w.loss;
+    b.loss_per_block = w.loss_per_block;
+    segment(kBesideKindLoss, 0, b.loss_chunks * (uint32_t)w.L);
+  }
+  for (int i = segs; i <= kBesideMaxSegments; ++i) b.start[i] = at;
+  b.total = at;
+  return b;
 }
 
 // dX and dW of one linear layer as a group of two products.
@@ -1384,10 +1438,12 @@ tweo_status_t tweo_fp8_linear_bwd(const uint8_t* dyq, int64_t lddy, int32_t fmt_
                                    ws, ws_bytes, stream);
 }
 
-tweo_status_t tweo_fp8_linear_group(const tweo_linear_problem_t* problems, int32_t count, void* stream) {
-  TWEO_LOG_CALL("tweo_fp8_linear_group " "problems=%p count=%d", (const void*)problems, count);
+}  // extern "C"
+
+namespace {
+// The checked problems as the launcher takes them.
+tweo_status_t group_descs(const tweo_linear_problem_t* problems, int32_t count, GroupDesc* d) {
   if (!problems || count < 1 || count > TWEO_MAX_GROUP) return TWEO_ERR_INVALID_ARG;
-  GroupDesc d[TWEO_MAX_GROUP];
   for (int i = 0; i < count; ++i) {
     const tweo_linear_problem_t& q = problems[i];
     const int64_t M = q.M, N = q.N, K = q.K;
@@ -1427,7 +1483,44 @@ tweo_status_t tweo_fp8_linear_group(const tweo_linear_problem_t* problems, int32
     if (!tweo_detail::aligned16(d[i].a) || !tweo_detail::aligned16(d[i].b) || (d[i].lda & 15) || (d[i].ldb & 15))
       return TWEO_ERR_ALIGNMENT;
   }
-  return run_group(d, count, (cudaStream_t)stream);
+  return TWEO_OK;
+}
+}  // namespace
+
+extern "C" {
+
+tweo_status_t tweo_fp8_linear_group(const tweo_linear_problem_t* problems, int32_t count, void* stream) {
+  TWEO_LOG_CALL("tweo_fp8_linear_group " "problems=%p count=%d", (const void*)problems, count);
+  GroupDesc d[TWEO_MAX_GROUP];
+  const tweo_status_t s = group_descs(problems, count, d);
+  return s == TWEO_OK ? run_group(d, count, (cudaStream_t)stream) : s;
+}
+
+tweo_status_t tweo_fp8_linear_group_beside(const tweo_linear_problem_t* problems, int32_t count, const tweo_beside_t* work, void* ws,
+                                           size_t ws_bytes, void* stream) {
+  TWEO_LOG_CALL("tweo_fp8_linear_group_beside " "problems=%p count=%d n_casts=%d L=%d n=%lld ws_bytes=%zu", (const void*)problems, count,
+                work ? work->n_casts : 0, work ? work->L : 0, (long long)(work ? work->n_per_tensor : 0), ws_bytes);
+  GroupDesc d[TWEO_MAX_GROUP];
+  tweo_status_t s = group_descs(problems, count, d);
+  if (s != TWEO_OK) return s;
+  if (!work || work->n_casts < 0 || work->n_casts > TWEO_MAX_QUANT_BATCH || (work->n_casts > 0 && !work->casts) || work->L < 0)
+    return TWEO_ERR_INVALID_ARG;
+  for (int i = 0; i < work->n_casts; ++i) {
+    s = check_quant_desc(work->casts[i]);
+    if (s != TWEO_OK) return s;
+    if (work->casts[i].sat_count) return TWEO_ERR_INVALID_ARG;
+    if (work->casts[i].n > ((int64_t)1 << 40)) return TWEO_ERR_UNSUPPORTED_SHAPE;   // chunks are counted in 32 bits
+  }
+  if (work->L > 0) {
+    if (!work->grad) return TWEO_ERR_INVALID_ARG;
+    s = check_loss_args(work->a, work->L, work->n_per_tensor, work->tau, work->eps, 4.0f, work->loss, work->grad, TWEO_BF16);
+    if (s != TWEO_OK) return s;
+    if (work->n_per_tensor > ((int64_t)1 << 36)) return TWEO_ERR_UNSUPPORTED_SHAPE;
+  }
+  if (!ws || ws_bytes < tweo_workspace_bytes(TWEO_OP_BESIDE, work->n_per_tensor, work->L, 0)) return TWEO_ERR_WORKSPACE_TOO_SMALL;
+  if (!tweo_detail::aligned16(ws)) return TWEO_ERR_ALIGNMENT;
+  const Beside b = make_beside(*work, ws);
+  return b.total ? run_group_beside(d, count, b, (cudaStream_t)stream) : run_group(d, count, (cudaStream_t)stream);
 }
 
 tweo_status_t tweo_fp4_weight_linear(const uint8_t* xq, int64_t ldx, int32_t fmt_x, const float* sx_inv, const uint8_t* w4,

@@ -18,8 +18,11 @@
 // TMA like the bf16 tile (one operand stage less).  Every wait is bounded.
 #pragma once
 
+#include <type_traits>
+
 #include <cuda.h>
 
+#include "beside.cuh"
 #include "gemm_common.cuh"
 #include "tc_ptx.cuh"
 
@@ -53,7 +56,7 @@ struct alignas(64) PairGroupParams {
   int32_t tile_start[kGroupMaxProblems + 1];  // product i owns the tile numbers [tile_start[i], tile_start[i + 1])
   int32_t total_tiles;
   int32_t use_lists;     // the per-pair lists are valid (total_tiles <= LIST)
-  int32_t pad;
+  int32_t gemm_pairs;    // pairs that may have tiles: the first ones
   uint16_t first[kGroupMaxPairs + 1];  // pair p computes list[first[p]] .. list[first[p + 1] - 1], in that order
   uint16_t list[LIST];                 // tile numbers
 };
@@ -72,7 +75,7 @@ struct GroupSched {
       t = g.list[pos++];
     } else {
       t = t < 0 ? worker : t + workers;
-      if (t >= g.total_tiles) return false;
+      if (t >= g.total_tiles || worker >= workers) return false;
     }
     prob = 0;
     while (prob + 1 < g.n_problems && t >= g.tile_start[prob + 1]) ++prob;
@@ -95,9 +98,12 @@ __device__ __forceinline__ void group_tile_coords(const GroupProblem& q, int til
 // half of a tile's columns each -- the fused epilogue of a short contraction is bound by the issue rate of one
 // warp per scheduler).  EBUF: staging buffers per epilogue warp (2: a chunk is staged while the store of the
 // one before it drains; 1: half the staging memory, which buys an operand stage).
-template <int STAGES, int LIST, bool QST = false, int EPIW = 4, int EBUF = 2>
-__global__ void __launch_bounds__(64 + 32 * EPIW, 1)
-gemm_fp8_pair_group_kernel(const __grid_constant__ PairGroupParams<LIST> g) {
+// B: Beside, and eight warps more that do its work (beside.cuh); or NothingBeside.
+struct NothingBeside {};
+
+template <int STAGES, int LIST, bool QST = false, int EPIW = 4, int EBUF = 2, typename B = NothingBeside>
+__global__ void __launch_bounds__(64 + 32 * EPIW + (std::is_same<B, Beside>::value ? 32 * kBesideWarps : 0), 1)
+gemm_fp8_pair_group_kernel(const __grid_constant__ PairGroupParams<LIST> g, const __grid_constant__ B beside) {
   constexpr int BN = 256;                 // tile columns of the pair, at most
   constexpr uint32_t A_BYTES = BM * BK;   // this CTA's 128 rows of A
   constexpr uint32_t B_BYTES = 128 * BK;  // this CTA's half of the columns of B, at most 128
@@ -154,7 +160,7 @@ gemm_fp8_pair_group_kernel(const __grid_constant__ PairGroupParams<LIST> g) {
   chain_release();
 
   const int pair = blockIdx.x >> 1;
-  const int num_pairs = gridDim.x >> 1;
+  const int num_pairs = g.gemm_pairs;
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (both CTAs)
@@ -240,6 +246,12 @@ gemm_fp8_pair_group_kernel(const __grid_constant__ PairGroupParams<LIST> g) {
         acc ^= 1;
         if (acc == 0) acc_phase ^= 1u;
       }
+    }
+  } else if (std::is_same<B, Beside>::value && warp >= 2 + EPIW) {
+    // ------------------------------------------------------------ streaming work beside the products
+    if constexpr (std::is_same<B, Beside>::value) {
+      chain_wait();
+      beside_work(beside, lane, abort_flag);
     }
   } else {
     // ------------------------------------------------------------ epilogue (warps 2.., both CTAs)

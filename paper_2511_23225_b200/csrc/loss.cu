@@ -15,6 +15,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "stream_ops.cuh"
 
 namespace tweo_detail {
 
@@ -56,30 +57,15 @@ struct LossArgs {
   int parts_per_tensor;   // gridDim.x of the streaming kernel
 };
 
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xFFFFFFFFu, v, o);
-  return v;
-}
-
-// One 16-byte vector (8 bf16).  p = 4: packed binary32 pairs -- s = a*a is exact (8-bit significands), a^3 = s*a
-// too (24 bits), so g = fl32(k * a^3) rounds once; the a^4 terms are folded into the running pair `acc2` by a
-// fused multiply-add (acc2 += s*s), which the caller empties into its binary64 sum once per loop iteration.
+// One 16-byte vector (8 bf16).  p = 4: see penalty4_vec(); the caller empties acc2 once per loop iteration.
 // Other p: binary64 pow (keeps the 1e-5 budget for any p > 1), terms added to `vsum`.
 template <bool FAST, bool GRAD, bool GRAD_F32>
 __device__ __forceinline__ void process_vec(const uint4 v, float k, float p, uint64_t& acc2, float& vsum,
                                             uint4* gout_bf16, float4* gout_f32) {
   const uint32_t w[4] = {v.x, v.y, v.z, v.w};
   if (FAST) {
-    const uint64_t kk = pack_f32x2(k, k);
     uint64_t g2[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint64_t a2 = bf16x2_to_f32x2(w[j]);
-      const uint64_t s2 = mul_f32x2(a2, a2);
-      acc2 = fma_f32x2(s2, s2, acc2);
-      if (GRAD) g2[j] = mul_f32x2(kk, mul_f32x2(s2, a2));
-    }
+    penalty4_vec<GRAD>(v, k, acc2, g2);
     if (GRAD) {
       if (GRAD_F32) {
         float g[8];
@@ -246,23 +232,6 @@ void launch(dim3 grid, cudaStream_t st, const LossPtrs& ptrs, const LossArgs& ar
 
 // Argument checks, kernel arguments and launch shared by the two entry points; they differ only in where the
 // scratch memory (partial sums from byte 256; every one that is read was written by the same call) lives.
-tweo_status_t check_loss_args(const uint16_t* const* a, int32_t L, int64_t n_per_tensor, float tau, float eps, float p,
-                              const float* loss, void* const* grad, int32_t grad_dtype) {
-  if (!a || !loss || L < 1 || L > TWEO_MAX_BLOCKS || n_per_tensor < 0) return TWEO_ERR_INVALID_ARG;
-  if (!(p > 1.0f) || !(tau + eps > 0.0f)) return TWEO_ERR_INVALID_ARG;
-  if (grad && grad_dtype != TWEO_BF16 && grad_dtype != TWEO_F32) return TWEO_ERR_INVALID_ARG;
-  for (int l = 0; l < L; ++l) {
-    if (!a[l] && n_per_tensor > 0) return TWEO_ERR_INVALID_ARG;
-    if (!aligned16(a[l])) return TWEO_ERR_ALIGNMENT;
-    if (grad) {
-      if (!grad[l] && n_per_tensor > 0) return TWEO_ERR_INVALID_ARG;
-      if (!aligned16(grad[l])) return TWEO_ERR_ALIGNMENT;
-      if (grad_dtype == TWEO_F32 && grad[l] == (const void*)a[l] && n_per_tensor > 0) return TWEO_ERR_INVALID_ARG;
-    }
-  }
-  return TWEO_OK;
-}
-
 tweo_status_t launch_loss(const uint16_t* const* a, int32_t L, int64_t n_per_tensor, float tau, float eps, float p,
                           float grad_coeff, float* loss, float* loss_per_block, void* const* grad, int32_t grad_dtype,
                           void* scratch, int blocks_per_tensor, cudaStream_t st, const char* what) {
@@ -275,10 +244,7 @@ tweo_status_t launch_loss(const uint16_t* const* a, int32_t L, int64_t n_per_ten
   args.n = n_per_tensor;
   args.L = L;
   args.p = p;
-  const double d = (double)tau + (double)eps;
-  const double norm = (double)n_per_tensor * pow(d, (double)p);
-  args.inv_norm = n_per_tensor > 0 ? 1.0 / norm : 0.0;
-  args.k_grad = n_per_tensor > 0 ? (float)((double)grad_coeff * (double)p / norm) : 0.0f;
+  loss_factors(n_per_tensor, tau, eps, p, grad_coeff, &args.k_grad, &args.inv_norm);
   args.loss = loss;
   args.loss_per_block = loss_per_block;
   args.partials = reinterpret_cast<double*>(reinterpret_cast<char*>(scratch) + 256);
@@ -303,6 +269,32 @@ tweo_status_t launch_loss(const uint16_t* const* a, int32_t L, int64_t n_per_ten
 }
 
 }  // namespace
+
+namespace tweo_detail {
+tweo_status_t check_loss_args(const uint16_t* const* a, int32_t L, int64_t n_per_tensor, float tau, float eps, float p,
+                              const float* loss, void* const* grad, int32_t grad_dtype) {
+  if (!a || !loss || L < 1 || L > TWEO_MAX_BLOCKS || n_per_tensor < 0) return TWEO_ERR_INVALID_ARG;
+  if (!(p > 1.0f) || !(tau + eps > 0.0f)) return TWEO_ERR_INVALID_ARG;
+  if (grad && grad_dtype != TWEO_BF16 && grad_dtype != TWEO_F32) return TWEO_ERR_INVALID_ARG;
+  for (int l = 0; l < L; ++l) {
+    if (!a[l] && n_per_tensor > 0) return TWEO_ERR_INVALID_ARG;
+    if (!aligned16(a[l])) return TWEO_ERR_ALIGNMENT;
+    if (grad) {
+      if (!grad[l] && n_per_tensor > 0) return TWEO_ERR_INVALID_ARG;
+      if (!aligned16(grad[l])) return TWEO_ERR_ALIGNMENT;
+      if (grad_dtype == TWEO_F32 && grad[l] == (const void*)a[l] && n_per_tensor > 0) return TWEO_ERR_INVALID_ARG;
+    }
+  }
+  return TWEO_OK;
+}
+
+// k_grad = fl32(grad_coeff p / (n (tau + eps)^p)), rounded once, and 1 / (n (tau + eps)^p)
+void loss_factors(int64_t n, float tau, float eps, float p, float grad_coeff, float* k_grad, double* inv_norm) {
+  const double norm = (double)n * pow((double)tau + (double)eps, (double)p);
+  *inv_norm = n > 0 ? 1.0 / norm : 0.0;
+  *k_grad = n > 0 ? (float)((double)grad_coeff * (double)p / norm) : 0.0f;
+}
+}  // namespace tweo_detail
 
 extern "C" tweo_status_t tweo_loss_fwd_bwd(const uint16_t* const* a, int32_t L, int64_t n_per_tensor, float tau,
                                            float eps, float p, float grad_coeff, float* loss,

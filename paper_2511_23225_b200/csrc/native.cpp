@@ -229,24 +229,33 @@ FN(quantize, 5, {
   Py_RETURN_NONE;
 })
 
+// The casts of a batch, at least `least` of them.
+struct Casts {
+  Ref xs, outs, modes;
+  Py_ssize_t count;
+  Casts(PyObject* xs_, PyObject* outs_, PyObject* modes_, tweo_quant_desc_t* d, Py_ssize_t least)
+      : xs(PySequence_Fast(xs_, "xs must be a sequence")), outs(PySequence_Fast(outs_, "outs must be a sequence")),
+        modes(modes_ == Py_None ? Py_NewRef(Py_None) : PySequence_Fast(modes_, "modes must be a sequence")),
+        count(PySequence_Fast_GET_SIZE(xs.o)) {
+    if (count < least || count > TWEO_MAX_QUANT_BATCH || PySequence_Fast_GET_SIZE(outs.o) != count)
+      fail(PyExc_ValueError, "need 1..MAX_QUANT_BATCH tensors with one output record each");
+    if (modes.o != Py_None && PySequence_Fast_GET_SIZE(modes.o) < count) fail(PyExc_IndexError, "list index out of range");
+    for (Py_ssize_t i = 0; i < count; ++i) {
+      PyObject* o = PySequence_Fast_GET_ITEM(outs.o, i);
+      Ref fmt(PyObject_GetAttr(o, N.fmt));
+      fill_desc(d[i], PySequence_Fast_GET_ITEM(xs.o, i), o, i32(fmt.o),
+                modes.o == Py_None ? TWEO_SCALE_CURRENT : i32(PySequence_Fast_GET_ITEM(modes.o, i)), true);
+    }
+  }
+};
+
 // quantize_batch(xs, outs, modes or None, ws)
 FN(quantize_batch, 4, {
-  Ref xs(PySequence_Fast(a[0], "xs must be a sequence")), outs(PySequence_Fast(a[1], "outs must be a sequence"));
-  Ref modes(a[2] == Py_None ? Py_NewRef(Py_None) : PySequence_Fast(a[2], "modes must be a sequence"));
-  const Py_ssize_t count = PySequence_Fast_GET_SIZE(xs.o);
-  if (count < 1 || count > TWEO_MAX_QUANT_BATCH || PySequence_Fast_GET_SIZE(outs.o) != count)
-    fail(PyExc_ValueError, "need 1..MAX_QUANT_BATCH tensors with one output record each");
-  if (modes.o != Py_None && PySequence_Fast_GET_SIZE(modes.o) < count) fail(PyExc_IndexError, "list index out of range");
   tweo_quant_desc_t d[TWEO_MAX_QUANT_BATCH];
-  for (Py_ssize_t i = 0; i < count; ++i) {
-    PyObject* o = PySequence_Fast_GET_ITEM(outs.o, i);
-    Ref fmt(PyObject_GetAttr(o, N.fmt));
-    fill_desc(d[i], PySequence_Fast_GET_ITEM(xs.o, i), o, i32(fmt.o),
-              modes.o == Py_None ? TWEO_SCALE_CURRENT : i32(PySequence_Fast_GET_ITEM(modes.o, i)), true);
-  }
+  const Casts casts(a[0], a[1], a[2], d, 1);
   const Ws w = workspace(a[3], true);
   void* st = stream();
-  call("tweo_quantize_per_tensor_batch", [&] { return tweo_quantize_per_tensor_batch(d, (int32_t)count, w.p, w.n, st); });
+  call("tweo_quantize_per_tensor_batch", [&] { return tweo_quantize_per_tensor_batch(d, (int32_t)casts.count, w.p, w.n, st); });
   Py_RETURN_NONE;
 })
 
@@ -408,16 +417,18 @@ int32_t item_i32(PyObject* map, PyObject* key, int32_t otherwise, Held& held) {
   return v == Py_None ? otherwise : i32(v);
 }
 
-// linear_group(problems)
-FN(linear_group, 1, {
-  Ref list(PySequence_Fast(a[0], "problems must be a sequence"));
-  const Py_ssize_t count = PySequence_Fast_GET_SIZE(list.o);
-  constexpr Py_ssize_t most = TWEO_MAX_GROUP;
-  if (count < 1 || count > most) fail(PyExc_ValueError, "need 1..MAX_GROUP problems");
-  tweo_linear_problem_t pr[most] = {};
-  Epi epi[most];
+// The problems of a grouped launch.
+struct Group {
+  tweo_linear_problem_t pr[TWEO_MAX_GROUP] = {};
+  Epi epi[TWEO_MAX_GROUP];
   Held held;
-  for (Py_ssize_t i = 0; i < count; ++i) {
+  Ref list;
+  Py_ssize_t count;
+  explicit Group(PyObject* problems) : list(PySequence_Fast(problems, "problems must be a sequence")), count(PySequence_Fast_GET_SIZE(list.o)) {
+    if (count < 1 || count > TWEO_MAX_GROUP) fail(PyExc_ValueError, "need 1..MAX_GROUP problems");
+    for (Py_ssize_t i = 0; i < count; ++i) fill(i);
+  }
+  void fill(Py_ssize_t i) {
     PyObject* d = PySequence_Fast_GET_ITEM(list.o, i);
     tweo_linear_problem_t& p = pr[i];
     PyObject* fmt = item(d, N.q_fmt, held);
@@ -452,43 +463,91 @@ FN(linear_group, 1, {
     p.out = (uint16_t*)o.p;
     p.ldo = o.ld;
   }
+};
+
+// linear_group(problems)
+FN(linear_group, 1, {
+  const Group g(a[0]);
   void* st = stream();
-  call("tweo_fp8_linear_group", [&] { return tweo_fp8_linear_group(pr, (int32_t)count, st); });
+  call("tweo_fp8_linear_group", [&] { return tweo_fp8_linear_group(g.pr, (int32_t)g.count, st); });
   Py_RETURN_NONE;
+})
+
+// The block outputs of a penalty and its gradients (None: no gradients).
+struct Blocks {
+  Ref blocks, grads;
+  Py_ssize_t L;
+  const uint16_t* pa[TWEO_MAX_BLOCKS];
+  void* pg[TWEO_MAX_BLOCKS];
+  int64_t numel = 0;
+  Blocks(PyObject* blocks_, PyObject* grads_, int32_t gdt)
+      : blocks(PySequence_Fast(blocks_, "blocks must be a sequence")),
+        grads(grads_ == Py_None ? Py_NewRef(Py_None) : PySequence_Fast(grads_, "grads must be a sequence")),
+        L(PySequence_Fast_GET_SIZE(blocks.o)) {
+    if (L < 1) fail(PyExc_IndexError, "list index out of range");
+    if (L > TWEO_MAX_BLOCKS) call("tweo_loss_fwd_bwd", [] { return TWEO_ERR_INVALID_ARG; });
+    const Py_ssize_t ng = grads.o == Py_None ? 0 : PySequence_Fast_GET_SIZE(grads.o);
+    if (ng > L) fail(PyExc_IndexError, "more gradients than block outputs");
+    for (Py_ssize_t i = 0; i < L; ++i) {
+      const at::Tensor& t = tensor(PySequence_Fast_GET_ITEM(blocks.o, i), "block output");
+      if (i == 0) numel = t.numel();
+      if (t.numel() != numel || !t.is_contiguous()) fail(PyExc_ValueError, "block outputs must be contiguous and of equal size");
+      check_kind(t, kBf16, "block output");
+      pa[i] = (const uint16_t*)t.data_ptr();
+      pg[i] = nullptr;   // a missing gradient is refused by the library
+      if (i < ng) pg[i] = dev(PySequence_Fast_GET_ITEM(grads.o, i), gdt == TWEO_BF16 ? kBf16 : kF32, "grad");
+    }
+  }
+  at::Device device() const { return tensor(PySequence_Fast_GET_ITEM(blocks.o, 0), "block output").device(); }
+};
+
+// linear_group_beside(problems, xs, outs, modes or None, blocks or None, grads, tau, eps, grad_coeff, ws)
+//   -> None, or with blocks (loss, per-block losses)
+FN(linear_group_beside, 10, {
+  const Group g(a[0]);
+  tweo_quant_desc_t d[TWEO_MAX_QUANT_BATCH];
+  tweo_beside_t w = {};
+  Casts casts(a[1], a[2], a[3], d, 0);
+  w.casts = d;
+  w.n_casts = (int32_t)casts.count;
+  const Ws ws = workspace(a[9], true);
+  void* st = stream();
+  auto run = [&] {
+    call("tweo_fp8_linear_group_beside", [&] { return tweo_fp8_linear_group_beside(g.pr, (int32_t)g.count, &w, ws.p, ws.n, st); });
+  };
+  if (a[4] == Py_None) {
+    run();
+    Py_RETURN_NONE;
+  }
+  const Blocks b(a[4], a[5], TWEO_BF16);
+  w.a = b.pa;
+  w.grad = b.pg;
+  w.L = (int32_t)b.L;
+  w.n_per_tensor = b.numel;
+  w.tau = flt(a[6]);
+  w.eps = flt(a[7]);
+  w.grad_coeff = flt(a[8]);
+  const at::Tensor out = empty({1}, at::kFloat, b.device()), pb = empty({(int64_t)b.L}, at::kFloat, b.device());
+  w.loss = (float*)out.data_ptr();
+  w.loss_per_block = (float*)pb.data_ptr();
+  run();
+  Ref ro(wrap(out)), rp(wrap(pb));
+  return PyTuple_Pack(2, ro.o, rp.o);
 })
 
 // loss(blocks, tau, eps, p, grad_coeff, grads or None, grad_dtype, ws, per_block) -> (loss, per-block losses or None)
 FN(loss, 9, {
-  Ref blocks(PySequence_Fast(a[0], "blocks must be a sequence"));
-  Ref grads(a[5] == Py_None ? Py_NewRef(Py_None) : PySequence_Fast(a[5], "grads must be a sequence"));
-  const Py_ssize_t L = PySequence_Fast_GET_SIZE(blocks.o);
-  if (L < 1) fail(PyExc_IndexError, "list index out of range");
-  if (L > TWEO_MAX_BLOCKS) call("tweo_loss_fwd_bwd", [] { return TWEO_ERR_INVALID_ARG; });
-  const Py_ssize_t ng = grads.o == Py_None ? 0 : PySequence_Fast_GET_SIZE(grads.o);
-  if (ng > L) fail(PyExc_IndexError, "more gradients than block outputs");
   const int32_t gdt = i32(a[6]);
-  const uint16_t* pa[TWEO_MAX_BLOCKS];
-  void* pg[TWEO_MAX_BLOCKS];
-  int64_t numel = 0;
-  for (Py_ssize_t i = 0; i < L; ++i) {
-    const at::Tensor& t = tensor(PySequence_Fast_GET_ITEM(blocks.o, i), "block output");
-    if (i == 0) numel = t.numel();
-    if (t.numel() != numel || !t.is_contiguous()) fail(PyExc_ValueError, "block outputs must be contiguous and of equal size");
-    check_kind(t, kBf16, "block output");
-    pa[i] = (const uint16_t*)t.data_ptr();
-    pg[i] = nullptr;   // a missing gradient is refused by the library
-    if (i < ng) pg[i] = dev(PySequence_Fast_GET_ITEM(grads.o, i), gdt == TWEO_BF16 ? kBf16 : kF32, "grad");
-  }
+  const Blocks b(a[0], a[5], gdt);
   const float tau = flt(a[1]), eps = flt(a[2]), p = flt(a[3]), c = flt(a[4]);
   const Ws w = workspace(a[7], true);
-  const at::Device device = tensor(PySequence_Fast_GET_ITEM(blocks.o, 0), "block output").device();
-  const at::Tensor out = empty({1}, at::kFloat, device);
+  const at::Tensor out = empty({1}, at::kFloat, b.device());
   at::Tensor pb;
-  if (flag(a[8])) pb = empty({(int64_t)L}, at::kFloat, device);
+  if (flag(a[8])) pb = empty({(int64_t)b.L}, at::kFloat, b.device());
   void* st = stream();
   call("tweo_loss_fwd_bwd", [&] {
-    return tweo_loss_fwd_bwd(pa, (int32_t)L, numel, tau, eps, p, c, (float*)out.data_ptr(), pb.defined() ? (float*)pb.data_ptr() : nullptr,
-                             grads.o != Py_None ? pg : nullptr, gdt, w.p, w.n, st);
+    return tweo_loss_fwd_bwd(b.pa, (int32_t)b.L, b.numel, tau, eps, p, c, (float*)out.data_ptr(),
+                             pb.defined() ? (float*)pb.data_ptr() : nullptr, b.grads.o != Py_None ? b.pg : nullptr, gdt, w.p, w.n, st);
   });
   Ref ro(wrap(out)), rp(pb.defined() ? wrap(pb) : Py_NewRef(Py_None));
   return PyTuple_Pack(2, ro.o, rp.o);
@@ -683,7 +742,7 @@ PyObject* set_error(PyObject*, PyObject* cls) {
 PyMethodDef methods[] = {
     {"set_error", set_error, METH_O, nullptr},
     ENTRY(quantize), ENTRY(quantize_batch), ENTRY(linear_fwd), ENTRY(linear_fwd_act), ENTRY(linear_dgrad), ENTRY(linear_wgrad),
-    ENTRY(linear_bwd), ENTRY(linear_group), ENTRY(loss), ENTRY(w8a8), ENTRY(fp4_weight), ENTRY(block_output), ENTRY(layernorm),
+    ENTRY(linear_bwd), ENTRY(linear_group), ENTRY(linear_group_beside), ENTRY(loss), ENTRY(w8a8), ENTRY(fp4_weight), ENTRY(block_output), ENTRY(layernorm),
     ENTRY(delayed_scaling), ENTRY(absmax), ENTRY(int8_linear), ENTRY(residual_rows),
     {nullptr, nullptr, 0, nullptr}};
 

@@ -21,6 +21,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "stream_ops.cuh"
 
 namespace tweo_detail {
 tweo_status_t launch_amax_prologue(const uint16_t* x, int64_t n, float* amax, uint32_t* sat_count, const float* scale_in,
@@ -85,26 +86,6 @@ __global__ void __launch_bounds__(kThreads) amax_kernel(const uint16_t* x, int64
     if (i < n) m = absmax_bits(m, (uint32_t)x[i]);
   }
   cta_amax_to_global(absmax_fold(m), amax);
-}
-
-// 16 elements: two 16-byte loads -> one 16-byte store.  SAT counts elements whose scaled value
-// exceeds the format's range, AMAX folds |x| into the running maximum m2.  NaN inputs come out of the
-// converter as the code 0x7F (see cvt_fp8x2).
-template <int FMT, bool SAT, bool AMAX>
-__device__ __forceinline__ uint4 cast16(const uint4 a, const uint4 b, float scale, uint32_t& sat, float& m0, float& m1) {
-  const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-  uint32_t c[8];
-  const float fmax = FMT == TWEO_E4M3 ? kE4M3Max : kE5M2Max;
-  const uint64_t ss = pack_f32x2(scale, scale);
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    float lo, hi;
-    unpack_f32x2(mul_f32x2(bf16x2_to_f32x2(w[j]), ss), lo, hi);   // one packed multiply, each lane rounded once
-    if (SAT) sat += (fabsf(lo) > fmax) + (fabsf(hi) > fmax);
-    c[j] = cvt_fp8x2<FMT>(lo, hi);
-    if (AMAX) absmax_f32(m0, m1, w[j]);
-  }
-  return make_uint4(c[0] | (c[1] << 16), c[2] | (c[3] << 16), c[4] | (c[5] << 16), c[6] | (c[7] << 16));
 }
 
 // CURRENT mode reads *amax (finished by the previous kernel) and derives the scale;
@@ -208,16 +189,6 @@ __global__ void __launch_bounds__(kThreads) cast_codes_kernel(const uint16_t* x,
 //   kernel 2 (one launch per FP8 format present): every CTA first reduces the slots of a
 //             tensor to its amax (a few KB from L2), derives the scale and casts its share;
 //             CTA 0 writes amax, scale and scale_inv.
-struct QTensor {
-  const uint16_t* x;
-  uint8_t* q;
-  int64_t n;
-  float* scale;
-  float* scale_inv;
-  float* amax;
-  int32_t fmt;
-  int32_t mode;
-};
 struct QBatch {
   QTensor t[TWEO_MAX_QUANT_BATCH];
   int32_t count;
@@ -613,15 +584,6 @@ int grid_for(int64_t work_items, int per_cta, int ctas_per_sm) {
   return balanced_grid((work_items + per_cta - 1) / per_cta, (int64_t)sm_count() * ctas_per_sm);
 }
 
-tweo_status_t check_desc(const tweo_quant_desc_t& d) {
-  if (d.n < 0 || !d.scale || !d.scale_inv || !d.amax) return TWEO_ERR_INVALID_ARG;
-  if (d.n > 0 && (!d.x || !d.q)) return TWEO_ERR_INVALID_ARG;
-  if (d.fmt != TWEO_E4M3 && d.fmt != TWEO_E5M2) return TWEO_ERR_INVALID_ARG;
-  if (d.mode != TWEO_SCALE_CURRENT && d.mode != TWEO_SCALE_GIVEN) return TWEO_ERR_INVALID_ARG;
-  if (!aligned16(d.x) || !aligned16(d.q)) return TWEO_ERR_ALIGNMENT;
-  return TWEO_OK;
-}
-
 // One tensor as separate kernels: reset, amax (CURRENT only), cast.
 template <int FMT, bool GIVEN, bool SAT>
 cudaError_t launch_cast(const tweo_quant_desc_t& d, cudaStream_t st) {
@@ -658,7 +620,7 @@ tweo_status_t launch_single(const tweo_quant_desc_t& d, cudaStream_t st) {
 // batch kernels; the others are launched one by one.
 tweo_status_t quantize_many(const tweo_quant_desc_t* descs, int count, void* ws, size_t ws_bytes, cudaStream_t st) {
   for (int i = 0; i < count; ++i) {
-    tweo_status_t s = check_desc(descs[i]);
+    tweo_status_t s = check_quant_desc(descs[i]);
     if (s != TWEO_OK) return s;
   }
   if (all_small(descs, count)) return launch_small(descs, count, st);
@@ -687,6 +649,15 @@ tweo_status_t quantize_many(const tweo_quant_desc_t* descs, int count, void* ws,
 }  // namespace
 
 namespace tweo_detail {
+tweo_status_t check_quant_desc(const tweo_quant_desc_t& d) {
+  if (d.n < 0 || !d.scale || !d.scale_inv || !d.amax) return TWEO_ERR_INVALID_ARG;
+  if (d.n > 0 && (!d.x || !d.q)) return TWEO_ERR_INVALID_ARG;
+  if (d.fmt != TWEO_E4M3 && d.fmt != TWEO_E5M2) return TWEO_ERR_INVALID_ARG;
+  if (d.mode != TWEO_SCALE_CURRENT && d.mode != TWEO_SCALE_GIVEN) return TWEO_ERR_INVALID_ARG;
+  if (!aligned16(d.x) || !aligned16(d.q)) return TWEO_ERR_ALIGNMENT;
+  return TWEO_OK;
+}
+
 // The first launches of every one-tensor cast (FP8 here, FP4 in fp4.cu): the reset of amax (and of the saturation
 // counter; with a given scale also its reciprocal), then, for current scaling (scale_in == nullptr), the amax pass.
 tweo_status_t launch_amax_prologue(const uint16_t* x, int64_t n, float* amax, uint32_t* sat_count, const float* scale_in,

@@ -76,6 +76,8 @@ def batch_partition(n):
 class BlockStep:
     """Device buffers + the launch sequence for one configuration (1..4)."""
 
+    beside_ws = None   # workspace of the streaming work beside grouped launches; None: casts and GEMMs on two streams
+
     def __init__(self, cfg_idx: int, M: int | None = None, device="cuda", grad_fmt=tw.E5M2, variant: str = "plain"):
         if variant not in VARIANTS:
             raise ValueError(f"variant must be one of {VARIANTS}")
@@ -94,11 +96,12 @@ class BlockStep:
         self.loss_ws = tw.new_workspace(tw.OP_LOSS, n, self.n_blocks, device=device)
         self.quant_ws = tw.new_workspace(tw.OP_QUANTIZE, device=device)
         self.gemm_ws = tw.new_workspace(tw.OP_LINEAR_WGRAD, device=device)
+        self.beside_ws = tw.new_workspace(tw.OP_BESIDE, n, self.n_blocks, device=device)
         for lb in self.linears:
             lb.qdy.fmt = grad_fmt
         self.loss = None
         self.host = None
-        self.overlap = True   # casts and TWEO pass on a second stream, overlapping the GEMMs
+        self.overlap = True   # casts and TWEO pass beside the GEMMs (in their launches, or on a second stream)
         self.side = None
         self.tau, self.eps, self.p, self.lam = 3.0, 1e-6, 4.0, 0.01
         if extra:
@@ -156,12 +159,15 @@ class BlockStep:
         each tensor with its own per-tensor scale, in one batch call: current scaling in the plain variant; in the
         others delayed scaling, one pass per tensor with the scale from the history, the pass reporting this step's
         amax."""
+        tw.quantize_per_tensor_batch(*self.casts(lbs), ws=self.quant_ws)
+
+    def casts(self, lbs):
+        """The tensors, output records and modes of these casts."""
         if isinstance(lbs, LinearBuffers):
             lbs = [lbs]
         xs = [t for lb in lbs for t in (lb.x, lb.w, lb.dy)]
         qs = [q for lb in lbs for q in (lb.qx, lb.qw, lb.qdy)]
-        modes = None if self.variant == "plain" else [tw.SCALE_GIVEN] * len(xs)
-        tw.quantize_per_tensor_batch(xs, qs, modes, ws=self.quant_ws)
+        return xs, qs, None if self.variant == "plain" else [tw.SCALE_GIVEN] * len(xs)
 
     def batches(self):
         return batch_partition(len(self.linears))
@@ -205,6 +211,9 @@ class BlockStep:
 
     def gemms_grouped(self, lbs):
         """Forward, data-gradient and weight-gradient product of each of the given linears in ONE launch."""
+        tw.fp8_linear_group(self.problems(lbs))
+
+    def problems(self, lbs):
         probs = []
         for i, lb in lbs:
             fwd_epi, dgrad_epi = {}, {}
@@ -218,7 +227,7 @@ class BlockStep:
                            fmt_dy=self.grad_fmt, out=lb.dx, **dgrad_epi),
                       dict(product=tw.PRODUCT_WGRAD, xq=lb.qx.q, dyq=lb.qdy.q, sx_inv=lb.qx.scale_inv, sdy_inv=lb.qdy.scale_inv,
                            fmt_dy=self.grad_fmt, out=lb.dw)]
-        tw.fp8_linear_group(probs)
+        return probs
 
     def gemm_batches(self):
         """The linears in launch order: the cast batches where every product can share a grouped launch, else one by one."""
@@ -253,7 +262,8 @@ class BlockStep:
                                                             grads=self.ga, ws=self.loss_ws)
 
     def step(self):
-        """One pass of the hot path.  The linears of a configuration are independent problems (each has
+        """One pass of the hot path.  Where every linear can be part of a grouped launch: step_beside().  Else on two streams.
+        The linears of a configuration are independent problems (each has
         its own X, W, dY), so the casts run on a second stream and the GEMMs of linear i overlap the casts of
         linear i+1 and the TWEO pass: the casts are HBM-bound, the GEMMs tensor-bound, and they share the SMs.
         Fork / join on the calling stream, so the step can be captured into one CUDA graph."""
@@ -262,6 +272,9 @@ class BlockStep:
                 self.quantize_all([self.linears[i] for i in batch])
             self.all_gemms()
             self.tweo()
+            return
+        if self.beside_ws is not None and all(self.group_ok(lb) for lb in self.linears):
+            self.step_beside()
             return
         main = torch.cuda.current_stream()
         if self.side is None:
@@ -306,6 +319,29 @@ class BlockStep:
         launch_gemms()
         self.update_output_scales()
         main.wait_stream(side)
+
+    def step_beside(self):
+        """The step on the calling stream alone: the first batch's casts, then every batch's grouped launch with the casts of the
+        next batch, or the loss behind the last one, beside its products.  Against two streams, us, call by call / replayed:
+        GPT-2-small block, 8192 tokens, plain 242 / 254 -> 259 / 248, fused 260 / 236 -> 226 / 222; ViT-B/16, fused, 20000 tokens 741 / 722 ->
+        628 / 590; LLaMA-1B, fused, 16384 tokens 2300 / 2350 -> 2325 / 2345, plain, 3001 tokens 464 / 499 -> 460 / 448; config 1,
+        512 tokens 64 / 13 -> 25 / 17 (its host issues one stream's three calls in 19 us, two streams' in 64)."""
+        batches = self.batches()
+        self.quantize_all([self.linears[i] for i in batches[0]])
+        for batch, following in zip(batches, batches[1:] + [None]):
+            problems = self.problems([(i, self.linears[i]) for i in batch])
+            if following is not None:
+                tw.fp8_linear_group_beside(problems, *self.casts([self.linears[i] for i in following]), ws=self.beside_ws)
+            elif self.p == 4.0:
+                self.loss, self.loss_per_block = tw.fp8_linear_group_beside(
+                    problems, blocks=self.a, grads=self.ga, tau=self.tau, eps=self.eps, grad_coeff=self.lam / self.n_blocks,
+                    ws=self.beside_ws)
+            else:
+                tw.fp8_linear_group(problems)
+                self.tweo()
+            if self.variant == "unfused":
+                self.cast_outputs(batch)
+        self.update_output_scales()
 
     @property
     def flops_per_step(self) -> int:

@@ -1,0 +1,143 @@
+"""Streaming work beside a grouped launch: casts and the penalty must equal the calls of their own (codes, scales, maxima and gradients
+bit for bit; the loss, whose binary64 partial sums are added in another order, to one binary32 rounding), the products the launch without it."""
+import dataclasses
+
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def tw():
+    from paper_2511_23225_b200 import binding
+    binding.lib()
+    return binding
+
+
+def _x(n, seed, std=1.0):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    return (torch.randn(n, device="cuda", generator=g) * std).to(torch.bfloat16)
+
+
+def _record(tw, n, fmt, scale=1.0):
+    s = torch.full((3,), scale, device="cuda")
+    return tw.Quantized(torch.zeros(n, dtype=torch.uint8, device="cuda"), s[0:1], s[1:2], s[2:3], None, fmt)
+
+
+def _problems(tw, M, K, N):
+    q = lambda *s: torch.randint(0, 100, s, dtype=torch.uint8, device="cuda", generator=torch.Generator(device="cuda").manual_seed(9))
+    one, x, w, dy = torch.full((1,), 0.01, device="cuda"), q(M, K), q(N, K), q(M, N)
+    out = [torch.zeros(s, dtype=torch.bfloat16, device="cuda") for s in ((M, N), (M, K), (N, K))]
+    return out, [dict(product=tw.PRODUCT_FWD, xq=x, wq=w, sx_inv=one, sw_inv=one, out=out[0]),
+                 dict(product=tw.PRODUCT_DGRAD, dyq=dy, wq=w, sdy_inv=one, sw_inv=one, out=out[1]),
+                 dict(product=tw.PRODUCT_WGRAD, xq=x, dyq=dy, sx_inv=one, sdy_inv=one, out=out[2])]
+
+
+SIZES = [0, 1, 7, 8, 15, 16, 8191, 8192, 8193, 8200, 8208, 100003, 2_000_016]
+
+
+@pytest.mark.parametrize("given", [False, True, None])   # None: in turn
+@pytest.mark.parametrize("first", [0, 5])
+def test_casts_equal_the_batch_call(tw, given, first):
+    sizes = SIZES[first:first + 8]
+    xs = [_x(n, i, 10.0 ** (i % 3)) for i, n in enumerate(sizes)]
+    if len(xs[-1]):
+        xs[-1][0], xs[-1][-1] = float("nan"), float("inf") if given else 3e30
+    fmts = [tw.E4M3 if i % 2 else tw.E5M2 for i in range(8)]
+    modes = [tw.SCALE_GIVEN if (i % 3 == 0 if given is None else given) else tw.SCALE_CURRENT for i in range(8)]
+    want, got = ([_record(tw, len(x), f, 3.7) for x, f in zip(xs, fmts)] for _ in range(2))
+    tw.quantize_per_tensor_batch(xs, want, modes, ws=tw.new_workspace(tw.OP_QUANTIZE))
+    ws = tw.new_workspace(tw.OP_BESIDE)
+    ws.fill_(255)                                  # any contents
+    out, problems = _problems(tw, 300, 272, 528)
+    tw.fp8_linear_group(problems)
+    alone = [t.clone() for t in out]
+    for _ in range(2):                             # the workspace as the launch before left it
+        for g in got:
+            g.q.zero_(), g.amax.fill_(-1)
+        [t.zero_() for t in out]
+        assert tw.fp8_linear_group_beside(problems, xs, got, modes, ws=ws) is None
+        for w, g in zip(want, got):
+            assert torch.equal(w.q, g.q)
+            assert all(torch.equal(a.view(torch.int32), b.view(torch.int32)) for a, b in ((w.scale, g.scale), (w.scale_inv, g.scale_inv), (w.amax, g.amax)))
+        assert all(torch.equal(a, t) for a, t in zip(alone, out))
+    assert tw.read_device_status() == 0
+
+
+@pytest.mark.parametrize("n,L", [(8, 1), (8191, 2), (8193, 3), (300_007, 12), (40, 128), (5_000_000, 2)])
+def test_penalty_equals_the_call_of_its_own(tw, n, L):
+    blocks = [_x(n, i, 1.0 + i) for i in range(L)]
+    grads = [torch.zeros_like(b) for b in blocks]
+    loss, per, want = tw.loss_fwd_bwd(blocks, 3.0, 1e-6, 4.0, 0.01)
+    out, problems = _problems(tw, 130, 144, 160)
+    got, got_per = tw.fp8_linear_group_beside(problems, blocks=blocks, grads=grads, grad_coeff=0.01)
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(want, grads))
+    assert torch.allclose(got, loss, rtol=1.2e-7, atol=0) and torch.allclose(got_per, per, rtol=1.2e-7, atol=0)
+
+
+def test_casts_and_penalty_together_replayed(tw):
+    xs = [_x(3_000_000, 1), _x(70_001, 2)]
+    got, want = ([_record(tw, len(x), tw.E4M3) for x in xs] for _ in range(2))
+    blocks, grads = [_x(1_000_000, 3)], [torch.zeros(1_000_000, dtype=torch.bfloat16, device="cuda")]
+    ws = tw.new_workspace(tw.OP_BESIDE, 1_000_000, 1)
+    out, problems = _problems(tw, 2000, 512, 1024)
+    run = lambda: tw.fp8_linear_group_beside(problems, xs, got, None, blocks, grads, ws=ws)
+    run()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        loss, _ = run()
+    for seed in (4, 5):
+        for x in xs + blocks:
+            x.copy_(_x(len(x), seed))
+        graph.replay()
+        tw.quantize_per_tensor_batch(xs, want)
+        ref = tw.loss_fwd_bwd(blocks)
+        assert all(torch.equal(a.q, b.q) and torch.equal(a.scale, b.scale) for a, b in zip(want, got))
+        assert torch.equal(ref[2][0], grads[0]) and torch.allclose(ref[0], loss, rtol=1.2e-7, atol=0)
+    del graph
+
+
+def test_refused(tw):
+    out, problems = _problems(tw, 300, 272, 272)
+    x = _x(1024, 1)
+    rec = _record(tw, 1024, tw.E4M3)
+    counting = dataclasses.replace(rec, sat_count=torch.zeros(1, dtype=torch.int32, device="cuda"))
+    ws = tw.new_workspace(tw.OP_BESIDE)
+    with pytest.raises(tw.TweoError):
+        tw.fp8_linear_group_beside(problems, [x], [counting], ws=ws)
+    with pytest.raises(tw.TweoError):
+        tw.fp8_linear_group_beside(problems, [x], [rec], ws=ws[:128])
+    with pytest.raises(tw.TweoError):       # no gradient
+        tw.fp8_linear_group_beside(problems, blocks=[x], grads=[], ws=tw.new_workspace(tw.OP_BESIDE, 1024, 1))
+    with pytest.raises(ValueError):
+        tw.fp8_linear_group_beside(problems, [x] * 9, [rec] * 9, ws=ws)
+
+
+@pytest.mark.parametrize("cfg,M,variant", [(2, 300, "plain"), (2, 777, "fused"), (4, 256, "unfused"), (3, 200, "fused")])
+def test_step_equals_the_one_without_overlap(tw, cfg, M, variant):
+    from paper_2511_23225_b200.workload import BlockStep
+    a, b = (BlockStep(cfg, M=M, variant=variant) for _ in range(2))
+    for i, (la, lb) in enumerate(zip(a.linears, b.linears)):
+        for j, k in enumerate(("x", "w", "dy")):
+            v = getattr(la, k)
+            v.copy_(_x(v.numel(), 3 * i + j, (1.0, 0.02, 1e-3)[j]).view(v.shape))
+            getattr(lb, k).copy_(v)
+    for i, t in enumerate(a.a):
+        t.copy_(_x(t.numel(), 100 + i).view(t.shape))
+        b.a[i].copy_(t)
+    b.overlap = False
+    for _ in range(3):
+        a.step(), b.step()
+    torch.cuda.synchronize()
+    assert torch.allclose(a.loss, b.loss, rtol=1.2e-7, atol=0) and all(torch.equal(x, y) for x, y in zip(a.ga, b.ga))
+    for la, lb in zip(a.linears, b.linears):
+        for k in ("y", "dx", "dw", "yq", "dxq"):
+            x, y = getattr(la, k), getattr(lb, k)
+            assert x is None or torch.equal(x, y), k
+        for k in ("qx", "qw", "qdy"):
+            assert torch.equal(getattr(la, k).q, getattr(lb, k).q) and torch.equal(getattr(la, k).scale, getattr(lb, k).scale)
+    if variant != "plain":
+        assert torch.equal(a.hist_e, b.hist_e) and torch.equal(a.scale_g, b.scale_g)
+    assert tw.read_device_status() == 0
