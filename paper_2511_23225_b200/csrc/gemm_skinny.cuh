@@ -36,6 +36,7 @@ struct SkinnyParams {
   int32_t vec_out;         // y and ldy allow 8-byte stores
   int32_t w_early;         // every kernel enqueued before this call has completed, its writes visible, when this kernel starts
   int32_t stages;          // TMA ring depth (<= kSkinnyMaxStages)
+  int32_t prefetch;        // k-blocks of W brought into L2 before the dependency wait
   uint32_t stage_bytes;    // 16 KB of W + Mpad * 128 B of X, rounded up to 1 KB
   uint32_t w_tx_bytes;     // bytes one W load reports to its barrier: the 16 KB it writes, or 8 KB for packed 4-bit
                            // codes (the load counts the bytes it fetched, not the padded groups it writes)
@@ -208,7 +209,7 @@ gemm_fp8_skinny_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_
         load_w(i, kb0 + i);
       }
       if (!p.w_early && mt == 0)   // the token tiles of a slab read the same W
-        for (int kb = kb0; kb < kb1; ++kb) tma_prefetch_2d(&tmap_w, W_MN ? n0 : kb * BK, W_MN ? kb * BK : n0);
+        for (int kb = kb0; kb < min(kb1, kb0 + p.prefetch); ++kb) tma_prefetch_2d(&tmap_w, W_MN ? n0 : kb * BK, W_MN ? kb * BK : n0);
       chain_wait();
       for (int i = 0; i < pre; ++i) load_x(i, kb0 + i);
       int stage = pre == p.stages ? 0 : pre;
