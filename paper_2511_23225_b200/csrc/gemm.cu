@@ -739,7 +739,7 @@ struct SkinnyPlan {
 };
 
 // The most shared memory a launch asks for: the ring, and alignment and barriers.
-constexpr int skinny_smem(bool wide) { return (wide ? 200 : 100) * 1024 + 1024 + 256; }
+constexpr int skinny_smem(bool wide) { return (wide ? 200 : 100) * 1024 + 1024 + kSkinnyTail; }
 
 // Never launched: resident_clusters() asks how many clusters of it fit.  Asking about the few-token kernel itself, with
 // success, left its later launches slower (one token, 4-bit weights [8192x8192]: 15.4 us a pass against 10.9); the cause is not known.
@@ -844,7 +844,7 @@ bool skinny_pays(int64_t M, int64_t N, int64_t Kc) {
 // w_packed4: W holds packed E2M1 codes (two per byte, ldw in BYTES); the ring and the kernel are the same, only the
 // tensor map of W differs (and the operand format in p.idesc, set by the caller).
 // w_early: see gemm_skinny.cuh; only for a call whose own kernel in front waits before it releases.
-template <bool I8, bool W_MN = false>
+template <bool I8, bool W_MN = false, int XITEMS = 0>
 tweo_status_t launch_skinny(SkinnyParams& p, const void* xq, int64_t ldx, const void* wq, int64_t ldw, int64_t M, int64_t N,
                             int64_t K, cudaStream_t st, bool w_early, bool w_packed4 = false) {
   if (M > INT32_MAX || N > INT32_MAX || K > INT32_MAX) return TWEO_ERR_UNSUPPORTED_SHAPE;
@@ -870,13 +870,23 @@ tweo_status_t launch_skinny(SkinnyParams& p, const void* xq, int64_t ldx, const 
   CUtensorMap mw, mx;
   const bool w_ok = w_packed4 ? make_map_packed4(&mw, wq, K, N, ldw, BM)
                               : (W_MN ? make_map(&mw, wq, N, K, ldw, BK) : make_map(&mw, wq, K, N, ldw, BM));
-  if (!w_ok || !make_map(&mx, xq, K, M, ldx, p.Mpad)) {
+  if (XITEMS > 0) mx = mw;   // not read
+  if (!w_ok || (XITEMS == 0 && !make_map(&mx, xq, K, M, ldx, p.Mpad))) {
     cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
     return TWEO_ERR_CUDA;
   }
-  const size_t smem = (size_t)p.stages * p.stage_bytes + 1024 + 256;
+  size_t smem = (size_t)p.stages * p.stage_bytes + 1024 + 256;
+  if (XITEMS > 0) {   // W alone in the ring; behind it the slice's activations
+    const int blocks = (p.k_blocks + p.slices - 1) / p.slices;
+    const uint32_t x_bytes = (uint32_t)blocks * XITEMS * 16 * 128;
+    p.stage_bytes = BM * BK;
+    p.stages = std::min(kSkinnyMaxStages, (int)((100 * 1024 - x_bytes) / p.stage_bytes));
+    smem = (size_t)p.stages * p.stage_bytes + kSkinnyTail + x_bytes + 1024;
+  }
   const bool wide = p.Mpad > 128;
-  auto kern = wide ? gemm_fp8_skinny_kernel<I8, W_MN, true> : gemm_fp8_skinny_kernel<I8, W_MN, false>;
+  auto kern = gemm_fp8_skinny_kernel<I8, W_MN, false, XITEMS>;
+  if constexpr (XITEMS == 0)
+    if (wide) kern = gemm_fp8_skinny_kernel<I8, W_MN, true>;
   static std::atomic<uint64_t> attr_done[2];  // per device
   int attr_dev = 0;
   if (device_once_pending(attr_done[wide], &attr_dev)) {
@@ -902,6 +912,38 @@ tweo_status_t run_skinny(const uint8_t* xq, int64_t ldx, int fmt_x, const uint8_
   p.sx_is_scale = sx_is_scale ? 1 : 0;
   return w_mn ? launch_skinny<false, true>(p, xq, ldx, wq, ldw, M, N, K, st, w_early)
               : launch_skinny<false>(p, xq, ldx, wq, ldw, M, N, K, st, w_early);
+}
+
+// Whether the few-token kernel casts M tokens' bf16 activations itself.  Up to 48 tokens, with slices of at most 26 k-blocks and 64 KB of codes:
+// the ring keeps two stages at least, four in most cases.  Rotating weights, us a pass called one by one, a cast kernel in front / inside:
+//   1 token    [4096x4096] 7.8 / 6.3   [4096x11008] 11.9 / 10.0   [8192x8192] 15.8 / 13.7   29 k-blocks [11008x11008] 23.0 / 24.2
+//   16 tokens  [4096x4096] 8.5 / 6.9   [4096x11008] 12.7 / 10.7   [8192x8192] 16.7 / 14.6   [1024x4096] 6.2 / 5.1
+//   32 tokens  [4096x4096] 9.4 / 7.8   [4096x11008] 13.1 / 11.5   [8192x8192] 17.7 / 16.7
+//   48 tokens  [4096x4096] 10.2 / 8.7  [2048x11008] 8.4 / 8.0     66 KB [4096x11008] 13.6 / 13.4 (replayed 12.9 / 13.0)
+//   64 tokens  [4096x4096] 10.9 / 10.1 [2048x11008] 9.2 / 9.1 (replayed 8.5 / 8.9)
+bool skinny_casts(int64_t M, int64_t N, int64_t K) {
+  if (M > 48 || N > INT32_MAX || K > INT32_MAX) return false;
+  const int k_blocks = (int)((K + BK - 1) / BK);
+  const SkinnyPlan pl = plan_skinny(M, N, k_blocks);
+  const int blocks = (k_blocks + pl.slices - 1) / pl.slices;
+  return blocks <= 26 && blocks * pl.tokens * BK <= 64 * 1024;
+}
+
+// bf16 activations with the scale *sx, cast in the kernel.
+tweo_status_t run_skinny_cast(const uint16_t* x, const float* sx, const uint8_t* wq, int64_t ldw, const float* sw_inv, uint16_t* y,
+                              int64_t ldy, int64_t M, int64_t N, int64_t K, cudaStream_t st) {
+  SkinnyParams p{};
+  p.y = y;
+  p.ldy = ldy;
+  p.idesc = make_idesc(TWEO_E4M3, TWEO_E4M3, false, false, 0, BM);
+  p.sx_inv = sx;
+  p.sw_inv = sw_inv;
+  p.sx_is_scale = 1;
+  p.x = x;
+  p.K = (int32_t)K;
+  if (M <= 16) return launch_skinny<false, false, 1>(p, x, K, wq, ldw, M, N, K, st, false);
+  if (M <= 32) return launch_skinny<false, false, 2>(p, x, K, wq, ldw, M, N, K, st, false);
+  return launch_skinny<false, false, 3>(p, x, K, wq, ldw, M, N, K, st, false);
 }
 
 // The same with W as packed E2M1 codes: half the bytes of the stream that bounds the call.
@@ -1223,6 +1265,14 @@ unsigned int* device_status_word() {
     cached[dev] = static_cast<unsigned int*>(ptr);
   }
   return cached[dev];
+}
+
+// The static W8A8 linear on bf16 activations [M, K], where the product's kernel casts them itself (false: it does not).
+bool gemm_fwd_casting(const uint16_t* x, const float* sx, const uint8_t* wq, int64_t ldw, const float* sw_inv, uint16_t* y, int64_t ldy,
+                      int64_t M, int64_t N, int64_t K, cudaStream_t st, tweo_status_t* status) {
+  if (!skinny_casts(M, N, K)) return false;
+  *status = run_skinny_cast(x, sx, wq, ldw, sw_inv, y, ldy, M, N, K, st);
+  return true;
 }
 
 // Used by the static W8A8 entry point: forward product on already-cast activations.

@@ -9,6 +9,8 @@ tweo_status_t gemm_fwd_codes(const uint8_t* xq, int64_t ldx, int fmt_x, const ui
                              const float* sx_inv, const float* sw_inv, uint16_t* y, int64_t ldy, int64_t M,
                              int64_t N, int64_t K, const tweo_epilogue_t* epi, void* ws, size_t ws_bytes,
                              cudaStream_t st, bool sx_is_scale, bool inference, bool w_early);
+bool gemm_fwd_casting(const uint16_t* x, const float* sx, const uint8_t* wq, int64_t ldw, const float* sw_inv, uint16_t* y, int64_t ldy,
+                      int64_t M, int64_t N, int64_t K, cudaStream_t st, tweo_status_t* status);
 }
 
 extern "C" tweo_status_t tweo_w8a8_static_gemm(const void* x, int32_t x_dtype, int64_t ldx, const float* sx,
@@ -31,8 +33,10 @@ extern "C" tweo_status_t tweo_w8a8_static_gemm(const void* x, int32_t x_dtype, i
       // the cast runs over a dense tensor; a padded bf16 input would need a strided cast
       return TWEO_ERR_UNSUPPORTED_SHAPE;
     }
+    tweo_status_t s = TWEO_OK;   // few tokens: one kernel
+    if (gemm_fwd_casting(reinterpret_cast<const uint16_t*>(x), sx, wq, ldw, sw_inv, y, ldy, M, N, K, st, &s)) return s;
     uint8_t* codes = reinterpret_cast<uint8_t*>(ws) + 256;
-    tweo_status_t s = launch_cast_codes(reinterpret_cast<const uint16_t*>(x), M * K, sx, codes, st);
+    s = launch_cast_codes(reinterpret_cast<const uint16_t*>(x), M * K, sx, codes, st);
     if (s != TWEO_OK) return s;
     xq = codes;
     ldxq = K;
