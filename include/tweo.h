@@ -350,7 +350,7 @@ TWEO_API tweo_status_t tweo_fp8_linear_group_beside(const tweo_linear_problem_t*
  *   p = 4 (the paper's setting) runs a fast path; other p > 1 a generic one.
  *   Needs a workspace (TWEO_OP_LOSS, any contents); the sum is reduced in a fixed order,
  *   so results are bit-reproducible run to run.  Two kernels: the streaming pass and a
- *   one-CTA kernel that adds its partial sums.
+ *   one-CTA kernel that adds its partial sums; one kernel for a single tensor of up to 2^17 elements.
  */
 TWEO_API tweo_status_t tweo_loss_fwd_bwd(const uint16_t* const* a, int32_t L, int64_t n_per_tensor, float tau,
                                 float eps, float p, float grad_coeff, float* loss,

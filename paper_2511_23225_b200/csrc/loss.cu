@@ -6,10 +6,11 @@
 // sum |a|^p per vector in binary32 and across vectors in binary64, the CTA reduces with
 // shuffles and writes ONE partial sum to the scratch memory.  A second, one-CTA kernel
 // (launched in the same chain, so its launch and set-up overlap the first) adds the
-// partials in a fixed order and writes the losses: the result does not depend on
+// partials in a fixed order and writes the losses (a small tensor takes one launch of a cluster, see below): the result does not depend on
 // scheduling, and the streaming CTAs end without a fence, a ticket or a wait -- a
 // last-CTA-reduces scheme cost 3.4 us at the end of every call (fence, atomic, a dependent
 // round trip to L2 behind the slowest CTA), a third of the pass over a [8192 x 768] tensor.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
 #include <mutex>
@@ -105,6 +106,29 @@ __device__ __forceinline__ void process_vec(const uint4 v, float k, float p, uin
   }
 }
 
+// The last n % 8 elements, by the first threads of one CTA.
+template <bool FAST, bool GRAD, bool GRAD_F32>
+__device__ __forceinline__ double ragged_tail(const uint16_t* a, void* gptr, const LossArgs& args) {
+  const int64_t i = (args.n >> 3 << 3) + threadIdx.x;
+  if (threadIdx.x >= 8 || i >= args.n) return 0.0;
+  float af = __uint_as_float((uint32_t)a[i] << 16);
+  float t, g;
+  if (FAST) {
+    float s = af * af;
+    t = s * s;
+    g = __fmul_rn(args.k_grad, s * af);
+  } else {
+    double m = fabs((double)af);
+    t = (float)pow(m, (double)args.p);
+    g = af == 0.0f ? 0.0f : (float)((double)args.k_grad * copysign(pow(m, (double)args.p - 1.0), (double)af));
+  }
+  if (GRAD) {
+    if (GRAD_F32) reinterpret_cast<float*>(gptr)[i] = g;
+    else reinterpret_cast<uint16_t*>(gptr)[i] = (uint16_t)f32_to_bf16_bits(g);
+  }
+  return (double)t;
+}
+
 // The p = 4 variants are held to the registers that keep kLossCtasPerSm CTAs per SM resident: the grid is sized
 // for exactly that many, one wave.
 template <bool FAST, bool GRAD, bool GRAD_F32>
@@ -154,28 +178,7 @@ tweo_loss_kernel(const __grid_constant__ LossPtrs ptrs, const LossArgs args) {
       acc += (double)lo + (double)hi;
     }
   }
-  // ragged tail (n % 8 elements), handled by the first threads of CTA 0 of this tensor
-  if (blockIdx.x == 0) {
-    int64_t i = (nvec << 3) + threadIdx.x;
-    if (threadIdx.x < 8 && i < args.n) {
-      float af = __uint_as_float((uint32_t)a[i] << 16);
-      float t, g;
-      if (FAST) {
-        float s = af * af;
-        t = s * s;
-        g = __fmul_rn(args.k_grad, s * af);
-      } else {
-        double m = fabs((double)af);
-        t = (float)pow(m, (double)args.p);
-        g = af == 0.0f ? 0.0f : (float)((double)args.k_grad * copysign(pow(m, (double)args.p - 1.0), (double)af));
-      }
-      acc += (double)t;
-      if (GRAD) {
-        if (GRAD_F32) reinterpret_cast<float*>(gptr)[i] = g;
-        else reinterpret_cast<uint16_t*>(gptr)[i] = (uint16_t)f32_to_bf16_bits(g);
-      }
-    }
-  }
+  if (blockIdx.x == 0) acc += ragged_tail<FAST, GRAD, GRAD_F32>(a, gptr, args);
 
   // CTA reduction in a fixed order; one partial per CTA
   __shared__ double warp_part[kLossThreads / 32];
@@ -225,6 +228,86 @@ __global__ void __launch_bounds__(kLossThreads) tweo_loss_finish_kernel(const Lo
   }
 }
 
+// One small block output in one launch: a cluster of eight CTAs, whose sums meet in the first one's shared memory.  At these sizes
+// the second kernel (its launch, and one more kernel boundary) costs more than the bytes.
+constexpr int kSmallCluster = 8;
+constexpr int kSmallThreads = 512;
+
+template <bool FAST, bool GRAD, bool GRAD_F32>
+__global__ void __launch_bounds__(kSmallThreads) tweo_loss_small_kernel(const uint16_t* a, void* gptr, const LossArgs args) {
+  namespace cg = cooperative_groups;
+  __shared__ double warp_part[kSmallThreads / 32];
+  __shared__ double parts[kSmallCluster];   // used in the first CTA
+  cg::cluster_group cluster = cg::this_cluster();
+  cluster.barrier_arrive();   // this CTA has started: its peers may write into its parts[]
+  chain_wait();
+  chain_release();
+  const int rank = blockIdx.x;
+  const int64_t nvec = args.n >> 3;
+  const uint4* av = reinterpret_cast<const uint4*>(a);
+  constexpr int stride = kSmallCluster * kSmallThreads;
+  double acc = 0.0;
+  for (int64_t base = rank * kSmallThreads + threadIdx.x; base < nvec; base += stride * kLossUnroll) {
+    uint4 v[kLossUnroll];
+#pragma unroll
+    for (int u = 0; u < kLossUnroll; ++u) {
+      const int64_t i = base + (int64_t)u * stride;
+      v[u] = i < nvec ? __ldg(av + i) : make_uint4(0, 0, 0, 0);
+    }
+    uint64_t acc2 = 0ull;
+#pragma unroll
+    for (int u = 0; u < kLossUnroll; ++u) {
+      const int64_t i = base + (int64_t)u * stride;
+      if (i < nvec) {
+        float vsum = 0.0f;
+        uint4 gb;
+        float4 gf[2];
+        process_vec<FAST, GRAD, GRAD_F32>(v[u], args.k_grad, args.p, acc2, vsum, &gb, gf);
+        if (!FAST) acc += (double)vsum;
+        if (GRAD && GRAD_F32) {
+          reinterpret_cast<float4*>(gptr)[2 * i] = gf[0];
+          reinterpret_cast<float4*>(gptr)[2 * i + 1] = gf[1];
+        } else if (GRAD) {
+          reinterpret_cast<uint4*>(gptr)[i] = gb;
+        }
+      }
+    }
+    if (FAST) {
+      float lo, hi;
+      unpack_f32x2(acc2, lo, hi);
+      acc += (double)lo + (double)hi;
+    }
+  }
+  if (rank == 0) acc += ragged_tail<FAST, GRAD, GRAD_F32>(a, gptr, args);
+  acc = warp_sum(acc);
+  if ((threadIdx.x & 31) == 0) warp_part[threadIdx.x >> 5] = acc;
+  cluster.barrier_wait();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double s = 0.0;
+#pragma unroll
+    for (int w = 0; w < kSmallThreads / 32; ++w) s += warp_part[w];
+    *cluster.map_shared_rank(&parts[rank], 0) = s;
+  }
+  cluster.sync();
+  if (rank == 0 && threadIdx.x == 0) {
+    double s = 0.0;
+#pragma unroll
+    for (int c = 0; c < kSmallCluster; ++c) s += parts[c];
+    const float loss = (float)(s * args.inv_norm);
+    if (args.loss_per_block) *args.loss_per_block = loss;
+    *args.loss = loss;
+  }
+}
+
+template <bool FAST, bool GRAD, bool GRAD_F32>
+tweo_status_t launch_small(cudaStream_t st, const LossPtrs& ptrs, const LossArgs& args) {
+  TWEO_CUDA_TRY(launch_chain(tweo_loss_small_kernel<FAST, GRAD, GRAD_F32>, dim3(kSmallCluster), dim3(kSmallThreads), 0, st, kSmallCluster,
+                             ptrs.a[0], ptrs.g[0], args));
+  count_launch();
+  return check_launch("tweo_loss_small_kernel");
+}
+
 template <bool FAST, bool GRAD, bool GRAD_F32>
 void launch(dim3 grid, cudaStream_t st, const LossPtrs& ptrs, const LossArgs& args) {
   launch_chain(tweo_loss_kernel<FAST, GRAD, GRAD_F32>, grid, dim3(kLossThreads), 0, st, 0, ptrs, args);
@@ -254,6 +337,14 @@ tweo_status_t launch_loss(const uint16_t* const* a, int32_t L, int64_t n_per_ten
   const bool fast = (p == 4.0f);
   const bool has_grad = grad != nullptr;
   const bool f32 = grad_dtype == TWEO_F32;
+  // One tensor of up to 2^17 elements (any p but 4: 2^16).  us replayed, and called one by one, two kernels / one: 2^10 2.5 / 1.7, 12.4 / 6.5;
+  // 2^16 3.0 / 2.2, 11.2 / 4.5; 2^17 3.0 / 2.5, 6.9 / 4.5; 2^18 3.0 / 3.4, 6.7 / 4.3; p = 3: 2^14 30.7 / 12.1, 2^16 30.8 / 22.1, 2^17 30.8 / 41.6.
+  if (L == 1 && n_per_tensor <= (fast ? 1 << 17 : 1 << 16)) {
+    if (fast) return !has_grad ? launch_small<true, false, false>(st, ptrs, args)
+                               : (f32 ? launch_small<true, true, true>(st, ptrs, args) : launch_small<true, true, false>(st, ptrs, args));
+    return !has_grad ? launch_small<false, false, false>(st, ptrs, args)
+                     : (f32 ? launch_small<false, true, true>(st, ptrs, args) : launch_small<false, true, false>(st, ptrs, args));
+  }
   if (fast) {
     if (!has_grad) launch<true, false, false>(grid, st, ptrs, args);
     else if (f32) launch<true, true, true>(grid, st, ptrs, args);

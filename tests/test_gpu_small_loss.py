@@ -1,0 +1,39 @@
+"""The penalty of one tensor at the sizes where its one launch begins, ends and has remainders, against the oracle (loss and binary32 gradient
+to 1e-5, as everywhere), with and without gradients, p = 4 and the general power."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import tweo_oracle as orc
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def tw():
+    from paper_2511_23225_b200 import binding
+    binding.lib()
+    return binding
+
+
+@pytest.mark.parametrize("p", [4.0, 2.5])
+@pytest.mark.parametrize("n", [1, 7, 8, 9, 4096, 32767, 32769, 65536, 65537, 131071, 131072, 131073])
+def test_one_tensor(tw, n, p):
+    x = torch.randn(n, generator=torch.Generator().manual_seed(n)).mul_(2).to(torch.bfloat16)
+    if n > 8:
+        x[3], x[-1] = 0.0, 50.0
+    bits = x.view(torch.int16).numpy().view(np.uint16)
+    tau, eps, c = float(np.float32(3.0)), float(np.float32(1e-6)), float(np.float32(0.01))
+    loss, grad = orc.tweo_loss_block(bits, tau, eps, p), orc.tweo_grad_block(bits, tau, eps, p, c)
+    xd = x.cuda()
+    ws = tw.new_workspace(tw.OP_LOSS, n, 1).fill_(255)
+    for dt in (tw.F32, tw.BF16, None):
+        got, per, g = tw.loss_fwd_bwd([xd], 3.0, 1e-6, p, 0.01, want_grad=dt is not None, grad_dtype=dt or tw.BF16, ws=ws)
+        assert abs(got.item() - loss) <= 1e-5 * loss and per.item() == got.item()
+        if dt == tw.F32:
+            assert np.abs(g[0].cpu().numpy().astype(np.float64) - grad).max() <= 1e-5 * np.abs(grad).max()
+            f32 = g[0]
+        elif dt == tw.BF16:
+            assert torch.equal(g[0], f32.to(torch.bfloat16))
+    again = tw.loss_fwd_bwd([xd], 3.0, 1e-6, p, 0.01, ws=ws)[0]
+    assert torch.equal(again, got)
