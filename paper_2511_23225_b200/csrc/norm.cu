@@ -6,6 +6,9 @@
 // the warp is contiguous), so mean, centred variance and output take one read of x.  gamma and
 // beta are staged once per CTA in shared memory.  The maximum of |y| travels in registers and
 // ends in one atomicMax per warp (the caller's amax is zeroed on the stream first).
+// What bounds it where rows are few per warp: gamma and beta from shared memory (96 of 330 cycles of a row of 768 when two lanes met in every
+// bank) and the latencies of its two reductions.  [12608x768] 12.0 -> 11.2 us with the planes below, [16384x2048] 27.1 -> 25.0; the first row
+// under way before gamma and beta: [1000x768] 4.5 -> 4.2.  Packed arithmetic alone gave nothing, four CTAs per SM (64 registers) 12.1, two 13.7.
 #include <cuda_runtime.h>
 
 #include "common.cuh"
@@ -40,27 +43,22 @@ constexpr int kNormThreads = 256;
 // QFMT: -1 no FP8 output, else the tweo_fp8_t of the codes
 template <int VPL, int QFMT>
 __global__ void __launch_bounds__(kNormThreads) norm_rows_kernel(const NormArgs a) {
-  extern __shared__ __align__(16) float gb[];  // gamma [d], beta [d]
+  // gamma [d], beta [d]; of every eight elements the first four in one plane, the last four in another: a lane's eight side by side would
+  // have two lanes of a 16-byte access meet in every bank
+  extern __shared__ __align__(16) float gb[];
   chain_release();
   chain_wait();
-  float* s_gamma = gb;
-  float* s_beta = gb + a.d;
-  for (int j = threadIdx.x; j < a.d; j += kNormThreads) {
-    s_gamma[j] = __ldg(a.gamma + j);
-    s_beta[j] = a.beta ? __ldg(a.beta + j) : 0.0f;
-  }
-  __syncthreads();
-
   const int lane = threadIdx.x & 31;
   const int warps_per_cta = kNormThreads / 32;
   const int64_t warp_global = (int64_t)blockIdx.x * warps_per_cta + (threadIdx.x >> 5);
   const int64_t warp_stride = (int64_t)gridDim.x * warps_per_cta;
   const int nvec = a.d >> 3;
   const float inv_d = 1.0f / (float)a.d;
-  const float qs = QFMT >= 0 ? __ldg(a.q_scale) : 0.0f;
-  float run_amax = 0.0f;
+  const uint64_t qs2 = splat_f32x2(QFMT >= 0 ? __ldg(a.q_scale) : 0.0f);
+  float run_m0 = 0.0f, run_m1 = 0.0f;
 
-  // the next row's loads are issued before this row's reductions, so a warp always has a row in flight
+  // the next row's loads are issued before this row's reductions, so a warp always has a row in flight; the first row's before gamma and
+  // beta are fetched
   constexpr bool PREFETCH = VPL <= 8;
   uint4 nxt[PREFETCH ? VPL : 1];
   if (PREFETCH && warp_global < a.rows) {
@@ -71,6 +69,16 @@ __global__ void __launch_bounds__(kNormThreads) norm_rows_kernel(const NormArgs 
       nxt[i] = idx < nvec ? __ldcs(xr + idx) : make_uint4(0u, 0u, 0u, 0u);
     }
   }
+  float* s_gamma = gb;
+  float* s_beta = gb + a.d;
+  const int half = a.d >> 1;   // floats of a plane
+  for (int j = threadIdx.x; j < a.d; j += kNormThreads) {
+    const int at = (j & 4 ? half : 0) + (j >> 3) * 4 + (j & 3);
+    s_gamma[at] = __ldg(a.gamma + j);
+    s_beta[at] = a.beta ? __ldg(a.beta + j) : 0.0f;
+  }
+  __syncthreads();
+
   for (int64_t row = warp_global; row < a.rows; row += warp_stride) {
     uint4 v[VPL];
     if (PREFETCH) {
@@ -100,10 +108,17 @@ __global__ void __launch_bounds__(kNormThreads) norm_rows_kernel(const NormArgs 
       for (int i = 0; i < VPL; ++i) {
         const uint32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
 #pragma unroll
-        for (int k = 0; k < 4; ++k) s += bf16lo_to_f32(w[k]) + bf16hi_to_f32(w[k]);
+        for (int k = 0; k < 4; k += 2) {   // two sums lo + hi in one instruction, added in the order of the words
+          float s0, s1;
+          unpack_f32x2(add_f32x2(pack_f32x2(bf16lo_to_f32(w[k]), bf16lo_to_f32(w[k + 1])),
+                                 pack_f32x2(bf16hi_to_f32(w[k]), bf16hi_to_f32(w[k + 1]))), s0, s1);
+          s += s0;
+          s += s1;
+        }
       }
       mu = warp_sum(s) * inv_d;
     }
+    const uint64_t nmu2 = splat_f32x2(-mu);
     float ss = 0.0f;
 #pragma unroll
     for (int i = 0; i < VPL; ++i) {
@@ -111,7 +126,8 @@ __global__ void __launch_bounds__(kNormThreads) norm_rows_kernel(const NormArgs 
         const uint32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          const float c0 = bf16lo_to_f32(w[k]) - mu, c1 = bf16hi_to_f32(w[k]) - mu;
+          float c0, c1;
+          unpack_f32x2(add_f32x2(bf16x2_to_f32x2(w[k]), nmu2), c0, c1);
           ss = fmaf(c0, c0, ss);
           ss = fmaf(c1, c1, ss);
         }
@@ -119,6 +135,7 @@ __global__ void __launch_bounds__(kNormThreads) norm_rows_kernel(const NormArgs 
     }
     const float var = warp_sum(ss) * inv_d;
     const float rs = 1.0f / sqrtf(var + a.eps);
+    const uint64_t rs2 = splat_f32x2(rs);
     if (lane == 0) {
       if (a.mean) a.mean[row] = mu;
       if (a.rstd) a.rstd[row] = rs;
@@ -128,44 +145,33 @@ __global__ void __launch_bounds__(kNormThreads) norm_rows_kernel(const NormArgs 
       const int idx = lane + 32 * i;
       if (idx < nvec) {
         const uint32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
-        const float4 g0 = *reinterpret_cast<const float4*>(s_gamma + 8 * idx);
-        const float4 g1 = *reinterpret_cast<const float4*>(s_gamma + 8 * idx + 4);
-        const float4 b0 = *reinterpret_cast<const float4*>(s_beta + 8 * idx);
-        const float4 b1 = *reinterpret_cast<const float4*>(s_beta + 8 * idx + 4);
-        const float g[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
-        const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+        auto pairs = [&](const float* s) { return *reinterpret_cast<const ulonglong2*>(s + 4 * idx); };   // two pairs of binary32
+        const ulonglong2 g0 = pairs(s_gamma), g1 = pairs(s_gamma + half), b0 = pairs(s_beta), b1 = pairs(s_beta + half);
+        const uint64_t g[4] = {g0.x, g0.y, g1.x, g1.y}, b[4] = {b0.x, b0.y, b1.x, b1.y};
         uint32_t o[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const float y0 = fmaf((bf16lo_to_f32(w[k]) - mu) * rs, g[2 * k], b[2 * k]);
-          const float y1 = fmaf((bf16hi_to_f32(w[k]) - mu) * rs, g[2 * k + 1], b[2 * k + 1]);
-          o[k] = f32x2_to_bf16x2(y0, y1);
-        }
+        for (int k = 0; k < 4; ++k)
+          o[k] = f32x2_pair_to_bf16x2(fma_f32x2(mul_f32x2(add_f32x2(bf16x2_to_f32x2(w[k]), nmu2), rs2), g[k], b[k]));
         if (a.y) __stcs(reinterpret_cast<uint4*>(a.y + row * a.ldy) + idx, make_uint4(o[0], o[1], o[2], o[3]));
-        if (QFMT >= 0 || a.amax) {
-          float f[8];
+        if (a.amax) {
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            f[2 * k] = bf16lo_to_f32(o[k]);
-            f[2 * k + 1] = bf16hi_to_f32(o[k]);
-          }
-          if (a.amax) {
+          for (int k = 0; k < 4; ++k) absmax_f32(run_m0, run_m1, o[k]);
+        }
+        if (QFMT >= 0) {
+          uint32_t c[4];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) run_amax = fmaxf(run_amax, fabsf(f[k]));
+          for (int k = 0; k < 4; ++k) {  // NaN -> 0x7F inside cvt_fp8x2
+            float f0, f1;
+            unpack_f32x2(mul_f32x2(bf16x2_to_f32x2(o[k]), qs2), f0, f1);
+            c[k] = cvt_fp8x2<QFMT >= 0 ? QFMT : 0>(f0, f1);
           }
-          if (QFMT >= 0) {
-            uint32_t c[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k)  // NaN -> 0x7F inside cvt_fp8x2
-              c[k] = cvt_fp8x2<QFMT >= 0 ? QFMT : 0>(__fmul_rn(f[2 * k], qs), __fmul_rn(f[2 * k + 1], qs));
-            __stcs(reinterpret_cast<uint2*>(a.q + row * a.ldq) + idx, make_uint2(c[0] | (c[1] << 16), c[2] | (c[3] << 16)));
-          }
+          __stcs(reinterpret_cast<uint2*>(a.q + row * a.ldq) + idx, make_uint2(c[0] | (c[1] << 16), c[2] | (c[3] << 16)));
         }
       }
     }
   }
   if (a.amax) {
-    run_amax = warp_max(run_amax);
+    const float run_amax = warp_max(fmaxf(run_m0, run_m1));
     if (lane == 0 && run_amax > 0.0f) atomicMax(reinterpret_cast<unsigned int*>(a.amax), __float_as_uint(run_amax));
   }
 }
