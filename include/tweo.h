@@ -137,9 +137,9 @@ TWEO_API tweo_status_t tweo_quantize_per_tensor(const uint16_t* x, int64_t n, in
  * (own amax, own scale, own format and mode; results bit-identical).
  *   descs: HOST array of `count` descriptors (read during the call, not kept).
  *   ws: tweo_workspace_bytes(TWEO_OP_QUANTIZE) bytes, any contents.  A batch of small tensors
- *     (up to 2^18 to 2^20 elements, by their number, modes and formats), none with a sat_count,
+ *     (up to 2^17 to 2^20 elements, by their number, modes and formats), none with a sat_count,
  *     is one launch.  In other batches the tensors with CURRENT scaling and no sat_count share
- *     one amax kernel and one cast kernel per FP8 format; two or more GIVEN-scale tensors
+ *     one amax kernel and one cast kernel; two or more GIVEN-scale tensors
  *     without a sat_count share one reset kernel and one cast kernel per FP8 format; those with
  *     a sat_count (and those with CURRENT scaling when ws is NULL or too small) are launched one
  *     by one as tweo_quantize_per_tensor does.

@@ -7,12 +7,9 @@
 // maximum of the sign-stripped bf16 bit patterns (exact, order-independent; NaN
 // patterns are skipped), reduced by shuffles and one atomicMax per CTA.
 //
-// Two launch forms.  Without a workspace: a reset kernel, the amax kernel and the cast kernel.
-// With a workspace: two kernels for up to TWEO_MAX_QUANT_BATCH tensors at once -- one reduces
-// every tensor's amax into the workspace, the other casts every tensor with the scale derived
-// from it, and its last CTA writes the scalars out and leaves the workspace zeroed for the
-// next call (so no reset kernel).  A linear layer's three casts (X, W, dY) then cost two
-// launches instead of nine, which matters because the tensors of a transformer block are
+// Launch forms.  One tensor without a workspace: a reset kernel, the amax kernel and the cast kernel.  Up to TWEO_MAX_QUANT_BATCH tensors
+// at once with a workspace: two kernels, one for the maxima and one for the casts (see the batched form below).  Small tensors: one launch.
+// A linear layer's three casts (X, W, dY) are one or two launches, which matters because the tensors of a transformer block are
 // small enough for launch cost to rival streaming time.
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
@@ -183,126 +180,180 @@ __global__ void __launch_bounds__(kThreads) cast_codes_kernel(const uint16_t* x,
 }
 
 // ---------------------------------------------------------------------------------------
-// Batched form with a workspace (CURRENT scaling): no reset kernel and no atomics.
-//   kernel 1: every CTA writes the maximum of its share of each tensor to its own workspace
-//             slot (so the workspace needs no particular contents on entry);
-//   kernel 2 (one launch per FP8 format present): every CTA first reduces the slots of a
-//             tensor to its amax (a few KB from L2), derives the scale and casts its share;
-//             CTA 0 writes amax, scale and scale_inv.
+// Batched form, up to TWEO_MAX_QUANT_BATCH tensors in one sequence of chunks: a CTA takes every gridDim.x-th chunk of 8192 elements,
+// whatever tensor it is of, with the loads of the next one under way.  Tensor after tensor, each with its own reduction, first loads and
+// last ones, and (CURRENT) a launch per format, took for X, W and dY of a linear [8192x768] -> 768 18.5 us, for two of a GPT-2-small
+// block (40 M elements) 46.7, for its others (68 M) 67.9; now 11.8, 30.7 and 51.9 (rotating buffers; 6.5 TB/s at 5 bytes an element).
+// CURRENT scaling with a workspace, no reset kernel and no atomics in global memory:
+//   kernel 1: every CTA writes its maximum of each tensor to its own workspace slot (so the workspace needs no particular contents on entry);
+//   kernel 2: every CTA first reduces the slots, a warp per tensor, derives the scales and casts its chunks; CTA 0 writes amax, scale and scale_inv.
+// GIVEN (delayed / static) scales: a reset kernel, then kernel 2 with the scales read and one atomicMax per CTA and tensor.
 struct QBatch {
   QTensor t[TWEO_MAX_QUANT_BATCH];
   int32_t count;
-  int32_t amax_grid;  // CTAs of kernel 1 = slots per tensor
+  int32_t amax_grid;                              // CTAs of kernel 1 = slots per tensor
+  uint32_t chunk_start[TWEO_MAX_QUANT_BATCH + 1];  // first chunk of a tensor; of those beyond the last: their total
 };
 constexpr int kMaxAmaxGrid = 2048;  // slots per tensor in the workspace
+constexpr int kChunk = 8192;
+constexpr int kFlatCtasPerSm = 4;
 
-__device__ __forceinline__ uint32_t cta_max(uint32_t m, uint32_t* part) {
+__device__ __forceinline__ int chunk_tensor(const QBatch& b, uint32_t chunk) {
+  int ti = 0;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-  __syncthreads();  // part[] may still be read from the previous use
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = m;
+  for (int i = 1; i < TWEO_MAX_QUANT_BATCH; ++i) ti = chunk >= b.chunk_start[i] ? i : ti;
+  return ti;
+}
+
+// A warp's maximum (a bf16 pattern) into the CTA's, per tensor.
+__device__ __forceinline__ void fold_max(float& m0, float& m1, uint32_t* cta) {
+  const uint32_t m = __reduce_max_sync(0xFFFFFFFFu, absmax_f32_bits(m0, m1));
+  if ((threadIdx.x & 31) == 0 && m) atomicMax(cta, m);
+  m0 = m1 = 0.0f;
+}
+
+__global__ void __launch_bounds__(kThreads, kFlatCtasPerSm) amax_batch_kernel(const __grid_constant__ QBatch b, uint32_t* slots) {
+  __shared__ uint32_t most[TWEO_MAX_QUANT_BATCH];
+  chain_release();
+  if (threadIdx.x < TWEO_MAX_QUANT_BATCH) most[threadIdx.x] = 0u;
   __syncthreads();
-#pragma unroll
-  for (int w = 0; w < kThreads / 32; ++w) m = max(m, part[w]);
-  return m;
-}
-
-// U: 16-byte loads in flight per thread.  Large batches take the deeper variant (more bytes in flight per SM);
-// small ones the shallow one, whose smaller per-CTA share keeps all SMs busy to the end.
-template <int U>
-__global__ void __launch_bounds__(kThreads) amax_batch_kernel(const __grid_constant__ QBatch b, uint32_t* slots) {
-  __shared__ uint32_t part[kThreads / 32];
-  chain_release();
   chain_wait();
-#pragma unroll 1
-  for (int ti = 0; ti < b.count; ++ti) {
-    const int64_t n = b.t[ti].n;
-    const int64_t nvec = n >> 3;
-    const uint16_t* x = b.t[ti].x;
-    const uint4* xv = reinterpret_cast<const uint4*>(x);
-    const int64_t stride = (int64_t)gridDim.x * kThreads * U;
-    float m0 = 0.0f, m1 = 0.0f;
-    for (int64_t base = (int64_t)blockIdx.x * kThreads * U + threadIdx.x; base < nvec; base += stride) {
-      uint4 v[U];
+  const uint32_t total = b.chunk_start[TWEO_MAX_QUANT_BATCH];
+  uint4 v[4];
+  auto load = [&](uint32_t chunk) {
+    const int ti = chunk_tensor(b, chunk);
+    const int64_t at = (int64_t)(chunk - b.chunk_start[ti]) * (kChunk / 8) + threadIdx.x, nvec = b.t[ti].n >> 3;
+    const uint4* xv = reinterpret_cast<const uint4*>(b.t[ti].x);
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        int64_t i = base + (int64_t)u * kThreads;
-        v[u] = i < nvec ? __ldg(xv + i) : make_uint4(0, 0, 0, 0);
-      }
+    for (int u = 0; u < 4; ++u) v[u] = at + u * kThreads < nvec ? __ldg(xv + at + u * kThreads) : make_uint4(0u, 0u, 0u, 0u);
+  };
+  float m0 = 0.0f, m1 = 0.0f;
+  int ti = 0;
+  if (blockIdx.x < total) load(blockIdx.x);
+  for (uint32_t chunk = blockIdx.x; chunk < total; chunk += gridDim.x) {
+    const uint4 w[4] = {v[0], v[1], v[2], v[3]};
+    const int now = chunk_tensor(b, chunk);
+    if (chunk + gridDim.x < total) load(chunk + gridDim.x);
+    if (now != ti) fold_max(m0, m1, most + ti);
+    ti = now;
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        absmax_f32(m0, m1, v[u].x);
-        absmax_f32(m0, m1, v[u].y);
-        absmax_f32(m0, m1, v[u].z);
-        absmax_f32(m0, m1, v[u].w);
-      }
+    for (int u = 0; u < 4; ++u) {
+      absmax_f32(m0, m1, w[u].x);
+      absmax_f32(m0, m1, w[u].y);
+      absmax_f32(m0, m1, w[u].z);
+      absmax_f32(m0, m1, w[u].w);
     }
-    if (blockIdx.x == 0 && threadIdx.x < 8) {
-      int64_t i = (nvec << 3) + threadIdx.x;
-      if (i < n) absmax_f32(m0, m1, (uint32_t)x[i]);
-    }
-    const uint32_t m = cta_max(absmax_f32_bits(m0, m1), part);
-    if (threadIdx.x == 0) slots[ti * kMaxAmaxGrid + blockIdx.x] = m;
   }
+  fold_max(m0, m1, most + ti);
+  if (blockIdx.x == 0 && threadIdx.x < 8 * TWEO_MAX_QUANT_BATCH) {   // ragged tails: n % 8 elements
+    const int k = threadIdx.x >> 3;
+    const int64_t i = (k < b.count ? b.t[k].n >> 3 << 3 : 0) + (threadIdx.x & 7);
+    if (k < b.count && i < b.t[k].n) {
+      absmax_f32(m0, m1, (uint32_t)b.t[k].x[i]);
+      atomicMax(most + k, absmax_f32_bits(m0, m1));
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < b.count) slots[threadIdx.x * kMaxAmaxGrid + blockIdx.x] = most[threadIdx.x];
 }
 
-// U: pairs of 16-byte loads in flight per thread (see amax_batch_kernel)
-template <int FMT, int U>
-__global__ void __launch_bounds__(kThreads) cast_batch_kernel(const __grid_constant__ QBatch b, const uint32_t* slots) {
-  __shared__ uint32_t part[kThreads / 32];
+template <bool GIVEN>
+__global__ void __launch_bounds__(kThreads, kFlatCtasPerSm) cast_batch_kernel(const __grid_constant__ QBatch b, const uint32_t* slots) {
+  __shared__ float scales[TWEO_MAX_QUANT_BATCH];
+  __shared__ uint32_t most[TWEO_MAX_QUANT_BATCH];
+  static_assert(TWEO_MAX_QUANT_BATCH <= kThreads / 32, "a warp per tensor");
   chain_release();
   chain_wait();
-#pragma unroll 1
-  for (int ti = 0; ti < b.count; ++ti) {
-    if (b.t[ti].fmt != FMT) continue;
-    uint32_t m = 0;
-    for (int k = threadIdx.x; k < b.amax_grid; k += kThreads) m = max(m, __ldcg(slots + ti * kMaxAmaxGrid + k));
-    m = cta_max(m, part);
-    const float amax = __uint_as_float(m << 16);  // non-negative bf16 pattern -> binary32
-    const float s = scale_from_amax(amax, FMT);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-      *b.t[ti].amax = amax;
-      *b.t[ti].scale = s;
-      *b.t[ti].scale_inv = __fdiv_rn(1.0f, s);
-    }
-    const int64_t n = b.t[ti].n;
-    const int64_t n16 = n >> 4;
-    const uint16_t* x = b.t[ti].x;
-    uint8_t* q = b.t[ti].q;
-    const uint4* xv = reinterpret_cast<const uint4*>(x);
-    uint4* qv = reinterpret_cast<uint4*>(q);
-    const int64_t stride = (int64_t)gridDim.x * kThreads * U;
-    uint32_t sat = 0;
-    float mm0 = 0.0f, mm1 = 0.0f;
-    for (int64_t base = (int64_t)blockIdx.x * kThreads * U + threadIdx.x; base < n16; base += stride) {
-      uint4 v[U][2];
+  const uint32_t total = b.chunk_start[TWEO_MAX_QUANT_BATCH];
+  uint4 v[2][2];
+  auto load = [&](uint32_t chunk) {
+    const int ti = chunk_tensor(b, chunk);
+    const int64_t at = (int64_t)(chunk - b.chunk_start[ti]) * (kChunk / 16) + threadIdx.x, n16 = b.t[ti].n >> 4;
+    const uint4* xv = reinterpret_cast<const uint4*>(b.t[ti].x);
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        int64_t i = base + (int64_t)u * kThreads;
-        if (i < n16) {
-          v[u][0] = __ldcs(xv + 2 * i);
-          v[u][1] = __ldcs(xv + 2 * i + 1);
+    for (int u = 0; u < 2; ++u) {
+      const bool in = at + u * kThreads < n16;
+      v[u][0] = in ? __ldcs(xv + 2 * (at + u * kThreads)) : make_uint4(0u, 0u, 0u, 0u);
+      v[u][1] = in ? __ldcs(xv + 2 * (at + u * kThreads) + 1) : make_uint4(0u, 0u, 0u, 0u);
+    }
+  };
+  if (blockIdx.x < total) load(blockIdx.x);   // the first loads do not wait for the scales
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (warp < b.count) {
+    if (GIVEN) {
+      if (lane == 0) {
+        scales[warp] = *b.t[warp].scale;
+        most[warp] = 0u;
+      }
+    } else {
+      uint32_t m = 0;
+      for (int k0 = lane; k0 < b.amax_grid; k0 += 32 * 8) {
+        uint32_t w[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) w[k] = k0 + 32 * k < b.amax_grid ? __ldcg(slots + warp * kMaxAmaxGrid + k0 + 32 * k) : 0u;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) m = max(m, w[k]);
+      }
+      m = __reduce_max_sync(0xFFFFFFFFu, m);
+      if (lane == 0) {
+        const float amax = __uint_as_float(m << 16);  // non-negative bf16 pattern -> binary32
+        const float s = scale_from_amax(amax, b.t[warp].fmt);
+        scales[warp] = s;
+        if (blockIdx.x == 0) {
+          *b.t[warp].amax = amax;
+          *b.t[warp].scale = s;
+          *b.t[warp].scale_inv = __fdiv_rn(1.0f, s);
         }
       }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        int64_t i = base + (int64_t)u * kThreads;
-        if (i < n16) __stcs(qv + i, cast16<FMT, false, false>(v[u][0], v[u][1], s, sat, mm0, mm1));
-      }
     }
-    if (blockIdx.x == 0 && threadIdx.x < 16) {  // ragged tail: n % 16 elements
-      int64_t i = (n16 << 4) + threadIdx.x;
-      if (i < n) {
-        float v = __fmul_rn(bf16lo_to_f32((uint32_t)x[i]), s);
-        q[i] = (uint8_t)(cvt_fp8x2<FMT>(v, 0.0f) & 0xFFu);
+  }
+  __syncthreads();
+  float m0 = 0.0f, m1 = 0.0f;
+  int ti = 0;
+  for (uint32_t chunk = blockIdx.x; chunk < total; chunk += gridDim.x) {
+    const int now = chunk_tensor(b, chunk);
+    if (GIVEN && now != ti) fold_max(m0, m1, most + ti);
+    ti = now;
+    const uint4 w[2][2] = {{v[0][0], v[0][1]}, {v[1][0], v[1][1]}};
+    if (chunk + gridDim.x < total) load(chunk + gridDim.x);
+    const int64_t at = (int64_t)(chunk - b.chunk_start[ti]) * (kChunk / 16) + threadIdx.x, n16 = b.t[ti].n >> 4;
+    uint4* qv = reinterpret_cast<uint4*>(b.t[ti].q);
+    const float s = scales[ti];
+    uint32_t sat = 0;
+    uint4 c[2];
+    if (b.t[ti].fmt == TWEO_E4M3) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u) c[u] = cast16<TWEO_E4M3, false, GIVEN>(w[u][0], w[u][1], s, sat, m0, m1);
+    } else {
+#pragma unroll
+      for (int u = 0; u < 2; ++u) c[u] = cast16<TWEO_E5M2, false, GIVEN>(w[u][0], w[u][1], s, sat, m0, m1);
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+      if (at + u * kThreads < n16) __stcs(qv + at + u * kThreads, c[u]);
+  }
+  if (GIVEN) fold_max(m0, m1, most + ti);
+  if (blockIdx.x == 0 && threadIdx.x < 16 * TWEO_MAX_QUANT_BATCH) {  // ragged tails: n % 16 elements
+    const int k = threadIdx.x >> 4;
+    const int64_t i = (k < b.count ? b.t[k].n >> 4 << 4 : 0) + (threadIdx.x & 15);
+    if (k < b.count && i < b.t[k].n) {
+      const uint32_t w = b.t[k].x[i];
+      const float p = __fmul_rn(bf16lo_to_f32(w), scales[k]);
+      b.t[k].q[i] = (uint8_t)((b.t[k].fmt == TWEO_E4M3 ? cvt_fp8x2<TWEO_E4M3>(p, 0.0f) : cvt_fp8x2<TWEO_E5M2>(p, 0.0f)) & 0xFFu);
+      if (GIVEN) {
+        absmax_f32(m0, m1, w);
+        atomicMax(most + k, absmax_f32_bits(m0, m1));
       }
     }
   }
+  if (GIVEN) {
+    __syncthreads();
+    if (threadIdx.x < b.count && most[threadIdx.x])   // non-negative binary32 values order like their bit patterns
+      atomicMax(reinterpret_cast<unsigned int*>(b.t[threadIdx.x].amax), most[threadIdx.x] << 16);
+  }
 }
 
-// Batched form for GIVEN (delayed / static) scales: one reset kernel for all tensors of the batch, then one
-// single-pass cast kernel per FP8 format present; every CTA folds its share of a tensor into that tensor's amax
-// with one atomicMax.  Three launches for a linear's (or two linears') tensors instead of two per tensor.
+// GIVEN scales: amax to zero, the reciprocals.
 __global__ void init_batch_kernel(const __grid_constant__ QBatch b) {
   chain_release();
   chain_wait();
@@ -313,67 +364,23 @@ __global__ void init_batch_kernel(const __grid_constant__ QBatch b) {
   }
 }
 
-template <int FMT, int U>
-__global__ void __launch_bounds__(kThreads) cast_given_batch_kernel(const __grid_constant__ QBatch b) {
-  chain_release();
-  chain_wait();
-#pragma unroll 1
-  for (int ti = 0; ti < b.count; ++ti) {
-    if (b.t[ti].fmt != FMT) continue;
-    const float s = *b.t[ti].scale;
-    const int64_t n = b.t[ti].n;
-    const int64_t n16 = n >> 4;
-    const uint16_t* x = b.t[ti].x;
-    uint8_t* q = b.t[ti].q;
-    const uint4* xv = reinterpret_cast<const uint4*>(x);
-    uint4* qv = reinterpret_cast<uint4*>(q);
-    const int64_t stride = (int64_t)gridDim.x * kThreads * U;
-    uint32_t sat = 0;
-    float m0 = 0.0f, m1 = 0.0f;
-    for (int64_t base = (int64_t)blockIdx.x * kThreads * U + threadIdx.x; base < n16; base += stride) {
-      uint4 v[U][2];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        int64_t i = base + (int64_t)u * kThreads;
-        if (i < n16) {
-          v[u][0] = __ldcs(xv + 2 * i);
-          v[u][1] = __ldcs(xv + 2 * i + 1);
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        int64_t i = base + (int64_t)u * kThreads;
-        if (i < n16) __stcs(qv + i, cast16<FMT, false, true>(v[u][0], v[u][1], s, sat, m0, m1));
-      }
-    }
-    if (blockIdx.x == 0 && threadIdx.x < 16) {  // ragged tail: n % 16 elements
-      int64_t i = (n16 << 4) + threadIdx.x;
-      if (i < n) {
-        const uint32_t w = x[i];
-        q[i] = (uint8_t)(cvt_fp8x2<FMT>(__fmul_rn(bf16lo_to_f32(w), s), 0.0f) & 0xFFu);
-        absmax_f32(m0, m1, w);
-      }
-    }
-    __syncthreads();  // the reduction's shared array may still be read from the previous tensor
-    cta_amax_to_global(absmax_f32_bits(m0, m1), b.t[ti].amax);
-  }
-}
-
 // ---------------------------------------------------------------------------------------
-// Small tensors, either kind of scale, up to TWEO_MAX_QUANT_BATCH in ONE launch and without a workspace: a cluster of
-// eight CTAs per tensor, which write their maxima into each other's shared memory.  At these sizes the launches are the cost
-// (2 to 4 us each in a chain, two to four of them in the other forms), not the bytes: eight SMs read a tensor twice, the
-// second time from L1 or L2.
-constexpr int kSmallCluster = 8;
+// Small tensors, either kind of scale, up to TWEO_MAX_QUANT_BATCH in ONE launch and without a workspace: a cluster of eight or sixteen CTAs per
+// tensor, which write their maxima into each other's shared memory.  At these sizes the launches are the cost (2 to 4 us each in a chain,
+// two to four of them in the other forms), not the bytes: a few SMs read a tensor twice, the second time from L1 or L2.
+// Beyond 2^17 elements what an SM takes in bounds it, hence sixteen: three tensors of 2^20, current scaling, 10.0 -> 6.5 us, 2^18 4.3 -> 3.4
+// (with eight CTAs of twice the threads and loads 8.9 and 5.1).
 constexpr int kSmallThreads = 512;
+constexpr int64_t kSmallShort = 1 << 17;   // tensors of up to this many elements are cast by eight CTAs each, longer ones by sixteen
 
-template <int FMT, bool AMAX>
+// C: CTAs per tensor.
+template <int FMT, bool AMAX, int C>
 __device__ __forceinline__ void small_cast_share(const QTensor& t, float s, int rank, float& m0, float& m1) {
   const int64_t n16 = t.n >> 4;
   const uint4* xv = reinterpret_cast<const uint4*>(t.x);
   uint4* qv = reinterpret_cast<uint4*>(t.q);
   uint32_t sat = 0;
-  constexpr int stride = kSmallCluster * kSmallThreads;
+  constexpr int stride = C * kSmallThreads;
   for (int64_t i = rank * kSmallThreads + threadIdx.x; i < n16; i += 2 * stride) {
     const int64_t j = i + stride;
     const uint4 a0 = __ldg(xv + 2 * i), b0 = __ldg(xv + 2 * i + 1);
@@ -395,28 +402,29 @@ __device__ __forceinline__ void small_cast_share(const QTensor& t, float s, int 
   }
 }
 
+template <int C>
 __global__ void __launch_bounds__(kSmallThreads) small_cast_kernel(const __grid_constant__ QBatch b) {
   namespace cg = cooperative_groups;
   __shared__ uint32_t part[kSmallThreads / 32];
-  __shared__ uint32_t maxima[kSmallCluster];   // one per CTA of the cluster, written by it
+  __shared__ uint32_t maxima[C];   // one per CTA of the cluster, written by it
   cg::cluster_group cluster = cg::this_cluster();
   cluster.barrier_arrive();   // this CTA has started: its peers may write into its maxima[]
   chain_wait();
   chain_release();   // in this order the kernels behind do not crowd in early (train step of a small linear: 21.5 -> 20.2 us)
-  const int ti = blockIdx.x / kSmallCluster;
-  const int rank = blockIdx.x - ti * kSmallCluster;
+  const int ti = blockIdx.x / C;
+  const int rank = blockIdx.x - ti * C;
   const QTensor& t = b.t[ti];
   const bool given = t.mode == TWEO_SCALE_GIVEN;   // uniform over the cluster
   float m0 = 0.0f, m1 = 0.0f;
   float s = 1.0f;
   if (given) {
     s = *t.scale;
-    if (t.fmt == TWEO_E4M3) small_cast_share<TWEO_E4M3, true>(t, s, rank, m0, m1);
-    else small_cast_share<TWEO_E5M2, true>(t, s, rank, m0, m1);
+    if (t.fmt == TWEO_E4M3) small_cast_share<TWEO_E4M3, true, C>(t, s, rank, m0, m1);
+    else small_cast_share<TWEO_E5M2, true, C>(t, s, rank, m0, m1);
   } else {
     const int64_t n16 = t.n >> 4;
     const uint4* xv = reinterpret_cast<const uint4*>(t.x);
-    constexpr int stride = kSmallCluster * kSmallThreads;
+    constexpr int stride = C * kSmallThreads;
     for (int64_t i = rank * kSmallThreads + threadIdx.x; i < n16; i += 2 * stride) {
       const int64_t j = i + stride < n16 ? i + stride : i;
       const uint4 v[4] = {__ldg(xv + 2 * i), __ldg(xv + 2 * i + 1), __ldg(xv + 2 * j), __ldg(xv + 2 * j + 1)};
@@ -439,10 +447,10 @@ __global__ void __launch_bounds__(kSmallThreads) small_cast_kernel(const __grid_
   __syncthreads();
   if (threadIdx.x < 32) {
     m = __reduce_max_sync(0xFFFFFFFFu, threadIdx.x < kSmallThreads / 32 ? part[threadIdx.x] : 0u);
-    if (threadIdx.x < kSmallCluster) *cluster.map_shared_rank(&maxima[rank], threadIdx.x) = m;
+    if (threadIdx.x < C) *cluster.map_shared_rank(&maxima[rank], threadIdx.x) = m;
   }
   cluster.sync();   // all maxima are there; nobody reaches into another CTA after this
-  m = __reduce_max_sync(0xFFFFFFFFu, (threadIdx.x & 31) < kSmallCluster ? maxima[threadIdx.x & 31] : 0u);
+  m = __reduce_max_sync(0xFFFFFFFFu, (threadIdx.x & 31) < C ? maxima[threadIdx.x & 31] : 0u);
   const float amax = __uint_as_float(m << 16);   // non-negative bf16 pattern -> binary32
   if (!given) s = scale_from_amax(amax, t.fmt);
   if (rank == 0 && threadIdx.x == 0) {
@@ -451,23 +459,25 @@ __global__ void __launch_bounds__(kSmallThreads) small_cast_kernel(const __grid_
     *t.scale_inv = __fdiv_rn(1.0f, s);
   }
   if (!given) {
-    if (t.fmt == TWEO_E4M3) small_cast_share<TWEO_E4M3, false>(t, s, rank, m0, m1);
-    else small_cast_share<TWEO_E5M2, false>(t, s, rank, m0, m1);
+    if (t.fmt == TWEO_E4M3) small_cast_share<TWEO_E4M3, false, C>(t, s, rank, m0, m1);
+    else small_cast_share<TWEO_E5M2, false, C>(t, s, rank, m0, m1);
   }
 }
 
 int grid_for(int64_t work_items, int per_cta, int ctas_per_sm);
 
-// Where one cluster per tensor is no slower than the other forms.  Microseconds per call replayed from a graph, this form /
-// the others (all tensors in one format; in parentheses: in both):
-//   one, given       2^10 1.8 / 2.2   2^14 2.1 / 2.3   2^17 2.35 / 2.40  2^19 4.2 / 2.4
-//   one, current     2^10 2.2 / 2.9   2^14 2.6 / 3.3   2^17 2.9 / 3.5    2^19 6.0 / 3.6
-//   two, given       2^16 2.1 / 3.5   2^18 3.1 / 3.7   2^19 4.3 / 3.9 (4.3 / 5.1)   2^20 6.2 / 4.9 (6.2 / 6.1)
-//   three, given     2^16 2.2 / 4.6   2^19 4.3 / 5.5   2^20 6.3 / 6.2 (6.4 / 7.6)
-//   four, given      2^16 2.3 / 5.4   2^19 4.2 / 7.2   2^20 6.4 / 9.1
-//   two, current     2^16 2.7 / 5.1   2^19 6.0 / 6.2   2^20 9.7 / 8.4
-//   three, current   2^16 2.7 / 6.8   2^19 6.0 / 10.2  2^20 9.7 / 14.0   2^21 17 / 16
-// Issued call by call the one launch also saves its host the others, 2 us each.
+// Up to which sizes a call is one launch.  Microseconds per call replayed from a graph, this form / the others with a workspace (all tensors in
+// one format; in parentheses: in both):
+//   one, given       2^14 2.2 / 2.2   2^17 2.7 / 2.6
+//   one, current     2^14 2.7 / 3.4   2^17 3.2 / 3.6
+//   two, given       2^17 2.6 / 3.1   2^18 2.8 / 3.1   (2^19 3.4 / 4.7)
+//   three, given     2^17 2.7 / 3.1   2^19 3.3 / 3.1   (2^20 4.6 / 5.9)
+//   four, given      2^17 2.8 / 3.2   2^20 4.7 / 4.3
+//   two, current     2^17 3.2 / 3.6   2^19 4.5 / 4.4
+//   three, current   2^17 3.2 / 3.6   2^19 4.4 / 4.5   2^20 6.5 / 5.1
+//   six, current     2^17 3.2 / 4.0   2^20 6.5 / 7.3
+// Issued call by call the one launch also saves its host the others, 2 us each; without a workspace the other form is three launches for every
+// tensor with current scaling.
 int64_t small_limit(const tweo_quant_desc_t* descs, int count) {
   if (count == 1) return 1 << 17;
   bool given = true, both = false;
@@ -493,86 +503,61 @@ tweo_status_t launch_small(const tweo_quant_desc_t* descs, int count, cudaStream
     const tweo_quant_desc_t& d = descs[i];
     b.t[i] = QTensor{d.x, d.q, d.n, d.scale, d.scale_inv, d.amax, d.fmt, d.mode};
   }
-  TWEO_CUDA_TRY(launch_chain(small_cast_kernel, dim3((unsigned)(kSmallCluster * count)), dim3(kSmallThreads), 0, st, kSmallCluster, b));
+  int64_t most = 0;
+  for (int i = 0; i < count; ++i) most = std::max(most, descs[i].n);
+  if (most <= kSmallShort) {
+    TWEO_CUDA_TRY(launch_chain(small_cast_kernel<8>, dim3((unsigned)(8 * count)), dim3(kSmallThreads), 0, st, 8, b));
+  } else {
+    static std::atomic<uint64_t> attr_done{0};  // per device
+    int attr_dev = 0;
+    if (device_once_pending(attr_done, &attr_dev)) {
+      TWEO_CUDA_TRY(cudaFuncSetAttribute(small_cast_kernel<16>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+      device_once_done(attr_done, attr_dev);
+    }
+    TWEO_CUDA_TRY(launch_chain(small_cast_kernel<16>, dim3((unsigned)(16 * count)), dim3(kSmallThreads), 0, st, 16, b));
+  }
   count_launch();
   return check_launch("small_cast_kernel");
 }
 
-// Launches the batched form for descs[idx[0..count)] (all CURRENT scaling, no saturation count).
-tweo_status_t launch_batch(const tweo_quant_desc_t* descs, const int* idx, int count, void* ws, cudaStream_t st) {
+QBatch make_batch(const tweo_quant_desc_t* descs, const int* idx, int count) {
   QBatch b;
   b.count = count;
-  int64_t vec8 = 0, vec16[2] = {0, 0};
-  for (int i = 0; i < count; ++i) {
+  b.amax_grid = 0;
+  uint32_t at = 0;
+  for (int i = 0; i <= TWEO_MAX_QUANT_BATCH; ++i) {
+    b.chunk_start[i] = at;
+    if (i >= count) continue;
     const tweo_quant_desc_t& d = descs[idx[i]];
     b.t[i] = QTensor{d.x, d.q, d.n, d.scale, d.scale_inv, d.amax, d.fmt, d.mode};
-    vec8 += d.n >> 3;
-    vec16[d.fmt] += d.n >> 4;
+    at += (uint32_t)((d.n + kChunk - 1) / kChunk);
   }
-  // the deeper variants once a launch has at least two full sweeps of the capped grid at their depth
-  const int64_t sweep = (int64_t)sm_count() * 8 * kThreads;
-  const bool deep_amax = vec8 >= 2 * sweep * 8;
-  b.amax_grid = grid_for(vec8, kThreads * (deep_amax ? 8 : 4), 8);
-  if (b.amax_grid > kMaxAmaxGrid) b.amax_grid = kMaxAmaxGrid;
+  return b;
+}
+
+// Launches the batched form for descs[idx[0..count)] (all CURRENT scaling, no saturation count).
+tweo_status_t launch_batch(const tweo_quant_desc_t* descs, const int* idx, int count, void* ws, cudaStream_t st) {
+  QBatch b = make_batch(descs, idx, count);
+  b.amax_grid = std::min(kMaxAmaxGrid, balanced_grid(b.chunk_start[TWEO_MAX_QUANT_BATCH], (int64_t)sm_count() * kFlatCtasPerSm));
   uint32_t* slots = reinterpret_cast<uint32_t*>(ws);
-  if (deep_amax) TWEO_CUDA_TRY(launch_chain(amax_batch_kernel<8>, dim3(b.amax_grid), dim3(kThreads), 0, st, 0, b, slots));
-  else TWEO_CUDA_TRY(launch_chain(amax_batch_kernel<4>, dim3(b.amax_grid), dim3(kThreads), 0, st, 0, b, slots));
-  count_launch();
-  bool has[2] = {false, false};
-  for (int i = 0; i < count; ++i) has[b.t[i].fmt] = true;
-  if (has[TWEO_E4M3]) {
-    if (vec16[TWEO_E4M3] >= 2 * sweep * 4)
-      TWEO_CUDA_TRY(launch_chain(cast_batch_kernel<TWEO_E4M3, 4>, dim3(grid_for(vec16[TWEO_E4M3], kThreads * 4, 8)), dim3(kThreads), 0, st, 0, b,
-                                 (const uint32_t*)slots));
-    else
-      TWEO_CUDA_TRY(launch_chain(cast_batch_kernel<TWEO_E4M3, 2>, dim3(grid_for(vec16[TWEO_E4M3], kThreads * 2, 8)), dim3(kThreads), 0, st, 0, b,
-                                 (const uint32_t*)slots));
-    count_launch();
-  }
-  if (has[TWEO_E5M2]) {
-    if (vec16[TWEO_E5M2] >= 2 * sweep * 4)
-      TWEO_CUDA_TRY(launch_chain(cast_batch_kernel<TWEO_E5M2, 4>, dim3(grid_for(vec16[TWEO_E5M2], kThreads * 4, 8)), dim3(kThreads), 0, st, 0, b,
-                                 (const uint32_t*)slots));
-    else
-      TWEO_CUDA_TRY(launch_chain(cast_batch_kernel<TWEO_E5M2, 2>, dim3(grid_for(vec16[TWEO_E5M2], kThreads * 2, 8)), dim3(kThreads), 0, st, 0, b,
-                                 (const uint32_t*)slots));
-    count_launch();
-  }
+  TWEO_CUDA_TRY(launch_chain(amax_batch_kernel, dim3(b.amax_grid), dim3(kThreads), 0, st, 0, b, slots));
+  TWEO_CUDA_TRY(launch_chain(cast_batch_kernel<false>, dim3(b.amax_grid), dim3(kThreads), 0, st, 0, b, (const uint32_t*)slots));
+  count_launch(2);
   return check_launch("quantize batch kernels");
 }
 
 // Launches the given-scale batched form for descs[idx[0..count)] (no saturation count).
 tweo_status_t launch_given_batch(const tweo_quant_desc_t* descs, const int* idx, int count, cudaStream_t st) {
-  QBatch b;
-  b.count = count;
-  b.amax_grid = 0;
-  int64_t vec16[2] = {0, 0};
-  for (int i = 0; i < count; ++i) {
-    const tweo_quant_desc_t& d = descs[idx[i]];
-    b.t[i] = QTensor{d.x, d.q, d.n, d.scale, d.scale_inv, d.amax, d.fmt, d.mode};
-    vec16[d.fmt] += d.n >> 4;
-  }
-  TWEO_CUDA_TRY(launch_chain(init_batch_kernel, dim3(1), dim3(32), 0, st, 0, b));
+  TWEO_CUDA_TRY(launch_chain(init_batch_kernel, dim3(1), dim3(32), 0, st, 0, make_batch(descs, idx, count)));
   count_launch();
-  const int64_t sweep = (int64_t)sm_count() * 8 * kThreads;
-  bool has[2] = {false, false};
-  for (int i = 0; i < count; ++i) has[b.t[i].fmt] = true;
-  if (has[TWEO_E4M3]) {
-    if (vec16[TWEO_E4M3] >= 2 * sweep * 4)
-      TWEO_CUDA_TRY(launch_chain(cast_given_batch_kernel<TWEO_E4M3, 4>, dim3(grid_for(vec16[TWEO_E4M3], kThreads * 4, 8)),
-                                 dim3(kThreads), 0, st, 0, b));
-    else
-      TWEO_CUDA_TRY(launch_chain(cast_given_batch_kernel<TWEO_E4M3, 2>, dim3(grid_for(vec16[TWEO_E4M3], kThreads * 2, 8)),
-                                 dim3(kThreads), 0, st, 0, b));
-    count_launch();
-  }
-  if (has[TWEO_E5M2]) {
-    if (vec16[TWEO_E5M2] >= 2 * sweep * 4)
-      TWEO_CUDA_TRY(launch_chain(cast_given_batch_kernel<TWEO_E5M2, 4>, dim3(grid_for(vec16[TWEO_E5M2], kThreads * 4, 8)),
-                                 dim3(kThreads), 0, st, 0, b));
-    else
-      TWEO_CUDA_TRY(launch_chain(cast_given_batch_kernel<TWEO_E5M2, 2>, dim3(grid_for(vec16[TWEO_E5M2], kThreads * 2, 8)),
-                                 dim3(kThreads), 0, st, 0, b));
+  for (int fmt : {TWEO_E4M3, TWEO_E5M2}) {   // one kernel per format present
+    int of[TWEO_MAX_QUANT_BATCH], n = 0;
+    for (int i = 0; i < count; ++i)
+      if (descs[idx[i]].fmt == fmt) of[n++] = idx[i];
+    if (n == 0) continue;
+    const QBatch b = make_batch(descs, of, n);
+    const int grid = balanced_grid(b.chunk_start[TWEO_MAX_QUANT_BATCH], (int64_t)sm_count() * kFlatCtasPerSm);
+    TWEO_CUDA_TRY(launch_chain(cast_batch_kernel<true>, dim3(grid), dim3(kThreads), 0, st, 0, b, (const uint32_t*)nullptr));
     count_launch();
   }
   return check_launch("quantize given-scale batch kernels");
@@ -623,8 +608,8 @@ tweo_status_t quantize_many(const tweo_quant_desc_t* descs, int count, void* ws,
     tweo_status_t s = check_quant_desc(descs[i]);
     if (s != TWEO_OK) return s;
   }
-  if (all_small(descs, count)) return launch_small(descs, count, st);
   const bool have_ws = ws && ws_bytes >= kBatchWsBytes && aligned16(ws);
+  if (all_small(descs, count)) return launch_small(descs, count, st);
   int idx[TWEO_MAX_QUANT_BATCH], idxg[TWEO_MAX_QUANT_BATCH];
   int nb = 0, ng = 0;
   for (int i = 0; i < count; ++i) {
