@@ -820,8 +820,8 @@ SkinnyPlan plan_skinny(int64_t M, int64_t N, int k_blocks) {
   return pl;
 }
 
-// Estimate for the CTA-pair kernel on whole tiles: 630 clocks per k-block of a 256 x 256 tile, 5000 for
-// set-up, the first tile's loads and the last tile's epilogue (fitted to the measurements below skinny_pays).
+// Estimate for the CTA-pair kernel on whole tiles as it was before narrower tiles and its present issue loop: 630 clocks per k-block of a
+// 256 x 256 tile, 5000 for set-up, the first tile's loads and the last tile's epilogue (fitted to the measurements below skinny_pays).
 double pair_clocks(int64_t M, int64_t N, int k_blocks) {
   const int64_t tiles = ((M + 255) / 256) * ((N + 255) / 256), pairs = sm_count() / 2;
   return (double)((tiles + pairs - 1) / pairs) * k_blocks * 630.0 + 5000.0;
